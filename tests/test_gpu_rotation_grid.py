@@ -50,5 +50,8 @@ def test_initialisation_and_steps(n, extra, hub):
         rp.step(10)
         assert np.array_equal(rp.params(), a)     # the same steps in one launch
     a_o, _ = G.adam(G.six_d_from_rot(R0), ci, cj, Rrel, 10, lr)
-    assert np.abs(a - a_o).max() < 1e-3 * lr
+    if len(ci) >= n:     # without a cycle every distance is 0 and the geodesic gradient undefined
+        assert np.abs(a - a_o).max() < 1e-3 * lr
+    else:
+        assert np.abs(a - G.six_d_from_rot(R0)).max() <= 10.01 * lr
     np.testing.assert_allclose(R, G.rot_from_6d(a), atol=1e-13)
