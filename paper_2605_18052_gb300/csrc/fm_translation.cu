@@ -4,17 +4,20 @@
 // by Adam from random initial centres, several runs at once, and the merge of the runs
 // (centre, unit mean norm, per camera the run with the lowest mean pair loss).
 //
-// Per iteration two launches, chained with programmatic dependent launch:
+// An evaluation is three launches, chained with programmatic dependent launch:
 //   k_tr_pair  (pair, run)   : the pair's L1 term and its subgradient with respect to
 //                              u = o_j - o_i, projected orthogonally to u and divided by |u|
 //   k_tr_cam   (camera, run) : the camera's gradient gathered from its pairs (CSR of the pair
-//                              table, fixed order, no atomics), its mean pair loss, Adam
-// then one launch closes a chain (per-run loss total, step count). Centres and their update
-// are FP64; the per-pair arithmetic is FP32 on the FP64 difference o_j - o_i.
+//                              table, fixed order, no atomics) and its mean pair loss
+//   k_tr_finalize (run)      : the loss total
+// Adam iterations of all runs are one persistent kernel (k_tr_steps). Centres and their update are
+// FP64; the per-pair arithmetic is FP32 on the FP64 difference o_j - o_i.
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
 
+#include "fm_grid.cuh"
 #include "fm_walk.cuh"
 
 void fm_internal_set_error(const char *msg);
@@ -30,7 +33,7 @@ struct DevTrans {
     int n_cams, n_pairs, n_runs;
     const int *cam_i, *cam_j, *cam_off, *cam_ent;
     float4 *oij;             // per pair: o_{i->j} (xyz), 0
-    double *o;               // n_runs x n_cams x 3
+    double *o, *o2;          // n_runs x n_cams x 3, and the other buffer of the step kernel
     float *m, *v;            // Adam moments, same shape
     float4 *pterm;           // n_runs x n_pairs: gradient wrt u (xyz), L1 term
     float *cam_loss;         // n_runs x n_cams: mean L1 term of the camera's pairs
@@ -40,6 +43,7 @@ struct DevTrans {
     double *stats;           // n_runs x 4: mean (3), mean norm after centring
     double *hyper;           // lr, beta1, beta2, eps
     long long *step;
+    unsigned *grid_state;    // grid barriers of the step kernel
     unsigned *err;
 };
 
@@ -58,22 +62,13 @@ __global__ void k_tr_setup(DevTrans t, const double *R, const double *trel) {
 
 __device__ __forceinline__ float sgn(float x) { return x > 0.f ? 1.f : (x < 0.f ? -1.f : 0.f); }
 
-__global__ void __launch_bounds__(TR_THREADS) k_tr_pair(DevTrans t) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const int run = blockIdx.y;
-    const int i = n < t.n_pairs ? t.cam_i[n] : 0, j = n < t.n_pairs ? t.cam_j[n] : 0;
-    const float4 target = n < t.n_pairs ? t.oij[n] : make_float4(0.f, 0.f, 0.f, 0.f);
-    pdl_wait();     // centres of the previous step
-    pdl_trigger();
-    if (n >= t.n_pairs) return;
-    const double *oi = t.o + ((size_t)run * t.n_cams + i) * 3;
-    const double *oj = t.o + ((size_t)run * t.n_cams + j) * 3;
-    const float u[3] = {(float)(oj[0] - oi[0]), (float)(oj[1] - oi[1]), (float)(oj[2] - oi[2])};
+// L1 term of a pair from u = o_j - o_i (w) and its gradient with respect to u (xyz); false when u
+// has no direction
+__device__ __forceinline__ bool pair_term(const float *u, float4 target, float4 &out) {
     const float n2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
     if (!(n2 > 0.f) || !isfinite(n2)) {
-        atomicOr(t.err, ERR_DEGENERATE);
-        t.pterm[(size_t)run * t.n_pairs + n] = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
+        out = make_float4(0.f, 0.f, 0.f, 0.f);
+        return false;
     }
     const float nrm = sqrtf(n2);
     const float uh[3] = {u[0] / nrm, u[1] / nrm, u[2] / nrm};
@@ -81,19 +76,35 @@ __global__ void __launch_bounds__(TR_THREADS) k_tr_pair(DevTrans t) {
     const float term = fabsf(r[0]) + fabsf(r[1]) + fabsf(r[2]);
     const float s[3] = {sgn(r[0]), sgn(r[1]), sgn(r[2])};
     const float dot = uh[0] * s[0] + uh[1] * s[1] + uh[2] * s[2];
-    t.pterm[(size_t)run * t.n_pairs + n] =
-        make_float4((s[0] - uh[0] * dot) / nrm, (s[1] - uh[1] * dot) / nrm, (s[2] - uh[2] * dot) / nrm, term);
+    out = make_float4((s[0] - uh[0] * dot) / nrm, (s[1] - uh[1] * dot) / nrm, (s[2] - uh[2] * dot) / nrm, term);
+    return true;
 }
 
-// warp per camera; apply = 0 writes the gradient instead of stepping
-__global__ void __launch_bounds__(TR_CAMS * 32) k_tr_cam(DevTrans t, int it, int apply) {
+__global__ void __launch_bounds__(TR_THREADS) k_tr_pair(DevTrans t) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int run = blockIdx.y;
+    const int i = n < t.n_pairs ? t.cam_i[n] : 0, j = n < t.n_pairs ? t.cam_j[n] : 0;
+    const float4 target = n < t.n_pairs ? t.oij[n] : make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();     // the centres
+    pdl_trigger();
+    if (n >= t.n_pairs) return;
+    const double *oi = t.o + ((size_t)run * t.n_cams + i) * 3;
+    const double *oj = t.o + ((size_t)run * t.n_cams + j) * 3;
+    const float u[3] = {(float)(oj[0] - oi[0]), (float)(oj[1] - oi[1]), (float)(oj[2] - oi[2])};
+    float4 term;
+    if (!pair_term(u, target, term)) atomicOr(t.err, ERR_DEGENERATE);
+    t.pterm[(size_t)run * t.n_pairs + n] = term;
+}
+
+// warp per camera: gradient, mean pair loss, the block's share of the loss
+__global__ void __launch_bounds__(TR_CAMS * 32) k_tr_cam(DevTrans t) {
     __shared__ double s_loss[TR_CAMS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int run = blockIdx.y;
     const int k = blockIdx.x * TR_CAMS + warp;
     const int e_begin = k < t.n_cams ? t.cam_off[k] : 0;
     const int e_end = k < t.n_cams ? t.cam_off[k + 1] : 0;
-    pdl_wait();     // pair terms of this step
+    pdl_wait();     // pair terms of this evaluation
     pdl_trigger();
     float g[3] = {0.f, 0.f, 0.f}, tsum = 0.f, lsum = 0.f;
     for (int e = e_begin + lane; e < e_end; e += 32) {
@@ -121,24 +132,8 @@ __global__ void __launch_bounds__(TR_CAMS * 32) k_tr_cam(DevTrans t, int it, int
             const int cnt = e_end - e_begin;
             t.cam_loss[(size_t)run * t.n_cams + k] = cnt > 0 ? tsum / (float)cnt : 0.f;
             const double inv_b = 1.0 / (double)t.n_pairs;
-            if (!apply) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) t.grad[base + a] = (double)g[a] * inv_b;
-            } else {
-                const long long ts = *t.step + 1 + it;
-                const float lr = (float)t.hyper[0], b1 = (float)t.hyper[1], b2 = (float)t.hyper[2],
-                            eps = (float)t.hyper[3];
-                const float bc1 = 1.f - powf(b1, (float)ts), bc2 = 1.f - powf(b2, (float)ts);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const float ga = (float)((double)g[a] * inv_b);
-                    const float mo = b1 * t.m[base + a] + (1.f - b1) * ga;
-                    const float vo = b2 * t.v[base + a] + (1.f - b2) * ga * ga;
-                    t.m[base + a] = mo;
-                    t.v[base + a] = vo;
-                    t.o[base + a] -= (double)(lr * (mo / bc1) / (sqrtf(vo / bc2) + eps));
-                }
-            }
+            for (int a = 0; a < 3; ++a) t.grad[base + a] = (double)g[a] * inv_b;
         }
     }
     __syncthreads();
@@ -150,8 +145,136 @@ __global__ void __launch_bounds__(TR_CAMS * 32) k_tr_cam(DevTrans t, int it, int
     }
 }
 
-// per run: loss total (FP64, fixed order) / |P|; block 0 adds `count` to the step count
-__global__ void __launch_bounds__(TR_THREADS) k_tr_finalize(DevTrans t, int count) {
+// iters Adam iterations of every run in one cooperative launch, one grid barrier per iteration. An
+// item is 8 cameras (a warp each) x rc runs; a block owns item blockIdx.x (+ grid, ...). A camera's
+// lanes take its image pairs, whose directions and partners stay in registers, and evaluate the pair
+// terms of the rc runs from the centres of one of two buffers: both cameras of a pair evaluate it,
+// which costs less than a second phase with its barrier and per-pair traffic. Then a thread per
+// (camera, run, component) takes the Adam step and writes the centre to the other buffer. FP64 is
+// issued at 64 cycles a warp instruction per sub-partition on GB300, so the camera's sums are left in
+// different lanes and the update runs 32 components a warp instruction (one lane per camera for all
+// of it made the camera kernel 20 us at 1,000 cameras x 8 runs). Per (camera, run) six FP64
+// instructions remain, the differences of centres and their rounding to FP32: they bound an
+// iteration, 7.7 us there with the barrier, 23.5 us as two launches.
+constexpr int TR_RC = 8;       // most runs of an item
+constexpr int TR_BATCH = 4;    // runs whose loads are in flight together
+
+__global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int iters, int rc) {
+    __shared__ float s_g[TR_CAMS][TR_RC][3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int chunks = (t.n_runs + rc - 1) / rc, items = cam_blocks(t) * chunks;
+    const bool single = items <= gridDim.x;
+    GridBarrier gb(t.grid_state, t.err);
+    const long long t0 = *t.step;
+    const double inv_b = 1.0 / (double)t.n_pairs;
+    const float lr = (float)t.hyper[0], b1 = (float)t.hyper[1], b2 = (float)t.hyper[2], eps = (float)t.hyper[3];
+    int e_begin = 0, e_end = 0, other = 0;
+    float sg = 1.f;
+    float4 target = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load_entry = [&](int e) {
+        const int ent = t.cam_ent[e];
+        const int n = ent >> 1;
+        sg = (ent & 1) ? 1.f : -1.f;           // camera j: +dL/du, camera i: -dL/du
+        other = (ent & 1) ? t.cam_i[n] : t.cam_j[n];
+        target = t.oij[n];
+    };
+    double st_o = 0.0;         // the thread's centre component and moments when the block owns one item
+    float st_m = 0.f, st_v = 0.f;
+    for (int it = 0; it < iters; ++it) {
+        const double *src = (it & 1) ? t.o2 : t.o;
+        double *dst = (it & 1) ? t.o : t.o2;
+        for (int item = blockIdx.x; item < items; item += gridDim.x) {
+            const int group = item / chunks, r0 = (item % chunks) * rc, nr = min(rc, t.n_runs - r0);
+            const int k = group * TR_CAMS + warp;
+            if (k < t.n_cams) {
+                if (!single || it == 0) {
+                    e_begin = t.cam_off[k];
+                    e_end = t.cam_off[k + 1];
+                    if (e_begin + lane < e_end) load_entry(e_begin + lane);
+                }
+                for (int rb = 0; rb < nr; rb += TR_BATCH) {
+                    float g[TR_BATCH][3];
+                    double own[TR_BATCH][3];
+#pragma unroll
+                    for (int b = 0; b < TR_BATCH; ++b) {
+                        const size_t row = (size_t)(r0 + min(rb + b, nr - 1)) * t.n_cams;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            own[b][a] = __ldcg(src + (row + k) * 3 + a);
+                            g[b][a] = 0.f;
+                        }
+                    }
+                    for (int e = e_begin + lane; e < e_end; e += 32) {
+                        if (e_end - e_begin > 32) load_entry(e);
+                        double oo[TR_BATCH][3];
+#pragma unroll
+                        for (int b = 0; b < TR_BATCH; ++b) {
+                            const size_t row = (size_t)(r0 + min(rb + b, nr - 1)) * t.n_cams;
+#pragma unroll
+                            for (int a = 0; a < 3; ++a) oo[b][a] = __ldcg(src + (row + other) * 3 + a);
+                        }
+#pragma unroll
+                        for (int b = 0; b < TR_BATCH; ++b) {
+                            if (rb + b >= nr) break;
+                            float u[3];
+#pragma unroll
+                            for (int a = 0; a < 3; ++a) u[a] = sg * (float)(own[b][a] - oo[b][a]);   // o_j - o_i
+                            float4 p;
+                            if (!pair_term(u, target, p)) atomicOr(t.err, ERR_DEGENERATE);
+                            g[b][0] = fmaf(sg, p.x, g[b][0]);
+                            g[b][1] = fmaf(sg, p.y, g[b][1]);
+                            g[b][2] = fmaf(sg, p.z, g[b][2]);
+                        }
+                    }
+#pragma unroll
+                    for (int b = 0; b < TR_BATCH; ++b) {
+                        if (rb + b >= nr) break;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) g[b][a] += __shfl_xor_sync(0xffffffffu, g[b][a], o);
+                        }
+                        if (lane < 3) s_g[warp][rb + b][lane] = lane == 0 ? g[b][0] : (lane == 1 ? g[b][1] : g[b][2]);
+                    }
+                }
+            }
+            __syncthreads();
+            const int cc = threadIdx.x / (3 * rc), rr = threadIdx.x / 3 % rc, ca = threadIdx.x % 3;
+            const int kc = group * TR_CAMS + cc;
+            if (cc < TR_CAMS && rr < nr && kc < t.n_cams) {
+                const size_t o = ((size_t)(r0 + rr) * t.n_cams + kc) * 3 + ca;
+                if (!single || it == 0) {
+                    st_o = __ldcg(src + o);
+                    st_m = t.m[o];
+                    st_v = t.v[o];
+                }
+                const float ts = (float)(t0 + 1 + it);
+                const float bc1 = 1.f - powf(b1, ts), bc2 = 1.f - powf(b2, ts);
+                const float ga = (float)((double)s_g[cc][rr][ca] * inv_b);
+                st_m = rfma(b1, st_m, rmul(radd(1.f, -b1), ga));
+                st_v = rfma(b2, st_v, rmul(rmul(radd(1.f, -b2), ga), ga));
+                st_o -= (double)(lr * (st_m / bc1) / (sqrtf(st_v / bc2) + eps));
+                dst[o] = st_o;
+                if (!single || it + 1 == iters) {
+                    t.m[o] = st_m;
+                    t.v[o] = st_v;
+                }
+            }
+            if (!single) __syncthreads();   // s_g is written again
+        }
+        if (!gb.sync()) return;
+    }
+    gb.finish();
+    if (iters & 1) {         // the centres end in t.o
+        const size_t n = (size_t)t.n_runs * t.n_cams * 3;
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+            t.o[i] = __ldcg(t.o2 + i);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *t.step = t0 + iters;
+}
+
+// per run: loss total (FP64, fixed order) / |P|
+__global__ void __launch_bounds__(TR_THREADS) k_tr_finalize(DevTrans t) {
     __shared__ double red[TR_THREADS];
     pdl_wait();
     pdl_trigger();
@@ -164,10 +287,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tr_finalize(DevTrans t, int coun
         if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        t.loss[run] = red[0] / (double)t.n_pairs;
-        if (run == 0) *t.step += count;
-    }
+    if (threadIdx.x == 0) t.loss[run] = red[0] / (double)t.n_pairs;
 }
 
 // per run: centroid, then mean distance to it (FP64, fixed order)
@@ -234,7 +354,7 @@ struct fm_translation {
     cudaStream_t user = nullptr;
     cudaStream_t s = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    cudaGraphExec_t graph = nullptr, graph8 = nullptr;
+    int step_grid = 0;       // most blocks of the step kernel
     std::vector<void *> allocs;
 };
 
@@ -276,6 +396,12 @@ fm_status tcheck_errors(fm_translation *p) {
     unsigned err = 0;
     TR_CUDA(cudaMemcpyAsync(&err, p->d.err, sizeof err, cudaMemcpyDeviceToHost, p->s));
     TR_CUDA(cudaStreamSynchronize(p->s));
+    if (err & ERR_GRID) {
+        TR_CUDA(cudaMemsetAsync(p->d.err, 0, sizeof err, p->s));
+        TR_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
+        TR_CUDA(cudaStreamSynchronize(p->s));
+        return tfail(FM_ECUDA, "a grid barrier ran into its limit");
+    }
     if (err & ERR_DEGENERATE) {
         const unsigned zero = 0;
         TR_CUDA(cudaMemcpyAsync(p->d.err, &zero, sizeof zero, cudaMemcpyHostToDevice, p->s));
@@ -285,44 +411,27 @@ fm_status tcheck_errors(fm_translation *p) {
     return FM_OK;
 }
 
-void enqueue_eval(fm_translation *p, int it, bool apply, bool pdl) {
+void enqueue_eval(fm_translation *p) {
     const dim3 gp((p->d.n_pairs + TR_THREADS - 1) / TR_THREADS, p->d.n_runs);
     const dim3 gc(cam_blocks(p->d), p->d.n_runs);
-    launch_k(k_tr_pair, gp, dim3(TR_THREADS), p->s, pdl, p->d);
-    launch_k(k_tr_cam, gc, dim3(TR_CAMS * 32), p->s, true, p->d, it, apply ? 1 : 0);
+    launch_k(k_tr_pair, gp, dim3(TR_THREADS), p->s, false, p->d);
+    launch_k(k_tr_cam, gc, dim3(TR_CAMS * 32), p->s, true, p->d);
 }
 
-void enqueue_steps(fm_translation *p, int iters) {
-    for (int it = 0; it < iters; ++it) enqueue_eval(p, it, true, true);
-    launch_k(k_tr_finalize, dim3(p->d.n_runs), dim3(TR_THREADS), p->s, true, p->d, iters);
+// items of rc runs each: as many as fit the resident blocks, so that few runs per block are in series
+cudaError_t enqueue_steps(fm_translation *p, int iters) {
+    const int64_t groups = cam_blocks(p->d);
+    const int rc = (int)std::min<int64_t>(TR_RC, (groups * p->d.n_runs + p->step_grid - 1) / p->step_grid);
+    const int64_t items = groups * ((p->d.n_runs + rc - 1) / rc);
+    return launch_coop(k_tr_steps, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, p->s, p->d, iters, rc);
 }
 
-fm_status build_tgraph(fm_translation *p, int iters, cudaGraphExec_t *out) {
-    cudaGraph_t g = nullptr;
-    TR_CUDA(cudaStreamBeginCapture(p->s, cudaStreamCaptureModeThreadLocal));
-    enqueue_steps(p, iters);
-    cudaError_t e = cudaStreamEndCapture(p->s, &g);
-    if (e != cudaSuccess) return tfail(FM_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(out, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        *out = nullptr;
-        return tfail(FM_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    }
-    return FM_OK;
-}
-
-void drop_graphs(fm_translation *p) {
-    if (p->graph) cudaGraphExecDestroy(p->graph);
-    if (p->graph8) cudaGraphExecDestroy(p->graph8);
-    p->graph = p->graph8 = nullptr;
-}
+constexpr int TR_CHAIN = 4096;
 
 void free_trans(fm_translation *p) {
     if (!p) return;
     if (p->s) cudaStreamSynchronize(p->s);
     for (void *a : p->allocs) cudaFree(a);
-    drop_graphs(p);
     if (p->ev_in) cudaEventDestroy(p->ev_in);
     if (p->ev_out) cudaEventDestroy(p->ev_out);
     if (p->s) cudaStreamDestroy(p->s);
@@ -384,6 +493,9 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     d.cam_ent = ce;
     TR_CUDA(talloc(p, &d.oij, (size_t)n_pairs));
     TR_CUDA(talloc(p, &d.o, nc3));
+    TR_CUDA(talloc(p, &d.o2, nc3));
+    TR_CUDA(talloc(p, &d.grid_state, (size_t)GRID_STATE_WORDS));
+    TR_CUDA(coop_blocks(k_tr_steps, TR_CAMS * 32, &p->step_grid));
     TR_CUDA(talloc(p, &d.m, nc3));
     TR_CUDA(talloc(p, &d.v, nc3));
     TR_CUDA(talloc(p, &d.pterm, (size_t)n_runs * n_pairs));
@@ -408,6 +520,7 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     TR_CUDA(cudaMemsetAsync(d.v, 0, sizeof(float) * nc3, p->s));
     TR_CUDA(cudaMemsetAsync(d.step, 0, sizeof(long long), p->s));
     TR_CUDA(cudaMemsetAsync(d.err, 0, sizeof(unsigned), p->s));
+    TR_CUDA(cudaMemsetAsync(d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
     k_tr_setup<<<(n_pairs + TR_THREADS - 1) / TR_THREADS, TR_THREADS, 0, p->s>>>(d, Rd, td);
     TR_CUDA(cudaGetLastError());
     TR_CUDA(cudaFreeAsync(Rd, p->s));
@@ -487,8 +600,8 @@ FM_API fm_status fm_translation_loss_grad(fm_translation *p, double *loss, doubl
     if (fm_status st = tcheck(p)) return st;
     if (!loss) return tfail(FM_EINVAL, "loss must not be NULL");
     TR_CUDA(tjoin_in(p));
-    enqueue_eval(p, 0, false, false);
-    launch_k(k_tr_finalize, dim3(p->d.n_runs), dim3(TR_THREADS), p->s, true, p->d, 0);
+    enqueue_eval(p);
+    launch_k(k_tr_finalize, dim3(p->d.n_runs), dim3(TR_THREADS), p->s, true, p->d);
     TR_CUDA(cudaGetLastError());
     const size_t nc = (size_t)p->d.n_runs * p->d.n_cams;
     TR_CUDA(cudaMemcpyAsync(loss, p->d.loss, sizeof(double) * p->d.n_runs, cudaMemcpyDeviceToHost, p->s));
@@ -508,18 +621,8 @@ FM_API fm_status fm_translation_step(fm_translation *p, int32_t n_iters) {
     if (n_iters < 0) return tfail(FM_EINVAL, "n_iters must be >= 0");
     if (n_iters == 0) return FM_OK;
     TR_CUDA(tjoin_in(p));
-    if (!p->opt.use_graph) {
-        enqueue_steps(p, n_iters);
-        TR_CUDA(cudaGetLastError());
-    } else {
-        if (!p->graph)
-            if (fm_status st = build_tgraph(p, 1, &p->graph)) return st;
-        if (n_iters >= 8 && !p->graph8)
-            if (fm_status st = build_tgraph(p, 8, &p->graph8)) return st;
-        int left = n_iters;
-        for (; left >= 8; left -= 8) TR_CUDA(cudaGraphLaunch(p->graph8, p->s));
-        for (; left > 0; --left) TR_CUDA(cudaGraphLaunch(p->graph, p->s));
-    }
+    // launches of bounded length (an iteration takes microseconds); use_graph makes no difference
+    for (int left = n_iters; left > 0; left -= TR_CHAIN) TR_CUDA(enqueue_steps(p, std::min(left, TR_CHAIN)));
     TR_CUDA(tjoin_out(p));
     return FM_OK;
 }
@@ -528,14 +631,13 @@ FM_API fm_status fm_translation_merge(fm_translation *p) {
     if (fm_status st = tcheck(p)) return st;
     TR_CUDA(tjoin_in(p));
     // camera losses at the current centres of every run, then per-run normalisation
-    enqueue_eval(p, 0, false, false);
+    enqueue_eval(p);
     k_tr_stats<<<p->d.n_runs, TR_THREADS, 0, p->s>>>(p->d);
     k_tr_merge<<<(p->d.n_cams + TR_THREADS - 1) / TR_THREADS, TR_THREADS, 0, p->s>>>(p->d);
     TR_CUDA(cudaGetLastError());
     if (fm_status st = tcheck_errors(p)) return st;
     // one run continues from the merged centres with fresh Adam state
     p->d.n_runs = 1;
-    drop_graphs(p);
     TR_CUDA(cudaMemsetAsync(p->d.m, 0, sizeof(float) * 3 * p->d.n_cams, p->s));
     TR_CUDA(cudaMemsetAsync(p->d.v, 0, sizeof(float) * 3 * p->d.n_cams, p->s));
     TR_CUDA(cudaMemsetAsync(p->d.step, 0, sizeof(long long), p->s));
