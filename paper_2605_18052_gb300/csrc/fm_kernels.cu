@@ -327,10 +327,9 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // over the lanes (a pair that spans many ranges does not hold up one lane). The warp reduces
 // the 6 gradient components and the loss with a compensated (TwoSum) FP32 butterfly, so each
 // sum is carried as an unevaluated hi + lo pair.
-// Phase 2: warp 0, one camera per lane: the final per-camera gradient hi + lo in FP64, the
-// Adam update (FP32 moments), R <- Exp(phi) R and Gram-Schmidt re-orthonormalisation in FP64,
-// the centre update in FP64 and the new camera record. Keeping the FP64 work lane-parallel
-// matters on GB300, whose FP64 pipe charges a whole warp instruction per operation.
+// Phase 2: warp 0, a lane per component of each of the block's cameras: the Adam update (FP32
+// moments), R <- Exp(phi) R and Gram-Schmidt re-orthonormalisation in FP64, the centre update in
+// FP64 and the new camera record (camera_update).
 // Geometry comes from the pair records, never from another camera's record, which another
 // block may be updating. The loss of a pair is counted by its first camera only; each camera's
 // FP64 loss share goes to cam_loss[camera], and the next kernel (the next pass, pair setup or
@@ -425,24 +424,24 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
                 for (int q = 0; q < NV; ++q) two_sum_acc(hi[q], lo[q], contrib[q], 0.f);
             }
         }
-        warp_two_sum_reduce<NV>(hi, lo);
-        if (lane == 0) {
+        warp_two_sum_spread<NV>(hi, lo, lane);
 #pragma unroll
-            for (int q = 0; q < STEP_VALS; ++q) {
-                s_hi[q][warp] = q < NV ? hi[q] : 0.f;
-                s_lo[q][warp] = lo[q];
+        for (int q = 0; q < NV; ++q)
+            if (lane == spread_lane(NV, q)) {
+                s_hi[q][warp] = hi[0];
+                s_lo[q][warp] = lo[0];
             }
-        }
     }
     __syncthreads();
-    if (warp == 0 && lane < STEP_CAMS) {
-        const int kc = blockIdx.x * STEP_CAMS + lane;
-        const double bl = kc < d.n_cams
-            ? camera_update<FOCAL>(d, kc, &s_hi[0][lane], &s_lo[0][lane], STEP_CAMS, s_mv[lane], s_Rc[lane],
-                                   s_R32[lane], s_hyper, t_step, apply, d.cam + (size_t)kc * CAMREC)
-            : 0.0;
+    if (warp == 0) {
+        const int cc = lane / 3, ca = lane % 3, kc = blockIdx.x * STEP_CAMS + cc;
+        const bool on = cc < STEP_CAMS && kc < d.n_cams;
+        const int sc = on ? cc : 0;
+        const double bl = camera_update<FOCAL>(d, kc, on, ca, 3 * cc, &s_hi[0][sc], &s_lo[0][sc], STEP_CAMS, s_mv[sc],
+                                               s_Rc[sc], s_R32[sc], s_hyper, t_step, apply,
+                                               d.cam + (size_t)kc * CAMREC);
         if (apply && next_geo) __threadfence();   // the record reaches L2 before any count below
-        if (kc < d.n_cams) d.cam_loss[kc] = bl;
+        if (on && ca == 0) d.cam_loss[kc] = bl;
     }
     if (!(apply && next_geo)) return;
     __syncthreads();   // the block's new records are written
@@ -454,36 +453,39 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
     }
 }
 
-// Adam step with a given gradient (d.grad, FP64), one camera per thread: the same update as the
-// camera-step kernel (camera_update with the gradient split into FP32 hi + lo parts, whose FP32
+// Adam step with a given gradient (d.grad, FP64), a warp for STEP_CAMS cameras: the same update as
+// the camera-step kernel (camera_update with the gradient split into FP32 hi + lo parts, whose FP32
 // sum is the gradient rounded to FP32, as there); the step count is advanced by k_bump_step.
-__global__ void k_apply_gradient(DevProblem d) {
-    const int kc = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kc >= d.n_cams) return;
+__global__ void __launch_bounds__(32) k_apply_gradient(DevProblem d) {
+    const int lane = threadIdx.x, cc = lane / 3, ca = lane % 3;
+    const int kc = blockIdx.x * STEP_CAMS + cc;
+    const bool on = cc < STEP_CAMS && kc < d.n_cams;
+    const size_t k = on ? kc : 0;
     const long long t_step = *d.step + 1;
     float hi[STEP_VALS], lo[STEP_VALS], mv[12], rec[10];
     double Rc[12], hyper[6];
 #pragma unroll
     for (int q = 0; q < STEP_VALS; ++q) {
-        const double g = q < 6 ? d.grad[(size_t)kc * 6 + q] : 0.0;
+        const double g = q < 6 ? d.grad[k * 6 + q] : 0.0;
         hi[q] = (float)g;
         lo[q] = (float)__dsub_rn(g, (double)hi[q]);
     }
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-        mv[q] = d.m[(size_t)kc * 6 + q];
-        mv[6 + q] = d.v[(size_t)kc * 6 + q];
+        mv[q] = d.m[k * 6 + q];
+        mv[6 + q] = d.v[k * 6 + q];
         hyper[q] = d.hyper[q];
     }
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        Rc[q] = d.R[(size_t)kc * 9 + q];
-        rec[q] = d.cam[(size_t)kc * CAMREC + q];
+        Rc[q] = d.R[k * 9 + q];
+        rec[q] = d.cam[k * CAMREC + q];
     }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) Rc[9 + q] = d.c[(size_t)kc * 3 + q];
-    rec[9] = d.cam[(size_t)kc * CAMREC + 15];
-    camera_update<false>(d, kc, hi, lo, 1, mv, Rc, rec, hyper, t_step, 1, d.cam + (size_t)kc * CAMREC);
+    for (int q = 0; q < 3; ++q) Rc[9 + q] = d.c[k * 3 + q];
+    rec[9] = d.cam[k * CAMREC + 15];
+    __syncwarp();   // every lane has read its camera's state before a lane replaces part of it
+    camera_update<false>(d, kc, on, ca, 3 * cc, hi, lo, 1, mv, Rc, rec, hyper, t_step, 1, d.cam + (size_t)kc * CAMREC);
 }
 
 __global__ void k_bump_step(DevProblem d) { *d.step += 1; }
@@ -575,7 +577,7 @@ void loss_scales(const DevProblem &d, float &gscale, float &lscale) {
 }
 
 void launch_apply_gradient(const DevProblem &d, cudaStream_t s) {
-    k_apply_gradient<<<blocks_for(d.n_cams, 64), 64, 0, s>>>(d);
+    k_apply_gradient<<<blocks_for(d.n_cams, STEP_CAMS), 32, 0, s>>>(d);
     k_bump_step<<<1, 1, 0, s>>>(d);
 }
 

@@ -160,7 +160,7 @@ __global__ void k_quad_combine(DevProblem d) {
 //   q = g0 + W d,  loss = c0 + d^T (g0 + q),  d = E'_n - e0,
 // and the chain rule to camera k. Both cameras of a pair evaluate it (O(1) each), which
 // removes a per-pair launch and the wait on it. The warp reduces with compensated butterflies,
-// then lanes 0..7 of warp 0 do the FP64 update of the block's cameras and write the new
+// then warp 0 does the FP64 update of the block's cameras and writes the new
 // records to cam_dst: the records of this step's poses stay intact in cam_src for the other
 // blocks. The Adam step count is *d.step + 1 + it; the launch that closes the chain adds
 // the chain's length to *d.step.
@@ -262,23 +262,23 @@ k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gs
 #pragma unroll
             for (int w = 0; w < NV; ++w) two_sum_acc(hi[w], lo[w], contrib[w], 0.f);
         }
-        warp_two_sum_reduce<NV>(hi, lo);
-        if (lane == 0) {
+        warp_two_sum_spread<NV>(hi, lo, lane);
 #pragma unroll
-            for (int q = 0; q < STEP_VALS; ++q) {
-                s_hi[q][warp] = q < NV ? hi[q] : 0.f;
-                s_lo[q][warp] = lo[q];
+        for (int q = 0; q < NV; ++q)
+            if (lane == spread_lane(NV, q)) {
+                s_hi[q][warp] = hi[0];
+                s_lo[q][warp] = lo[0];
             }
-        }
     }
     __syncthreads();
-    if (warp == 0 && lane < STEP_CAMS) {
-        const int kc = blockIdx.x * STEP_CAMS + lane;
-        const double bl = kc < d.n_cams
-            ? camera_update<FOCAL>(d, kc, &s_hi[0][lane], &s_lo[0][lane], STEP_CAMS, s_mv[lane], s_Rc[lane], s_R32[lane], s_hyper,
-                            t_step, apply, cam_dst + (size_t)kc * CAMREC)
-            : 0.0;
-        if (kc < d.n_cams) d.cam_loss[kc] = bl;
+    if (warp == 0) {
+        const int cc = lane / 3, ca = lane % 3, kc = blockIdx.x * STEP_CAMS + cc;
+        const bool on = cc < STEP_CAMS && kc < d.n_cams;
+        const int sc = on ? cc : 0;
+        const double bl = camera_update<FOCAL>(d, kc, on, ca, 3 * cc, &s_hi[0][sc], &s_lo[0][sc], STEP_CAMS, s_mv[sc],
+                                               s_Rc[sc], s_R32[sc], s_hyper, t_step, apply,
+                                               cam_dst + (size_t)kc * CAMREC);
+        if (on && ca == 0) d.cam_loss[kc] = bl;
     }
 }
 

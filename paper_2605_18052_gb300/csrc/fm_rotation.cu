@@ -75,18 +75,6 @@ __device__ __forceinline__ void warp_sum(double *v) {
 // Warp-wide sums of N doubles that leave value i with lane spread_lane(N, i): at each butterfly
 // level a lane keeps half of its values and hands the other half over, so N = 9 takes 12 additions
 // instead of 45. The order of every sum is the butterfly's.
-constexpr int spread_lane(int n, int i) {
-    int lane = 0;
-    for (int o = 16; n > 1; o >>= 1) {
-        const int h = (n + 1) / 2;
-        if (i >= h) {
-            lane |= o;
-            i -= h;
-        }
-        n = h;
-    }
-    return lane;
-}
 template <int N>
 __device__ __forceinline__ double warp_sum_spread(double (&v)[N], int lane) {
     int cnt = N;

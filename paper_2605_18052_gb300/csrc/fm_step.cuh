@@ -57,11 +57,11 @@ __device__ __forceinline__ double rsqrt64(double x) {
     return y;
 }
 
-// Exp(phi) - I = a K + b K^2 (K = [phi]_x) in FP32. A rotation increment is small, so its
+// Row r of Exp(phi) - I = a K + b K^2 (K = [phi]_x) in FP32. A rotation increment is small, so its
 // FP32 relative error (a few ulp) is an absolute error of a few 1e-7 |phi|, the same order as
 // that of phi itself, which Adam computes in FP32. For |phi| < 0.1 the Taylor series of a and b
 // through the t^6 terms (truncation below 1e-13); otherwise sin and b = 2 sin^2(t/2) / t^2.
-__device__ __forceinline__ void so3_exp_minus_identity(const float *phi, float *A) {
+__device__ __forceinline__ void so3_exp_minus_identity_row(const float *phi, int r, float *A) {
     const float th2 = rdot3(phi[0], phi[0], phi[1], phi[1], phi[2], phi[2]);
     float a, b;
     if (th2 < 0.01f) {
@@ -74,13 +74,14 @@ __device__ __forceinline__ void so3_exp_minus_identity(const float *phi, float *
         b = __fdiv_rn(rmul(rmul(2.f, sh), sh), th2);
     }
     const float K[9] = {0.f, -phi[2], phi[1], phi[2], 0.f, -phi[0], -phi[1], phi[0], 0.f};
+    float k[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int c = 0; c < 3; ++c) k[c] = r == 0 ? K[c] : (r == 1 ? K[3 + c] : K[6 + c]);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float k2 = rdot3(K[3 * r], K[c], K[3 * r + 1], K[3 + c], K[3 * r + 2], K[6 + c]);
-            A[3 * r + c] = rfma(b, k2, rmul(a, K[3 * r + c]));
-        }
+    for (int c = 0; c < 3; ++c) {
+        const float k2 = rdot3(k[0], K[c], k[1], K[3 + c], k[2], K[6 + c]);
+        A[c] = rfma(b, k2, rmul(a, k[c]));
+    }
 }
 
 // Gram-Schmidt on the rows: r0 normalised, r1 orthogonalised and normalised, r2 = r0 x r1
@@ -207,72 +208,94 @@ __device__ __forceinline__ void pair_chain_rule(const float *gr, int role, const
 }
 
 
-// warp-wide TwoSum butterfly of N (hi, lo) pairs: every lane ends with the total
+// Warp-wide TwoSum sums of N (hi, lo) pairs: value i ends in hi[0], lo[0] of lane spread_lane(N, i).
+// TwoSum is symmetric in its operands, so this is the butterfly's result bit for bit, with 9 of
+// these accumulations for N = 7 where the butterfly takes 35.
 template <int N>
-__device__ __forceinline__ void warp_two_sum_reduce(float *hi, float *lo) {
+__device__ __forceinline__ void warp_two_sum_spread(float *hi, float *lo, int lane) {
+    int cnt = N;
 #pragma unroll
-    for (int q = 0; q < N; ++q)
+    for (int o = 16; o > 0; o >>= 1) {
+        if (cnt > 1) {
+            const int h = (cnt + 1) / 2;
+            const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float bh = __shfl_xor_sync(0xffffffffu, hi[q], o);
-            const float bl = __shfl_xor_sync(0xffffffffu, lo[q], o);
-            two_sum_acc(hi[q], lo[q], bh, bl);
+            for (int i = 0; i < N; ++i) {
+                if (i >= h) break;
+                const float oh = h + i < cnt ? hi[h + i] : 0.f, ol = h + i < cnt ? lo[h + i] : 0.f;
+                const float gh = up ? hi[i] : oh, gl = up ? lo[i] : ol;
+                hi[i] = up ? oh : hi[i];
+                lo[i] = up ? ol : lo[i];
+                const float bh = __shfl_xor_sync(0xffffffffu, gh, o);
+                const float bl = __shfl_xor_sync(0xffffffffu, gl, o);
+                two_sum_acc(hi[i], lo[i], bh, bl);
+            }
+            cnt = h;
+        } else {
+            const float bh = __shfl_xor_sync(0xffffffffu, hi[0], o);
+            const float bl = __shfl_xor_sync(0xffffffffu, lo[0], o);
+            two_sum_acc(hi[0], lo[0], bh, bl);
         }
+    }
 }
 
-// Phase 2 of a step for camera kc, one lane. apply = 0: the gradient (FP64 sum of its hi + lo
-// parts) and the focal gradient are written, nothing else. apply = 1: one Adam step (FP32
-// moments) and the new pose: R <- R + (Exp(phi) - I) R and c <- c + delta_c in FP64, where the
-// small increment (Exp(phi) - I) R is formed in FP32 from the camera's FP32 record rotation R32
-// (its error, a few 1e-7 |phi|, is of the order of phi's own FP32 error), then Gram-Schmidt on
-// the rows in FP64 on every eighth step (steps 1, 9, 17, ...) and the new camera record at
-// rec_out. hi/lo hold STEP_VALS values (6 pose gradient components, the loss, the
+// Phase 2 of a step, by one warp: lane 3 c + a holds component a of camera kc (the block's camera c;
+// `on` for lanes that have one), so that the warp finishes up to ten cameras at once. apply = 0: the
+// gradient (FP64 sum of its hi + lo parts) and the focal gradient are written, nothing else. apply =
+// 1: one Adam step (FP32 moments) and the new pose: R <- R + (Exp(phi) - I) R and c <- c + delta_c in
+// FP64, where the small increment (Exp(phi) - I) R is formed in FP32 from the camera's FP32 record
+// rotation R32 (its error, a few 1e-7 |phi|, is of the order of phi's own FP32 error), then
+// Gram-Schmidt on the rows in FP64 on every eighth step (steps 1, 9, 17, ...) and the new camera
+// record at rec_out. hi/lo hold STEP_VALS values (6 pose gradient components, the loss, the
 // keypoint-scale gradient) `stride` apart; mv = the camera's Adam m (6) and v (6); Rc = its R
 // (9) and c (3) in FP64; rec = its current record's rotation (9 floats) and keypoint scale
 // (rec[9]); hyper = lr_rot, lr_c, beta1, beta2, eps, lr_focal. With focal refinement
 // rho = log s takes its own Adam step (gradient s dL/ds); without, the record keeps its scale.
 // Returns the camera's loss share.
-// GB300 executes FP64 on a narrow pipe at whole-warp cost per instruction, and every block of a
-// step reaches this phase at the same moment, so the update keeps its FP64 work to the state
-// itself: the two sums and the record (about 45 operations), and the re-orthonormalisation
-// (about 40) only every eighth step. Between two of them R leaves SO(3) by the FP32 rounding of
-// the increments, a few 1e-7 |phi| per step, far below the FP32 camera record's resolution.
+// GB300 issues an FP64 instruction (conversions included) of a warp over 64 cycles, whatever its
+// active lanes, and every block of a step reaches this phase at the same moment. So the update keeps
+// its FP64 work to the state itself (two sums, the record; re-orthonormalisation, about 40
+// operations, only every eighth step), and spreads a camera's components over lanes: about 21 FP64
+// instructions where a lane per camera took 48, and a third of the FP32 chain. Between two
+// re-orthonormalisations R leaves SO(3) by the FP32 rounding of the increments, a few 1e-7 |phi| per
+// step, far below the FP32 camera record's resolution.
 template <bool FOCAL>
-__device__ __forceinline__ double camera_update(const DevProblem &d, int kc, const float *hi, const float *lo,
-                                                int stride, const float *mv, const double *Rc, const float *rec,
-                                                const double *hyper, long long t_step, int apply,
+__device__ __forceinline__ double camera_update(const DevProblem &d, int kc, bool on, int a, int base, const float *hi,
+                                                const float *lo, int stride, const float *mv, const double *Rc,
+                                                const float *rec, const double *hyper, long long t_step, int apply,
                                                 float *rec_out) {
     const float *R32 = rec;
     const double bl = (double)hi[6 * stride] + (double)lo[6 * stride];
-    const double s_cur = FOCAL ? camera_scale(d, kc) : 1.0;
+    const double s_cur = FOCAL && on ? camera_scale(d, kc) : 1.0;
     const double g_rho = FOCAL ? s_cur * ((double)hi[7 * stride] + (double)lo[7 * stride]) : 0.0;
     if (!apply) {
         bool ok = isfinite(hi[6 * stride]);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
+        for (int h = 0; h < 2; ++h) {
+            const int q = 3 * h + a;
             const double g = (double)hi[q * stride] + (double)lo[q * stride];
             ok = ok && isfinite(g);
-            d.grad[(size_t)kc * 6 + q] = g;
+            if (on) d.grad[(size_t)kc * 6 + q] = g;
         }
-        if (!ok) atomicOr(d.err, ERR_NONFINITE);
-        if (d.grad_rho) d.grad_rho[kc] = g_rho;
+        if (on && !ok) atomicOr(d.err, ERR_NONFINITE);
+        if (on && a == 0 && d.grad_rho) d.grad_rho[kc] = g_rho;
         return bl;
     }
     // the FP32 gradient: hi is the rounded value of hi + lo (TwoSum keeps |lo| within half an
     // ulp of hi), so hi + lo in FP32 is the same number the FP64 sum would round to
-    float gq[6];
+    float gq[2];
     bool ok = isfinite(hi[6 * stride]);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        gq[q] = radd(hi[q * stride], lo[q * stride]);
-        ok = ok && isfinite(gq[q]);
+    for (int h = 0; h < 2; ++h) {
+        gq[h] = radd(hi[(3 * h + a) * stride], lo[(3 * h + a) * stride]);
+        ok = ok && isfinite(gq[h]);
     }
-    if (!ok) atomicOr(d.err, ERR_NONFINITE);
+    if (on && !ok) atomicOr(d.err, ERR_NONFINITE);
     float s_new = rec[9];
     const float b1 = (float)hyper[2], b2 = (float)hyper[3], eps = (float)hyper[4];
-    const float lr_r = (float)hyper[0], lr_c = (float)hyper[1];
+    const float lr[2] = {(float)hyper[0], (float)hyper[1]};
     const float bc1 = radd(1.f, -powf(b1, (float)t_step)), bc2 = radd(1.f, -powf(b2, (float)t_step));
-    if (FOCAL) {
+    if (FOCAL && on && a == 0) {
         const float g1 = (float)g_rho;
         const float mo = rfma(b1, d.rho_m[kc], rmul(radd(1.f, -b1), g1));
         const float vo = rfma(b2, d.rho_v[kc], rmul(rmul(radd(1.f, -b2), g1), g1));
@@ -284,37 +307,51 @@ __device__ __forceinline__ double camera_update(const DevProblem &d, int kc, con
         d.grad_rho[kc] = g_rho;
         s_new = (float)exp(r);
     }
-    float dl[6], mo[6], vo[6];
+    float dl[2], mo[2], vo[2];   // phi_a and c_a
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        mo[q] = rfma(b1, mv[q], rmul(radd(1.f, -b1), gq[q]));
-        vo[q] = rfma(b2, mv[6 + q], rmul(rmul(radd(1.f, -b2), gq[q]), gq[q]));
-        dl[q] = __fdiv_rn(rmul(-(q < 3 ? lr_r : lr_c), __fdiv_rn(mo[q], bc1)),
-                          radd(__fsqrt_rn(__fdiv_rn(vo[q], bc2)), eps));
+    for (int h = 0; h < 2; ++h) {
+        const int q = 3 * h + a;
+        mo[h] = rfma(b1, mv[q], rmul(radd(1.f, -b1), gq[h]));
+        vo[h] = rfma(b2, mv[6 + q], rmul(rmul(radd(1.f, -b2), gq[h]), gq[h]));
+        dl[h] = __fdiv_rn(rmul(-lr[h], __fdiv_rn(mo[h], bc1)), radd(__fsqrt_rn(__fdiv_rn(vo[h], bc2)), eps));
     }
-    float A[9];
-    so3_exp_minus_identity(dl, A);
-    double Rn[9], cn[3];
+    float phi[3], A[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int q = 0; q < 3; ++q) phi[q] = __shfl_sync(0xffffffffu, dl[0], base + q);
+    so3_exp_minus_identity_row(phi, a, A);
+    double Rn[3];   // row a
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-            Rn[3 * r + c] = __dadd_rn(Rc[3 * r + c], (double)rdot3(A[3 * r], R32[c], A[3 * r + 1], R32[3 + c],
-                                                                     A[3 * r + 2], R32[6 + c]));
-    if ((t_step & 7) == 1) orthonormalize_rows(Rn);
+    for (int c = 0; c < 3; ++c)
+        Rn[c] = __dadd_rn(Rc[3 * a + c], (double)rdot3(A[0], R32[c], A[1], R32[3 + c], A[2], R32[6 + c]));
+    if ((t_step & 7) == 1) {
+        double M[9];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) cn[q] = __dadd_rn(Rc[9 + q], (double)dl[3 + q]);
+        for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        const size_t o = (size_t)kc * 6 + q;
-        d.m[o] = mo[q];
-        d.v[o] = vo[q];
+            for (int c = 0; c < 3; ++c) M[3 * r + c] = __shfl_sync(0xffffffffu, Rn[c], base + r);
+        orthonormalize_rows(M);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Rn[c] = a == 0 ? M[c] : (a == 1 ? M[3 + c] : M[6 + c]);
     }
+    const double cn = __dadd_rn(Rc[9 + a], (double)dl[1]);
+    if (on) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) d.R[(size_t)kc * 9 + q] = Rn[q];
+        for (int h = 0; h < 2; ++h) {
+            const size_t o = (size_t)kc * 6 + 3 * h + a;
+            d.m[o] = mo[h];
+            d.v[o] = vo[h];
+        }
 #pragma unroll
-    for (int q = 0; q < 3; ++q) d.c[(size_t)kc * 3 + q] = cn[q];
-    write_camrec(rec_out, Rn, cn, s_new);
+        for (int c = 0; c < 3; ++c) {
+            d.R[(size_t)kc * 9 + 3 * a + c] = Rn[c];
+            rec_out[3 * a + c] = (float)Rn[c];
+        }
+        d.c[(size_t)kc * 3 + a] = cn;
+        const float c_hi = (float)cn;
+        rec_out[9 + a] = c_hi;
+        rec_out[12 + a] = (float)__dsub_rn(cn, (double)c_hi);
+        if (a == 0) rec_out[15] = s_new;
+    }
     return bl;
 }
 
