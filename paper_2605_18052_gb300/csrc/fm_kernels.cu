@@ -11,22 +11,37 @@
 //   irls_weights / residuals: the same streaming walk writing one value per point pair
 #include <math.h>
 
+#include <type_traits>
+
 #include "fm_step.cuh"
 
 namespace fm {
 
-// prev_loss > 0: this pass follows an optimiser camera step (which also wrote this pass's
-// geometry records); block 0 first finishes that step's loss total (over prev_loss per-camera
+// W warps per block, a range each, staged in shared memory S chunks deep (walk_range_staged). The last
+// block has no range: when the pass follows an optimiser camera step (prev_loss > 0; that step also
+// wrote this pass's geometry records), it finishes the step's loss total (over prev_loss per-camera
 // shares) and step count.
-template <int STORE, int MODE>
-__global__ void __launch_bounds__(CTA_WARPS * 32, 4) k_stream_loss(DevProblem d, int prev_loss) {
-    pdl_wait();     // pair geometry of this pass
-    pdl_trigger();  // the per-camera step may be scheduled once the last wave has started
-    if (prev_loss > 0 && blockIdx.x == 0) finish_step(d, prev_loss, 1);
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
-    if (r >= d.n_ranges) return;
+// Bound by HBM on large scenes, by the latency of a range's loads and by the launches around the pass
+// on small ones. Loading 4 groups per warp into registers after the wait for the launch before
+// (8 warps a block) left the memory system idle while a pass filled up and drained. An iteration of
+// fm_step, before -> now: 119 k point pairs FP32 18.7 -> 15.1 us, 3.1 M FP32 28.0 -> 19.2, 12 M FP16
+// 39.6 -> 31.2, 49 M FP32 161 -> 154, 49 M FP16 92.3 -> 84.5, 141 M FP16 227.9 -> 219.5.
+template <int STORE, int MODE, int S, int W>
+__global__ void __launch_bounds__(32 * W) k_stream_loss(DevProblem d, int prev_loss) {
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
+    if (r >= d.n_ranges) {
+        pdl_wait();
+        pdl_trigger();
+        if (prev_loss > 0 && blockIdx.x == gridDim.x - 1)
+            finish_step<32 * W>(d, prev_loss, 1, reinterpret_cast<double *>(stage));
+        return;
+    }
     LossBody<MODE> body(d);
-    walk_range<STORE, MODE == MODE_LOSS_IRLS>(d, r, threadIdx.x & 31, body);
+    walk_range_staged<STORE, MODE == MODE_LOSS_IRLS, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {
+        pdl_wait();     // pair geometry of this pass
+        pdl_trigger();  // the per-camera step may be scheduled once the last wave has started
+    });
 }
 
 // The first pass of an IRLS round fused with the round's reweighting: the residual at the
@@ -72,25 +87,21 @@ struct ReweightLossBody {
     }
 };
 
-template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32, 4) k_stream_reweight(DevProblem d) {
-    __shared__ unsigned cta_kept;
-    if (threadIdx.x == 0) cta_kept = 0;
-    __syncthreads();
-    pdl_wait();     // pair geometry of this pass
-    pdl_trigger();
-    const float tau = (float)d.hyper[6];
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
-    if (r < d.n_ranges) {
-        ReweightLossBody<STORE> body(d, tau);
-        walk_range<STORE, false>(d, r, threadIdx.x & 31, body);
-        unsigned k = body.kept;
+template <int STORE, int S, int W>
+__global__ void __launch_bounds__(32 * W) k_stream_reweight(DevProblem d) {
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
+    if (r >= d.n_ranges) return;
+    ReweightLossBody<STORE> body(d, 0.f);
+    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [&] {
+        pdl_wait();     // pair geometry of this pass, the threshold
+        pdl_trigger();
+        body.tau = (float)d.hyper[6];
+    });
+    unsigned k = body.kept;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&cta_kept, k);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && cta_kept) atomicAdd(d.counter, (unsigned long long)cta_kept);
+    for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    if ((threadIdx.x & 31) == 0 && k) atomicAdd(d.counter, (unsigned long long)k);
 }
 
 // ---- per-point-pair maps (IRLS weights, residual export) ------------------------------------------
@@ -183,7 +194,8 @@ __global__ void __launch_bounds__(256) k_pair_setup(DevProblem d, int prev_loss)
     const int i = n < d.n_pairs ? d.cam_i[n] : 0, j = n < d.n_pairs ? d.cam_j[n] : 0;
     pdl_wait();     // camera records of the previous step
     pdl_trigger();
-    if (prev_loss > 0 && blockIdx.x == 0) finish_step(d, prev_loss, 1);
+    __shared__ double red[FIN_THREADS];
+    if (prev_loss > 0 && blockIdx.x == 0) finish_step(d, prev_loss, 1, red);
     if (n >= d.n_pairs) return;
     pair_geometry(d, n, i, j);
 }
@@ -494,7 +506,8 @@ __global__ void k_bump_step(DevProblem d) { *d.step += 1; }
 __global__ void __launch_bounds__(FIN_THREADS) k_finalize(DevProblem d, int n_loss, int count) {
     pdl_wait();
     pdl_trigger();
-    finish_step(d, n_loss, count);
+    __shared__ double red[FIN_THREADS];
+    finish_step(d, n_loss, count, red);
 }
 
 // camera records copied back from the alternate buffer (one float4 per thread)
@@ -529,23 +542,48 @@ void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cu
     launch_k(k_finalize, dim3(1), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count);
 }
 
-void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
-    static_assert(CTA_WARPS * 32 == FIN_THREADS, "block 0 of the pass finishes a step");
-    const dim3 grid(blocks_for(d.n_ranges, CTA_WARPS)), block(CTA_WARPS * 32);
-    const int prev = after_step ? d.n_cams : 0;
+// Depth and block size of the staged passes. FP32: 4 chunks (512 point pairs) a warp; the whole range,
+// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 15.5 ->
+// 15.1 us an iteration, 245 ranges 17.5 -> 16.8; 733 ranges 17.9 -> 19.2). FP16: 2 chunks (512 point
+// pairs). One warp per block, so that a finished range makes room for the next at once, but four from
+// 300 ranges per SM on, where the block launches count (FP16: 68,633 ranges 223.6 -> 219.5 us, 23,860
+// ranges 84.5 -> 85.8).
+constexpr int FEW_RANGES = 2 * 152, MANY_RANGES = 300 * 152;
+
+template <class Launch>
+static void with_stages(const DevProblem &d, Launch launch) {
+    using std::integral_constant;
     if (d.storage == FM_STORE_FP32) {
-        if (d.loss == FM_LOSS_IRLS) launch_k(k_stream_loss<FM_STORE_FP32, MODE_LOSS_IRLS>, grid, block, s, pdl, d, prev);
-        else launch_k(k_stream_loss<FM_STORE_FP32, MODE_LOSS_L1>, grid, block, s, pdl, d, prev);
+        integral_constant<int, FM_STORE_FP32> st;
+        if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>(), integral_constant<int, 1>());
+        else if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 4>(), integral_constant<int, 1>());
+        else launch(st, integral_constant<int, 4>(), integral_constant<int, 4>());
     } else {
-        if (d.loss == FM_LOSS_IRLS) launch_k(k_stream_loss<FM_STORE_FP16, MODE_LOSS_IRLS>, grid, block, s, pdl, d, prev);
-        else launch_k(k_stream_loss<FM_STORE_FP16, MODE_LOSS_L1>, grid, block, s, pdl, d, prev);
+        integral_constant<int, FM_STORE_FP16> st;
+        if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 2>(), integral_constant<int, 1>());
+        else launch(st, integral_constant<int, 2>(), integral_constant<int, 4>());
     }
 }
 
+void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
+    const int prev = after_step ? d.n_cams : 0;
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        static_assert(S * W * STAGE_BYTES >= FIN_THREADS * sizeof(double), "the last block finishes a step in its stage");
+        const dim3 grid(blocks_for(d.n_ranges, W) + 1), block(32 * W);
+        if (d.loss == FM_LOSS_IRLS)
+            launch_smem(k_stream_loss<STORE, MODE_LOSS_IRLS, S, W>, grid, block, S * W * STAGE_BYTES, s, pdl, d, prev);
+        else
+            launch_smem(k_stream_loss<STORE, MODE_LOSS_L1, S, W>, grid, block, S * W * STAGE_BYTES, s, pdl, d, prev);
+    });
+}
+
 void launch_stream_reweight(const DevProblem &d, cudaStream_t s, bool pdl) {
-    const dim3 grid(blocks_for(d.n_ranges, CTA_WARPS)), block(CTA_WARPS * 32);
-    if (d.storage == FM_STORE_FP32) launch_k(k_stream_reweight<FM_STORE_FP32>, grid, block, s, pdl, d);
-    else launch_k(k_stream_reweight<FM_STORE_FP16>, grid, block, s, pdl, d);
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        launch_smem(k_stream_reweight<STORE, S, W>, dim3(blocks_for(d.n_ranges, W)), dim3(32 * W), S * W * STAGE_BYTES, s,
+                    pdl, d);
+    });
 }
 
 void launch_combine(const DevProblem &d, cudaStream_t s) {

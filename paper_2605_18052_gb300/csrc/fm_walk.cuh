@@ -18,12 +18,12 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
-                            bool pdl, Args... args) {
+static cudaError_t launch_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               bool pdl, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -31,6 +31,12 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
+                            bool pdl, Args... args) {
+    return launch_smem(kernel, grid, block, 0, s, pdl, args...);
 }
 
 // Warp sums of n values that hand half of a lane's values over at each butterfly level leave value i
@@ -181,63 +187,135 @@ __device__ __forceinline__ unsigned atomic_add_acq_rel(unsigned *p, unsigned v) 
 // contiguous 512 B block. The image pair changes only at sorted boundaries: a group that lies
 // inside the current pair takes the fast path; a group that crosses a boundary is processed in
 // passes, one pass per image pair it meets, and `body.segment_end` closes each finished pair.
+struct WalkState {
+    int64_t p_begin, p_end;
+    int seg;
+    int64_t seg_end;
+    float E[9];
+    __device__ __forceinline__ WalkState(const DevProblem &d, int r)
+        : p_begin((int64_t)r * WR), p_end(min(p_begin + (int64_t)WR, d.n_pp)), seg(d.range_pair[r]),
+          seg_end(d.pair_off[seg + 1]) {}
+};
+
+template <int STORE, class Body>
+__device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, const typename Fmt<STORE>::Raw &raw, int64_t gb,
+                                           int r, int lane, Body &body) {
+    using F = Fmt<STORE>;
+    constexpr int PPL = F::PPL;
+    constexpr int GROUP = 32 * PPL;
+    if (gb + GROUP <= st.seg_end) {
+#pragma unroll
+        for (int k = 0; k < PPL; ++k) {
+            float x1, y1, x2, y2, w;
+            F::get(raw, k, x1, y1, x2, y2, w);
+            body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+        }
+    } else {
+        int64_t lo = gb;
+        const int64_t g_end = min(gb + GROUP, st.p_end);
+        while (true) {
+            const int64_t hi = min(st.seg_end, st.p_end);
+#pragma unroll
+            for (int k = 0; k < PPL; ++k) {
+                const int64_t q = gb + lane * PPL + k;
+                if (q >= lo && q < hi) {
+                    float x1, y1, x2, y2, w;
+                    F::get(raw, k, x1, y1, x2, y2, w);
+                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+                }
+            }
+            if (st.seg_end >= g_end) break;
+            body.segment_end(st.seg, r, lane, false);
+            lo = st.seg_end;
+            ++st.seg;
+            st.seg_end = d.pair_off[st.seg + 1];
+            load_E(d.geo, st.seg, st.E);
+            body.segment_begin(st.seg);
+        }
+    }
+    body.group_done(gb, st.p_end, lane);
+}
+
 // U groups are loaded before any is processed (loads in flight per warp).
 template <int STORE, bool NEED_W, class Body, int U = 4>
 __device__ __forceinline__ void walk_range(const DevProblem &d, int r, int lane, Body &body) {
     using F = Fmt<STORE>;
-    constexpr int PPL = F::PPL;
-    constexpr int GROUP = 32 * PPL;
+    constexpr int GROUP = 32 * F::PPL;
     static_assert(WR % (U * GROUP) == 0, "range must be whole unrolled groups");
-    const int64_t p_begin = (int64_t)r * WR;
-    const int64_t p_end = min(p_begin + (int64_t)WR, d.n_pp);
-    int seg = d.range_pair[r];
-    int64_t seg_end = d.pair_off[seg + 1];
-    float E[9];
-    load_E(d.geo, seg, E);
-    body.segment_begin(seg);
+    WalkState st(d, r);
+    load_E(d.geo, st.seg, st.E);
+    body.segment_begin(st.seg);
     const uint64_t pol = evict_first_policy();
-    for (int64_t g0 = p_begin; g0 < p_end; g0 += U * GROUP) {
+    for (int64_t g0 = st.p_begin; g0 < st.p_end; g0 += U * GROUP) {
         typename F::Raw raw[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) raw[u] = F::load(d, g0 + u * GROUP + lane * PPL, NEED_W, pol);
+        for (int u = 0; u < U; ++u) raw[u] = F::load(d, g0 + u * GROUP + lane * F::PPL, NEED_W, pol);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t gb = g0 + u * GROUP;
-            if (gb >= p_end) break;
-            if (gb + GROUP <= seg_end) {
-#pragma unroll
-                for (int k = 0; k < PPL; ++k) {
-                    float x1, y1, x2, y2, w;
-                    F::get(raw[u], k, x1, y1, x2, y2, w);
-                    body.point(k, epi(E, x1, y1, x2, y2), x1, y1, x2, y2, w);
-                }
-            } else {
-                int64_t lo = gb;
-                const int64_t g_end = min(gb + GROUP, p_end);
-                while (true) {
-                    const int64_t hi = min(seg_end, p_end);
-#pragma unroll
-                    for (int k = 0; k < PPL; ++k) {
-                        const int64_t q = gb + lane * PPL + k;
-                        if (q >= lo && q < hi) {
-                            float x1, y1, x2, y2, w;
-                            F::get(raw[u], k, x1, y1, x2, y2, w);
-                            body.point(k, epi(E, x1, y1, x2, y2), x1, y1, x2, y2, w);
-                        }
-                    }
-                    if (seg_end >= g_end) break;
-                    body.segment_end(seg, r, lane, false);
-                    lo = seg_end;
-                    ++seg;
-                    seg_end = d.pair_off[seg + 1];
-                    load_E(d.geo, seg, E);
-                    body.segment_begin(seg);
-                }
-            }
-            body.group_done(gb, p_end, lane);
+            if (gb >= st.p_end) break;
+            walk_group<STORE>(d, st, raw[u], gb, r, lane, body);
         }
     }
-    body.segment_end(seg, r, lane, true);
+    body.segment_end(st.seg, r, lane, true);
+}
+
+// The same walk with the range staged in shared memory by asynchronous copies, a chunk of 4 groups
+// (2 KB of keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the
+// launch before this one; the first S chunks are requested ahead of it, so they arrive while that
+// launch finishes. (Keypoints are static. Weights are written at least two launches earlier: a pass
+// that writes them is followed by the camera step, which lets this launch start only after its own
+// wait for that pass.)
+constexpr int STAGE_GROUPS = 4;
+constexpr int STAGE_BYTES = STAGE_GROUPS * 32 * (16 + 4);
+
+__device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int STORE, bool NEED_W, int S, class Body, class Before>
+__device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, int lane, Body &body, unsigned char *stage,
+                                                  Before before) {
+    using F = Fmt<STORE>;
+    constexpr int GROUP = 32 * F::PPL;
+    constexpr int CHUNK = STAGE_GROUPS * GROUP;
+    static_assert(WR % CHUNK == 0, "range must be whole chunks");
+    WalkState st(d, r);
+    const int n_chunks = (int)((st.p_end - st.p_begin + CHUNK - 1) / CHUNK);
+    const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + st.p_begin * (16 / F::PPL);
+    const unsigned char *wp = static_cast<const unsigned char *>(d.w) + st.p_begin * (4 / F::PPL);
+    auto request = [&](int c) {
+        if (c < n_chunks) {
+            unsigned char *dst = stage + (c % S) * STAGE_BYTES;
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u)
+                cp_async16(dst + (u * 32 + lane) * 16, kp + (size_t)c * (STAGE_GROUPS * 512) + (u * 32 + lane) * 16);
+            if (NEED_W) cp_async16(dst + STAGE_GROUPS * 512 + lane * 16, wp + (size_t)c * (STAGE_GROUPS * 128) + lane * 16);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < S; ++c) request(c);
+    before();
+    load_E(d.geo, st.seg, st.E);
+    body.segment_begin(st.seg);
+    for (int c = 0; c < n_chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
+        __syncwarp();   // a lane's weights were copied by another lane
+        const unsigned char *src = stage + (c % S) * STAGE_BYTES;
+#pragma unroll
+        for (int u = 0; u < STAGE_GROUPS; ++u) {
+            const int64_t gb = st.p_begin + (int64_t)c * CHUNK + u * GROUP;
+            if (gb >= st.p_end) break;
+            typename F::Raw raw;
+            raw.kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
+            raw.w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
+            walk_group<STORE>(d, st, raw, gb, r, lane, body);
+        }
+        if (S < WR / CHUNK) __syncwarp();   // every lane has read the chunk before it is overwritten
+        request(c + S);
+    }
+    body.segment_end(st.seg, r, lane, true);
 }
 
 // ---- packed FP32 pairs -----------------------------------------------------------------------------
@@ -440,10 +518,10 @@ __device__ __forceinline__ void pair_geometry(const DevProblem &d, int n, int i,
 // launch that finishes a step produces the same bits.
 constexpr int FIN_THREADS = 256;
 
+// `red` is shared memory for FIN_THREADS doubles.
 template <int NT = FIN_THREADS>
-__device__ __forceinline__ void finish_step(const DevProblem &d, int n_loss, int count) {
+__device__ __forceinline__ void finish_step(const DevProblem &d, int n_loss, int count, double *red) {
     static_assert(FIN_THREADS % NT == 0, "block must divide FIN_THREADS");
-    __shared__ double red[FIN_THREADS];
 #pragma unroll
     for (int v = threadIdx.x; v < FIN_THREADS; v += NT) {
         double s = 0.0;
