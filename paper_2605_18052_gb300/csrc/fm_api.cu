@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "fm_grid.cuh"
 #include "fm_internal.cuh"
 
 using namespace fm;
@@ -52,6 +53,7 @@ struct fm_problem {
     double lr_focal = 1e-3;               // Adam step size of rho = log(f0/f)
     bool quad_alloc = false;              // d.qslots, d.quad, d.pair_rec allocated
     bool quad_valid = false;              // d.quad holds the form of the current weights
+    bool quad_persistent = false;         // the cameras fit the persistent steps on the form
     cudaGraphExec_t qgraph = nullptr, qgraph8 = nullptr;  // quadratic-path iterations
     // timing events per timed pass (fm_pass_time), pairs (start, end)
     std::vector<cudaEvent_t> tev[FM_NUM_PASSES];
@@ -93,6 +95,12 @@ fm_status check_device_errors(fm_problem *p) {
     unsigned err = 0;
     FM_CUDA(cudaMemcpyAsync(&err, p->d.err, sizeof(unsigned), cudaMemcpyDeviceToHost, p->s));
     FM_CUDA(cudaStreamSynchronize(p->s));
+    if (err & ERR_GRID) {
+        FM_CUDA(cudaMemsetAsync(p->d.err, 0, sizeof(unsigned), p->s));
+        FM_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
+        FM_CUDA(cudaStreamSynchronize(p->s));
+        return fail(FM_ECUDA, "a grid barrier ran into its limit");
+    }
     if (err & (ERR_DEGENERATE | ERR_NONFINITE)) {
         FM_CUDA(cudaMemsetAsync(p->d.err, 0, sizeof(unsigned), p->s));
         FM_CUDA(cudaStreamSynchronize(p->s));
@@ -1013,6 +1021,11 @@ fm_status quad_prepare(fm_problem *p) {
     FM_CUDA(dalloc(p, &p->d.qslots, (size_t)QSLOT * ((size_t)p->d.n_pairs + p->d.n_ranges)));
     FM_CUDA(dalloc(p, &p->d.quad, (size_t)QREC * p->d.n_pairs));
     FM_CUDA(dalloc(p, &p->d.cam_alt, (size_t)CAMREC * p->d.n_cams));
+    FM_CUDA(dalloc(p, &p->d.grid_state, GRID_STATE_WORDS));
+    FM_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
+    int blocks = 0;
+    FM_CUDA(quad_steps_capacity(p->d.refine_focal != 0, &blocks));
+    p->quad_persistent = camera_step_blocks(p->d) <= blocks;
     p->quad_alloc = true;
     return FM_OK;
 }
@@ -1082,7 +1095,11 @@ FM_API fm_status fm_step_quadratic(fm_problem *p, int32_t n_iters) {
     if (fm_status st = quad_check(p)) return st;
     if (n_iters == 0) return FM_OK;
     FM_CUDA(join_in(p));
-    if (!p->opt.use_graph) {
+    if (p->quad_persistent) {   // launches of bounded length (an iteration takes microseconds)
+        constexpr int QUAD_CHAIN = 4096;
+        for (int left = n_iters; left > 0; left -= QUAD_CHAIN)
+            FM_CUDA(launch_quad_steps(p->d, std::min(left, QUAD_CHAIN), p->s));
+    } else if (!p->opt.use_graph) {
         enqueue_iterations(p, p->s, false, n_iters, true);
         FM_CUDA(cudaGetLastError());
     } else {

@@ -77,10 +77,11 @@ struct GridBarrier {
 
 // cooperative launch (all blocks resident at once, or an error)
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_coop(void (*kernel)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
+static cudaError_t launch_coop(void (*kernel)(KArgs...), int grid, int block, int smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -92,11 +93,11 @@ static cudaError_t launch_coop(void (*kernel)(KArgs...), int grid, int block, cu
 
 // most blocks of a cooperative launch on the current device
 template <typename K>
-static cudaError_t coop_blocks(K kernel, int block, int *out) {
+static cudaError_t coop_blocks(K kernel, int block, int *out, int smem = 0) {
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, smem);
     *out = sms * per;
     if (e == cudaSuccess && *out < 1) e = cudaErrorLaunchOutOfResources;
     return e;

@@ -91,6 +91,7 @@ struct DevProblem {
     float *quad;            // n_pairs x QREC: c0, g0(9), M(36), e0(9), pad
     float *cam_alt;         // n_cams x CAMREC: second camera-record buffer of the fused step
     unsigned *pair_cnt;     // per pair: cameras updated by camera steps with the geometry phase
+    unsigned *grid_state;   // grid barriers of the persistent steps on the form
 };
 
 // c0 = sum w eps0^2, g0 = sum w eps0 a (9), M = the 36 distinct entries of W = sum w a a^T
@@ -119,6 +120,11 @@ void launch_quad_combine(const DevProblem &d, cudaStream_t s);
 // camera records read from cam_src and written to cam_dst (apply = false: gradient and loss only)
 void launch_quad_step(const DevProblem &d, int it, const float *cam_src, float *cam_dst, bool apply,
                       cudaStream_t s, bool pdl);
+
+// `iters` of these steps in one persistent launch, the loss total and the step count included; for
+// at most `blocks` camera-step blocks (quad_steps_capacity, which also prepares the kernel)
+cudaError_t quad_steps_capacity(bool focal, int *blocks);
+cudaError_t launch_quad_steps(const DevProblem &d, int iters, cudaStream_t s);
 
 // pair statistics of the current residuals (pstat), then features -> MLP -> weights, or the
 // features themselves (input order) for training

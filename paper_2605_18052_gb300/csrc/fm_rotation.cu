@@ -1060,9 +1060,9 @@ FM_API fm_status fm_rotation_initialize(fm_rotation *p, int32_t *cg_iters, doubl
     // column 1: sum ||x_j - R_p x_i||^2, anchored x_0 = e1; column 2: (1/|P|) sum ||y_j - R_p y_i||^2 +
     // (1/N) sum (x_k^T y_k)^2, anchored y_0 = e2
     RT_CUDA(cudaMemsetAsync(p->d.scal, 0, sizeof(double) * 8, p->s));
-    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, p->s, p->d, 0, 1.0, 0.0, (int)p->opt.cg_max_iters,
+    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 0, 1.0, 0.0, (int)p->opt.cg_max_iters,
                         p->opt.cg_tol));
-    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, p->s, p->d, 1, 1.0 / n_pairs, 1.0 / n_cams,
+    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 1, 1.0 / n_pairs, 1.0 / n_cams,
                         (int)p->opt.cg_max_iters, p->opt.cg_tol));
     double sc[8] = {};
     RT_CUDA(cudaMemcpyAsync(sc, p->d.scal, sizeof sc, cudaMemcpyDeviceToHost, p->s));
@@ -1129,7 +1129,7 @@ FM_API fm_status fm_rotation_step(fm_rotation *p, int32_t n_iters) {
     RT_CUDA(rjoin_in(p));
     // launches of bounded length (a step takes microseconds); use_graph makes no difference
     for (int left = n_iters; left > 0; left -= ROT_CHAIN)
-        RT_CUDA(launch_coop(k_rot_steps, p->step_grid, RT_CAMS * 32, p->s, p->d, std::min(left, ROT_CHAIN)));
+        RT_CUDA(launch_coop(k_rot_steps, p->step_grid, RT_CAMS * 32, 0, p->s, p->d, std::min(left, ROT_CHAIN)));
     RT_CUDA(rjoin_out(p));
     return FM_OK;
 }

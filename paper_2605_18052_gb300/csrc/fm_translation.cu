@@ -423,7 +423,7 @@ cudaError_t enqueue_steps(fm_translation *p, int iters) {
     const int64_t groups = cam_blocks(p->d);
     const int rc = (int)std::min<int64_t>(TR_RC, (groups * p->d.n_runs + p->step_grid - 1) / p->step_grid);
     const int64_t items = groups * ((p->d.n_runs + rc - 1) / rc);
-    return launch_coop(k_tr_steps, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, p->s, p->d, iters, rc);
+    return launch_coop(k_tr_steps, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, 0, p->s, p->d, iters, rc);
 }
 
 constexpr int TR_CHAIN = 4096;
