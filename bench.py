@@ -76,7 +76,7 @@ KERNEL_SOURCES = {
     "stream_loss": ("fm_kernels.cu", "fm_walk.cuh", "fm_internal.cuh"),
     "stream_reweight": ("fm_kernels.cu", "fm_walk.cuh", "fm_internal.cuh"),
     "quad_accumulate": ("fm_quad.cu", "fm_walk.cuh", "fm_internal.cuh"),
-    "learned_loss": ("fm_mlp.cu", "fm_tcgen05.cuh", "fm_walk.cuh", "fm_internal.cuh"),
+    "learned_loss": ("fm_mlp.cu", "fm_walk.cuh", "fm_internal.cuh"),
 }
 
 

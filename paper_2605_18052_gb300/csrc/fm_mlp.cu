@@ -6,10 +6,9 @@
 //
 // Numerics (shared by inference and training): features, weights and hidden activations are
 // rounded to BF16, every product is accumulated in FP32, biases are FP32.
-//   * inference runs inside the streaming walk on the tensor cores (mma.sync m16n8k16 BF16,
-//     FP32 accumulate): 16 point pairs per tile, 14 MMAs per tile; the FP32 accumulator
-//     fragments of one layer are the BF16 A fragments of the next after packing, so no
-//     shuffles are needed between layers;
+//   * inference runs inside the streaming walk on the tensor cores (mma.sync BF16, FP32
+//     accumulate): 16 point pairs per tile, 19 MMAs per tile; the FP32 accumulator fragments of
+//     one layer are the BF16 A fragments of the next after packing;
 //   * training runs tiles of samples as register-tiled FP32 products (forward and backward), sums
 //     the gradient per block in a fixed order and applies FP32 Adam to FP32 master parameters.
 #include <cuda_bf16.h>
@@ -19,7 +18,6 @@
 #include <cstring>
 #include <string>
 
-#include "fm_tcgen05.cuh"
 #include "fm_walk.cuh"
 
 namespace fm {
@@ -71,12 +69,24 @@ __global__ void k_pair_stats_combine(DevProblem d) {
     reinterpret_cast<float4 *>(d.pstat)[n] = make_float4(s0 / cnt, s1 / cnt, logf(cnt) * 0.1f, 0.f);
 }
 
-// ---- tensor-core MLP on 16-row tiles ------------------------------------------------------------
-__device__ __forceinline__ void mma_bf16(float *c, const unsigned *a, unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+// ---- the network on the tensor cores ---------------------------------------------------------------
+// c (16 x 8, FP32) += a (16 x 16, BF16) b (16 x 8), and the same with 8 columns of a
+__device__ __forceinline__ void mma_k16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
                  "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_k16_first(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+                 "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+                 : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+__device__ __forceinline__ void mma_k8(float (&c)[4], unsigned a0, unsigned a1, unsigned b0) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(b0));
 }
 
 __device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
@@ -92,97 +102,86 @@ __device__ __forceinline__ unsigned pack_relu_bf16(float lo, float hi) {
     return d;
 }
 
-// The per-lane B fragments and bias slices of the three layers.
-// For lane (g = lane / 4, t = lane % 4): B fragment of an n-tile j holds W[k][8j + g] for
-// k = 2t, 2t+1 (b0) and k = 2t+8, 2t+9 (b1); accumulator columns are 8j + 2t, 8j + 2t + 1.
-struct MlpFrag {
-    unsigned w1[4];        // layer 1: K = 8 (padded to 16: b1 = 0), 4 n-tiles
-    unsigned w2[2][4][2];  // layer 2: 2 k-tiles x 4 n-tiles x (b0, b1)
-    unsigned w3[2][2];     // layer 3: 2 k-tiles x (b0, b1), only column 0 real
-    float b1[4][2], b2[4][2], b3;
+// v = hi + mid + lo with three BF16 values (exact for FP32 v up to the last bit of lo)
+__device__ __forceinline__ void bf16_split3(float v, float &hi, float &mid, float &lo) {
+    hi = __bfloat162float(__float2bfloat16_rn(v));
+    mid = __bfloat162float(__float2bfloat16_rn(v - hi));
+    lo = v - hi - mid;
+}
+
+// The B operands of the three layers, in registers. For lane (g = lane / 4, t = lane % 4) and the n-tile
+// j the register b0 holds W[k][8j + g] for k = 2t, 2t + 1, b1 for k = 2t + 8, 2t + 9. A layer's bias
+// is three BF16 parts (hi + mid + lo = b) against three constant-1 columns of its A operand, so
+// that it is added inside the FP32 accumulation: layer 1 in columns 8..10 beside the 8 features, layers
+// 2 and 3 as a slice of 8 columns after their 32 inputs. The output layer has its vector in every column,
+// so that every lane of a row's quad gets the row's value.
+struct NetFrag {
+    unsigned w1[4][2], w2[2][4][2], b2[4], w3[2][2], b3;
+    unsigned ones;        // the lane's pair of the constant columns
+    __device__ __forceinline__ void load(const float *master, const __nv_bfloat16 *wbf, int lane) {
+        const int g = lane >> 2, t = lane & 3;
+        const __nv_bfloat16 *W1 = wbf, *W2 = wbf + MLP_IN * MLP_H, *W3 = W2 + MLP_H * MLP_H;
+        auto pk = [](__nv_bfloat16 lo, __nv_bfloat16 hi) {
+            return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
+        };
+        auto bias = [&](float v) {   // the lane's pair of (hi, mid, lo, 0, ...)
+            float h, m, l;
+            bf16_split3(v, h, m, l);
+            return t == 0 ? pack_bf16(h, m) : (t == 1 ? pack_bf16(l, 0.f) : 0u);
+        };
+        ones = t == 0 ? pack_bf16(1.f, 1.f) : (t == 1 ? pack_bf16(1.f, 0.f) : 0u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            w1[j][0] = pk(W1[(2 * t) * MLP_H + 8 * j + g], W1[(2 * t + 1) * MLP_H + 8 * j + g]);
+            w1[j][1] = bias(master[MLP_OFF_B1 + 8 * j + g]);
+            b2[j] = bias(master[MLP_OFF_B2 + 8 * j + g]);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = 16 * s + 8 * h + 2 * t;
+                    w2[s][j][h] = pk(W2[k * MLP_H + 8 * j + g], W2[(k + 1) * MLP_H + 8 * j + g]);
+                }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) w3[s][h] = pk(W3[16 * s + 8 * h + 2 * t], W3[16 * s + 8 * h + 2 * t + 1]);
+        b3 = bias(master[MLP_OFF_B3]);
+    }
+    // the network's logit of a tile's 16 rows: z0 of row g, z1 of row g + 8; f0, f1: the lane's pair of
+    // the features of those rows
+    __device__ __forceinline__ void tile(unsigned f0, unsigned f1, float &z0, float &z1) const {
+        const unsigned a1[4] = {f0, f1, ones, ones};
+        float h[4][4];
+        unsigned a[2][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_k16_first(h[j], a1, w1[j][0], w1[j][1]);
+        auto pack = [&]() {   // an accumulator tile of one layer is an A operand of the next
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                a[s][0] = pack_relu_bf16(h[2 * s][0], h[2 * s][1]);
+                a[s][1] = pack_relu_bf16(h[2 * s][2], h[2 * s][3]);
+                a[s][2] = pack_relu_bf16(h[2 * s + 1][0], h[2 * s + 1][1]);
+                a[s][3] = pack_relu_bf16(h[2 * s + 1][2], h[2 * s + 1][3]);
+            }
+        };
+        pack();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_k16_first(h[j], a[0], w2[0][j][0], w2[0][j][1]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_k16(h[j], a[1], w2[1][j][0], w2[1][j][1]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_k8(h[j], ones, ones, b2[j]);
+        pack();
+        float z[4];
+        mma_k16_first(z, a[0], w3[0][0], w3[0][1]);
+        mma_k16(z, a[1], w3[1][0], w3[1][1]);
+        mma_k8(z, ones, ones, b3);
+        z0 = z[0];
+        z1 = z[2];
+    }
 };
-
-__device__ __forceinline__ void load_frag(MlpFrag &f, const float *master, const __nv_bfloat16 *wbf, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    const __nv_bfloat16 *W1 = wbf, *W2 = wbf + MLP_IN * MLP_H, *W3 = W2 + MLP_H * MLP_H;
-    auto pk = [](__nv_bfloat16 lo, __nv_bfloat16 hi) {
-        return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
-    };
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        f.w1[j] = pk(W1[(2 * t) * MLP_H + 8 * j + g], W1[(2 * t + 1) * MLP_H + 8 * j + g]);
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const int k0 = 16 * kk + 2 * t;
-            f.w2[kk][j][0] = pk(W2[k0 * MLP_H + 8 * j + g], W2[(k0 + 1) * MLP_H + 8 * j + g]);
-            f.w2[kk][j][1] = pk(W2[(k0 + 8) * MLP_H + 8 * j + g], W2[(k0 + 9) * MLP_H + 8 * j + g]);
-        }
-        f.b1[j][0] = master[MLP_OFF_B1 + 8 * j + 2 * t];
-        f.b1[j][1] = master[MLP_OFF_B1 + 8 * j + 2 * t + 1];
-        f.b2[j][0] = master[MLP_OFF_B2 + 8 * j + 2 * t];
-        f.b2[j][1] = master[MLP_OFF_B2 + 8 * j + 2 * t + 1];
-    }
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-        const int k0 = 16 * kk + 2 * t;
-        f.w3[kk][0] = g == 0 ? pk(W3[k0], W3[k0 + 1]) : 0u;
-        f.w3[kk][1] = g == 0 ? pk(W3[k0 + 8], W3[k0 + 9]) : 0u;
-    }
-    f.b3 = master[MLP_OFF_B3];
-}
-
-// p = sigmoid(MLP(x)) for `ntiles` tiles of 16 rows of xs (BF16, 8 features per row)
-__device__ __forceinline__ void mlp_tiles(const MlpFrag &f, const __nv_bfloat16 (*xs)[MLP_IN], float *ps,
-                                          int ntiles, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    for (int tile = 0; tile < ntiles; ++tile) {
-        const int r0 = 16 * tile + g, r1 = r0 + 8;
-        const unsigned a1[4] = {*reinterpret_cast<const unsigned *>(&xs[r0][2 * t]),
-                                *reinterpret_cast<const unsigned *>(&xs[r1][2 * t]), 0u, 0u};
-        float h1[4][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            h1[j][0] = f.b1[j][0];
-            h1[j][1] = f.b1[j][1];
-            h1[j][2] = f.b1[j][0];
-            h1[j][3] = f.b1[j][1];
-            mma_bf16(h1[j], a1, f.w1[j], 0u);
-        }
-        unsigned a2[2][4];
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            a2[kk][0] = pack_relu_bf16(h1[2 * kk][0], h1[2 * kk][1]);
-            a2[kk][1] = pack_relu_bf16(h1[2 * kk][2], h1[2 * kk][3]);
-            a2[kk][2] = pack_relu_bf16(h1[2 * kk + 1][0], h1[2 * kk + 1][1]);
-            a2[kk][3] = pack_relu_bf16(h1[2 * kk + 1][2], h1[2 * kk + 1][3]);
-        }
-        float h2[4][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            h2[j][0] = f.b2[j][0];
-            h2[j][1] = f.b2[j][1];
-            h2[j][2] = f.b2[j][0];
-            h2[j][3] = f.b2[j][1];
-            mma_bf16(h2[j], a2[0], f.w2[0][j][0], f.w2[0][j][1]);
-            mma_bf16(h2[j], a2[1], f.w2[1][j][0], f.w2[1][j][1]);
-        }
-        unsigned a3[2][4];
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            a3[kk][0] = pack_relu_bf16(h2[2 * kk][0], h2[2 * kk][1]);
-            a3[kk][1] = pack_relu_bf16(h2[2 * kk][2], h2[2 * kk][3]);
-            a3[kk][2] = pack_relu_bf16(h2[2 * kk + 1][0], h2[2 * kk + 1][1]);
-            a3[kk][3] = pack_relu_bf16(h2[2 * kk + 1][2], h2[2 * kk + 1][3]);
-        }
-        float z[4] = {t == 0 ? f.b3 : 0.f, 0.f, t == 0 ? f.b3 : 0.f, 0.f};
-        mma_bf16(z, a3[0], f.w3[0][0], f.w3[0][1]);
-        mma_bf16(z, a3[1], f.w3[1][0], f.w3[1][1]);
-        if (t == 0) {
-            ps[r0] = __frcp_rn(1.f + __expf(-z[0]));
-            ps[r1] = __frcp_rn(1.f + __expf(-z[2]));
-        }
-    }
-}
 
 // learned IRLS weight p / max(|eps|, delta) (fast quotient, within 2 ulp; every learned kernel
 // uses this one expression, so the fused and separate passes agree bit for bit)
@@ -194,21 +193,16 @@ __device__ __forceinline__ float learned_weight(float p, float ae, float delta) 
 //  0 log(|e|+1e-6) - log(tau)      1 log(|e|+1e-6) - pair mean log    2 log(|e_prev|+1e-6) - log(|e|+1e-6)
 //  3 match score                   4 pair fraction with |e| <= tau    5 log(pair count) / 10
 //  6 round / 10                    7 log(|e_prev|+1e-6) - log(tau)
-template <int STORE, bool COLLECT>
-struct LearnedBody {
+template <int STORE>
+struct CollectBody {
     static constexpr int PPL = Fmt<STORE>::PPL;
-    static constexpr int GROUP = 32 * PPL;
     const DevProblem &d;
-    float log_tau, tau_cap, delta, wscale, round_f;
+    float log_tau, round_f;
     int hist_valid;
     float st_mean, st_frac, st_cnt;
-    float ae[PPL], le[PPL], sm[PPL], sf[PPL], sc[PPL];
-    unsigned kept;
-    MlpFrag frag;     // the network's B fragments, in registers
-    __nv_bfloat16 (*xs)[MLP_IN];
-    float *ps;
+    float le[PPL], sm[PPL], sf[PPL], sc[PPL];
     __nv_bfloat16 *feat_out;
-    __device__ LearnedBody(const DevProblem &dd) : d(dd), kept(0) {}
+    __device__ CollectBody(const DevProblem &dd) : d(dd) {}
     __device__ __forceinline__ void segment_begin(int seg) {
         const float4 p = reinterpret_cast<const float4 *>(d.pstat)[seg];
         st_mean = p.x;
@@ -216,8 +210,7 @@ struct LearnedBody {
         st_cnt = p.z;
     }
     __device__ __forceinline__ void point(int k, float e, float, float, float, float, float) {
-        ae[k] = fabsf(e);
-        le[k] = __logf(ae[k] + LOG_FLOOR);
+        le[k] = __logf(fabsf(e) + LOG_FLOOR);
         sm[k] = st_mean;
         sf[k] = st_frac;
         sc[k] = st_cnt;
@@ -233,604 +226,259 @@ struct LearnedBody {
         }
 #pragma unroll
         for (int k = 0; k < PPL; ++k) {
-            float f[MLP_IN];
-            f[0] = le[k] - log_tau;
-            f[1] = le[k] - sm[k];
-            f[2] = lp[k] - le[k];
-            f[3] = sco[k];
-            f[4] = sf[k];
-            f[5] = sc[k];
-            f[6] = round_f;
-            f[7] = lp[k] - log_tau;
-            __align__(16) __nv_bfloat16 fb[MLP_IN];
-#pragma unroll
-            for (int i = 0; i < MLP_IN; ++i) fb[i] = __float2bfloat16_rn(f[i]);
-            if (COLLECT) {
-                if (q + k < p_end) {
-                    const int64_t dst = d.perm ? d.perm[q + k] : q + k;
-                    *reinterpret_cast<uint4 *>(feat_out + dst * MLP_IN) = *reinterpret_cast<const uint4 *>(fb);
-                }
-            } else {
-                *reinterpret_cast<uint4 *>(xs[lane * PPL + k]) = *reinterpret_cast<const uint4 *>(fb);
-            }
-        }
-        if (!COLLECT) {
-            __syncwarp();
-            mlp_tiles(frag, xs, ps, GROUP / 16, lane);
-            __syncwarp();
-            float w[PPL];
-#pragma unroll
-            for (int k = 0; k < PPL; ++k) {
-                const bool in = q + k < p_end && ae[k] <= tau_cap;
-                w[k] = in ? learned_weight(ps[lane * PPL + k], ae[k], delta) : 0.f;
-                kept += in ? 1u : 0u;
-            }
-            if (STORE == FM_STORE_FP32) {
-                static_cast<float *>(d.w)[q] = w[0];
-            } else {
-                reinterpret_cast<__half2 *>(d.w)[q >> 1] = __floats2half2_rn(w[0] * wscale, w[PPL - 1] * wscale);
-            }
-            __syncwarp();
+            if (q + k >= p_end) continue;
+            const int64_t dst = d.perm ? d.perm[q + k] : q + k;
+            *reinterpret_cast<uint4 *>(feat_out + dst * MLP_IN) =
+                make_uint4(pack_bf16(le[k] - log_tau, le[k] - sm[k]), pack_bf16(lp[k] - le[k], sco[k]),
+                           pack_bf16(sf[k], sc[k]), pack_bf16(round_f, lp[k] - log_tau));
+            d.le_hist[q + k] = __float2half_rn(le[k]);
         }
 #pragma unroll
-        for (int k = 0; k < PPL; ++k)
-            if (q + k < p_end) d.le_hist[q + k] = __float2half_rn(le[k]);
-#pragma unroll
-        for (int k = 0; k < PPL; ++k) ae[k] = le[k] = 0.f;
+        for (int k = 0; k < PPL; ++k) le[k] = 0.f;
     }
 };
 
-template <int STORE, bool COLLECT>
-__global__ void __launch_bounds__(CTA_WARPS * 32, 2)
-k_learned(DevProblem d, const float *master, const __nv_bfloat16 *wbf, float tau, float tau_cap,
-          int round, int hist_valid, __nv_bfloat16 *feat_out) {
-    constexpr int GROUP = 32 * Fmt<STORE>::PPL;
-    __shared__ __align__(16) __nv_bfloat16 xs[CTA_WARPS][GROUP][MLP_IN];
-    __shared__ float ps[CTA_WARPS][GROUP];
-    __shared__ unsigned cta_kept;
-    if (threadIdx.x == 0) cta_kept = 0;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    const int r = blockIdx.x * CTA_WARPS + w;
-    if (r < d.n_ranges) {
-        LearnedBody<STORE, COLLECT> body(d);
-        if (!COLLECT) load_frag(body.frag, master, wbf, lane);
-        body.log_tau = __logf(tau);
-        body.tau_cap = tau_cap;
-        body.delta = (float)d.delta;
-        body.wscale = d.w_scale;
-        body.round_f = round * 0.1f;
-        body.hist_valid = hist_valid;
-        body.xs = xs[w];
-        body.ps = ps[w];
-        body.feat_out = feat_out;
-        // one group in flight: the fragments take the registers a deeper unroll would use
-        walk_range<STORE, false, LearnedBody<STORE, COLLECT>, 1>(d, r, lane, body);
-        unsigned k = body.kept;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-        if (lane == 0) atomicAdd(&cta_kept, k);
-    }
-    __syncthreads();
-    if (!COLLECT && threadIdx.x == 0 && cta_kept) atomicAdd(d.counter, (unsigned long long)cta_kept);
-}
-
-// ---- the learned reweighting fused with the round's first loss + adjoint pass -------------------
-// Same arithmetic as k_learned followed by k_stream_loss, one read of the keypoints instead of
-// two. Every group of 32 * PPL point pairs is handled in two phases:
-//   A: residual, features (with the statistics of each point pair's own image pair), the MLP on
-//      the group's rows (tensor cores, mma.sync), the weight (written, FP16-quantised for FP16
-//      storage), the residual history;
-//   B: the loss and adjoint sums of the group with those weights, closing every image pair that
-//      ended inside the group (warp butterfly into its slot n + r, as the streaming pass does).
-// Phase A walks the group's image pairs forward; phase B revisits the same image pairs from the
-// group's first one. The network's B fragments stay in registers for the whole kernel (reading
-// them from shared memory for every 16-row tile would move about 330 B of shared memory per
-// point pair); to make room, the keypoints stay packed between the phases and the current image
-// pair's E'_n and statistics are reloaded (from L1) at the start of every group.
 template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32, 2)
-k_learned_loss(DevProblem d, const float *master, const __nv_bfloat16 *wbf, float tau, float tau_cap, int round,
-               int hist_valid) {
-    using F = Fmt<STORE>;
-    constexpr int PPL = F::PPL;
-    constexpr int GROUP = 32 * PPL;
-    __shared__ __align__(16) __nv_bfloat16 xs[CTA_WARPS][GROUP][MLP_IN];
-    __shared__ float ps[CTA_WARPS][GROUP];
-    __shared__ unsigned cta_kept;
-    if (threadIdx.x == 0) cta_kept = 0;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    MlpFrag frag;
-    load_frag(frag, master, wbf, lane);
-    pdl_wait();     // pair geometry and statistics of this pass
-    pdl_trigger();
-    __syncthreads();
-    const int r = blockIdx.x * CTA_WARPS + wid;
-    unsigned kept = 0;
-    if (r < d.n_ranges) {
-        const float log_tau = __logf(tau), delta = (float)d.delta, wscale = d.w_scale, round_f = round * 0.1f;
-        const int64_t p_begin = (int64_t)r * WR;
-        const int64_t p_end = min(p_begin + (int64_t)WR, d.n_pp);
-        int seg = d.range_pair[r];
-        int64_t seg_end = d.pair_off[seg + 1];
-        LossBody<MODE_LOSS_IRLS> loss(d);
-        const uint64_t pol = evict_first_policy();
-        for (int64_t gb = p_begin; gb < p_end; gb += GROUP) {
-            const int64_t q0 = gb + lane * PPL;
-            const typename F::Raw raw = F::load(d, q0, false, pol);
-            // score and history of the lane's point pairs (PPL consecutive halves)
-            float sco[PPL], lp[PPL];
-            if (PPL == 2) {
-                const float2 sv = __half22float2(reinterpret_cast<const __half2 *>(d.score)[q0 >> 1]);
-                const float2 hv = __half22float2(reinterpret_cast<const __half2 *>(d.le_hist)[q0 >> 1]);
-                sco[0] = sv.x;
-                sco[PPL - 1] = sv.y;
-                lp[0] = hv.x;
-                lp[PPL - 1] = hv.y;
-            } else {
-                sco[0] = __half2float(d.score[q0]);
-                lp[0] = __half2float(d.le_hist[q0]);
-            }
-            float e[PPL], le[PPL];
-#pragma unroll
-            for (int k = 0; k < PPL; ++k) e[k] = le[k] = 0.f;
-            // phase A
-            const int seg0 = seg;
-            const int64_t seg0_end = seg_end;
-            const int64_t g_end = min(gb + GROUP, p_end);
-            float E[9];
-            load_E(d.geo, seg, E);
-            float4 st = reinterpret_cast<const float4 *>(d.pstat)[seg];
-            int64_t lo = gb;
-            while (true) {
-                const int64_t hi = min(seg_end, p_end);
-#pragma unroll
-                for (int k = 0; k < PPL; ++k) {
-                    const int64_t q = q0 + k;
-                    if (q >= lo && q < hi) {
-                        float x1, y1, x2, y2, unused;
-                        F::get(raw, k, x1, y1, x2, y2, unused);
-                        e[k] = epi(E, x1, y1, x2, y2);
-                        le[k] = __logf(fabsf(e[k]) + LOG_FLOOR);
-                        const float lpk = hist_valid ? lp[k] : le[k];
-                        float f[MLP_IN];
-                        f[0] = le[k] - log_tau;
-                        f[1] = le[k] - st.x;
-                        f[2] = lpk - le[k];
-                        f[3] = sco[k];
-                        f[4] = st.y;
-                        f[5] = st.z;
-                        f[6] = round_f;
-                        f[7] = lpk - log_tau;
-                        __align__(16) __nv_bfloat16 fb[MLP_IN];
-#pragma unroll
-                        for (int i = 0; i < MLP_IN; ++i) fb[i] = __float2bfloat16_rn(f[i]);
-                        *reinterpret_cast<uint4 *>(xs[wid][lane * PPL + k]) = *reinterpret_cast<const uint4 *>(fb);
-                    }
-                }
-                if (seg_end >= g_end) break;
-                lo = seg_end;
-                ++seg;
-                seg_end = d.pair_off[seg + 1];
-                load_E(d.geo, seg, E);
-                st = reinterpret_cast<const float4 *>(d.pstat)[seg];
-            }
-#pragma unroll
-            for (int k = 0; k < PPL; ++k)   // rows past the end of the range: any finite input
-                if (q0 + k >= p_end) *reinterpret_cast<uint4 *>(xs[wid][lane * PPL + k]) = make_uint4(0u, 0u, 0u, 0u);
-            __syncwarp();
-            mlp_tiles(frag, xs[wid], ps[wid], GROUP / 16, lane);
-            __syncwarp();
-            float w[PPL];
-#pragma unroll
-            for (int k = 0; k < PPL; ++k) {
-                const float ae = fabsf(e[k]);
-                const bool in = q0 + k < p_end && ae <= tau_cap;
-                const float wf = in ? learned_weight(ps[wid][lane * PPL + k], ae, delta) : 0.f;
-                w[k] = STORE == FM_STORE_FP32 ? wf : __half2float(__float2half_rn(wf * wscale));
-                kept += in ? 1u : 0u;
-            }
-            if (STORE == FM_STORE_FP32) {
-                static_cast<float *>(d.w)[q0] = w[0];
-                if (q0 < p_end) d.le_hist[q0] = __float2half_rn(le[0]);
-            } else {
-                reinterpret_cast<__half2 *>(d.w)[q0 >> 1] = __floats2half2_rn(w[0], w[PPL - 1]);
-                const __half2 hv = __floats2half2_rn(le[0], le[PPL - 1]);
-                if (q0 + 1 < p_end) reinterpret_cast<__half2 *>(d.le_hist)[q0 >> 1] = hv;
-                else if (q0 < p_end) d.le_hist[q0] = __low2half(hv);
-            }
-            __syncwarp();
-            // phase B
-            int sb = seg0;
-            int64_t sb_end = seg0_end;
-            lo = gb;
-            while (true) {
-                const int64_t hi = min(sb_end, p_end);
-#pragma unroll
-                for (int k = 0; k < PPL; ++k) {
-                    const int64_t q = q0 + k;
-                    if (q >= lo && q < hi) {
-                        float x1, y1, x2, y2, unused;
-                        F::get(raw, k, x1, y1, x2, y2, unused);
-                        loss.point(k, e[k], x1, y1, x2, y2, w[k]);
-                    }
-                }
-                if (sb == seg) break;
-                loss.segment_end(sb, r, lane, false);
-                lo = sb_end;
-                ++sb;
-                sb_end = d.pair_off[sb + 1];
-            }
-        }
-        loss.segment_end(seg, r, lane, true);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
-    if (lane == 0 && kept) atomicAdd(&cta_kept, kept);
-    __syncthreads();
-    if (threadIdx.x == 0 && cta_kept) atomicAdd(d.counter, (unsigned long long)cta_kept);
+__global__ void __launch_bounds__(CTA_WARPS * 32)
+k_collect_features(DevProblem d, float tau, int round, int hist_valid, __nv_bfloat16 *feat_out) {
+    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
+    if (r >= d.n_ranges) return;
+    CollectBody<STORE> body(d);
+    body.log_tau = __logf(tau);
+    body.round_f = round * 0.1f;
+    body.hist_valid = hist_valid;
+    body.feat_out = feat_out;
+    walk_range<STORE, false, CollectBody<STORE>, 1>(d, r, threadIdx.x & 31, body);
 }
 
-// ---- the learned reweighting on the fifth-generation tensor cores (tcgen05) ---------------------
-// A CTA is one warpgroup (4 warps); each warp streams its own warp range as in the other passes,
-// and for every group of 32 * PPL point pairs per warp the warpgroup's 128 x PPL rows go through
-// the network as MMAs of M = 128 rows with FP32 accumulators in TMEM (k = the lane's k-th point
-// pair of the group, one MMA row block per k):
-//   L1  D1[k] (128 x 32) = A1[k] (128 x 16: 8 features, three 1s, 5 zeros) . B1^T
-//        B1 (32 x 16) = W1^T with b1 in its columns 8..10 as three BF16 parts (hi + mid + lo = b1)
-//   L2  D2[k] (128 x 32) = A2[k] (128 x 48: bf16(relu(D1)), three 1s, zeros) . B2^T (W2^T, b2 parts)
-//   L3  D3[k] (128 x 16, column 0 used) = A3[k] (A2's layout, from D2) . B3^T (row 0: W3, b3 parts)
-// so the biases are added inside the FP32 accumulation and every row's epilogue is one TMEM load,
-// one ReLU-and-round instruction per two values and four 16-byte shared-memory stores. One thread
-// issues the MMAs and commits them to an mbarrier; the warpgroup waits on it (bounded: a wait that
-// runs out records ERR_NONFINITE and the warpgroup leaves the loop together).
-// Footprint (the pass is bound by the latency of the MMA round trips, so what matters is how many
-// row blocks an SM keeps in flight): D1, D2 and D3 of row block k share TMEM columns 32 k .. 32 k
-// + 31 (each layer's result is read before the next layer's MMA is issued), 64 columns per CTA;
-// A1 lives inside A2's buffer: the features take A2's first K core matrix and layer 1 reads its
-// second K core matrix from A2's fifth (the constant bias inputs), through the descriptor's
-// leading byte offset.
-// FUSE: also accumulate the loss + adjoint sums with the new weights (the round's first pass).
-constexpr int TC_THREADS = 128;
-constexpr uint32_t TC_COLS = 64;
-constexpr int TC_K1 = 16, TC_K2 = 48;      // padded K of layer 1 and of layers 2 and 3
-constexpr long long TC_WAIT_CYCLES = 2000000000LL;   // about one second
-
-struct TcSmem {
-    alignas(128) unsigned char a2[2][128 * TC_K2 * 2];
-    alignas(128) unsigned char b1[32 * TC_K1 * 2];
-    alignas(128) unsigned char b2[32 * TC_K2 * 2];
-    alignas(128) unsigned char b3[16 * TC_K2 * 2];
-    alignas(8) uint64_t mbar;
-    uint32_t tmem;
-    int fail;
-    unsigned kept;
-};
-
-__device__ __forceinline__ void put_bf16(unsigned char *base, uint32_t r, uint32_t k, uint32_t kp, float v) {
-    *reinterpret_cast<__nv_bfloat16 *>(base + tc_offset(r, k, kp)) = __float2bfloat16_rn(v);
-}
-
-// v = hi + mid + lo with three BF16 values (exact for FP32 v up to the last bit of lo)
-__device__ __forceinline__ void bf16_split3(float v, float &hi, float &mid, float &lo) {
-    hi = __bfloat162float(__float2bfloat16_rn(v));
-    mid = __bfloat162float(__float2bfloat16_rn(v - hi));
-    lo = v - hi - mid;
-}
-
-// the network's B operands and the constant columns of the A operands, by the whole CTA
-__device__ __forceinline__ void tc_setup(TcSmem &sm, const float *master, const __nv_bfloat16 *wbf) {
-    const int tid = threadIdx.x;
-    const __nv_bfloat16 *W1 = wbf, *W2 = wbf + MLP_IN * MLP_H, *W3 = W2 + MLP_H * MLP_H;
-    for (int i = tid; i < 32 * TC_K1; i += TC_THREADS) {
-        const int n = i / TC_K1, k = i % TC_K1;
-        float v = 0.f;
-        if (k < MLP_IN) v = __bfloat162float(W1[k * MLP_H + n]);
-        else if (k < MLP_IN + 3) {
-            float h, m, l;
-            bf16_split3(master[MLP_OFF_B1 + n], h, m, l);
-            v = k == MLP_IN ? h : (k == MLP_IN + 1 ? m : l);
-        }
-        put_bf16(sm.b1, n, k, TC_K1, v);
-    }
-    for (int i = tid; i < 32 * TC_K2; i += TC_THREADS) {
-        const int n = i / TC_K2, k = i % TC_K2;
-        float v = 0.f;
-        if (k < MLP_H) v = __bfloat162float(W2[k * MLP_H + n]);
-        else if (k < MLP_H + 3) {
-            float h, m, l;
-            bf16_split3(master[MLP_OFF_B2 + n], h, m, l);
-            v = k == MLP_H ? h : (k == MLP_H + 1 ? m : l);
-        }
-        put_bf16(sm.b2, n, k, TC_K2, v);
-    }
-    for (int i = tid; i < 16 * TC_K2; i += TC_THREADS) {
-        const int n = i / TC_K2, k = i % TC_K2;
-        float v = 0.f;
-        if (n == 0 && k < MLP_H) v = __bfloat162float(W3[k]);
-        else if (n == 0 && k < MLP_H + 3) {
-            float h, m, l;
-            bf16_split3(master[MLP_OFF_B3], h, m, l);
-            v = k == MLP_H ? h : (k == MLP_H + 1 ? m : l);
-        }
-        put_bf16(sm.b3, n, k, TC_K2, v);
-    }
-    // A2 columns 32..47: three 1s (the bias inputs of every layer) and zeros
-    for (int i = tid; i < 2 * 128 * (TC_K2 - MLP_H); i += TC_THREADS) {
-        const int kk = i / (128 * (TC_K2 - MLP_H)), rem = i % (128 * (TC_K2 - MLP_H));
-        const int r = rem / (TC_K2 - MLP_H), k = MLP_H + rem % (TC_K2 - MLP_H);
-        put_bf16(sm.a2[kk], r, k, TC_K2, k < MLP_H + 3 ? 1.f : 0.f);
-    }
-}
-
-// bf16(relu(x)) of 32 accumulator columns into row `row` of an A operand (K padded to TC_K2)
-__device__ __forceinline__ void tc_relu_row(unsigned char *a, int row, const uint32_t (&acc)[32]) {
-#pragma unroll
-    for (int kb = 0; kb < 4; ++kb) {
-        uint4 v;
-        v.x = pack_relu_bf16(__uint_as_float(acc[8 * kb + 0]), __uint_as_float(acc[8 * kb + 1]));
-        v.y = pack_relu_bf16(__uint_as_float(acc[8 * kb + 2]), __uint_as_float(acc[8 * kb + 3]));
-        v.z = pack_relu_bf16(__uint_as_float(acc[8 * kb + 4]), __uint_as_float(acc[8 * kb + 5]));
-        v.w = pack_relu_bf16(__uint_as_float(acc[8 * kb + 6]), __uint_as_float(acc[8 * kb + 7]));
-        *reinterpret_cast<uint4 *>(a + tc_offset(row, 8 * kb, TC_K2)) = v;
-    }
-}
-
-// all warpgroup threads: make the A rows visible to the tensor core and hand over to the issuer;
-// returns whether an earlier wait ran out (then everybody leaves)
-__device__ __forceinline__ bool tc_handover(TcSmem &sm) {
-    fence_smem_async();
-    tc_fence_before_sync();
-    named_sync(1, TC_THREADS);
-    return sm.fail != 0;
-}
-
-__device__ __forceinline__ void tc_wait(TcSmem &sm, uint32_t &phase) {
-    if (!mbar_wait(smem_addr(&sm.mbar), phase, TC_WAIT_CYCLES)) sm.fail = 1;
-    phase ^= 1u;
-    tc_fence_after_sync();
-}
+// ---- the learned reweighting -------------------------------------------------------------------------
+// A warp streams its range in blocks of 64 point pairs, two per lane: features, the network's logit, the
+// weight (written, and rounded as the storage keeps it), the residual history; FUSE: also the loss
+// and adjoint sums with the new weights (the round's first pass), closing every image pair that ends in
+// the block, in the streaming pass's order.
+// The network runs on mma.sync tiles of 16 rows, four per block, wholly in registers: the accumulators
+// of one layer, rounded by one instruction per two values, are the A operand of the next, the weights
+// stay in 34 registers for the whole range, and there is no barrier. Row g of tile T is the first point
+// pair of lane 4 g + T and row g + 8 its second, so that only the features change lanes (one 16-byte
+// shared store per point pair, one ldmatrix per two tiles) and a lane finds its own logits in its
+// accumulators. On fifth-generation tensor memory (tcgen05, M = 128 over a warpgroup) the same products
+// are an eighth of the tensor work, but three MMA round trips through shared memory, an mbarrier and
+// TMEM per 128 rows, and 296 instructions per point pair: 837 us on 48.9 M point pairs (FP16,
+// fused), 127 us on 3.1 M (FP32, weights only). Both give the same bits (each product of 16 terms and
+// its FP32 accumulation are rounded alike; compared on 3.3 M random outputs). Now 618 and 56 us, at 240
+// instructions per point pair; the tensor pipe is 62% busy (8.3 cycles per mma.sync and
+// sub-partition: 415 us on 48.9 M if it never waited), the rest is the latency of a block's phases with
+// four warps per sub-partition. Two tiles interleaved by hand, with 4 or 3 blocks per SM, changed
+// nothing (619, 637 us); 5 blocks spill (818 us).
+constexpr int LP_WARPS = 4;
+constexpr int LP_BLOCK = 64;                // point pairs per warp and step
+constexpr int LP_STAGES = 4;                // steps whose loads are in flight
+constexpr int LP_STAGE_BYTES = LP_BLOCK * (16 + 2 + 2);   // keypoints (FP32 size), scores, history
 
 template <int STORE, bool FUSE>
-__global__ void __launch_bounds__(TC_THREADS, 5)
-k_learned_tc(DevProblem d, const float *master, const __nv_bfloat16 *wbf, float tau, float tau_cap, int round,
-             int hist_valid) {
+__global__ void __launch_bounds__(LP_WARPS * 32, 4)
+k_learned_pass(DevProblem d, const float *master, const __nv_bfloat16 *wbf, float tau, float tau_cap, int round,
+               int hist_valid) {
     using F = Fmt<STORE>;
-    constexpr int PPL = F::PPL;
-    constexpr int GROUP = 32 * PPL;
-    constexpr int NG = WR / GROUP;
-    __shared__ TcSmem sm;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int row = 32 * wid + lane;
-    if (wid == 0) {
-        tmem_alloc(smem_addr(&sm.tmem), TC_COLS);
-        tmem_relinquish();
-    }
-    if (threadIdx.x == 0) {
-        mbar_init(smem_addr(&sm.mbar), 1);
-        sm.fail = 0;
-        sm.kept = 0;
-    }
-    tc_setup(sm, master, wbf);
+    constexpr int PPL = F::PPL, SUBS = 2 / PPL, GROUP = 32 * PPL;   // SUBS groups of GROUP point pairs per step
+    constexpr int KP_BYTES = LP_BLOCK * (STORE == FM_STORE_FP32 ? 16 : 8);
+    __shared__ __align__(16) unsigned char s_stage[LP_WARPS][LP_STAGES][LP_STAGE_BYTES];
+    __shared__ __align__(16) uint4 s_feat[LP_WARPS][2 * 36];        // [slot][tile][row], 9 rows a tile
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 3;
+    NetFrag net;
+    net.load(master, wbf, lane);
     pdl_wait();     // pair geometry and statistics of this pass
     pdl_trigger();
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tm = sm.tmem + ((uint32_t)(32 * wid) << 16);   // this warp's TMEM lanes
-    const uint32_t id1 = tc_idesc_bf16(128, 32), id3 = tc_idesc_bf16(128, 16);
-    // operand descriptors (loop-invariant; K slice sl of layers 2 and 3 adds sl * 2 * TC_LBO to
-    // the start address field, i.e. sl * 16 in 16-byte units)
-    const uint64_t dA1[2] = {tc_desc(smem_addr(sm.a2[0]), TC_K2 * 16, 4 * TC_LBO),
-                             tc_desc(smem_addr(sm.a2[1]), TC_K2 * 16, 4 * TC_LBO)};
-    const uint64_t dA2[2] = {tc_desc(smem_addr(sm.a2[0]), TC_K2 * 16), tc_desc(smem_addr(sm.a2[1]), TC_K2 * 16)};
-    const uint64_t dB1 = tc_desc(smem_addr(sm.b1), TC_K1 * 16), dB2 = tc_desc(smem_addr(sm.b2), TC_K2 * 16),
-                   dB3 = tc_desc(smem_addr(sm.b3), TC_K2 * 16);
-    constexpr uint64_t SLICE = (2 * TC_LBO) >> 4;
-    uint32_t phase = 0;
-
-    const int r = blockIdx.x * 4 + wid;
-    const bool r_ok = r < d.n_ranges;
+    const int r = blockIdx.x * LP_WARPS + warp;
+    if (r >= d.n_ranges) return;
     const float log_tau = __logf(tau), delta = (float)d.delta, wscale = d.w_scale, round_f = round * 0.1f;
-    const int64_t p_begin = (int64_t)r * WR;
-    const int64_t p_end = r_ok ? min(p_begin + (int64_t)WR, d.n_pp) : p_begin;
-    int seg = r_ok ? d.range_pair[r] : 0;
-    int64_t seg_end = r_ok ? d.pair_off[seg + 1] : 0;
+    const int p_begin = r * WR, p_end = (int)min((int64_t)p_begin + WR, d.n_pp);
+    const int steps = (p_end - p_begin + LP_BLOCK - 1) / LP_BLOCK;
+    auto request = [&](int c) {
+        if (c < steps) {
+            unsigned char *dst = s_stage[warp][c % LP_STAGES];
+            const size_t q = (size_t)p_begin + (size_t)c * LP_BLOCK;
+            const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + q * (KP_BYTES / LP_BLOCK);
+#pragma unroll
+            for (int u = 0; u < KP_BYTES / 512; ++u) cp_async16(dst + (u * 32 + lane) * 16, kp + (u * 32 + lane) * 16);
+            if (lane < 16) {   // 64 scores (lanes 0..7) and 64 history values (8..15)
+                const __half *src = lane < 8 ? d.score : d.le_hist;
+                cp_async16(dst + KP_BYTES + lane * 16, src + q + (lane & 7) * 8);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < LP_STAGES; ++c) request(c);
+    int seg = d.range_pair[r], seg_end = d.pair_off[seg + 1];
     LossBody<MODE_LOSS_IRLS> loss(d);
     unsigned kept = 0;
-    const uint64_t pol = evict_first_policy();
-    // the keypoints, scores and history of the next group are loaded one group ahead, so their
-    // latency overlaps the current group's MMAs
-    typename F::Raw nraw;
-    unsigned nsc = 0u, nhi = 0u;
-    auto fetch = [&](int64_t gq) {
-        nraw = F::load(d, gq, false, pol);
-        if (PPL == 2) {
-            nsc = *reinterpret_cast<const unsigned *>(d.score + gq);
-            nhi = *reinterpret_cast<const unsigned *>(d.le_hist + gq);
-        } else {
-            nsc = __half_as_ushort(d.score[gq]);
-            nhi = __half_as_ushort(d.le_hist[gq]);
-        }
-    };
-    if (p_begin < p_end) fetch(p_begin + lane * PPL);
-    for (int g = 0; g < NG; ++g) {
-        const int64_t gb = p_begin + (int64_t)g * GROUP;
-        const bool active = gb < p_end;   // warp-uniform
-        const int64_t q0 = gb + lane * PPL;
-        typename F::Raw raw = nraw;
-        const unsigned csc = nsc, chi = nhi;
-        if (gb + GROUP < p_end) fetch(q0 + GROUP);
-        float sco[PPL], lp[PPL], e[PPL], le[PPL];
+    float E[9];
+    load_E(d.geo, seg, E);
+    float4 st = reinterpret_cast<const float4 *>(d.pstat)[seg];
+    uint4 *feat = s_feat[warp];
+    const int my_row = (lane & 3) * 9 + (lane >> 2);
+    const uint32_t frag_row = (uint32_t)__cvta_generic_to_shared(feat + ((lane >> 3) & 1) * 36 + (lane >> 4) * 9 + (lane & 7));
+    for (int c = 0; c < steps; ++c) {
+        const int b0 = p_begin + c * LP_BLOCK;
+        asm volatile("cp.async.wait_group %0;" ::"n"(LP_STAGES - 1) : "memory");
+        __syncwarp();
+        const unsigned char *src = s_stage[warp][c % LP_STAGES];
+        uint4 kp[SUBS];
 #pragma unroll
-        for (int k = 0; k < PPL; ++k) sco[k] = lp[k] = e[k] = le[k] = 0.f;
-        int seg0 = seg;
-        int64_t seg0_end = seg_end;
-        // ---- phase A: features of the lane's point pairs into A1[k], row `row`
-        uint4 feat[PPL];
-#pragma unroll
-        for (int k = 0; k < PPL; ++k) feat[k] = make_uint4(0u, 0u, 0u, 0u);
-        if (active) {
+        for (int u = 0; u < SUBS; ++u) kp[u] = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
+        float sco[2], lp[2];
+        {
+            const __half *sc = reinterpret_cast<const __half *>(src + KP_BYTES), *hs = sc + LP_BLOCK;
             if (PPL == 2) {
-                const float2 sv = __half22float2(*reinterpret_cast<const __half2 *>(&csc));
-                const float2 hv = __half22float2(*reinterpret_cast<const __half2 *>(&chi));
-                sco[0] = sv.x;
-                sco[PPL - 1] = sv.y;
-                lp[0] = hv.x;
-                lp[PPL - 1] = hv.y;
+                const float2 a = __half22float2(reinterpret_cast<const __half2 *>(sc)[lane]);
+                const float2 b = __half22float2(reinterpret_cast<const __half2 *>(hs)[lane]);
+                sco[0] = a.x;
+                sco[1] = a.y;
+                lp[0] = b.x;
+                lp[1] = b.y;
             } else {
-                sco[0] = __half2float(__ushort_as_half((unsigned short)csc));
-                lp[0] = __half2float(__ushort_as_half((unsigned short)chi));
-            }
-            const int64_t g_end = min(gb + GROUP, p_end);
-            float E[9];
-            load_E(d.geo, seg, E);
-            float4 st = reinterpret_cast<const float4 *>(d.pstat)[seg];
-            int64_t lo = gb;
-            while (true) {
-                const int64_t hi = min(seg_end, p_end);
 #pragma unroll
-                for (int k = 0; k < PPL; ++k) {
-                    const int64_t q = q0 + k;
-                    if (q >= lo && q < hi) {
-                        float x1, y1, x2, y2, unused;
-                        F::get(raw, k, x1, y1, x2, y2, unused);
-                        e[k] = epi(E, x1, y1, x2, y2);
-                        le[k] = __logf(fabsf(e[k]) + LOG_FLOOR);
-                        const float lpk = hist_valid ? lp[k] : le[k];
-                        feat[k] = make_uint4(pack_bf16(le[k] - log_tau, le[k] - st.x),
-                                             pack_bf16(lpk - le[k], sco[k]), pack_bf16(st.y, st.z),
-                                             pack_bf16(round_f, lpk - log_tau));
-                    }
+                for (int k = 0; k < 2; ++k) {
+                    sco[k] = __half2float(sc[32 * k + lane]);
+                    lp[k] = __half2float(hs[32 * k + lane]);
                 }
-                if (seg_end >= g_end) break;
-                lo = seg_end;
-                ++seg;
-                seg_end = d.pair_off[seg + 1];
-                load_E(d.geo, seg, E);
-                st = reinterpret_cast<const float4 *>(d.pstat)[seg];
             }
         }
+        // ---- features of the lane's two point pairs
+        const int seg0 = seg, seg0_end = seg_end;
+        float x1[2], y1[2], x2[2], y2[2], e[2], le[2];
 #pragma unroll
-        for (int k = 0; k < PPL; ++k) *reinterpret_cast<uint4 *>(sm.a2[k] + tc_offset(row, 0, TC_K2)) = feat[k];
-        // ---- layer 1
-        if (tc_handover(sm)) break;
-        if (threadIdx.x == 0) {
-            tc_fence_after_sync();
-#pragma unroll
-            for (int k = 0; k < PPL; ++k)
-                tc_mma_bf16(sm.tmem + 32 * k, dA1[k], dB1, id1, 0u);
-            tc_commit(smem_addr(&sm.mbar));
+        for (int k = 0; k < 2; ++k) {
+            typename F::Raw raw;
+            raw.kp = kp[k / PPL];
+            raw.w = 0u;
+            float unused;
+            F::get(raw, k % PPL, x1[k], y1[k], x2[k], y2[k], unused);
+            e[k] = le[k] = 0.f;
         }
-        tc_wait(sm, phase);
+        auto feature = [&](int k) {
+            e[k] = epi(E, x1[k], y1[k], x2[k], y2[k]);
+            le[k] = __logf(fabsf(e[k]) + LOG_FLOOR);
+            const float lpk = hist_valid ? lp[k] : le[k];
+            feat[k * 36 + my_row] = make_uint4(pack_bf16(le[k] - log_tau, le[k] - st.x), pack_bf16(lpk - le[k], sco[k]),
+                                               pack_bf16(st.y, st.z), pack_bf16(round_f, lpk - log_tau));
+        };
+        const bool whole = b0 + LP_BLOCK <= seg_end;   // one image pair, no end of the range
+        if (whole) {
+            feature(0);
+            feature(1);
+        } else {
 #pragma unroll
-        for (int k = 0; k < PPL; ++k) {
-            uint32_t acc[32];
-            tmem_ld32(tm + 32 * k, acc);
-            tc_relu_row(sm.a2[k], row, acc);
+            for (int u = 0; u < SUBS; ++u) {
+                const int gb = b0 + u * GROUP, g_end = min(gb + GROUP, p_end);
+                int lo = gb;
+                while (lo < g_end) {
+                    const int hi = min(seg_end, g_end);
+#pragma unroll
+                    for (int k = 0; k < PPL; ++k) {
+                        const int q = gb + lane * PPL + k;
+                        if (q >= lo && q < hi) feature(u * PPL + k);
+                    }
+                    lo = hi;
+                    if (seg_end >= g_end) break;
+                    ++seg;
+                    seg_end = d.pair_off[seg + 1];
+                    load_E(d.geo, seg, E);
+                    st = reinterpret_cast<const float4 *>(d.pstat)[seg];
+                }
+#pragma unroll
+                for (int k = 0; k < PPL; ++k)   // rows past the end of the range: any finite input
+                    if (gb + lane * PPL + k >= p_end) feat[(u * PPL + k) * 36 + my_row] = make_uint4(0u, 0u, 0u, 0u);
+            }
         }
-        // ---- layer 2
-        if (tc_handover(sm)) break;
-        if (threadIdx.x == 0) {
-            tc_fence_after_sync();
+        __syncwarp();
+        // ---- the network
+        float z[2] = {0.f, 0.f};
 #pragma unroll
-            for (int k = 0; k < PPL; ++k)
+        for (int m = 0; m < 2; ++m) {
+            unsigned f[4];
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
+                         : "r"(frag_row + (uint32_t)(m * 2 * 9 * 16))
+                         : "memory");
 #pragma unroll
-                for (int sl = 0; sl < TC_K2 / 16; ++sl)
-                    tc_mma_bf16(sm.tmem + 32 * k, dA2[k] + sl * SLICE, dB2 + sl * SLICE, id1, sl > 0 ? 1u : 0u);
-            tc_commit(smem_addr(&sm.mbar));
+            for (int h = 0; h < 2; ++h) {
+                float z0, z1;
+                net.tile(f[2 * h], f[2 * h + 1], z0, z1);
+                z[0] = t == 2 * m + h ? z0 : z[0];
+                z[1] = t == 2 * m + h ? z1 : z[1];
+            }
         }
-        tc_wait(sm, phase);
-#pragma unroll
-        for (int k = 0; k < PPL; ++k) {
-            uint32_t acc[32];
-            tmem_ld32(tm + 32 * k, acc);
-            tc_relu_row(sm.a2[k], row, acc);
-        }
-        // ---- layer 3
-        if (tc_handover(sm)) break;
-        if (threadIdx.x == 0) {
-            tc_fence_after_sync();
-#pragma unroll
-            for (int k = 0; k < PPL; ++k)
-#pragma unroll
-                for (int sl = 0; sl < TC_K2 / 16; ++sl)
-                    tc_mma_bf16(sm.tmem + 32 * k, dA2[k] + sl * SLICE, dB3 + sl * SLICE, id3, sl > 0 ? 1u : 0u);
-            tc_commit(smem_addr(&sm.mbar));
-        }
-        tc_wait(sm, phase);
-        float z[PPL];
-#pragma unroll
-        for (int k = 0; k < PPL; ++k) z[k] = __uint_as_float(tmem_ld1(tm + 32 * k));
-        tc_fence_before_sync();
-        if (!active) continue;
+        __syncwarp();   // the features and the stage have been read
+        request(c + LP_STAGES);
         // ---- weights, history, kept count
-        float w[PPL];
+        float w[2];
 #pragma unroll
-        for (int k = 0; k < PPL; ++k) {
+        for (int k = 0; k < 2; ++k) {
+            const int q = b0 + (k / PPL) * GROUP + lane * PPL + k % PPL;
             const float pk = __frcp_rn(1.f + __expf(-z[k]));
             const float ae = fabsf(e[k]);
-            const bool in = q0 + k < p_end && ae <= tau_cap;
+            const bool in = q < p_end && ae <= tau_cap;
             const float wf = in ? learned_weight(pk, ae, delta) : 0.f;
             w[k] = STORE == FM_STORE_FP32 ? wf : __half2float(__float2half_rn(wf * wscale));
             kept += in ? 1u : 0u;
         }
-        if (STORE == FM_STORE_FP32) {
-            static_cast<float *>(d.w)[q0] = w[0];
-            if (q0 < p_end) d.le_hist[q0] = __float2half_rn(le[0]);
+        if (PPL == 2) {
+            const int q = b0 + 2 * lane;
+            reinterpret_cast<__half2 *>(d.w)[q >> 1] = __floats2half2_rn(w[0], w[1]);
+            const __half2 hv = __floats2half2_rn(le[0], le[1]);
+            if (q + 1 < p_end) reinterpret_cast<__half2 *>(d.le_hist)[q >> 1] = hv;
+            else if (q < p_end) d.le_hist[q] = __low2half(hv);
         } else {
-            reinterpret_cast<__half2 *>(d.w)[q0 >> 1] = __floats2half2_rn(w[0], w[PPL - 1]);
-            const __half2 hv = __floats2half2_rn(le[0], le[PPL - 1]);
-            if (q0 + 1 < p_end) reinterpret_cast<__half2 *>(d.le_hist)[q0 >> 1] = hv;
-            else if (q0 < p_end) d.le_hist[q0] = __low2half(hv);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int q = b0 + 32 * k + lane;
+                static_cast<float *>(d.w)[q] = w[k];
+                if (q < p_end) d.le_hist[q] = __float2half_rn(le[k]);
+            }
         }
         if (!FUSE) continue;
-        // ---- phase B: loss and adjoint sums with the new weights
-        int sb = seg0;
-        int64_t sb_end = seg0_end, lo = gb;
-        while (true) {
-            const int64_t hi = min(sb_end, p_end);
+        // ---- loss and adjoint sums with the new weights
+        if (whole) {
 #pragma unroll
-            for (int k = 0; k < PPL; ++k) {
-                const int64_t q = q0 + k;
-                if (q >= lo && q < hi) {
-                    float x1, y1, x2, y2, unused;
-                    F::get(raw, k, x1, y1, x2, y2, unused);
-                    loss.point(k, e[k], x1, y1, x2, y2, w[k]);
+            for (int k = 0; k < 2; ++k) loss.point(k, e[k], x1[k], y1[k], x2[k], y2[k], w[k]);
+        } else {
+            int sb = seg0, sb_end = seg0_end;
+#pragma unroll
+            for (int u = 0; u < SUBS; ++u) {
+                const int gb = b0 + u * GROUP, g_end = min(gb + GROUP, p_end);
+                int lo = gb;
+                while (lo < g_end) {
+                    const int hi = min(sb_end, g_end);
+#pragma unroll
+                    for (int k = 0; k < PPL; ++k) {
+                        const int q = gb + lane * PPL + k, i = u * PPL + k;
+                        if (q >= lo && q < hi) loss.point(i, e[i], x1[i], y1[i], x2[i], y2[i], w[i]);
+                    }
+                    lo = hi;
+                    if (sb_end >= g_end) break;
+                    loss.segment_end(sb, r, lane, false);
+                    ++sb;
+                    sb_end = d.pair_off[sb + 1];
                 }
             }
-            if (sb == seg) break;
-            loss.segment_end(sb, r, lane, false);
-            lo = sb_end;
-            ++sb;
-            sb_end = d.pair_off[sb + 1];
         }
     }
-    if (FUSE && r_ok) loss.segment_end(seg, r, lane, true);
+    if (FUSE) loss.segment_end(seg, r, lane, true);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
-    if (lane == 0 && kept) atomicAdd(&sm.kept, kept);
-    tc_fence_before_sync();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (sm.kept) atomicAdd(d.counter, (unsigned long long)sm.kept);
-        if (sm.fail) atomicOr(d.err, ERR_NONFINITE);
-    }
-    if (wid == 0) {
-        tc_fence_after_sync();
-        tmem_dealloc(sm.tmem, TC_COLS);
-    }
+    if (lane == 0 && kept) atomicAdd(d.counter, (unsigned long long)kept);
 }
 
 static inline int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 void launch_learned_loss(const DevProblem &d, const float *master, const __nv_bfloat16 *wbf, float tau,
                          float tau_cap, int round, int hist_valid, cudaStream_t s, bool pdl) {
-    const dim3 grid(blocks_for(d.n_ranges, TC_THREADS / 32)), block(TC_THREADS);
+    const dim3 grid(blocks_for(d.n_ranges, LP_WARPS)), block(LP_WARPS * 32);
     if (d.storage == FM_STORE_FP32)
-        launch_k(k_learned_tc<FM_STORE_FP32, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
+        launch_k(k_learned_pass<FM_STORE_FP32, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
     else
-        launch_k(k_learned_tc<FM_STORE_FP16, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
+        launch_k(k_learned_pass<FM_STORE_FP16, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
 }
 
 void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
@@ -842,20 +490,20 @@ void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
 
 void launch_learned_weights(const DevProblem &d, const float *master, const __nv_bfloat16 *wbf, float tau,
                             float tau_cap, int round, int hist_valid, cudaStream_t s) {
-    const dim3 grid(blocks_for(d.n_ranges, TC_THREADS / 32)), block(TC_THREADS);
+    const dim3 grid(blocks_for(d.n_ranges, LP_WARPS)), block(LP_WARPS * 32);
     if (d.storage == FM_STORE_FP32)
-        launch_k(k_learned_tc<FM_STORE_FP32, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
+        launch_k(k_learned_pass<FM_STORE_FP32, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
     else
-        launch_k(k_learned_tc<FM_STORE_FP16, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
+        launch_k(k_learned_pass<FM_STORE_FP16, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
 }
 
 void launch_collect_features(const DevProblem &d, float tau, int round, int hist_valid,
                              __nv_bfloat16 *feat, cudaStream_t s) {
     const int grid = blocks_for(d.n_ranges, CTA_WARPS);
     if (d.storage == FM_STORE_FP32)
-        k_learned<FM_STORE_FP32, true><<<grid, CTA_WARPS * 32, 0, s>>>(d, nullptr, nullptr, tau, INFINITY, round, hist_valid, feat);
+        k_collect_features<FM_STORE_FP32><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau, round, hist_valid, feat);
     else
-        k_learned<FM_STORE_FP16, true><<<grid, CTA_WARPS * 32, 0, s>>>(d, nullptr, nullptr, tau, INFINITY, round, hist_valid, feat);
+        k_collect_features<FM_STORE_FP16><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau, round, hist_valid, feat);
 }
 
 // ---- training: register-tiled forward and backward, block-level gradient sums, FP32 Adam --------
