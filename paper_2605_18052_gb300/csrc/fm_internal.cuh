@@ -19,7 +19,6 @@ namespace fm {
 // advances n or r, so n + r is unique per non-empty intersection and there are at most
 // n_pairs + n_ranges slots.
 constexpr int WR = 2048;           // point pairs per warp range
-constexpr int CTA_WARPS = 8;       // warps per CTA of the streaming kernels
 constexpr int SLOT = 12;           // floats per slot: G'(9), loss, 2 pad (48 B)
 constexpr int GEO = 40;            // floats per pair geometry record (160 B)
 constexpr int CAMREC = 16;         // floats per camera record

@@ -11,8 +11,6 @@
 //   irls_weights / residuals: the same streaming walk writing one value per point pair
 #include <math.h>
 
-#include <type_traits>
-
 #include "fm_step.cuh"
 
 namespace fm {
@@ -73,8 +71,8 @@ struct ReweightLossBody {
     __device__ __forceinline__ void segment_end(int seg, int r, int lane, bool last) {
         loss.segment_end(seg, r, lane, last);
     }
-    __device__ __forceinline__ void group_done(int64_t gb, int64_t p_end, int lane) {
-        const int64_t q = gb + lane * Fmt<STORE>::PPL;
+    __device__ __forceinline__ void group_done(int gb, int p_end, int lane) {
+        const int q = gb + lane * Fmt<STORE>::PPL;
         if (STORE == FM_STORE_FP32) {
             static_cast<float *>(d.w)[q] = q < p_end ? out[0] : 0.f;
         } else {
@@ -124,8 +122,8 @@ struct WeightBody {
     }
     __device__ __forceinline__ void segment_begin(int) {}
     __device__ __forceinline__ void segment_end(int, int, int, bool) {}
-    __device__ __forceinline__ void group_done(int64_t gb, int64_t p_end, int lane) {
-        const int64_t q = gb + lane * Fmt<STORE>::PPL;
+    __device__ __forceinline__ void group_done(int gb, int p_end, int lane) {
+        const int q = gb + lane * Fmt<STORE>::PPL;
         if (STORE == FM_STORE_FP32) {
             static_cast<float *>(d.w)[q] = q < p_end ? out[0] : 0.f;
         } else {
@@ -137,22 +135,17 @@ struct WeightBody {
     }
 };
 
-template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32) k_irls_weights(DevProblem d, float tau) {
-    __shared__ unsigned cta_kept;
-    if (threadIdx.x == 0) cta_kept = 0;
-    __syncthreads();
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
-    if (r < d.n_ranges) {
-        WeightBody<STORE> body(d, tau);
-        walk_range<STORE, false>(d, r, threadIdx.x & 31, body);
-        unsigned k = body.kept;
+template <int STORE, int S, int W>
+__global__ void __launch_bounds__(32 * W) k_irls_weights(DevProblem d, float tau) {
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * W + warp;
+    if (r >= d.n_ranges) return;
+    WeightBody<STORE> body(d, tau);
+    walk_range_staged<STORE, false, S>(d, r, lane, body, stage + warp * S * STAGE_BYTES, [] {});
+    unsigned k = body.kept;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&cta_kept, k);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && cta_kept) atomicAdd(d.counter, (unsigned long long)cta_kept);
+    for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    if (lane == 0 && k) atomicAdd(d.counter, (unsigned long long)k);
 }
 
 template <int STORE>
@@ -165,20 +158,21 @@ struct ResidualBody {
     }
     __device__ __forceinline__ void segment_begin(int) {}
     __device__ __forceinline__ void segment_end(int, int, int, bool) {}
-    __device__ __forceinline__ void group_done(int64_t gb, int64_t p_end, int lane) {
-        const int64_t q = gb + lane * Fmt<STORE>::PPL;
+    __device__ __forceinline__ void group_done(int gb, int p_end, int lane) {
+        const int q = gb + lane * Fmt<STORE>::PPL;
 #pragma unroll
         for (int k = 0; k < Fmt<STORE>::PPL; ++k)
             if (q + k < p_end) out_sorted[q + k] = out[k];
     }
 };
 
-template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32) k_residuals(DevProblem d, float *out) {
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
+template <int STORE, int S, int W>
+__global__ void __launch_bounds__(32 * W) k_residuals(DevProblem d, float *out) {
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
     if (r >= d.n_ranges) return;
     ResidualBody<STORE> body(out);
-    walk_range<STORE, false>(d, r, threadIdx.x & 31, body);
+    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
 }
 
 __global__ void k_cam_prep(DevProblem d) {
@@ -542,29 +536,6 @@ void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cu
     launch_k(k_finalize, dim3(1), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count);
 }
 
-// Depth and block size of the staged passes. FP32: 4 chunks (512 point pairs) a warp; the whole range,
-// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 15.5 ->
-// 15.1 us an iteration, 245 ranges 17.5 -> 16.8; 733 ranges 17.9 -> 19.2). FP16: 2 chunks (512 point
-// pairs). One warp per block, so that a finished range makes room for the next at once, but four from
-// 300 ranges per SM on, where the block launches count (FP16: 68,633 ranges 223.6 -> 219.5 us, 23,860
-// ranges 84.5 -> 85.8).
-constexpr int FEW_RANGES = 2 * 152, MANY_RANGES = 300 * 152;
-
-template <class Launch>
-static void with_stages(const DevProblem &d, Launch launch) {
-    using std::integral_constant;
-    if (d.storage == FM_STORE_FP32) {
-        integral_constant<int, FM_STORE_FP32> st;
-        if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>(), integral_constant<int, 1>());
-        else if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 4>(), integral_constant<int, 1>());
-        else launch(st, integral_constant<int, 4>(), integral_constant<int, 4>());
-    } else {
-        integral_constant<int, FM_STORE_FP16> st;
-        if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 2>(), integral_constant<int, 1>());
-        else launch(st, integral_constant<int, 2>(), integral_constant<int, 4>());
-    }
-}
-
 void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
     const int prev = after_step ? d.n_cams : 0;
     with_stages(d, [&](auto store, auto depth, auto warps) {
@@ -632,15 +603,17 @@ void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pd
 }
 
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {
-    const int grid = blocks_for(d.n_ranges, CTA_WARPS);
-    if (d.storage == FM_STORE_FP32) k_irls_weights<FM_STORE_FP32><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau);
-    else k_irls_weights<FM_STORE_FP16><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau);
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        k_irls_weights<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau);
+    });
 }
 
 void launch_residuals(const DevProblem &d, float *out_sorted, cudaStream_t s) {
-    const int grid = blocks_for(d.n_ranges, CTA_WARPS);
-    if (d.storage == FM_STORE_FP32) k_residuals<FM_STORE_FP32><<<grid, CTA_WARPS * 32, 0, s>>>(d, out_sorted);
-    else k_residuals<FM_STORE_FP16><<<grid, CTA_WARPS * 32, 0, s>>>(d, out_sorted);
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        k_residuals<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, out_sorted);
+    });
 }
 
 }  // namespace fm

@@ -45,15 +45,16 @@ struct StatsBody {
         }
         acc[0] = acc[1] = 0.f;
     }
-    __device__ __forceinline__ void group_done(int64_t, int64_t, int) {}
+    __device__ __forceinline__ void group_done(int, int, int) {}
 };
 
-template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32) k_pair_stats(DevProblem d, float tau) {
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
+template <int STORE, int S, int W>
+__global__ void __launch_bounds__(32 * W) k_pair_stats(DevProblem d, float tau) {
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
     if (r >= d.n_ranges) return;
     StatsBody body(d, tau);
-    walk_range<STORE, false>(d, r, threadIdx.x & 31, body);
+    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
 }
 
 __global__ void k_pair_stats_combine(DevProblem d) {
@@ -216,8 +217,8 @@ struct CollectBody {
         sc[k] = st_cnt;
     }
     __device__ __forceinline__ void segment_end(int, int, int, bool) {}
-    __device__ __forceinline__ void group_done(int64_t gb, int64_t p_end, int lane) {
-        const int64_t q = gb + lane * PPL;
+    __device__ __forceinline__ void group_done(int gb, int p_end, int lane) {
+        const int q = gb + lane * PPL;
         float lp[PPL], sco[PPL];
 #pragma unroll
         for (int k = 0; k < PPL; ++k) {
@@ -238,17 +239,18 @@ struct CollectBody {
     }
 };
 
-template <int STORE>
-__global__ void __launch_bounds__(CTA_WARPS * 32)
+template <int STORE, int S, int W>
+__global__ void __launch_bounds__(32 * W)
 k_collect_features(DevProblem d, float tau, int round, int hist_valid, __nv_bfloat16 *feat_out) {
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
+    extern __shared__ __align__(16) unsigned char stage[];
+    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
     if (r >= d.n_ranges) return;
     CollectBody<STORE> body(d);
     body.log_tau = __logf(tau);
     body.round_f = round * 0.1f;
     body.hist_valid = hist_valid;
     body.feat_out = feat_out;
-    walk_range<STORE, false, CollectBody<STORE>, 1>(d, r, threadIdx.x & 31, body);
+    walk_range_staged<STORE, false, S, 1>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
 }
 
 // ---- the learned reweighting -------------------------------------------------------------------------
@@ -482,9 +484,10 @@ void launch_learned_loss(const DevProblem &d, const float *master, const __nv_bf
 }
 
 void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
-    const int grid = blocks_for(d.n_ranges, CTA_WARPS);
-    if (d.storage == FM_STORE_FP32) k_pair_stats<FM_STORE_FP32><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau);
-    else k_pair_stats<FM_STORE_FP16><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau);
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        k_pair_stats<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau);
+    });
     k_pair_stats_combine<<<blocks_for(d.n_pairs, 128), 128, 0, s>>>(d);
 }
 
@@ -499,11 +502,11 @@ void launch_learned_weights(const DevProblem &d, const float *master, const __nv
 
 void launch_collect_features(const DevProblem &d, float tau, int round, int hist_valid,
                              __nv_bfloat16 *feat, cudaStream_t s) {
-    const int grid = blocks_for(d.n_ranges, CTA_WARPS);
-    if (d.storage == FM_STORE_FP32)
-        k_collect_features<FM_STORE_FP32><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau, round, hist_valid, feat);
-    else
-        k_collect_features<FM_STORE_FP16><<<grid, CTA_WARPS * 32, 0, s>>>(d, tau, round, hist_valid, feat);
+    with_stages(d, [&](auto store, auto depth, auto warps) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
+        k_collect_features<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau, round, hist_valid,
+                                                                                                   feat);
+    });
 }
 
 // ---- training: register-tiled forward and backward, block-level gradient sums, FP32 Adam --------

@@ -49,17 +49,27 @@ struct QuadBody {
         // c0 and g0 = sum (w eps o2) (x) o1
         const float we = w * e;
         acc[0] = fmaf(we, e, acc[0]);
-        const float t2[3] = {we * x2, we * y2, we};
-        const float o1[3] = {x1, y1, 1.f};
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) acc[1 + 3 * p + q] = fmaf(t2[p], o1[q], acc[1 + 3 * p + q]);
+        float tx, ty;                       // w eps o2 = (tx, ty, we)
+        mul2(tx, ty, we, we, x2, y2);
+        fma2(acc[1], acc[2], tx, tx, x1, y1);
+        fma2(acc[4], acc[5], ty, ty, x1, y1);
+        fma2(acc[7], acc[8], we, we, x1, y1);
+        add2(acc[3], acc[6], tx, ty);
+        acc[9] += we;
         // M[u][v] += (w m2_u) m1_v, two neighbouring entries of a row per packed instruction (the
         // pass is bound by instruction issue, not by the FP32 pipe)
-        const float wx2 = w * x2, wy2 = w * y2;
-        const float u[6] = {wx2 * x2, wx2 * y2, wx2, wy2 * y2, wy2, w};
-        const float v[6] = {x1 * x1, x1 * y1, x1, y1 * y1, y1, 1.f};
+        float wx2, wy2, u[6], v[6];
+        mul2(wx2, wy2, w, w, x2, y2);
+        mul2(u[0], u[1], wx2, wx2, x2, y2);
+        u[2] = wx2;
+        u[3] = wy2 * y2;
+        u[4] = wy2;
+        u[5] = w;
+        mul2(v[0], v[1], x1, x1, x1, y1);
+        v[2] = x1;
+        v[3] = y1 * y1;
+        v[4] = y1;
+        v[5] = 1.f;
 #pragma unroll
         for (int a = 0; a < 6; ++a)
 #pragma unroll
@@ -86,9 +96,9 @@ struct QuadBody {
 #pragma unroll
         for (int i = 0; i < QSUMS; ++i) acc[i] = 0.f;
     }
-    __device__ __forceinline__ void group_done(int64_t gb, int64_t p_end, int lane) {
+    __device__ __forceinline__ void group_done(int gb, int p_end, int lane) {
         if (!REWEIGHT) return;
-        const int64_t q = gb + lane * Fmt<STORE>::PPL;
+        const int q = gb + lane * Fmt<STORE>::PPL;
         if (STORE == FM_STORE_FP32) {
             static_cast<float *>(d.w)[q] = q < p_end ? out[0] : 0.f;
         } else {
@@ -101,34 +111,24 @@ struct QuadBody {
     }
 };
 
-// groups in flight per warp and resident CTAs per SM of the accumulation pass (the 46 running
-// sums leave room for few of either)
-#ifndef FM_QUAD_UNROLL
-#define FM_QUAD_UNROLL 4
-#endif
-#ifndef FM_QUAD_MIN_CTAS
-#define FM_QUAD_MIN_CTAS 2
-#endif
+// One warp per block and range, staged 3 chunks deep, two groups of a chunk in straight code: 94
+// registers, 20 warps per SM. Bound by instruction issue and the FP32 pipe (66 operations a point pair).
+// The 46 sums leave no registers for loads in flight, and four groups in straight code overran the
+// instruction cache; with 4 groups loaded ahead and 16 warps per SM in blocks of 8 the pass took, on
+// 48.9 M point pairs with / without reweighting, FP16 224 / 189 us and FP32 309 / 246 us; now 183 / 152
+// and 184 / 159 (3.1 M: FP16 30 / 27 -> 25 / 21, FP32 35 / 29 -> 26 / 23).
+constexpr int QUAD_STAGES = 3, QUAD_UNROLL = 2, QUAD_WARPS_PER_SM = 20;
 
 template <int STORE, bool REWEIGHT>
-__global__ void __launch_bounds__(CTA_WARPS * 32, FM_QUAD_MIN_CTAS) k_quad_accumulate(DevProblem d, float tau) {
-    __shared__ unsigned cta_kept;
-    if (threadIdx.x == 0) cta_kept = 0;
-    __syncthreads();
-    const int r = blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
-    if (r < d.n_ranges) {
-        QuadBody<STORE, REWEIGHT> body(d, tau);
-        walk_range<STORE, !REWEIGHT, QuadBody<STORE, REWEIGHT>, FM_QUAD_UNROLL>(d, r, threadIdx.x & 31, body);
-        if (REWEIGHT) {
-            unsigned k = body.kept;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-            if ((threadIdx.x & 31) == 0) atomicAdd(&cta_kept, k);
-        }
-    }
+__global__ void __launch_bounds__(32, QUAD_WARPS_PER_SM) k_quad_accumulate(DevProblem d, float tau) {
+    __shared__ __align__(16) unsigned char stage[QUAD_STAGES * STAGE_BYTES];
+    QuadBody<STORE, REWEIGHT> body(d, tau);
+    walk_range_staged<STORE, !REWEIGHT, QUAD_STAGES, QUAD_UNROLL>(d, blockIdx.x, threadIdx.x, body, stage, [] {});
     if (REWEIGHT) {
-        __syncthreads();
-        if (threadIdx.x == 0 && cta_kept) atomicAdd(d.counter, (unsigned long long)cta_kept);
+        unsigned k = body.kept;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+        if (threadIdx.x == 0 && k) atomicAdd(d.counter, (unsigned long long)k);
     }
 }
 
@@ -391,8 +391,7 @@ static inline int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); 
 
 // tau < 0: keep the current weights; otherwise reweight with threshold tau in the same pass
 void launch_quad_accumulate(const DevProblem &d, float tau, cudaStream_t s) {
-    const int grid = blocks_for(d.n_ranges, CTA_WARPS);
-    const dim3 block(CTA_WARPS * 32);
+    const int grid = d.n_ranges, block = 32;
     if (tau < 0.f) {
         if (d.storage == FM_STORE_FP32) k_quad_accumulate<FM_STORE_FP32, false><<<grid, block, 0, s>>>(d, tau);
         else k_quad_accumulate<FM_STORE_FP16, false><<<grid, block, 0, s>>>(d, tau);

@@ -1,7 +1,9 @@
 // Device building blocks shared by the streaming kernels: programmatic-dependent-launch
-// helpers, evict-first streaming loads, the two keypoint storage formats and the warp-range
-// walk over the pair-sorted point pairs.
+// helpers, the two keypoint storage formats and the warp-range walk over the pair-sorted point
+// pairs.
 #pragma once
+
+#include <type_traits>
 
 #include "fm_internal.cuh"
 
@@ -54,30 +56,6 @@ constexpr int spread_lane(int n, int i) {
     return lane;
 }
 
-// ---- streaming loads: 16 B vectors, no L1 allocation, evict-first in L2 -----------------------
-// The point-pair arrays are read once per pass and are 10-100x larger than L2; marking them
-// evict-first keeps the small per-pair and per-camera tables (geometry, partial sums, camera
-// lists, poses) resident in L2 across passes, which the latency-bound per-camera step needs.
-__device__ __forceinline__ uint64_t evict_first_policy() {
-    uint64_t pol;
-    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-__device__ __forceinline__ uint4 ld_stream_v4(const void *p, uint64_t pol) {
-    uint4 r;
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-        : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-        : "l"(p), "l"(pol));
-    return r;
-}
-
-__device__ __forceinline__ unsigned ld_stream_u32(const void *p, uint64_t pol) {
-    unsigned r;
-    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(r) : "l"(p), "l"(pol));
-    return r;
-}
-
 // ---- storage formats -----------------------------------------------------------------------------
 template <int STORE>
 struct Fmt;
@@ -90,12 +68,6 @@ struct Fmt<FM_STORE_FP32> {
         uint4 kp;
         unsigned w;
     };
-    __device__ static Raw load(const DevProblem &d, int64_t q, bool need_w, uint64_t pol) {
-        Raw r;
-        r.kp = ld_stream_v4(static_cast<const float4 *>(d.kp) + q, pol);
-        r.w = need_w ? ld_stream_u32(static_cast<const float *>(d.w) + q, pol) : 0u;
-        return r;
-    }
     __device__ static void get(const Raw &r, int, float &x1, float &y1, float &x2, float &y2,
                                float &w) {
         x1 = __uint_as_float(r.kp.x);
@@ -115,12 +87,6 @@ struct Fmt<FM_STORE_FP16> {
         uint4 kp;
         unsigned w;
     };
-    __device__ static Raw load(const DevProblem &d, int64_t q, bool need_w, uint64_t pol) {
-        Raw r;
-        r.kp = ld_stream_v4(static_cast<const uint2 *>(d.kp) + q, pol);
-        r.w = need_w ? ld_stream_u32(static_cast<const __half *>(d.w) + q, pol) : 0u;
-        return r;
-    }
     __device__ static void get(const Raw &r, int k, float &x1, float &y1, float &x2, float &y2,
                                float &w) {
         const unsigned a = k == 0 ? r.kp.x : r.kp.z;
@@ -187,18 +153,17 @@ __device__ __forceinline__ unsigned atomic_add_acq_rel(unsigned *p, unsigned v) 
 // contiguous 512 B block. The image pair changes only at sorted boundaries: a group that lies
 // inside the current pair takes the fast path; a group that crosses a boundary is processed in
 // passes, one pass per image pair it meets, and `body.segment_end` closes each finished pair.
+// Positions are 32-bit (n_pp < 2^31 - 2^16, so also past the end of the padded arrays).
 struct WalkState {
-    int64_t p_begin, p_end;
-    int seg;
-    int64_t seg_end;
+    int p_begin, p_end, seg, seg_end;
     float E[9];
     __device__ __forceinline__ WalkState(const DevProblem &d, int r)
-        : p_begin((int64_t)r * WR), p_end(min(p_begin + (int64_t)WR, d.n_pp)), seg(d.range_pair[r]),
+        : p_begin(r * WR), p_end((int)min((int64_t)p_begin + WR, d.n_pp)), seg(d.range_pair[r]),
           seg_end(d.pair_off[seg + 1]) {}
 };
 
 template <int STORE, class Body>
-__device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, const typename Fmt<STORE>::Raw &raw, int64_t gb,
+__device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, const typename Fmt<STORE>::Raw &raw, int gb,
                                            int r, int lane, Body &body) {
     using F = Fmt<STORE>;
     constexpr int PPL = F::PPL;
@@ -211,13 +176,13 @@ __device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, c
             body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
         }
     } else {
-        int64_t lo = gb;
-        const int64_t g_end = min(gb + GROUP, st.p_end);
+        int lo = gb;
+        const int g_end = min(gb + GROUP, st.p_end);
         while (true) {
-            const int64_t hi = min(st.seg_end, st.p_end);
+            const int hi = min(st.seg_end, st.p_end);
 #pragma unroll
             for (int k = 0; k < PPL; ++k) {
-                const int64_t q = gb + lane * PPL + k;
+                const int q = gb + lane * PPL + k;
                 if (q >= lo && q < hi) {
                     float x1, y1, x2, y2, w;
                     F::get(raw, k, x1, y1, x2, y2, w);
@@ -236,32 +201,7 @@ __device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, c
     body.group_done(gb, st.p_end, lane);
 }
 
-// U groups are loaded before any is processed (loads in flight per warp).
-template <int STORE, bool NEED_W, class Body, int U = 4>
-__device__ __forceinline__ void walk_range(const DevProblem &d, int r, int lane, Body &body) {
-    using F = Fmt<STORE>;
-    constexpr int GROUP = 32 * F::PPL;
-    static_assert(WR % (U * GROUP) == 0, "range must be whole unrolled groups");
-    WalkState st(d, r);
-    load_E(d.geo, st.seg, st.E);
-    body.segment_begin(st.seg);
-    const uint64_t pol = evict_first_policy();
-    for (int64_t g0 = st.p_begin; g0 < st.p_end; g0 += U * GROUP) {
-        typename F::Raw raw[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) raw[u] = F::load(d, g0 + u * GROUP + lane * F::PPL, NEED_W, pol);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t gb = g0 + u * GROUP;
-            if (gb >= st.p_end) break;
-            walk_group<STORE>(d, st, raw[u], gb, r, lane, body);
-        }
-    }
-    body.segment_end(st.seg, r, lane, true);
-}
-
-// The same walk with the range staged in shared memory by asynchronous copies, a chunk of 4 groups
-// (2 KB of keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the
+// The walk of a range, staged in shared memory by asynchronous copies, a chunk of 4 groups (2 KB of keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the
 // launch before this one; the first S chunks are requested ahead of it, so they arrive while that
 // launch finishes. (Keypoints are static. Weights are written at least two launches earlier: a pass
 // that writes them is followed by the camera step, which lets this launch start only after its own
@@ -274,7 +214,8 @@ __device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) 
                  : "memory");
 }
 
-template <int STORE, bool NEED_W, int S, class Body, class Before>
+// UNROLL: groups of a chunk in straight code (1 for bodies of many instructions).
+template <int STORE, bool NEED_W, int S, int UNROLL = STAGE_GROUPS, class Body, class Before>
 __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, int lane, Body &body, unsigned char *stage,
                                                   Before before) {
     using F = Fmt<STORE>;
@@ -282,9 +223,9 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
     constexpr int CHUNK = STAGE_GROUPS * GROUP;
     static_assert(WR % CHUNK == 0, "range must be whole chunks");
     WalkState st(d, r);
-    const int n_chunks = (int)((st.p_end - st.p_begin + CHUNK - 1) / CHUNK);
-    const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + st.p_begin * (16 / F::PPL);
-    const unsigned char *wp = static_cast<const unsigned char *>(d.w) + st.p_begin * (4 / F::PPL);
+    const int n_chunks = (st.p_end - st.p_begin + CHUNK - 1) / CHUNK;
+    const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + (size_t)st.p_begin * (16 / F::PPL);
+    const unsigned char *wp = static_cast<const unsigned char *>(d.w) + (size_t)st.p_begin * (4 / F::PPL);
     auto request = [&](int c) {
         if (c < n_chunks) {
             unsigned char *dst = stage + (c % S) * STAGE_BYTES;
@@ -303,9 +244,9 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
         asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
         __syncwarp();   // a lane's weights were copied by another lane
         const unsigned char *src = stage + (c % S) * STAGE_BYTES;
-#pragma unroll
+#pragma unroll UNROLL
         for (int u = 0; u < STAGE_GROUPS; ++u) {
-            const int64_t gb = st.p_begin + (int64_t)c * CHUNK + u * GROUP;
+            const int gb = st.p_begin + c * CHUNK + u * GROUP;
             if (gb >= st.p_end) break;
             typename F::Raw raw;
             raw.kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
@@ -316,6 +257,29 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
         request(c + S);
     }
     body.segment_end(st.seg, r, lane, true);
+}
+
+// Depth and block size of the staged passes. FP32: 4 chunks (512 point pairs) a warp; the whole range,
+// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 15.5 ->
+// 15.1 us an iteration, 245 ranges 17.5 -> 16.8; 733 ranges 17.9 -> 19.2). FP16: 2 chunks (512 point
+// pairs). One warp per block, so that a finished range makes room for the next at once, but four from
+// 300 ranges per SM on, where the block launches count (FP16: 68,633 ranges 223.6 -> 219.5 us, 23,860
+// ranges 84.5 -> 85.8).
+constexpr int FEW_RANGES = 2 * 152, MANY_RANGES = 300 * 152;
+
+template <class Launch>
+static void with_stages(const DevProblem &d, Launch launch) {
+    using std::integral_constant;
+    if (d.storage == FM_STORE_FP32) {
+        integral_constant<int, FM_STORE_FP32> st;
+        if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>(), integral_constant<int, 1>());
+        else if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 4>(), integral_constant<int, 1>());
+        else launch(st, integral_constant<int, 4>(), integral_constant<int, 4>());
+    } else {
+        integral_constant<int, FM_STORE_FP16> st;
+        if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 2>(), integral_constant<int, 1>());
+        else launch(st, integral_constant<int, 2>(), integral_constant<int, 4>());
+    }
 }
 
 // ---- packed FP32 pairs -----------------------------------------------------------------------------
@@ -401,7 +365,7 @@ struct LossBody {
 #pragma unroll
         for (int i = 0; i < 10; ++i) acc[i] = 0.f;
     }
-    __device__ __forceinline__ void group_done(int64_t, int64_t, int) {}
+    __device__ __forceinline__ void group_done(int, int, int) {}
 };
 
 // ---- per pair: relative pose and folded essential matrix ------------------------------------------
