@@ -175,6 +175,15 @@ FM_API fm_status fm_loss_grad(fm_problem *p, double *loss, double *grad);
 /* Same, asynchronous, into device memory the caller owns (either pointer may be NULL). */
 FM_API fm_status fm_loss_grad_device(fm_problem *p, double *d_loss, double *d_grad);
 
+/*
+ * Euclidean pose gradients from a gradient d_grad (n_cams x 6 FP64, ordered as above) at rotations d_R
+ * (n_cams x 9 FP64): d_gR = 0.5 s [g_phi]_x R (n_cams x 9; its inner product with any rotation
+ * perturbation [dphi]_x R is s g_phi . dphi) and d_gc = s g_c (n_cams x 3), s = *d_scale (1 FP64). All
+ * pointers are device pointers; asynchronous on `stream` (a cudaStream_t, NULL = legacy default).
+ */
+FM_API fm_status fm_pose_gradient(int32_t n_cams, const double *d_grad, const double *d_R, const double *d_scale,
+                                  double *d_gR, double *d_gc, void *stream);
+
 /* Residuals eps = x2^T E_n x1 at the current poses, FP32, input order, host. Synchronises. */
 FM_API fm_status fm_residuals(fm_problem *p, float *eps);
 

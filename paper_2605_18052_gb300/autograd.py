@@ -9,11 +9,16 @@ quantity. With recompute=True the forward keeps nothing and backward runs the pa
 Gradients: the library returns the left-trivialised gradient g_phi (R <- Exp(phi) R) and
 g_c. For R the backward returns the tangent-space Euclidean gradient 0.5 [g_phi]_x R, whose
 inner product with any rotation perturbation [dphi]_x R equals g_phi . dphi, so autograd
-through any rotation parameterisation (exponential map, 6D, quaternions) is exact.
+through any rotation parameterisation (exponential map, 6D, quaternions) is exact. Contiguous
+float64 inputs take one kernel for this (fm_pose_gradient; as torch operations it was 13 launches,
+one of them a 70 us batched FP64 matrix product); other types and layouts, and a backward that is itself
+differentiated (create_graph), take the torch operations.
 """
 from __future__ import annotations
 
 import torch
+
+from .binding import pose_gradient
 
 
 def _hat(v: torch.Tensor) -> torch.Tensor:
@@ -27,7 +32,7 @@ def _loss_grad(problem, R, c):
     R = R.detach().to(torch.float64).contiguous()
     c = c.detach().to(torch.float64).contiguous()
     problem.set_params_device(R, c)
-    loss = torch.empty(1, dtype=torch.float64, device=R.device)
+    loss = torch.empty((), dtype=torch.float64, device=R.device)
     grad = torch.empty(R.shape[0], 6, dtype=torch.float64, device=R.device)
     problem.loss_grad_device(loss, grad)
     return loss, grad
@@ -43,7 +48,7 @@ class EpipolarLoss(torch.autograd.Function):
             ctx.save_for_backward(R, c)
         else:
             ctx.save_for_backward(R, grad)
-        return loss[0]
+        return loss
 
     @staticmethod
     def backward(ctx, grad_out):
@@ -52,6 +57,10 @@ class EpipolarLoss(torch.autograd.Function):
             _, grad = _loss_grad(ctx.problem, R, c)
         else:
             R, grad = ctx.saved_tensors
+        if (not torch.is_grad_enabled() and R.dtype == grad.dtype == grad_out.dtype == torch.float64
+                and R.is_cuda and grad_out.device == R.device and R.is_contiguous()
+                and type(R) is type(grad_out) is torch.Tensor):
+            return None, *pose_gradient(grad, R, grad_out), None
         g = grad * grad_out
         gR = 0.5 * _hat(g[:, :3]) @ R.to(torch.float64)
         return None, gR.to(R.dtype), g[:, 3:].to(R.dtype), None

@@ -21,7 +21,7 @@ PASS_STREAM_LOSS, PASS_STREAM_REWEIGHT, PASS_QUAD_ACCUMULATE, PASS_LEARNED_LOSS,
 EXPORTED = [
     "fm_default_options", "fm_create_problem", "fm_destroy_problem", "fm_problem_info",
     "fm_get_poses", "fm_set_poses", "fm_get_params", "fm_set_params", "fm_set_params_device", "fm_set_weights", "fm_get_weights", "fm_irls_weights",
-    "fm_loss_grad", "fm_loss_grad_device", "fm_residuals", "fm_step", "fm_step_irls", "fm_last_loss",
+    "fm_loss_grad", "fm_loss_grad_device", "fm_pose_gradient", "fm_residuals", "fm_step", "fm_step_irls", "fm_last_loss",
     "fm_set_learning_rate", "fm_reset_optimizer", "fm_get_state", "fm_set_state",
     "fm_synchronize", "fm_apply_gradient", "fm_enable_kernel_timing", "fm_kernel_time", "fm_pass_time",
     "fm_loss_grad_noalloc",
@@ -87,6 +87,7 @@ def load_library(path: str = LIB_PATH):
         "fm_irls_weights": (I32, [P, D, P]),
         "fm_loss_grad": (I32, [P, P, P]),
         "fm_loss_grad_device": (I32, [P, P, P]),
+        "fm_pose_gradient": (I32, [I32, P, P, P, P, P, P]),
         "fm_residuals": (I32, [P, P]),
         "fm_step": (I32, [P, I32]),
         "fm_step_irls": (I32, [P, D, I32, P]),
@@ -622,6 +623,17 @@ class Rotation:
     def set_params(self, a6):
         a6 = np.ascontiguousarray(_host(a6, np.float64).reshape(self.n_cams, 6))
         _check(load_library().fm_rotation_set_params(self._h, _ptr(a6)))
+
+
+def pose_gradient(grad, R, scale):
+    """(0.5 s [g_phi]_x R, s g_c) from grad (N, 6), R (N, 3, 3) and the 0-dim scale s, contiguous
+    float64 CUDA tensors, in one launch on the current stream (fm_pose_gradient)."""
+    import torch
+    gR = torch.empty_like(R)
+    gc = torch.empty(R.shape[0], 3, dtype=R.dtype, device=R.device)
+    _check(load_library().fm_pose_gradient(R.shape[0], grad.data_ptr(), R.data_ptr(), scale.data_ptr(), gR.data_ptr(),
+                                           gc.data_ptr(), _current_stream()))
+    return gR, gc
 
 
 def focal_vote(F, candidates, tau: float, f1_known=None, f2_known=None, timed: bool = False, stream=None):

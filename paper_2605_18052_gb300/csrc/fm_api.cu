@@ -204,6 +204,17 @@ void enqueue_iteration(fm_problem *p, cudaStream_t s, bool timed, bool first, bo
     launch_camera_step(p->d, true, s, !t, true);
 }
 
+// loss and gradient at the current poses, chained like an iteration; the caller's device memory
+// (either may be null) is written by the kernels that compute the values
+void enqueue_loss_grad(fm_problem *p, double *d_loss, double *d_grad) {
+    DevProblem d = p->d;
+    if (d_grad) d.grad = d_grad;
+    launch_pair_setup(d, p->s, true, false);
+    launch_stream_loss(d, p->s, true);
+    launch_camera_step(d, false, p->s, true);
+    launch_finalize(d, false, p->s, true, d_loss);
+}
+
 // `iters` chained iterations and the closing finalize launch (reweight: the first pass fused
 // with the round's reweighting); `quad`: fused steps on the pre-aggregated quadratic form (one
 // launch per iteration), alternating between the two camera-record buffers; after an odd count
@@ -604,11 +615,8 @@ FM_API fm_status fm_set_params(fm_problem *p, const double *R, const double *c) 
 FM_API fm_status fm_set_params_device(fm_problem *p, const double *d_R, const double *d_c) {
     if (fm_status st = check_problem(p)) return st;
     if (!d_R || !d_c) return fail(FM_EINVAL, "d_R and d_c must not be NULL");
-    const int n = p->d.n_cams;
     FM_CUDA(join_in(p));
-    FM_CUDA(cudaMemcpyAsync(p->d.R, d_R, sizeof(double) * 9 * n, cudaMemcpyDeviceToDevice, p->s));
-    FM_CUDA(cudaMemcpyAsync(p->d.c, d_c, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, p->s));
-    launch_cam_prep(p->d, p->s);
+    launch_set_params(p->d, d_R, d_c, p->s);
     FM_CUDA(cudaGetLastError());
     FM_CUDA(join_out(p));
     return FM_OK;
@@ -794,14 +802,8 @@ FM_API fm_status fm_irls_weights(fm_problem *p, double tau, int64_t *n_active) {
 FM_API fm_status fm_loss_grad_device(fm_problem *p, double *d_loss, double *d_grad) {
     if (fm_status st = check_problem(p)) return st;
     FM_CUDA(join_in(p));
-    launch_pair_setup(p->d, p->s);
-    launch_stream_loss(p->d, p->s);
-    launch_camera_step(p->d, false, p->s);
-    launch_finalize(p->d, false, p->s);
+    enqueue_loss_grad(p, d_loss, d_grad);
     FM_CUDA(cudaGetLastError());
-    if (d_loss) FM_CUDA(cudaMemcpyAsync(d_loss, p->d.loss_out, sizeof(double), cudaMemcpyDeviceToDevice, p->s));
-    if (d_grad)
-        FM_CUDA(cudaMemcpyAsync(d_grad, p->d.grad, sizeof(double) * 6 * p->d.n_cams, cudaMemcpyDeviceToDevice, p->s));
     FM_CUDA(join_out(p));
     return FM_OK;
 }
@@ -810,15 +812,20 @@ FM_API fm_status fm_loss_grad(fm_problem *p, double *loss, double *grad) {
     if (fm_status st = check_problem(p)) return st;
     if (!loss) return fail(FM_EINVAL, "loss must not be NULL");
     FM_CUDA(join_in(p));
-    launch_pair_setup(p->d, p->s);
-    launch_stream_loss(p->d, p->s);
-    launch_camera_step(p->d, false, p->s);
-    launch_finalize(p->d, false, p->s);
+    enqueue_loss_grad(p, nullptr, nullptr);
     FM_CUDA(cudaGetLastError());
     FM_CUDA(cudaMemcpyAsync(loss, p->d.loss_out, sizeof(double), cudaMemcpyDeviceToHost, p->s));
     if (grad)
         FM_CUDA(cudaMemcpyAsync(grad, p->d.grad, sizeof(double) * 6 * p->d.n_cams, cudaMemcpyDeviceToHost, p->s));
     return check_device_errors(p);
+}
+
+FM_API fm_status fm_pose_gradient(int32_t n_cams, const double *d_grad, const double *d_R, const double *d_scale,
+                                  double *d_gR, double *d_gc, void *stream) {
+    if (n_cams < 1) return fail(FM_EINVAL, "n_cams must be >= 1");
+    if (!d_grad || !d_R || !d_scale || !d_gR || !d_gc) return fail(FM_EINVAL, "device pointers must not be NULL");
+    FM_CUDA(launch_pose_gradient(n_cams, d_grad, d_R, d_scale, d_gR, d_gc, static_cast<cudaStream_t>(stream)));
+    return FM_OK;
 }
 
 FM_API fm_status fm_residuals(fm_problem *p, float *eps) {

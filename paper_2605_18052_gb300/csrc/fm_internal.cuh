@@ -138,14 +138,19 @@ void launch_learned_loss(const DevProblem &d, const float *mlp_master, const __n
 
 // ---- kernels launched by the API layer (fm_kernels.cu) ----------------------------------------
 void launch_cam_prep(const DevProblem &d, cudaStream_t s);
+void launch_set_params(const DevProblem &d, const double *R, const double *c, cudaStream_t s);
+cudaError_t launch_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR,
+                                 double *gc, cudaStream_t s);
 // pdl: launch with programmatic stream serialisation (overlaps the predecessor's tail)
 // after_step: the previous kernel was an optimiser camera step whose loss total and step
 // count this launch finishes
 void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl = false, bool after_step = false);
 // loss total of the last camera step (and the step count after an optimiser step)
-void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl = false);
+// (loss_copy: also written to the caller's device memory)
+void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl = false, double *loss_copy = nullptr);
 // the same with `count` steps added, and camera records copied back from copy_src if not null
-void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl);
+void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl,
+                       double *loss_copy = nullptr);
 int camera_step_blocks(const DevProblem &d);
 // factors applied to the raw sums of the loss (Sum w eps^2 or Sum |eps|, weights stored as
 // w * s): gradient 2/(Z s) and loss 1/(Z s) for IRLS, 1/Z for L1

@@ -181,6 +181,30 @@ __global__ void k_cam_prep(DevProblem d) {
     write_camrec(d.cam + (size_t)k * CAMREC, d.R + 9 * (size_t)k, d.c + 3 * (size_t)k, (float)camera_scale(d, k));
 }
 
+// new parameters from the caller's device memory, and their camera records
+__global__ void k_set_params(DevProblem d, const double *R, const double *c) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= d.n_cams) return;
+    double Rk[9], ck[3];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) d.R[9 * (size_t)k + q] = Rk[q] = R[9 * (size_t)k + q];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) d.c[3 * (size_t)k + q] = ck[q] = c[3 * (size_t)k + q];
+    write_camrec(d.cam + (size_t)k * CAMREC, Rk, ck, (float)camera_scale(d, k));
+}
+
+// g_R = 0.5 s [g_phi]_x R and g_c = s g_c of every camera, a thread per row
+__global__ void k_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR, double *gc) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = i / 3, a = i % 3;
+    if (k >= n_cams) return;
+    const double s = *scale, *g = grad + 6 * (size_t)k, *Rk = R + 9 * (size_t)k;
+    const int b = (a + 1) % 3, c = (a + 2) % 3;   // row a of [g]_x: -g_c at column b, g_b at column c
+    const double hb = -0.5 * (g[c] * s), hc = 0.5 * (g[b] * s);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) gR[9 * (size_t)k + 3 * a + q] = hb * Rk[3 * b + q] + hc * Rk[3 * c + q];
+    gc[3 * (size_t)k + a] = g[3 + a] * s;
+}
+
 // prev_loss > 0: this pass follows an optimiser step with that many per-camera loss shares;
 // block 0 (with 256 threads) finishes that step's loss total and step count.
 __global__ void __launch_bounds__(256) k_pair_setup(DevProblem d, int prev_loss) {
@@ -497,11 +521,13 @@ __global__ void __launch_bounds__(32) k_apply_gradient(DevProblem d) {
 __global__ void k_bump_step(DevProblem d) { *d.step += 1; }
 
 // closes a chain of steps: loss of the last step and `count` steps added to the step count
-__global__ void __launch_bounds__(FIN_THREADS) k_finalize(DevProblem d, int n_loss, int count) {
+// (loss_copy: the caller's loss, or null)
+__global__ void __launch_bounds__(FIN_THREADS) k_finalize(DevProblem d, int n_loss, int count, double *loss_copy) {
     pdl_wait();
     pdl_trigger();
     __shared__ double red[FIN_THREADS];
     finish_step(d, n_loss, count, red);
+    if (loss_copy && threadIdx.x == 0) *loss_copy = red[0];
 }
 
 // camera records copied back from the alternate buffer (one float4 per thread)
@@ -525,15 +551,19 @@ void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl, bool after
     launch_k(k_pair_setup, dim3(blocks_for(d.n_pairs, 256)), dim3(256), s, pdl, d, after_step ? d.n_cams : 0);
 }
 
-void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl) {
-    launch_finalize_n(d, count_step ? 1 : 0, nullptr, s, pdl);
+void launch_set_params(const DevProblem &d, const double *R, const double *c, cudaStream_t s) {
+    k_set_params<<<blocks_for(d.n_cams, 64), 64, 0, s>>>(d, R, c);
 }
 
-void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl) {
+void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl, double *loss_copy) {
+    launch_finalize_n(d, count_step ? 1 : 0, nullptr, s, pdl, loss_copy);
+}
+
+void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl, double *loss_copy) {
     if (copy_src)
         launch_k(k_copy_records, dim3(blocks_for((int64_t)d.n_cams * (CAMREC / 4), 256)), dim3(256), s, pdl, d,
                  reinterpret_cast<const float4 *>(copy_src));
-    launch_k(k_finalize, dim3(1), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count);
+    launch_k(k_finalize, dim3(1), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count, loss_copy);
 }
 
 void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
@@ -614,6 +644,12 @@ void launch_residuals(const DevProblem &d, float *out_sorted, cudaStream_t s) {
         constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
         k_residuals<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, out_sorted);
     });
+}
+
+cudaError_t launch_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR,
+                                 double *gc, cudaStream_t s) {
+    k_pose_gradient<<<blocks_for(3 * (int64_t)n_cams, 96), 96, 0, s>>>(n_cams, grad, R, scale, gR, gc);
+    return cudaGetLastError();
 }
 
 }  // namespace fm
