@@ -9,6 +9,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "fm_grid.cuh"
@@ -77,6 +78,26 @@ cudaError_t dalloc(fm_problem *p, T **ptr, size_t count) {
     return e;
 }
 
+// Several arrays of a problem in one allocation (a cudaMalloc and its cudaFree take 20 us; a problem has
+// 33 arrays): add() notes where each array's pointer goes, commit() allocates and fills them in.
+// Arrays lie in the order of add(), each on a 256-byte boundary.
+struct Arena {
+    std::vector<std::pair<void **, size_t>> items;
+    size_t bytes = 0;
+    template <class T>
+    void add(T **ptr, size_t count) {
+        items.emplace_back(reinterpret_cast<void **>(ptr), bytes);
+        bytes += (sizeof(T) * (count ? count : 1) + 255) / 256 * 256;
+    }
+    cudaError_t commit(fm_problem *p) {
+        char *base = nullptr;
+        cudaError_t e = dalloc(p, &base, bytes);
+        if (e == cudaSuccess)
+            for (auto &it : items) *it.first = base + it.second;
+        return e;
+    }
+};
+
 // order the problem's stream after the caller's stream
 cudaError_t join_in(fm_problem *p) {
     cudaError_t e = cudaEventRecord(p->ev_in, p->user);
@@ -117,13 +138,14 @@ bool finite_all(const double *a, size_t n) {
     return true;
 }
 
-// host poses (R, t) -> device (R, c = -R^T t) and camera records
-fm_status upload_poses(fm_problem *p, const double *R, const double *t) {
+// host poses (R, t) -> device (R, c = -R^T t) and camera records; R and `c` stay as they are until the
+// stream has been waited for
+fm_status upload_poses(fm_problem *p, const double *R, const double *t, std::vector<double> &c) {
     const int n = p->d.n_cams;
     if (!R || !t) return fail(FM_EINVAL, "R and t must not be NULL");
     if (!finite_all(R, 9 * (size_t)n) || !finite_all(t, 3 * (size_t)n))
         return fail(FM_EINVAL, "poses must be finite");
-    std::vector<double> c(3 * (size_t)n);
+    c.resize(3 * (size_t)n);
     for (int k = 0; k < n; ++k) {
         const double *Rk = R + 9 * (size_t)k;
         double dev = 0.0;
@@ -140,14 +162,14 @@ fm_status upload_poses(fm_problem *p, const double *R, const double *t) {
     FM_CUDA(cudaMemcpyAsync(p->d.c, c.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice, p->s));
     launch_cam_prep(p->d, p->s);
     FM_CUDA(cudaGetLastError());
-    FM_CUDA(cudaStreamSynchronize(p->s));
     return FM_OK;
 }
 
+// the optimiser's constants for later steps (by value in a launch: nothing to wait for)
 fm_status upload_hyper(fm_problem *p) {
     const double h[6] = {p->opt.lr_rot, p->opt.lr_c, p->opt.beta1, p->opt.beta2, p->opt.adam_eps, p->lr_focal};
-    FM_CUDA(cudaMemcpyAsync(p->d.hyper, h, sizeof h, cudaMemcpyHostToDevice, p->s));
-    FM_CUDA(cudaStreamSynchronize(p->s));
+    launch_set_hyper(p->d, h, p->s);
+    FM_CUDA(cudaGetLastError());
     return FM_OK;
 }
 
@@ -326,85 +348,67 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
         }
     }
 
-    FM_CUDA(dalloc(p, &d.R, 9 * (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.c, 3 * (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.m, 6 * (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.v, 6 * (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.rho, (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.grad_rho, (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.rho_m, (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.rho_v, (size_t)n_cams));
+    const size_t nc = (size_t)n_cams, np = (size_t)n_pairs;
     d.refine_focal = p->opt.refine_focal;
-    FM_CUDA(dalloc(p, &d.cam_loss, (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.hyper, 8));
-    FM_CUDA(dalloc(p, &d.step, 1));
-    FM_CUDA(dalloc(p, &d.cam, (size_t)CAMREC * n_cams));
-    FM_CUDA(dalloc(p, &d.pair_cnt, (size_t)n_pairs));
-    FM_CUDA(dalloc(p, &d.cen, (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.cam_i, (size_t)n_pairs));
-    FM_CUDA(dalloc(p, &d.cam_j, (size_t)n_pairs));
-    FM_CUDA(dalloc(p, &d.pair_off, (size_t)n_pairs + 1));
-    FM_CUDA(dalloc(p, &d.range_pair, (size_t)d.n_ranges));
-    FM_CUDA(dalloc(p, &d.cam_off, (size_t)n_cams + 1));
-    FM_CUDA(dalloc(p, &d.cam_ent, 2 * (size_t)n_pairs));
-    if (d.storage == FM_STORE_FP32) {
-        float4 *kp;
-        float *w;
-        FM_CUDA(dalloc(p, &kp, (size_t)d.n_pad));
-        FM_CUDA(dalloc(p, &w, (size_t)d.n_pad));
-        d.kp = kp;
-        d.w = w;
-    } else {
-        uint2 *kp;
-        __half *w;
-        FM_CUDA(dalloc(p, &kp, (size_t)d.n_pad));
-        FM_CUDA(dalloc(p, &w, (size_t)d.n_pad));
-        d.kp = kp;
-        d.w = w;
-    }
-    FM_CUDA(dalloc(p, &d.score, (size_t)d.n_pad));
-    FM_CUDA(dalloc(p, &d.le_hist, (size_t)d.n_pad));
-    {
-        float4 *ps;
-        FM_CUDA(dalloc(p, &ps, (size_t)n_pairs));
-        d.pstat = reinterpret_cast<float *>(ps);
-    }
-    FM_CUDA(dalloc(p, &d.geo, (size_t)GEO * n_pairs));
-    FM_CUDA(dalloc(p, &d.slots, (size_t)SLOT * ((size_t)n_pairs + d.n_ranges)));
-    FM_CUDA(dalloc(p, &d.pair_grad, (size_t)PG * n_pairs));
-    FM_CUDA(dalloc(p, &d.grad, 6 * (size_t)n_cams));
-    FM_CUDA(dalloc(p, &d.loss_out, 1));
-    FM_CUDA(dalloc(p, &d.err, 1));
-    FM_CUDA(dalloc(p, &d.counter, 1));
+    Arena arena;
+    arena.add(&d.R, 9 * nc);         // R, c and the error word are read together (read_params)
+    arena.add(&d.c, 3 * nc);
+    arena.add(&d.err, 1);            // from here to pair_cnt: zero at the start
+    arena.add(&d.m, 6 * nc);
+    arena.add(&d.v, 6 * nc);
+    arena.add(&d.rho, nc);
+    arena.add(&d.grad_rho, nc);
+    arena.add(&d.rho_m, nc);
+    arena.add(&d.rho_v, nc);
+    arena.add(&d.step, 1);
+    arena.add(&d.cen, nc);
+    arena.add(&d.geo, GEO * np);
+    arena.add(&d.pair_cnt, np);
+    arena.add(&d.cam_loss, nc);
+    arena.add(&d.hyper, 8);
+    arena.add(&d.cam, CAMREC * nc);
+    arena.add(&d.cam_i, np);
+    arena.add(&d.cam_j, np);
+    arena.add(&d.pair_off, np + 1);
+    arena.add(&d.range_pair, (size_t)d.n_ranges);
+    arena.add(&d.cam_off, nc + 1);
+    arena.add(&d.cam_ent, 2 * np);
+    float4 *ps = nullptr;
+    arena.add(&ps, np);
+    arena.add(&d.slots, SLOT * (np + d.n_ranges));
+    arena.add(&d.pair_grad, PG * np);
+    arena.add(&d.grad, 6 * nc);
+    arena.add(&d.loss_out, 1);
+    arena.add(&d.counter, 1);
+    const size_t kp_bytes = d.storage == FM_STORE_FP32 ? sizeof(float4) : sizeof(uint2);
+    const size_t w_bytes = d.storage == FM_STORE_FP32 ? sizeof(float) : sizeof(__half);
+    char *kp = nullptr, *w = nullptr;
+    arena.add(&kp, kp_bytes * d.n_pad);
+    arena.add(&w, w_bytes * d.n_pad);
+    arena.add(&d.score, (size_t)d.n_pad);
+    arena.add(&d.le_hist, (size_t)d.n_pad);
+    FM_CUDA(arena.commit(p));
+    d.kp = kp;
+    d.w = w;
+    d.pstat = reinterpret_cast<float *>(ps);
     d.perm = nullptr;
     d.fbuf = nullptr;
 
-    FM_CUDA(cudaMemsetAsync(d.err, 0, sizeof(unsigned), p->s));
-    FM_CUDA(cudaMemsetAsync(d.m, 0, sizeof(float) * 6 * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.v, 0, sizeof(float) * 6 * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.rho, 0, sizeof(double) * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.grad_rho, 0, sizeof(double) * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.rho_m, 0, sizeof(float) * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.rho_v, 0, sizeof(float) * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.step, 0, sizeof(long long), p->s));
-    FM_CUDA(cudaMemsetAsync(d.cen, 0, sizeof(float2) * n_cams, p->s));
-    FM_CUDA(cudaMemsetAsync(d.geo, 0, sizeof(float) * GEO * n_pairs, p->s));
-    FM_CUDA(cudaMemsetAsync(d.pair_cnt, 0, sizeof(unsigned) * n_pairs, p->s));
+    FM_CUDA(cudaMemsetAsync(d.err, 0, (char *)d.cam_loss - (char *)d.err, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_i, cam_i, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_j, cam_j, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_off, cam_off.data(), sizeof(int) * (n_cams + 1), cudaMemcpyHostToDevice, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_ent, cam_ent.data(), sizeof(int) * 2 * n_pairs, cudaMemcpyHostToDevice, p->s));
 
-    // point pairs on the device (temporaries when they come from the host)
+    // point pairs on the device (temporaries when they come from the host, in one allocation)
     const int *d_pid = pair_id;
     const float2 *d_x1 = reinterpret_cast<const float2 *>(x1);
     const float2 *d_x2 = reinterpret_cast<const float2 *>(x2);
-    int *t_pid = nullptr;
-    float2 *t_x1 = nullptr, *t_x2 = nullptr;
+    char *t_in = nullptr, *t_sort = nullptr;
     if (!pp_on_device) {
-        FM_CUDA(cudaMallocAsync(&t_pid, sizeof(int) * n_pp, p->s));
-        FM_CUDA(cudaMallocAsync(&t_x1, sizeof(float2) * n_pp, p->s));
-        FM_CUDA(cudaMallocAsync(&t_x2, sizeof(float2) * n_pp, p->s));
+        FM_CUDA(cudaMallocAsync(&t_in, (sizeof(float2) * 2 + sizeof(int)) * n_pp, p->s));
+        float2 *t_x1 = reinterpret_cast<float2 *>(t_in), *t_x2 = t_x1 + n_pp;
+        int *t_pid = reinterpret_cast<int *>(t_x2 + n_pp);
         FM_CUDA(cudaMemcpyAsync(t_pid, pair_id, sizeof(int) * n_pp, cudaMemcpyHostToDevice, p->s));
         FM_CUDA(cudaMemcpyAsync(t_x1, x1, sizeof(float2) * n_pp, cudaMemcpyHostToDevice, p->s));
         FM_CUDA(cudaMemcpyAsync(t_x2, x2, sizeof(float2) * n_pp, cudaMemcpyHostToDevice, p->s));
@@ -413,11 +417,9 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
         d_x2 = t_x2;
     }
     auto release_temps = [&]() {
-        if (t_pid) cudaFreeAsync(t_pid, p->s);
-        if (t_x1) cudaFreeAsync(t_x1, p->s);
-        if (t_x2) cudaFreeAsync(t_x2, p->s);
-        t_pid = nullptr;
-        t_x1 = t_x2 = nullptr;
+        if (t_in) cudaFreeAsync(t_in, p->s);
+        if (t_sort) cudaFreeAsync(t_sort, p->s);
+        t_in = t_sort = nullptr;
     };
 
     launch_validate(d_pid, d_x1, d_x2, n_pp, n_pairs, d.err, p->s);
@@ -434,46 +436,56 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     p->input_was_sorted = (err & ERR_UNSORTED) ? 0 : 1;
 
     const int *keys = d_pid;
-    int *sorted_keys = nullptr;
+    float4 *sorted = nullptr;   // point pairs in pair order, when they did not come so
     if (!p->input_was_sorted) {
         FM_CUDA(dalloc(p, &d.perm, (size_t)n_pp));
-        FM_CUDA(cudaMallocAsync(&sorted_keys, sizeof(int) * n_pp, p->s));
-        FM_CUDA(sort_by_pair(d_pid, n_pp, n_pairs, sorted_keys, d.perm, p->s));
+        const size_t kb = (sizeof(int) * n_pp + 255) / 256 * 256;
+        const size_t gather = d.storage == FM_STORE_FP16 ? sizeof(float4) * n_pp : 0;
+        FM_CUDA(cudaMallocAsync(&t_sort, kb + std::max(sort_scratch_bytes(n_pp), gather), p->s));
+        int *sorted_keys = reinterpret_cast<int *>(t_sort);
+        FM_CUDA(sort_by_pair(d_pid, n_pp, n_pairs, sorted_keys, d.perm, t_sort + kb, p->s));
         keys = sorted_keys;
+        if (gather) {   // the sort's scratch is free again
+            sorted = reinterpret_cast<float4 *>(t_sort + kb);
+            launch_gather_points(d, d_x1, d_x2, sorted, p->s);
+        }
     }
     launch_pair_offsets(keys, n_pp, n_pairs, d.pair_off, d.err, p->s);
     FM_CUDA(cudaGetLastError());
     FM_CUDA(cudaMemcpyAsync(&err, d.err, sizeof(unsigned), cudaMemcpyDeviceToHost, p->s));
     FM_CUDA(cudaStreamSynchronize(p->s));
     if (err & ERR_EMPTY_PAIR) {
-        if (sorted_keys) cudaFreeAsync(sorted_keys, p->s);
         release_temps();
         cudaStreamSynchronize(p->s);
         return fail(FM_EINVAL, "every image pair needs at least one point pair");
     }
     launch_range_pairs(d.pair_off, n_pairs, d.n_ranges, d.range_pair, p->s);
-    if (d.storage == FM_STORE_FP16) {
-        unsigned long long *sums = nullptr;
-        FM_CUDA(cudaMallocAsync(&sums, sizeof(unsigned long long) * 2 * n_cams, p->s));
-        launch_centroids(d, keys, d_x1, d_x2, sums, p->s);
-        FM_CUDA(cudaFreeAsync(sums, p->s));
-    }
-    launch_pack(d, keys, d_x1, d_x2, p->s);
-    launch_fill_weights(d, 1.0f, p->s);
-    launch_fill_half(d.score, d.n_pad, 0.5f, p->s);
-    launch_fill_half(d.le_hist, d.n_pad, 0.0f, p->s);
+    if (d.storage == FM_STORE_FP16)   // d.grad is free until the first evaluation: the sums of 2 words a camera
+        launch_centroids(d, d_x1, d_x2, sorted, reinterpret_cast<unsigned long long *>(d.grad), p->s);
+    launch_pack(d, keys, d_x1, d_x2, sorted, p->s);
     FM_CUDA(cudaGetLastError());
-    if (sorted_keys) FM_CUDA(cudaFreeAsync(sorted_keys, p->s));
     release_temps();
     FM_CUDA(cudaMemsetAsync(d.err, 0, sizeof(unsigned), p->s));
+    std::vector<double> c;
+    fm_status st = upload_poses(p, R, t, c);
+    if (st == FM_OK) st = upload_hyper(p);
+    if (st == FM_OK) FM_CUDA(join_out(p));
     FM_CUDA(cudaStreamSynchronize(p->s));
+    return st;
+}
 
-    fm_status st = upload_poses(p, R, t);
-    if (st != FM_OK) return st;
-    st = upload_hyper(p);
-    if (st != FM_OK) return st;
-    FM_CUDA(join_out(p));
-    return FM_OK;
+// R, c and the device's error word in one copy (they are neighbours in the arena); reports errors as
+// check_device_errors does
+fm_status read_params(fm_problem *p, double *R, double *c) {
+    const size_t n = (size_t)p->d.n_cams, span = (char *)p->d.err - (char *)p->d.R;
+    std::vector<char> buf(span + sizeof(unsigned));
+    FM_CUDA(cudaMemcpyAsync(buf.data(), p->d.R, buf.size(), cudaMemcpyDeviceToHost, p->s));
+    FM_CUDA(cudaStreamSynchronize(p->s));
+    unsigned err;
+    std::memcpy(&err, buf.data() + span, sizeof err);
+    std::memcpy(R, buf.data(), sizeof(double) * 9 * n);
+    std::memcpy(c, buf.data() + ((char *)p->d.c - (char *)p->d.R), sizeof(double) * 3 * n);
+    return err ? check_device_errors(p) : FM_OK;
 }
 
 fm_status check_problem(const fm_problem *p) {
@@ -567,9 +579,7 @@ FM_API fm_status fm_get_poses(fm_problem *p, double *R, double *t) {
     const int n = p->d.n_cams;
     std::vector<double> c(3 * (size_t)n);
     FM_CUDA(join_in(p));
-    FM_CUDA(cudaMemcpyAsync(R, p->d.R, sizeof(double) * 9 * n, cudaMemcpyDeviceToHost, p->s));
-    FM_CUDA(cudaMemcpyAsync(c.data(), p->d.c, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, p->s));
-    if (fm_status st = check_device_errors(p)) return st;
+    if (fm_status st = read_params(p, R, c.data())) return st;
     for (int k = 0; k < n; ++k) {
         const double *Rk = R + 9 * (size_t)k;
         for (int a = 0; a < 3; ++a)
@@ -581,7 +591,9 @@ FM_API fm_status fm_get_poses(fm_problem *p, double *R, double *t) {
 FM_API fm_status fm_set_poses(fm_problem *p, const double *R, const double *t) {
     if (fm_status st = check_problem(p)) return st;
     FM_CUDA(join_in(p));
-    fm_status st = upload_poses(p, R, t);
+    std::vector<double> c;
+    fm_status st = upload_poses(p, R, t, c);
+    FM_CUDA(cudaStreamSynchronize(p->s));
     if (st != FM_OK) return st;
     FM_CUDA(join_out(p));
     return FM_OK;
@@ -591,9 +603,7 @@ FM_API fm_status fm_get_params(fm_problem *p, double *R, double *c) {
     if (fm_status st = check_problem(p)) return st;
     if (!R || !c) return fail(FM_EINVAL, "R and c must not be NULL");
     FM_CUDA(join_in(p));
-    FM_CUDA(cudaMemcpyAsync(R, p->d.R, sizeof(double) * 9 * p->d.n_cams, cudaMemcpyDeviceToHost, p->s));
-    FM_CUDA(cudaMemcpyAsync(c, p->d.c, sizeof(double) * 3 * p->d.n_cams, cudaMemcpyDeviceToHost, p->s));
-    return check_device_errors(p);
+    return read_params(p, R, c);
 }
 
 FM_API fm_status fm_set_params(fm_problem *p, const double *R, const double *c) {
@@ -832,15 +842,12 @@ FM_API fm_status fm_residuals(fm_problem *p, float *eps) {
     if (fm_status st = check_problem(p)) return st;
     if (!eps) return fail(FM_EINVAL, "eps must not be NULL");
     FM_CUDA(join_in(p));
-    float *sorted = nullptr, *ordered = nullptr;
-    FM_CUDA(cudaMallocAsync(&sorted, sizeof(float) * p->d.n_pp, p->s));
+    float *ordered = nullptr;
     FM_CUDA(cudaMallocAsync(&ordered, sizeof(float) * p->d.n_pp, p->s));
     launch_pair_setup(p->d, p->s);
-    launch_residuals(p->d, sorted, p->s);
-    launch_unpermute(p->d, sorted, ordered, p->s);
+    launch_residuals(p->d, ordered, p->s);
     FM_CUDA(cudaGetLastError());
     FM_CUDA(cudaMemcpyAsync(eps, ordered, sizeof(float) * p->d.n_pp, cudaMemcpyDeviceToHost, p->s));
-    FM_CUDA(cudaFreeAsync(sorted, p->s));
     FM_CUDA(cudaFreeAsync(ordered, p->s));
     return check_device_errors(p);
 }
@@ -866,9 +873,8 @@ FM_API fm_status fm_step_irls(fm_problem *p, double tau, int32_t n_iters, int64_
     if (n_iters < 1) return fail(FM_EINVAL, "n_iters must be >= 1");
     if (p->d.loss != FM_LOSS_IRLS) return fail(FM_EINVAL, "the fused reweighting needs the IRLS objective");
     FM_CUDA(join_in(p));
-    const double tv = std::isinf(tau) ? INFINITY : (double)(float)tau;
-    FM_CUDA(cudaMemcpyAsync(p->d.hyper + 6, &tv, sizeof tv, cudaMemcpyHostToDevice, p->s));
-    FM_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(unsigned long long), p->s));
+    launch_begin_round(p->d, std::isinf(tau) ? INFINITY : (double)(float)tau, p->s);
+    FM_CUDA(cudaGetLastError());
     p->quad_valid = false;
     if (p->timing || !p->opt.use_graph) {
         enqueue_iterations(p, p->s, p->timing, n_iters, false, true);
@@ -1025,10 +1031,12 @@ namespace {
 fm_status quad_prepare(fm_problem *p) {
     if (p->d.loss != FM_LOSS_IRLS) return fail(FM_EINVAL, "the quadratic form needs the IRLS objective");
     if (p->quad_alloc) return FM_OK;
-    FM_CUDA(dalloc(p, &p->d.qslots, (size_t)QSLOT * ((size_t)p->d.n_pairs + p->d.n_ranges)));
-    FM_CUDA(dalloc(p, &p->d.quad, (size_t)QREC * p->d.n_pairs));
-    FM_CUDA(dalloc(p, &p->d.cam_alt, (size_t)CAMREC * p->d.n_cams));
-    FM_CUDA(dalloc(p, &p->d.grid_state, GRID_STATE_WORDS));
+    Arena arena;
+    arena.add(&p->d.qslots, (size_t)QSLOT * ((size_t)p->d.n_pairs + p->d.n_ranges));
+    arena.add(&p->d.quad, (size_t)QREC * p->d.n_pairs);
+    arena.add(&p->d.cam_alt, (size_t)CAMREC * p->d.n_cams);
+    arena.add(&p->d.grid_state, GRID_STATE_WORDS);
+    FM_CUDA(arena.commit(p));
     FM_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
     int blocks = 0;
     FM_CUDA(quad_steps_capacity(p->d.refine_focal != 0, &blocks));

@@ -7,13 +7,14 @@
 // is already known uses it instead of the candidate (the paper's several-camera procedure).
 //
 // One thread evaluates one (candidate, pair) term: E from F (FP32, F normalised to unit
-// Frobenius norm on the host, which leaves the ratio unchanged), M = E^T E, its eigenvalues by
+// Frobenius norm first, which leaves the ratio unchanged), M = E^T E, its eigenvalues by
 // four sweeps of cyclic Jacobi rotations (each 2x2 step uses the cancellation-free rotation
 // angle, so nearly equal eigenvalues keep their relative accuracy, unlike the closed-form cubic
 // roots), lambda_1 / lambda_2 = sqrt(mu_1 / mu_2). A block covers 256 pairs and VOTE_CANDS
 // candidates; per-block sums are reduced in a fixed order, then added per candidate in FP64 in
 // block order: the votes are bit-reproducible.
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -73,6 +74,25 @@ __device__ __forceinline__ float vote_term(const float *F, float f1, float f2, f
     if (!(mid > 0.f)) return 0.f;
     const float ratio = sqrtf(hi / mid);
     return expf((1.f - ratio) * inv_tau);
+}
+
+// F normalised to unit Frobenius norm and rounded to FP32 (the arithmetic in FP64), a thread per pair.
+// *bad ends as the smallest 2 n + (0: not finite, 1: zero) of a refused matrix n.
+__global__ void k_focal_prepare(const double *F, int n_pairs, float *out, unsigned long long *bad) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= n_pairs) return;
+    double v[9], nrm = 0.0;
+    bool finite = true;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        v[q] = F[(size_t)n * 9 + q];
+        finite = finite && isfinite(v[q]);
+        nrm = __fma_rn(v[q], v[q], nrm);
+    }
+    if (!finite || !(nrm > 0.0)) atomicMin(bad, 2ull * n + (finite ? 1 : 0));
+    const double inv = 1.0 / sqrt(nrm);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) out[(size_t)n * 9 + q] = (float)(v[q] * inv);
 }
 
 // grid (pair blocks, candidate chunks); partial[c * n_blocks + block] for candidate c
@@ -147,72 +167,64 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
     if ((int64_t)n_cand > 65535LL * VOTE_CANDS) return fv_fail(FM_EINVAL, "n_cand must be <= 1048560");
     if (!F || !cand || !votes) return fv_fail(FM_EINVAL, "F, cand and votes must not be NULL");
     if (!(tau > 0.0) || !std::isfinite(tau)) return fv_fail(FM_EINVAL, "tau must be finite and > 0");
-    std::vector<float> hF((size_t)n_pairs * 9), hk1, hk2, hc(n_cand);
-    for (int n = 0; n < n_pairs; ++n) {
-        double nrm = 0.0;
-        for (int q = 0; q < 9; ++q) {
-            const double v = F[(size_t)n * 9 + q];
-            if (!std::isfinite(v)) return fv_fail(FM_EINVAL, "F must be finite");
-            nrm += v * v;
-        }
-        if (!(nrm > 0.0)) return fv_fail(FM_EINVAL, "F of pair " + std::to_string(n) + " is zero");
-        const double inv = 1.0 / std::sqrt(nrm);
-        for (int q = 0; q < 9; ++q) hF[(size_t)n * 9 + q] = (float)(F[(size_t)n * 9 + q] * inv);
-    }
-    auto known = [&](const double *src, std::vector<float> &dst) -> bool {
+    // one host buffer for the small inputs: candidates, then the known focal lengths that are given
+    std::vector<float> small(n_cand + (size_t)n_pairs * ((f1_known ? 1 : 0) + (f2_known ? 1 : 0)));
+    float *k1 = small.data() + n_cand, *k2 = k1 + (f1_known ? n_pairs : 0);
+    auto known = [&](const double *src, float *dst) -> bool {
         if (!src) return true;
-        dst.resize(n_pairs);
         for (int n = 0; n < n_pairs; ++n) {
             if (!(src[n] >= 0.0) || !std::isfinite(src[n])) return false;
             dst[n] = (float)src[n];
         }
         return true;
     };
-    if (!known(f1_known, hk1) || !known(f2_known, hk2))
+    if (!known(f1_known, k1) || !known(f2_known, k2))
         return fv_fail(FM_EINVAL, "known focal lengths must be finite and >= 0 (0 = the candidate)");
     for (int c = 0; c < n_cand; ++c) {
         if (!(cand[c] > 0.0) || !std::isfinite(cand[c])) return fv_fail(FM_EINVAL, "candidates must be finite and > 0");
-        hc[c] = (float)cand[c];
+        small[c] = (float)cand[c];
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n_blocks = (n_pairs + VOTE_THREADS - 1) / VOTE_THREADS;
     const int n_chunks = (n_cand + VOTE_CANDS - 1) / VOTE_CANDS;
-    float *dF = nullptr, *dk1 = nullptr, *dk2 = nullptr, *dc = nullptr, *dpart = nullptr;
-    double *dv = nullptr;
+    // one device allocation (a stream-ordered one takes 30 us): the votes and the refusal word, read back
+    // together; F as given; F in FP32; the small inputs; the block sums
+    const size_t votes_b = sizeof(double) * ((size_t)n_cand + 1), in_b = sizeof(double) * 9 * (size_t)n_pairs,
+                 f_b = sizeof(float) * 9 * (size_t)n_pairs, small_b = sizeof(float) * small.size(),
+                 part_b = sizeof(float) * (size_t)n_blocks * n_cand;
+    char *base = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaSuccess;
     auto step = [&](cudaError_t r) {
         if (e == cudaSuccess) e = r;
     };
-    step(cudaMallocAsync(&dF, sizeof(float) * hF.size(), s));
-    if (!hk1.empty()) step(cudaMallocAsync(&dk1, sizeof(float) * n_pairs, s));
-    if (!hk2.empty()) step(cudaMallocAsync(&dk2, sizeof(float) * n_pairs, s));
-    step(cudaMallocAsync(&dc, sizeof(float) * n_cand, s));
-    step(cudaMallocAsync(&dpart, sizeof(float) * (size_t)n_blocks * n_cand, s));
-    step(cudaMallocAsync(&dv, sizeof(double) * n_cand, s));
-    step(cudaMemcpyAsync(dF, hF.data(), sizeof(float) * hF.size(), cudaMemcpyHostToDevice, s));
-    if (dk1) step(cudaMemcpyAsync(dk1, hk1.data(), sizeof(float) * n_pairs, cudaMemcpyHostToDevice, s));
-    if (dk2) step(cudaMemcpyAsync(dk2, hk2.data(), sizeof(float) * n_pairs, cudaMemcpyHostToDevice, s));
-    step(cudaMemcpyAsync(dc, hc.data(), sizeof(float) * n_cand, cudaMemcpyHostToDevice, s));
-    if (elapsed_ms) {
-        step(cudaEventCreate(&e0));
-        step(cudaEventCreate(&e1));
-        if (e == cudaSuccess) step(cudaEventRecord(e0, s));
+    step(cudaMallocAsync(&base, votes_b + in_b + f_b + small_b + part_b, s));
+    double *dv = reinterpret_cast<double *>(base), *dF64 = reinterpret_cast<double *>(base + votes_b);
+    unsigned long long *dbad = reinterpret_cast<unsigned long long *>(dv + n_cand);
+    float *dF = reinterpret_cast<float *>(base + votes_b + in_b), *dc = dF + 9 * (size_t)n_pairs;
+    float *dk1 = f1_known ? dc + n_cand : nullptr, *dk2 = f2_known ? dc + (k2 - small.data()) : nullptr;
+    float *dpart = dc + small.size();
+    std::vector<double> out((size_t)n_cand + 1);
+    if (e == cudaSuccess) {
+        step(cudaMemcpyAsync(dF64, F, in_b, cudaMemcpyHostToDevice, s));
+        step(cudaMemcpyAsync(dc, small.data(), small_b, cudaMemcpyHostToDevice, s));
+        step(cudaMemsetAsync(dbad, 0xff, sizeof *dbad, s));
     }
     if (e == cudaSuccess) {
+        k_focal_prepare<<<(n_pairs + 63) / 64, 64, 0, s>>>(dF64, n_pairs, dF, dbad);
+        if (elapsed_ms) {
+            step(cudaEventCreate(&e0));
+            step(cudaEventCreate(&e1));
+            if (e == cudaSuccess) step(cudaEventRecord(e0, s));
+        }
         k_focal_vote<<<dim3(n_blocks, n_chunks), VOTE_THREADS, 0, s>>>(dF, dk1, dk2, n_pairs, dc, n_cand,
                                                                       (float)(1.0 / tau), dpart);
         k_focal_vote_sum<<<(n_cand + 7) / 8, 256, 0, s>>>(dpart, n_blocks, n_cand, dv);
         step(cudaGetLastError());
     }
     if (elapsed_ms && e == cudaSuccess) step(cudaEventRecord(e1, s));
-    if (e == cudaSuccess) step(cudaMemcpyAsync(votes, dv, sizeof(double) * n_cand, cudaMemcpyDeviceToHost, s));
-    cudaFreeAsync(dF, s);
-    if (dk1) cudaFreeAsync(dk1, s);
-    if (dk2) cudaFreeAsync(dk2, s);
-    cudaFreeAsync(dc, s);
-    cudaFreeAsync(dpart, s);
-    cudaFreeAsync(dv, s);
+    if (e == cudaSuccess) step(cudaMemcpyAsync(out.data(), dv, votes_b, cudaMemcpyDeviceToHost, s));
+    if (base) cudaFreeAsync(base, s);
     const cudaError_t es = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = es;
     if (elapsed_ms && e == cudaSuccess) e = cudaEventElapsedTime(elapsed_ms, e0, e1);
@@ -220,5 +232,10 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess)
         return fv_fail(e == cudaErrorMemoryAllocation ? FM_ENOMEM : FM_ECUDA, cudaGetErrorString(e));
+    unsigned long long bad;
+    std::memcpy(&bad, &out[n_cand], sizeof bad);
+    if (bad != ~0ull)
+        return fv_fail(FM_EINVAL, (bad & 1) ? "F of pair " + std::to_string(bad / 2) + " is zero" : std::string("F must be finite"));
+    std::memcpy(votes, out.data(), sizeof(double) * n_cand);
     return FM_OK;
 }

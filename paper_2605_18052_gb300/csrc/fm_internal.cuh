@@ -138,6 +138,8 @@ void launch_learned_loss(const DevProblem &d, const float *mlp_master, const __n
 
 // ---- kernels launched by the API layer (fm_kernels.cu) ----------------------------------------
 void launch_cam_prep(const DevProblem &d, cudaStream_t s);
+void launch_set_hyper(const DevProblem &d, const double *h, cudaStream_t s);   // h: 6 constants, by value
+void launch_begin_round(const DevProblem &d, double tau, cudaStream_t s);      // hyper[6] = tau, counter = 0
 void launch_set_params(const DevProblem &d, const double *R, const double *c, cudaStream_t s);
 cudaError_t launch_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR,
                                  double *gc, cudaStream_t s);
@@ -171,31 +173,31 @@ void launch_apply_gradient(const DevProblem &d, cudaStream_t s);
 // (with apply, when d.pair_cnt is allocated): also the geometry records of the new poses
 void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pdl = false, bool next_geo = false);
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s);
-void launch_residuals(const DevProblem &d, float *out_sorted, cudaStream_t s);
+void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s);
 
 // ---- layout kernels (fm_layout.cu) -------------------------------------------------------------
 // Validate pair ids / coordinates and detect whether the input is grouped by pair.
 void launch_validate(const int *pair_id, const float2 *x1, const float2 *x2, int64_t n_pp,
                      int n_pairs, unsigned *err, cudaStream_t s);
 // Stable sort of point pairs by pair id: writes perm (sorted -> input) and sorted keys.
+size_t sort_scratch_bytes(int64_t n_pp);
 cudaError_t sort_by_pair(const int *pair_id, int64_t n_pp, int n_pairs, int *keys_out,
-                         int *perm_out, cudaStream_t s);
+                         int *perm_out, void *scratch, cudaStream_t s);
 void launch_pair_offsets(const int *sorted_keys, int64_t n_pp, int n_pairs, int *pair_off,
                          unsigned *err, cudaStream_t s);
 void launch_range_pairs(const int *pair_off, int n_pairs, int n_ranges, int *range_pair,
                         cudaStream_t s);
-// FP16 storage: per-image centroids into d.cen (needs d.cam_off/cam_ent/pair_off/range_pair/perm);
+// point pairs in pair order from an unsorted input (d.perm), for the two launches below
+void launch_gather_points(const DevProblem &d, const float2 *x1, const float2 *x2, float4 *out, cudaStream_t s);
+// FP16 storage: per-image centroids into d.cen (needs d.cam_off/cam_ent/pair_off/range_pair);
 // `sums` is scratch for 2 * n_cams int64.
-void launch_centroids(const DevProblem &d, const int *sorted_keys, const float2 *x1,
-                      const float2 *x2, unsigned long long *sums, cudaStream_t s);
-void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2,
+void launch_centroids(const DevProblem &d, const float2 *x1, const float2 *x2, const float4 *sorted,
+                      unsigned long long *sums, cudaStream_t s);
+// keypoints in the streaming format, initial weights, scores and history
+void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2, const float4 *sorted,
                  cudaStream_t s);
-void launch_fill_weights(const DevProblem &d, float value, cudaStream_t s);
 void launch_set_weights(const DevProblem &d, const float *w_input_order, cudaStream_t s);
 void launch_get_weights(const DevProblem &d, float *w_input_order, cudaStream_t s);
-void launch_unpermute(const DevProblem &d, const float *sorted, float *input_order,
-                      cudaStream_t s);
-void launch_fill_half(__half *p, int64_t n, float value, cudaStream_t s);
 // match scores in input order -> d.score (sorted order, FP16); values outside [0, 1] -> ERR_WEIGHT
 void launch_set_scores(const DevProblem &d, const float *score_input_order, cudaStream_t s);
 

@@ -150,9 +150,10 @@ __global__ void __launch_bounds__(32 * W) k_irls_weights(DevProblem d, float tau
 
 template <int STORE>
 struct ResidualBody {
-    float *out_sorted;
+    const int *perm;
+    float *out_input;   // input order
     float out[2];
-    __device__ explicit ResidualBody(float *o) : out_sorted(o) { out[0] = out[1] = 0.f; }
+    __device__ ResidualBody(const DevProblem &d, float *o) : perm(d.perm), out_input(o) { out[0] = out[1] = 0.f; }
     __device__ __forceinline__ void point(int k, float e, float, float, float, float, float) {
         out[k] = e;
     }
@@ -162,7 +163,7 @@ struct ResidualBody {
         const int q = gb + lane * Fmt<STORE>::PPL;
 #pragma unroll
         for (int k = 0; k < Fmt<STORE>::PPL; ++k)
-            if (q + k < p_end) out_sorted[q + k] = out[k];
+            if (q + k < p_end) out_input[perm ? perm[q + k] : q + k] = out[k];
     }
 };
 
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(32 * W) k_residuals(DevProblem d, float *out) 
     extern __shared__ __align__(16) unsigned char stage[];
     const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
     if (r >= d.n_ranges) return;
-    ResidualBody<STORE> body(out);
+    ResidualBody<STORE> body(d, out);
     walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
 }
 
@@ -179,6 +180,17 @@ __global__ void k_cam_prep(DevProblem d) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= d.n_cams) return;
     write_camrec(d.cam + (size_t)k * CAMREC, d.R + 9 * (size_t)k, d.c + 3 * (size_t)k, (float)camera_scale(d, k));
+}
+
+struct Hyper {
+    double v[6];
+};
+__global__ void k_set_hyper(DevProblem d, Hyper h) { d.hyper[threadIdx.x] = h.v[threadIdx.x]; }
+
+// threshold and kept count of a round whose first pass is fused with the reweighting
+__global__ void k_begin_round(DevProblem d, double tau) {
+    d.hyper[6] = tau;
+    *d.counter = 0;
 }
 
 // new parameters from the caller's device memory, and their camera records
@@ -551,6 +563,14 @@ void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl, bool after
     launch_k(k_pair_setup, dim3(blocks_for(d.n_pairs, 256)), dim3(256), s, pdl, d, after_step ? d.n_cams : 0);
 }
 
+void launch_set_hyper(const DevProblem &d, const double *h, cudaStream_t s) {
+    Hyper v;
+    for (int q = 0; q < 6; ++q) v.v[q] = h[q];
+    k_set_hyper<<<1, 6, 0, s>>>(d, v);
+}
+
+void launch_begin_round(const DevProblem &d, double tau, cudaStream_t s) { k_begin_round<<<1, 1, 0, s>>>(d, tau); }
+
 void launch_set_params(const DevProblem &d, const double *R, const double *c, cudaStream_t s) {
     k_set_params<<<blocks_for(d.n_cams, 64), 64, 0, s>>>(d, R, c);
 }
@@ -639,10 +659,10 @@ void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {
     });
 }
 
-void launch_residuals(const DevProblem &d, float *out_sorted, cudaStream_t s) {
+void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s) {
     with_stages(d, [&](auto store, auto depth, auto warps) {
         constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        k_residuals<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, out_sorted);
+        k_residuals<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, out_input_order);
     });
 }
 
