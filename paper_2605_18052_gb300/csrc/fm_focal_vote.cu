@@ -10,9 +10,16 @@
 // Frobenius norm first, which leaves the ratio unchanged), M = E^T E, its eigenvalues by
 // four sweeps of cyclic Jacobi rotations (each 2x2 step uses the cancellation-free rotation
 // angle, so nearly equal eigenvalues keep their relative accuracy, unlike the closed-form cubic
-// roots), lambda_1 / lambda_2 = sqrt(mu_1 / mu_2). A block covers 256 pairs and VOTE_CANDS
-// candidates; per-block sums are reduced in a fixed order, then added per candidate in FP64 in
-// block order: the votes are bit-reproducible.
+// roots), lambda_1 / lambda_2 = sqrt(mu_1 / mu_2). A block covers 256 pairs and one candidate;
+// per-block sums are reduced in a fixed order, then added per candidate in FP64 in block order:
+// the votes are bit-reproducible.
+//
+// What bounds it: the chain of 24 divisions, 12 square roots and 12 reciprocal roots of a term, so
+// the number of independent terms in flight. Candidates one after the other in a block (16) left
+// short rows on a few SMs and a last wave at 5 of 7 blocks: one candidate a block takes 101 instead of
+// 119 us for 11,669 pairs x 256 candidates, 355 for 373 at 47,903 x 256, 15 for 68 at 300 x 256 and
+// 17 for 66 at 11,669 x 16; the matrix of a pair is read again per candidate, from L2. Two
+// candidates a block are within 3% at every size.
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -24,7 +31,7 @@ namespace fm {
 namespace {
 
 constexpr int VOTE_THREADS = 256;
-constexpr int VOTE_CANDS = 16;
+constexpr int VOTE_CANDS = 16;     // most candidates of a block (a grid has 65,535 rows of blocks)
 constexpr int JACOBI_SWEEPS = 4;
 
 // one Jacobi rotation of the symmetric 3x3 matrix (a00, a11, a22, a01, a02, a12) in plane (p, q)
@@ -95,13 +102,13 @@ __global__ void k_focal_prepare(const double *F, int n_pairs, float *out, unsign
     for (int q = 0; q < 9; ++q) out[(size_t)n * 9 + q] = (float)(v[q] * inv);
 }
 
-// grid (pair blocks, candidate chunks); partial[c * n_blocks + block] for candidate c
+// grid (pair blocks, rows of per_block <= VOTE_CANDS candidates); partial[c * n_blocks + block] for candidate c
 __global__ void __launch_bounds__(VOTE_THREADS)
 k_focal_vote(const float *F, const float *f1k, const float *f2k, int n_pairs, const float *cand, int n_cand,
-             float inv_tau, float *partial) {
+             int per_block, float inv_tau, float *partial) {
     __shared__ float red[VOTE_CANDS][VOTE_THREADS / 32];
     const int n = blockIdx.x * VOTE_THREADS + threadIdx.x;
-    const int c0 = blockIdx.y * VOTE_CANDS;
+    const int c0 = blockIdx.y * per_block;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float Fn[9];
     float k1 = 0.f, k2 = 0.f;
@@ -113,7 +120,7 @@ k_focal_vote(const float *F, const float *f1k, const float *f2k, int n_pairs, co
         k2 = f2k ? f2k[n] : 0.f;
     }
 #pragma unroll 1
-    for (int cc = 0; cc < VOTE_CANDS; ++cc) {
+    for (int cc = 0; cc < per_block; ++cc) {
         const int c = c0 + cc;
         float v = 0.f;
         if (valid && c < n_cand) {
@@ -125,7 +132,7 @@ k_focal_vote(const float *F, const float *f1k, const float *f2k, int n_pairs, co
         if (lane == 0) red[cc][warp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < VOTE_CANDS) {
+    if (threadIdx.x < per_block) {
         const int c = c0 + threadIdx.x;
         float s = 0.f;
 #pragma unroll
@@ -186,7 +193,8 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n_blocks = (n_pairs + VOTE_THREADS - 1) / VOTE_THREADS;
-    const int n_chunks = (n_cand + VOTE_CANDS - 1) / VOTE_CANDS;
+    const int per_block = (n_cand + 65534) / 65535;   // one candidate a block while the grid has rows for it
+    const int n_chunks = (n_cand + per_block - 1) / per_block;
     // one device allocation (a stream-ordered one takes 30 us): the votes and the refusal word, read back
     // together; F as given; F in FP32; the small inputs; the block sums
     const size_t votes_b = sizeof(double) * ((size_t)n_cand + 1), in_b = sizeof(double) * 9 * (size_t)n_pairs,
@@ -218,7 +226,7 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
             if (e == cudaSuccess) step(cudaEventRecord(e0, s));
         }
         k_focal_vote<<<dim3(n_blocks, n_chunks), VOTE_THREADS, 0, s>>>(dF, dk1, dk2, n_pairs, dc, n_cand,
-                                                                      (float)(1.0 / tau), dpart);
+                                                                      per_block, (float)(1.0 / tau), dpart);
         k_focal_vote_sum<<<(n_cand + 7) / 8, 256, 0, s>>>(dpart, n_blocks, n_cand, dv);
         step(cudaGetLastError());
     }

@@ -1,6 +1,6 @@
 """Problem creation from inputs that are and are not in pair order, at the edges of the layout kernels
 (four groups of 32 ahead in the centroid sums, ranges of 2,048, padding), and the refusals that the
-focal-length vote finds on the device. The centroids are fixed-point sums, so the order of the input may
+focal-length vote finds on the device and its grid's limit. The centroids are fixed-point sums, so the order of the input may
 not change a bit: residuals and the initial weights (1) are compared exactly."""
 import numpy as np
 import pytest
@@ -44,3 +44,13 @@ def test_focal_vote_names_the_refused_matrix(n):
         with pytest.raises(fm.FastMapError, match=text):
             fm.focal_vote(B, [400.0, 500.0], 0.1)
     np.testing.assert_array_equal(fm.focal_vote(F, [400.0, 500.0], 0.1), good)
+
+
+@pytest.mark.parametrize("n_cand", [65535, 65536, 131071])
+def test_focal_vote_with_more_candidates_than_rows_of_blocks(n_cand):
+    # every candidate list repeats the same 7 values: equal candidates get equal bits in any block
+    build.build()
+    F = np.random.default_rng(1).normal(size=(257, 3, 3))
+    c = np.resize(np.linspace(300.0, 900.0, 7), n_cand)
+    few = fm.focal_vote(F, c[:7], 0.1)
+    np.testing.assert_array_equal(fm.focal_vote(F, c, 0.1), np.resize(few, n_cand))
