@@ -22,8 +22,8 @@ namespace fm {
 // Bound by HBM on large scenes, by the latency of a range's loads and by the launches around the pass
 // on small ones. Loading 4 groups per warp into registers after the wait for the launch before
 // (8 warps a block) left the memory system idle while a pass filled up and drained. An iteration of
-// fm_step, before -> now: 119 k point pairs FP32 18.7 -> 15.1 us, 3.1 M FP32 28.0 -> 19.2, 12 M FP16
-// 39.6 -> 31.2, 49 M FP32 161 -> 154, 49 M FP16 92.3 -> 84.5, 141 M FP16 227.9 -> 219.5.
+// fm_step, before -> now: 119 k point pairs FP32 18.7 -> 13.7 us, 3.1 M FP32 28.0 -> 18.4, 12 M FP16
+// 39.6 -> 30.8, 49 M FP32 161 -> 153, 49 M FP16 92.3 -> 84, 141 M FP16 227.9 -> 216.
 template <int STORE, int MODE, int S, int W>
 __global__ void __launch_bounds__(32 * W) k_stream_loss(DevProblem d, int prev_loss) {
     extern __shared__ __align__(16) unsigned char stage[];

@@ -201,8 +201,8 @@ __device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, c
     body.group_done(gb, st.p_end, lane);
 }
 
-// The walk of a range, staged in shared memory by asynchronous copies, a chunk of 4 groups (2 KB of keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the
-// launch before this one; the first S chunks are requested ahead of it, so they arrive while that
+// The walk of a range, staged in shared memory by asynchronous copies, a chunk of 4 groups (2 KB of
+// keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the launch before this one; the first S chunks are requested ahead of it, so they arrive while that
 // launch finishes. (Keypoints are static. Weights are written at least two launches earlier: a pass
 // that writes them is followed by the camera step, which lets this launch start only after its own
 // wait for that pass.)
@@ -214,7 +214,12 @@ __device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) 
                  : "memory");
 }
 
-// UNROLL: groups of a chunk in straight code (1 for bodies of many instructions).
+// UNROLL: groups of a chunk in straight code (1 for bodies of many instructions). A chunk inside one image
+// pair takes one branch and reads its four groups before their sums: a warp that checks every group
+// issues the loads of one at a time, and where few warps share an SM the pass is that chain of latencies
+// (an iteration on 119 k point pairs 15.1 -> 13.7 us, 3.1 M FP32 19.2 -> 18.4; 141 M FP16 219.5 -> 216).
+// Where UNROLL is below a chunk (the quadratic-form pass) the second copy of the body costs
+// more than it gives: 403 -> 421 us for a round on 49 M.
 template <int STORE, bool NEED_W, int S, int UNROLL = STAGE_GROUPS, class Body, class Before>
 __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, int lane, Body &body, unsigned char *stage,
                                                   Before before) {
@@ -244,9 +249,28 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
         asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
         __syncwarp();   // a lane's weights were copied by another lane
         const unsigned char *src = stage + (c % S) * STAGE_BYTES;
+        const int cb = st.p_begin + c * CHUNK;
+        if (UNROLL == STAGE_GROUPS && cb + CHUNK <= st.seg_end) {
+            typename F::Raw raw[STAGE_GROUPS];
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u) {
+                raw[u].kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
+                raw[u].w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u) {
+#pragma unroll
+                for (int k = 0; k < F::PPL; ++k) {
+                    float x1, y1, x2, y2, w;
+                    F::get(raw[u], k, x1, y1, x2, y2, w);
+                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+                }
+                body.group_done(cb + u * GROUP, st.p_end, lane);
+            }
+        } else
 #pragma unroll UNROLL
         for (int u = 0; u < STAGE_GROUPS; ++u) {
-            const int gb = st.p_begin + c * CHUNK + u * GROUP;
+            const int gb = cb + u * GROUP;
             if (gb >= st.p_end) break;
             typename F::Raw raw;
             raw.kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
@@ -260,11 +284,12 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
 }
 
 // Depth and block size of the staged passes. FP32: 4 chunks (512 point pairs) a warp; the whole range,
-// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 15.5 ->
-// 15.1 us an iteration, 245 ranges 17.5 -> 16.8; 733 ranges 17.9 -> 19.2). FP16: 2 chunks (512 point
-// pairs). One warp per block, so that a finished range makes room for the next at once, but four from
-// 300 ranges per SM on, where the block launches count (FP16: 68,633 ranges 223.6 -> 219.5 us, 23,860
-// ranges 84.5 -> 85.8).
+// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 13.8 ->
+// 13.65 us an iteration, 245 ranges 16.3 -> 16.0; 733 ranges 16.6 -> 18.5). FP16: 2 chunks (512 point
+// pairs; 4 chunks: 5,860 ranges 30.8 -> 32.2, 48,829 ranges 163.5 -> 166.8). One warp per block, so that a
+// finished range makes room for the next at once, but four from 300 ranges per SM on, where the block
+// launches count (FP16: 48,829 ranges 163.5 -> 162.3 us, 68,633 ranges 223.6 -> 219.5, 23,860 ranges
+// 85.5 -> 85.9).
 constexpr int FEW_RANGES = 2 * 152, MANY_RANGES = 300 * 152;
 
 template <class Launch>
