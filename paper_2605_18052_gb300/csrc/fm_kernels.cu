@@ -369,9 +369,8 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // over the lanes (a pair that spans many ranges does not hold up one lane). The warp reduces
 // the 6 gradient components and the loss with a compensated (TwoSum) FP32 butterfly, so each
 // sum is carried as an unevaluated hi + lo pair.
-// Phase 2: warp 0, a lane per component of each of the block's cameras: the Adam update (FP32
-// moments), R <- Exp(phi) R and Gram-Schmidt re-orthonormalisation in FP64, the centre update in
-// FP64 and the new camera record (camera_update).
+// Phase 2: the update of the block's cameras, spread over warps (step_update). The two powers of its
+// bias corrections are formed before the wait.
 // Geometry comes from the pair records, never from another camera's record, which another
 // block may be updating. The loss of a pair is counted by its first camera only; each camera's
 // FP64 loss share goes to cam_loss[camera], and the next kernel (the next pass, pair setup or
@@ -387,26 +386,20 @@ template <bool FOCAL>
 __global__ void __launch_bounds__(STEP_CAMS * 32, 4)
 k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo) {
     constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;   // sums carried per camera
-    __shared__ float s_hi[STEP_VALS][STEP_CAMS], s_lo[STEP_VALS][STEP_CAMS];
+    __shared__ StepState<STEP_CAMS> st;
     __shared__ int4 s_item[STEP_CAMS][32];
     __shared__ __align__(16) float s_geo[STEP_CAMS][32][GEO];
-    __shared__ float s_mv[STEP_CAMS][12];     // Adam m (6) and v (6) of the block's cameras
-    __shared__ double s_Rc[STEP_CAMS][12];    // R (9) and c (3) of the block's cameras
-    __shared__ float s_R32[STEP_CAMS][10];    // their records' rotations (9) and keypoint scale
-    __shared__ double s_hyper[6];   // lr_rot, lr_c, beta1, beta2, eps, lr_focal
+    __shared__ float s_bc[2][2];
+    __shared__ long long s_step;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x * STEP_CAMS + warp;
-    {
-        const int cam0 = blockIdx.x * STEP_CAMS;
-        for (int i = threadIdx.x; i < STEP_CAMS * 12; i += STEP_CAMS * 32) {
-            const int cc = i / 12, q = i % 12;
-            if (cam0 + cc < d.n_cams) {
-                s_mv[cc][q] = q < 6 ? d.m[(size_t)(cam0 + cc) * 6 + q] : d.v[(size_t)(cam0 + cc) * 6 + q - 6];
-                s_Rc[cc][q] = q < 9 ? d.R[(size_t)(cam0 + cc) * 9 + q] : d.c[(size_t)(cam0 + cc) * 3 + q - 9];
-                if (q < 10) s_R32[cc][q] = d.cam[(size_t)(cam0 + cc) * CAMREC + (q < 9 ? q : 15)];
-            }
-        }
-        if (threadIdx.x < 6) s_hyper[threadIdx.x] = d.hyper[threadIdx.x];
+    st.load(d, d.cam, blockIdx.x * STEP_CAMS);
+    // bias corrections before the wait: the pass that runs now may or may not have added the step before
+    // this one to the count, so they are formed for both counts
+    if (warp == STEP_CAMS - 1 && lane < 4) {
+        const long long t = *reinterpret_cast<volatile long long *>(d.step);
+        s_bc[lane >> 1][lane & 1] = bias_correction((float)d.hyper[2 + (lane & 1)], t + 1 + (lane >> 1));
+        if (lane == 0) s_step = t;
     }
     const int e_begin = k < d.n_cams ? d.cam_off[k] : 0;
     const int e_end = k < d.n_cams ? d.cam_off[k + 1] : 0;
@@ -470,23 +463,22 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
 #pragma unroll
         for (int q = 0; q < NV; ++q)
             if (lane == spread_lane(NV, q)) {
-                s_hi[q][warp] = hi[0];
-                s_lo[q][warp] = lo[0];
+                st.hi[q][warp] = hi[0];
+                st.lo[q][warp] = lo[0];
             }
     }
     __syncthreads();
-    if (warp == 0) {
-        const int cc = lane / 3, ca = lane % 3, kc = blockIdx.x * STEP_CAMS + cc;
-        const bool on = cc < STEP_CAMS && kc < d.n_cams;
-        const int sc = on ? cc : 0;
-        const double bl = camera_update<FOCAL>(d, kc, on, ca, 3 * cc, &s_hi[0][sc], &s_lo[0][sc], STEP_CAMS, s_mv[sc],
-                                               s_Rc[sc], s_R32[sc], s_hyper, t_step, apply,
-                                               d.cam + (size_t)kc * CAMREC);
-        if (apply && next_geo) __threadfence();   // the record reaches L2 before any count below
-        if (on && ca == 0) d.cam_loss[kc] = bl;
+    if (warp <= rot_roles(STEP_CAMS)) {
+        const long long ahead = t_step - 1 - s_step;
+        float bc1 = s_bc[ahead & 1][0], bc2 = s_bc[ahead & 1][1];
+        if (ahead < 0 || ahead > 1) {   // the count moved by more than that step
+            bc1 = bias_correction(st.hyper[2], t_step);
+            bc2 = bias_correction(st.hyper[3], t_step);
+        }
+        step_update<FOCAL, false>(d, st, blockIdx.x * STEP_CAMS, warp, lane, bc1, bc2, t_step, apply, true, d.cam);
     }
     if (!(apply && next_geo)) return;
-    __syncthreads();   // the block's new records are written
+    __syncthreads();   // the block's new records are written (the releases below order them for the other blocks)
     if (k < d.n_cams) {
         for (int e = e_begin + lane; e < e_end; e += 32) {
             const int n = d.cam_ent[e] >> 1;
@@ -495,39 +487,23 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
     }
 }
 
-// Adam step with a given gradient (d.grad, FP64), a warp for STEP_CAMS cameras: the same update as
-// the camera-step kernel (camera_update with the gradient split into FP32 hi + lo parts, whose FP32
-// sum is the gradient rounded to FP32, as there); the step count is advanced by k_bump_step.
-__global__ void __launch_bounds__(32) k_apply_gradient(DevProblem d) {
-    const int lane = threadIdx.x, cc = lane / 3, ca = lane % 3;
-    const int kc = blockIdx.x * STEP_CAMS + cc;
-    const bool on = cc < STEP_CAMS && kc < d.n_cams;
-    const size_t k = on ? kc : 0;
+// Adam step with a given gradient (d.grad, FP64): the same update as the camera-step kernel (with the
+// gradient split into FP32 hi + lo parts, whose FP32 sum is the gradient rounded to FP32, as there); the
+// step count is advanced by k_bump_step.
+__global__ void __launch_bounds__(128) k_apply_gradient(DevProblem d) {
+    __shared__ StepState<STEP_CAMS> st;
+    const int cam0 = blockIdx.x * STEP_CAMS;
     const long long t_step = *d.step + 1;
-    float hi[STEP_VALS], lo[STEP_VALS], mv[12], rec[10];
-    double Rc[12], hyper[6];
-#pragma unroll
-    for (int q = 0; q < STEP_VALS; ++q) {
-        const double g = q < 6 ? d.grad[k * 6 + q] : 0.0;
-        hi[q] = (float)g;
-        lo[q] = (float)__dsub_rn(g, (double)hi[q]);
+    st.load(d, d.cam, cam0);
+    if (threadIdx.x < STEP_CAMS * STEP_VALS) {
+        const int q = threadIdx.x % STEP_VALS, cc = threadIdx.x / STEP_VALS;
+        const double g = q < 6 && cam0 + cc < d.n_cams ? d.grad[(size_t)(cam0 + cc) * 6 + q] : 0.0;
+        st.hi[q][cc] = (float)g;
+        st.lo[q][cc] = (float)__dsub_rn(g, (double)st.hi[q][cc]);
     }
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        mv[q] = d.m[k * 6 + q];
-        mv[6 + q] = d.v[k * 6 + q];
-        hyper[q] = d.hyper[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        Rc[q] = d.R[k * 9 + q];
-        rec[q] = d.cam[k * CAMREC + q];
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) Rc[9 + q] = d.c[k * 3 + q];
-    rec[9] = d.cam[k * CAMREC + 15];
-    __syncwarp();   // every lane has read its camera's state before a lane replaces part of it
-    camera_update<false>(d, kc, on, ca, 3 * cc, hi, lo, 1, mv, Rc, rec, hyper, t_step, 1, d.cam + (size_t)kc * CAMREC);
+    __syncthreads();
+    step_update<false, false>(d, st, cam0, threadIdx.x >> 5, threadIdx.x & 31, bias_correction(st.hyper[2], t_step),
+                              bias_correction(st.hyper[3], t_step), t_step, 1, true, d.cam);
 }
 
 __global__ void k_bump_step(DevProblem d) { *d.step += 1; }
@@ -636,7 +612,7 @@ void loss_scales(const DevProblem &d, float &gscale, float &lscale) {
 }
 
 void launch_apply_gradient(const DevProblem &d, cudaStream_t s) {
-    k_apply_gradient<<<blocks_for(d.n_cams, STEP_CAMS), 32, 0, s>>>(d);
+    k_apply_gradient<<<blocks_for(d.n_cams, STEP_CAMS), 128, 0, s>>>(d);
     k_bump_step<<<1, 1, 0, s>>>(d);
 }
 

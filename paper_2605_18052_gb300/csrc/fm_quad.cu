@@ -208,19 +208,14 @@ __device__ __forceinline__ void form_sums(const float4 *rec, const float *g, flo
 //   q = g0 + W d,  loss = c0 + d^T (g0 + q),  d = E'_n - e0,
 // and the chain rule to camera k. Both cameras of a pair evaluate it (O(1) each), which
 // removes a per-pair launch and the wait on it. The warp reduces with compensated butterflies,
-// then warp 0 does the FP64 update of the block's cameras and writes the new
-// records to cam_dst: the records of this step's poses stay intact in cam_src for the other
+// then the block updates its cameras (step_update) and writes the new records to cam_dst: the records of this step's poses stay intact in cam_src for the other
 // blocks. The Adam step count is *d.step + 1 + it; the launch that closes the chain adds
 // the chain's length to *d.step.
 template <bool FOCAL>
 __global__ void __launch_bounds__(STEP_CAMS * 32, 4)
 k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gscale, float lscale, int apply) {
     constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;   // sums carried per camera
-    __shared__ float s_hi[STEP_VALS][STEP_CAMS], s_lo[STEP_VALS][STEP_CAMS];
-    __shared__ float s_mv[STEP_CAMS][12];
-    __shared__ double s_Rc[STEP_CAMS][12];
-    __shared__ float s_R32[STEP_CAMS][10];    // the cameras' records' rotations (9) and keypoint scale
-    __shared__ double s_hyper[6];   // lr_rot, lr_c, beta1, beta2, eps, lr_focal
+    __shared__ StepState<STEP_CAMS> st;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x * STEP_CAMS + warp;
     const int e_begin = k < d.n_cams ? d.cam_off[k] : 0;
@@ -238,18 +233,7 @@ k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gs
     }
     pdl_wait();     // camera records, poses and moments of the previous step
     pdl_trigger();
-    {
-        const int cam0 = blockIdx.x * STEP_CAMS;
-        for (int i = threadIdx.x; i < STEP_CAMS * 12; i += STEP_CAMS * 32) {
-            const int cc = i / 12, q = i % 12;
-            if (cam0 + cc < d.n_cams) {
-                s_mv[cc][q] = q < 6 ? d.m[(size_t)(cam0 + cc) * 6 + q] : d.v[(size_t)(cam0 + cc) * 6 + q - 6];
-                s_Rc[cc][q] = q < 9 ? d.R[(size_t)(cam0 + cc) * 9 + q] : d.c[(size_t)(cam0 + cc) * 3 + q - 9];
-                if (q < 10) s_R32[cc][q] = cam_src[(size_t)(cam0 + cc) * CAMREC + (q < 9 ? q : 15)];
-            }
-        }
-        if (threadIdx.x < 6) s_hyper[threadIdx.x] = d.hyper[threadIdx.x];
-    }
+    st.load(d, cam_src, blockIdx.x * STEP_CAMS);
     const long long t_step = *d.step + 1 + it;
     if (k < d.n_cams) {
         float hi[STEP_VALS], lo[STEP_VALS];
@@ -276,20 +260,14 @@ k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gs
 #pragma unroll
         for (int q = 0; q < NV; ++q)
             if (lane == spread_lane(NV, q)) {
-                s_hi[q][warp] = hi[0];
-                s_lo[q][warp] = lo[0];
+                st.hi[q][warp] = hi[0];
+                st.lo[q][warp] = lo[0];
             }
     }
     __syncthreads();
-    if (warp == 0) {
-        const int cc = lane / 3, ca = lane % 3, kc = blockIdx.x * STEP_CAMS + cc;
-        const bool on = cc < STEP_CAMS && kc < d.n_cams;
-        const int sc = on ? cc : 0;
-        const double bl = camera_update<FOCAL>(d, kc, on, ca, 3 * cc, &s_hi[0][sc], &s_lo[0][sc], STEP_CAMS, s_mv[sc],
-                                               s_Rc[sc], s_R32[sc], s_hyper, t_step, apply,
-                                               cam_dst + (size_t)kc * CAMREC);
-        if (on && ca == 0) d.cam_loss[kc] = bl;
-    }
+    if (warp <= rot_roles(STEP_CAMS))
+        step_update<FOCAL, false>(d, st, blockIdx.x * STEP_CAMS, warp, lane, bias_correction(st.hyper[2], t_step),
+                                  bias_correction(st.hyper[3], t_step), t_step, apply, true, cam_dst);
 }
 
 // iters of these iterations in one cooperative launch, one grid barrier each, for as many cameras as
@@ -298,7 +276,8 @@ k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gs
 // lane: 16-byte loads free of bank conflicts). The same arithmetic as k_quad_step, bit for bit. What bounds
 // an iteration is its serial chain: other cameras' records from L2, geometry and chain rule,
 // the compensated sums, the FP64 update and the barrier. 25 iterations on 1,000 cameras and 11,700
-// pairs: 135 us, 5.4 us each (12.4 us as launches). More cameras than resident warps take k_quad_step, whose
+// pairs: 114 us, 4.5 us each (12.4 us as launches; 5.4 us with the update in one warp and the state
+// read back from memory each iteration). More cameras than resident warps take k_quad_step, whose
 // blocks then overlap each other's latencies (4,000 cameras: 500 blocks, 15 us an iteration).
 constexpr int QROW = 60;
 constexpr int QUAD_SMEM = STEP_CAMS * 32 * QROW * (int)sizeof(float);
@@ -308,11 +287,8 @@ __global__ void __launch_bounds__(STEP_CAMS * 32, 2)
 k_quad_steps(DevProblem d, int iters, float gscale, float lscale) {
     constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;   // sums carried per camera
     extern __shared__ __align__(16) float s_rec[];          // [STEP_CAMS][32][QROW]
-    __shared__ float s_hi[STEP_VALS][STEP_CAMS], s_lo[STEP_VALS][STEP_CAMS];
-    __shared__ float s_mv[STEP_CAMS][12];
-    __shared__ double s_Rc[STEP_CAMS][12];
-    __shared__ float s_R32[STEP_CAMS][10];
-    __shared__ double s_hyper[6];
+    __shared__ StepState<STEP_CAMS> st;                      // stays here from iteration to iteration
+    __shared__ float s_bc[2][2];                             // bias corrections of this and the next iteration
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cam0 = blockIdx.x * STEP_CAMS, k = cam0 + warp;
     GridBarrier gb(d.grid_state, d.err);
@@ -333,19 +309,12 @@ k_quad_steps(DevProblem d, int iters, float gscale, float lscale) {
 #pragma unroll
         for (int q = 0; q < QREC / 4; ++q) row[q] = rec[q];
     }
-    if (threadIdx.x < 6) s_hyper[threadIdx.x] = d.hyper[threadIdx.x];
     const long long t0 = *d.step;
+    st.load(d, d.cam, cam0);
+    if (threadIdx.x < 2) s_bc[0][threadIdx.x] = bias_correction((float)d.hyper[2 + threadIdx.x], t0 + 1);
     for (int it = 0; it < iters; ++it) {
         const float *src = (it & 1) ? d.cam_alt : d.cam;
         float *dst = (it & 1) ? d.cam : d.cam_alt;
-        for (int i = threadIdx.x; i < STEP_CAMS * 12; i += STEP_CAMS * 32) {
-            const int cc = i / 12, q = i % 12;
-            if (cam0 + cc < d.n_cams) {
-                s_mv[cc][q] = q < 6 ? d.m[(size_t)(cam0 + cc) * 6 + q] : d.v[(size_t)(cam0 + cc) * 6 + q - 6];
-                s_Rc[cc][q] = q < 9 ? d.R[(size_t)(cam0 + cc) * 9 + q] : d.c[(size_t)(cam0 + cc) * 3 + q - 9];
-                if (q < 10) s_R32[cc][q] = __ldcg(src + (size_t)(cam0 + cc) * CAMREC + (q < 9 ? q : 15));
-            }
-        }
         if (k < d.n_cams) {
             float hi[STEP_VALS], lo[STEP_VALS];
 #pragma unroll
@@ -364,20 +333,16 @@ k_quad_steps(DevProblem d, int iters, float gscale, float lscale) {
 #pragma unroll
             for (int q = 0; q < NV; ++q)
                 if (lane == spread_lane(NV, q)) {
-                    s_hi[q][warp] = hi[0];
-                    s_lo[q][warp] = lo[0];
+                    st.hi[q][warp] = hi[0];
+                    st.lo[q][warp] = lo[0];
                 }
         }
         __syncthreads();
-        if (warp == 0) {
-            const int cc = lane / 3, ca = lane % 3, kc = cam0 + cc;
-            const bool on = cc < STEP_CAMS && kc < d.n_cams;
-            const int sc = on ? cc : 0;
-            const double bl = camera_update<FOCAL>(d, kc, on, ca, 3 * cc, &s_hi[0][sc], &s_lo[0][sc], STEP_CAMS, s_mv[sc],
-                                                   s_Rc[sc], s_R32[sc], s_hyper, t0 + 1 + it, 1,
-                                                   dst + (size_t)kc * CAMREC);
-            if (on && ca == 0 && it + 1 == iters) d.cam_loss[kc] = bl;
-        }
+        if (warp <= rot_roles(STEP_CAMS))
+            step_update<FOCAL, true>(d, st, cam0, warp, lane, s_bc[it & 1][0], s_bc[it & 1][1], t0 + 1 + it, 1,
+                                     it + 1 == iters, dst);
+        else if (warp == STEP_CAMS - 1 && lane < 2)
+            s_bc[(it + 1) & 1][lane] = bias_correction(st.hyper[2 + lane], t0 + 2 + it);
         if (!gb.sync()) return;
     }
     gb.finish();

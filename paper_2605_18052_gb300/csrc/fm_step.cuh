@@ -239,120 +239,166 @@ __device__ __forceinline__ void warp_two_sum_spread(float *hi, float *lo, int la
     }
 }
 
-// Phase 2 of a step, by one warp: lane 3 c + a holds component a of camera kc (the block's camera c;
-// `on` for lanes that have one), so that the warp finishes up to ten cameras at once. apply = 0: the
-// gradient (FP64 sum of its hi + lo parts) and the focal gradient are written, nothing else. apply =
-// 1: one Adam step (FP32 moments) and the new pose: R <- R + (Exp(phi) - I) R and c <- c + delta_c in
-// FP64, where the small increment (Exp(phi) - I) R is formed in FP32 from the camera's FP32 record
-// rotation R32 (its error, a few 1e-7 |phi|, is of the order of phi's own FP32 error), then
-// Gram-Schmidt on the rows in FP64 on every eighth step (steps 1, 9, 17, ...) and the new camera
-// record at rec_out. hi/lo hold STEP_VALS values (6 pose gradient components, the loss, the
-// keypoint-scale gradient) `stride` apart; mv = the camera's Adam m (6) and v (6); Rc = its R
-// (9) and c (3) in FP64; rec = its current record's rotation (9 floats) and keypoint scale
-// (rec[9]); hyper = lr_rot, lr_c, beta1, beta2, eps, lr_focal. With focal refinement
-// rho = log s takes its own Adam step (gradient s dL/ds); without, the record keeps its scale.
-// Returns the camera's loss share.
-// GB300 issues an FP64 instruction (conversions included) of a warp over 64 cycles, whatever its
-// active lanes, and every block of a step reaches this phase at the same moment. So the update keeps
-// its FP64 work to the state itself (two sums, the record; re-orthonormalisation, about 40
-// operations, only every eighth step), and spreads a camera's components over lanes: about 21 FP64
-// instructions where a lane per camera took 48, and a third of the FP32 chain. Between two
-// re-orthonormalisations R leaves SO(3) by the FP32 rounding of the increments, a few 1e-7 |phi| per
-// step, far below the FP32 camera record's resolution.
-template <bool FOCAL>
-__device__ __forceinline__ double camera_update(const DevProblem &d, int kc, bool on, int a, int base, const float *hi,
-                                                const float *lo, int stride, const float *mv, const double *Rc,
-                                                const float *rec, const double *hyper, long long t_step, int apply,
-                                                float *rec_out) {
-    const float *R32 = rec;
-    const double bl = (double)hi[6 * stride] + (double)lo[6 * stride];
+// ---- the update of a block's C cameras ------------------------------------------------------------
+// What a block of a step kernel holds of its cameras: the sums of phase 1 (6 pose gradient components,
+// the loss, the keypoint-scale gradient, as hi + lo), Adam's m (6) and v (6), R (9) and c (3) in FP64,
+// the current record's rotation (9) and keypoint scale, and the hyper-parameters lr_rot, lr_c, beta1,
+// beta2, eps, lr_focal.
+template <int C>
+struct StepState {
+    float hi[STEP_VALS][C], lo[STEP_VALS][C], mv[C][12], rec[C][10], hyper[6];
+    double Rc[C][12];
+    __device__ __forceinline__ void load(const DevProblem &d, const float *cam, int cam0) {
+        for (int i = threadIdx.x; i < C * 12; i += blockDim.x) {
+            const int cc = i / 12, q = i % 12;
+            if (cam0 + cc < d.n_cams) {
+                const size_t k = cam0 + cc;
+                mv[cc][q] = q < 6 ? d.m[k * 6 + q] : d.v[k * 6 + q - 6];
+                Rc[cc][q] = q < 9 ? d.R[k * 9 + q] : d.c[k * 3 + q - 9];
+                if (q < 10) rec[cc][q] = cam[k * CAMREC + (q < 9 ? q : 15)];
+            }
+        }
+        if (threadIdx.x < 6) hyper[threadIdx.x] = (float)d.hyper[threadIdx.x];
+    }
+};
+
+// 1 - beta^t
+__device__ __forceinline__ float bias_correction(float beta, long long t) { return radd(1.f, -powf(beta, (float)t)); }
+
+// Adam's step of one component (gradient g; m and v are replaced)
+__device__ __forceinline__ float adam_delta(float g, float lr, const float *hyper, float bc1, float bc2, float &m, float &v) {
+    const float b1 = hyper[2], b2 = hyper[3], eps = hyper[4];
+    m = rfma(b1, m, rmul(radd(1.f, -b1), g));
+    v = rfma(b2, v, rmul(rmul(radd(1.f, -b2), g), g));
+    return __fdiv_rn(rmul(-lr, __fdiv_rn(m, bc1)), radd(__fsqrt_rn(__fdiv_rn(v, bc2)), eps));
+}
+
+// Phase 2 of a step, by the warps that take the roles 0 .. ROT_ROLES(C) of their block (a role a warp,
+// behind a block barrier after phase 1). One Adam step (FP32 moments) and the new pose:
+// R <- R + (Exp(phi) - I) R and c <- c + delta_c in FP64, where the small increment (Exp(phi) - I) R is
+// formed in FP32 from the camera's FP32 record rotation (its error, a few 1e-7 |phi|, is of the order of
+// phi's own FP32 error), then Gram-Schmidt on the rows in FP64 on every eighth step (steps 1, 9, 17, ...)
+// and the new camera record in `records`. apply = 0: the gradient (FP64 sum of its hi + lo parts) and the
+// focal gradient are written, nothing else. With focal refinement rho = log s takes its own Adam step
+// (gradient s dL/ds); without, the record keeps its scale. KEEP: the new state is left in `st` as well
+// and goes to memory only with `store` (a kernel of several steps).
+// The first roles take the rotations of three cameras each, lane 9 c + 3 r + q the entry (r, q); the
+// last role the centres, keypoint scales and loss shares of all, lane 3 c + a a component.
+// GB300 issues an FP64 instruction (conversions included) of a warp over 64 cycles, whatever its active
+// lanes, and every block of a step reaches this phase at the same moment. So the update keeps its FP64
+// work to the state itself and spreads it over lanes and over the SM's four sub-partitions, one role
+// each: 3 such instructions in series for a rotation (re-orthonormalisation, about 40, only every eighth
+// step) and 8 for a centre and its loss, where one warp with a lane per row of R took 26 with the
+// conversions of the hyper-parameters (and a lane per camera 48). An iteration on 119 k point pairs went
+// from 13.0 to 11.8 us, on 3.1 M from 19.8 to 18.2, a form iteration from 5.4 to 4.5. Between two re-orthonormalisations R leaves SO(3) by the FP32 rounding of the
+// increments, a few 1e-7 |phi| per step, far below the FP32 camera record's resolution.
+constexpr int rot_roles(int cams) { return (cams + 2) / 3; }
+
+template <bool FOCAL, bool KEEP, int C>
+__device__ __forceinline__ void step_update(const DevProblem &d, StepState<C> &st, int cam0, int role, int lane, float bc1,
+                                            float bc2, long long t_step, int apply, bool store, float *records) {
+    if (role < rot_roles(C)) {
+        if (!apply) return;
+        const int c9 = lane / 9, r = (lane % 9) / 3, q = lane % 3, base = 9 * c9;
+        const int cc = 3 * role + c9, kc = cam0 + cc;
+        const bool on = lane < 27 && cc < C && kc < d.n_cams;
+        const int s = on ? cc : 0;
+        // the FP32 gradient: hi is the rounded value of hi + lo (TwoSum keeps |lo| within half an
+        // ulp of hi), so hi + lo in FP32 is the same number the FP64 sum would round to
+        const float g = radd(st.hi[r][s], st.lo[r][s]);
+        if (on && !isfinite(g)) atomicOr(d.err, ERR_NONFINITE);
+        float m = st.mv[s][r], v = st.mv[s][6 + r], phi[3], A[3];
+        const float dl = adam_delta(g, st.hyper[0], st.hyper, bc1, bc2, m, v);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) phi[a] = __shfl_sync(0xffffffffu, dl, min(base + 3 * a, 31));
+        so3_exp_minus_identity_row(phi, r, A);
+        const float *R32 = st.rec[s];
+        double Rn = __dadd_rn(st.Rc[s][3 * r + q], (double)rdot3(A[0], R32[q], A[1], R32[3 + q], A[2], R32[6 + q]));
+        if ((t_step & 7) == 1) {
+            double M[9];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) M[i] = __shfl_sync(0xffffffffu, Rn, min(base + i, 31));
+            orthonormalize_rows(M);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) Rn = i == 3 * r + q ? M[i] : Rn;
+        }
+        if (KEEP) __syncwarp();   // every lane has read the rows that are replaced
+        if (on) {
+            records[(size_t)kc * CAMREC + 3 * r + q] = (float)Rn;
+            if (!KEEP || store) d.R[(size_t)kc * 9 + 3 * r + q] = Rn;
+            if (KEEP) {
+                st.Rc[s][3 * r + q] = Rn;
+                st.rec[s][3 * r + q] = (float)Rn;
+            }
+            if (q == 0) {
+                if (!KEEP || store) {
+                    d.m[(size_t)kc * 6 + r] = m;
+                    d.v[(size_t)kc * 6 + r] = v;
+                }
+                if (KEEP) {
+                    st.mv[s][r] = m;
+                    st.mv[s][6 + r] = v;
+                }
+            }
+        }
+        return;
+    }
+    const int cc = lane / 3, a = lane % 3, kc = cam0 + cc;
+    const bool on = cc < C && kc < d.n_cams;
+    const int s = on ? cc : 0;
+    const double bl = (double)st.hi[6][s] + (double)st.lo[6][s];
     const double s_cur = FOCAL && on ? camera_scale(d, kc) : 1.0;
-    const double g_rho = FOCAL ? s_cur * ((double)hi[7 * stride] + (double)lo[7 * stride]) : 0.0;
+    const double g_rho = FOCAL ? s_cur * ((double)st.hi[7][s] + (double)st.lo[7][s]) : 0.0;
+    if (on && a == 0 && (!KEEP || store)) d.cam_loss[kc] = bl;
     if (!apply) {
-        bool ok = isfinite(hi[6 * stride]);
+        bool ok = isfinite(st.hi[6][s]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int q = 3 * h + a;
-            const double g = (double)hi[q * stride] + (double)lo[q * stride];
+            const double g = (double)st.hi[q][s] + (double)st.lo[q][s];
             ok = ok && isfinite(g);
             if (on) d.grad[(size_t)kc * 6 + q] = g;
         }
         if (on && !ok) atomicOr(d.err, ERR_NONFINITE);
         if (on && a == 0 && d.grad_rho) d.grad_rho[kc] = g_rho;
-        return bl;
+        return;
     }
-    // the FP32 gradient: hi is the rounded value of hi + lo (TwoSum keeps |lo| within half an
-    // ulp of hi), so hi + lo in FP32 is the same number the FP64 sum would round to
-    float gq[2];
-    bool ok = isfinite(hi[6 * stride]);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        gq[h] = radd(hi[(3 * h + a) * stride], lo[(3 * h + a) * stride]);
-        ok = ok && isfinite(gq[h]);
-    }
-    if (on && !ok) atomicOr(d.err, ERR_NONFINITE);
-    float s_new = rec[9];
-    const float b1 = (float)hyper[2], b2 = (float)hyper[3], eps = (float)hyper[4];
-    const float lr[2] = {(float)hyper[0], (float)hyper[1]};
-    const float bc1 = radd(1.f, -powf(b1, (float)t_step)), bc2 = radd(1.f, -powf(b2, (float)t_step));
+    const float g = radd(st.hi[3 + a][s], st.lo[3 + a][s]);
+    if (on && !(isfinite(g) && isfinite(st.hi[6][s]))) atomicOr(d.err, ERR_NONFINITE);
+    float s_new = st.rec[s][9];
     if (FOCAL && on && a == 0) {
-        const float g1 = (float)g_rho;
+        const float b1 = st.hyper[2], b2 = st.hyper[3], g1 = (float)g_rho;
         const float mo = rfma(b1, d.rho_m[kc], rmul(radd(1.f, -b1), g1));
         const float vo = rfma(b2, d.rho_v[kc], rmul(rmul(radd(1.f, -b2), g1), g1));
         d.rho_m[kc] = mo;
         d.rho_v[kc] = vo;
-        const double r = d.rho[kc] - (double)__fdiv_rn(rmul((float)hyper[5], __fdiv_rn(mo, bc1)),
-                                                       radd(__fsqrt_rn(__fdiv_rn(vo, bc2)), eps));
+        const double r = d.rho[kc] - (double)__fdiv_rn(rmul(st.hyper[5], __fdiv_rn(mo, bc1)),
+                                                       radd(__fsqrt_rn(__fdiv_rn(vo, bc2)), st.hyper[4]));
         d.rho[kc] = r;
         d.grad_rho[kc] = g_rho;
         s_new = (float)exp(r);
     }
-    float dl[2], mo[2], vo[2];   // phi_a and c_a
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int q = 3 * h + a;
-        mo[h] = rfma(b1, mv[q], rmul(radd(1.f, -b1), gq[h]));
-        vo[h] = rfma(b2, mv[6 + q], rmul(rmul(radd(1.f, -b2), gq[h]), gq[h]));
-        dl[h] = __fdiv_rn(rmul(-lr[h], __fdiv_rn(mo[h], bc1)), radd(__fsqrt_rn(__fdiv_rn(vo[h], bc2)), eps));
-    }
-    float phi[3], A[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) phi[q] = __shfl_sync(0xffffffffu, dl[0], base + q);
-    so3_exp_minus_identity_row(phi, a, A);
-    double Rn[3];   // row a
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        Rn[c] = __dadd_rn(Rc[3 * a + c], (double)rdot3(A[0], R32[c], A[1], R32[3 + c], A[2], R32[6 + c]));
-    if ((t_step & 7) == 1) {
-        double M[9];
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) M[3 * r + c] = __shfl_sync(0xffffffffu, Rn[c], base + r);
-        orthonormalize_rows(M);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Rn[c] = a == 0 ? M[c] : (a == 1 ? M[3 + c] : M[6 + c]);
-    }
-    const double cn = __dadd_rn(Rc[9 + a], (double)dl[1]);
+    float m = st.mv[s][3 + a], v = st.mv[s][9 + a];
+    const float dl = adam_delta(g, st.hyper[1], st.hyper, bc1, bc2, m, v);
+    const double cn = __dadd_rn(st.Rc[s][9 + a], (double)dl);
     if (on) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const size_t o = (size_t)kc * 6 + 3 * h + a;
-            d.m[o] = mo[h];
-            d.v[o] = vo[h];
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            d.R[(size_t)kc * 9 + 3 * a + c] = Rn[c];
-            rec_out[3 * a + c] = (float)Rn[c];
-        }
-        d.c[(size_t)kc * 3 + a] = cn;
+        float *rec_out = records + (size_t)kc * CAMREC;
         const float c_hi = (float)cn;
         rec_out[9 + a] = c_hi;
         rec_out[12 + a] = (float)__dsub_rn(cn, (double)c_hi);
         if (a == 0) rec_out[15] = s_new;
+        if (!KEEP || store) {
+            d.c[(size_t)kc * 3 + a] = cn;
+            d.m[(size_t)kc * 6 + 3 + a] = m;
+            d.v[(size_t)kc * 6 + 3 + a] = v;
+        }
+        if (KEEP) {
+            st.Rc[s][9 + a] = cn;
+            st.mv[s][3 + a] = m;
+            st.mv[s][9 + a] = v;
+            if (a == 0) st.rec[s][9] = s_new;
+        }
     }
-    return bl;
 }
 
 }  // namespace fm
