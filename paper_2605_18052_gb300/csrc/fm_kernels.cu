@@ -359,16 +359,19 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 }
 
 // ---- per camera: Adam + exponential map (FP64) -----------------------------------------------------
-// Fused per-camera step, 8 cameras per 256-thread block (all blocks resident at once).
-// Before waiting for the streaming pass (griddepcontrol.wait) the block fetches everything that
-// is at least two kernels old: its cameras' Adam moments, poses and the step count, and for
+// Fused per-camera step, C cameras a block and W warps a camera (all blocks resident at once for up to
+// 4,864 cameras). Before waiting for the streaming pass (griddepcontrol.wait) the block fetches everything
+// that is at least two kernels old: its cameras' Adam moments, poses and the step count, and for
 // each camera the (pair, role) entries, their range-partial counts and the pairs' geometry
 // records (into shared memory). After the wait only the partial sums remain to be read.
-// Phase 1: warp w owns camera k = 8*block + w. The chain rule is linear in a pair's sums, so it
-// is applied to every (pair, warp-range partial) item separately; the items are spread evenly
-// over the lanes (a pair that spans many ranges does not hold up one lane). The warp reduces
-// the 6 gradient components and the loss with a compensated (TwoSum) FP32 butterfly, so each
-// sum is carried as an unevaluated hi + lo pair.
+// Phase 1: the chain rule is linear in a pair's sums, so it is applied to every (pair, warp-range partial)
+// item separately; the items are spread evenly over the lanes of the camera's warps, 32 a pass, W passes
+// at once (a pair that spans many ranges does not hold up one lane). Each sum is carried as an unevaluated
+// hi + lo pair (TwoSum); a lane's items are added in the order of their passes and the lanes by a
+// butterfly, whatever W is, so every W gives the same bits; with W > 1 the warps share the values out.
+// What bounds it is latency: a pass of loads and chain rule takes about 2,000 cycles, and a warp a camera
+// makes three of them in series on 1,000 cameras and 49 M point pairs. An iteration there 83.7 -> 79.2 us
+// (FP16), on 16 cameras and 119 k 11.6 -> 10.55, on 128 and 3.1 M (FP32) 16.9 -> 12.2.
 // Phase 2: the update of the block's cameras, spread over warps (step_update). The two powers of its
 // bias corrections are formed before the wait.
 // Geometry comes from the pair records, never from another camera's record, which another
@@ -376,27 +379,40 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // FP64 loss share goes to cam_loss[camera], and the next kernel (the next pass, pair setup or
 // the finalize kernel) adds them up in a fixed order and advances the step count.
 // Phase 3 (next_geo, with apply): the geometry records of the new poses, so the next pass
-// needs no pair-setup launch. Each camera's warp counts its image pairs in d.pair_cnt (one
+// needs no pair-setup launch. Each camera's warps count its image pairs in d.pair_cnt (one
 // acquire-release atomic per (pair, camera); every such step adds 2 to each pair's count); the
 // camera that finds an odd count is the pair's second, both records are then written, and it
 // computes the pair's record. A record is overwritten only after both of its readers in this
 // launch (the pair's two cameras) have passed phase 1, and the pass that read E'_n has
 // completed before this kernel's wait.
-template <bool FOCAL>
-__global__ void __launch_bounds__(STEP_CAMS * 32, 4)
+template <bool FOCAL, int C, int W>
+__global__ void __launch_bounds__(32 * C * W, 1024 / (32 * C * W))
 k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo) {
-    constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;   // sums carried per camera
-    __shared__ StepState<STEP_CAMS> st;
-    __shared__ int4 s_item[STEP_CAMS][32];
-    __shared__ __align__(16) float s_geo[STEP_CAMS][32][GEO];
+    constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;      // sums carried per camera
+    constexpr int NQ = W == 1 ? NV : (STEP_VALS + W - 1) / W;  // of which a warp adds up
+    __shared__ StepState<C> st;
+    __shared__ int4 s_item[C][32];
+    constexpr int ROW = GEO - 8 + 4;   // a record from its float 8 on; 16-byte reads free of bank conflicts
+    __shared__ __align__(16) float s_geo[8 + C * 32 * ROW];
+    __shared__ float s_con[W > 1 ? C : 1][W][STEP_VALS][32];   // contributions of W passes over the items
     __shared__ float s_bc[2][2];
     __shared__ long long s_step;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int k = blockIdx.x * STEP_CAMS + warp;
-    st.load(d, d.cam, blockIdx.x * STEP_CAMS);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cc = warp / W, sub = warp % W;
+    const int cam0 = blockIdx.x * C, k = cam0 + cc;
+    // the warps of a camera, barrier 1 + cc (literal ids: with an id in a register a block reserves all 16
+    // barriers, and an SM then holds only three blocks beside a pass)
+    static_assert(W == 1 || C <= 4, "a barrier per camera");
+    auto camera_sync = [&] {
+        if (W == 1) __syncwarp();
+        else if (C < 2 || cc == 0) asm volatile("bar.sync 1, %0;" ::"n"(32 * W) : "memory");
+        else if (C < 3 || cc == 1) asm volatile("bar.sync 2, %0;" ::"n"(32 * W) : "memory");
+        else if (cc == 2) asm volatile("bar.sync 3, %0;" ::"n"(32 * W) : "memory");
+        else asm volatile("bar.sync 4, %0;" ::"n"(32 * W) : "memory");
+    };
+    st.load(d, d.cam, cam0);
     // bias corrections before the wait: the pass that runs now may or may not have added the step before
     // this one to the count, so they are formed for both counts
-    if (warp == STEP_CAMS - 1 && lane < 4) {
+    if (warp == C * W - 1 && lane < 4) {
         const long long t = *reinterpret_cast<volatile long long *>(d.step);
         s_bc[lane >> 1][lane & 1] = bias_correction((float)d.hyper[2 + (lane & 1)], t + 1 + (lane >> 1));
         if (lane == 0) s_step = t;
@@ -405,6 +421,7 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
     const int e_end = k < d.n_cams ? d.cam_off[k + 1] : 0;
     // this camera's entries, 32 at a time: pair, role, first range and number of ranges; the
     // pair's geometry record goes to shared memory
+    int pair0 = 0, ci = 0, cj = 0;   // of the lane's first entry, for the geometry at the end
     auto load_chunk = [&](int base) -> int {
         const int e = base + lane;
         int n = 0, role = 0, r0 = 0, cnt = 0;
@@ -415,9 +432,14 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
             r0 = d.pair_off[n] / WR;
             cnt = (d.pair_off[n + 1] - 1) / WR - r0 + 1;
             const float4 *gv = reinterpret_cast<const float4 *>(d.geo + (size_t)n * GEO);
-            float4 *dst = reinterpret_cast<float4 *>(s_geo[warp][lane]);
+            float4 *dst = reinterpret_cast<float4 *>(s_geo + (cc * 32 + lane) * ROW);
 #pragma unroll
-            for (int q = 2; q < GEO / 4; ++q) dst[q] = gv[q];
+            for (int q = 2 + sub; q < GEO / 4; q += W) dst[q] = gv[q];
+            if (base == e_begin && sub == 0) {
+                pair0 = n;
+                ci = d.cam_i[n];
+                cj = d.cam_j[n];
+            }
         }
         int incl = cnt;
 #pragma unroll
@@ -425,64 +447,100 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
             const int x = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += x;
         }
-        s_item[warp][lane] = make_int4(incl - cnt, n, role, r0);
-        __syncwarp();
+        if (sub == 0) s_item[cc][lane] = make_int4(incl - cnt, n, role, r0);
+        camera_sync();
         return __shfl_sync(0xffffffffu, incl, 31);
     };
+    auto find = [&](int t) {   // the entry of item t
+        int lo = 0, hi = 31;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_item[cc][mid].x <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    };
     int total = load_chunk(e_begin);
+    const int first = find(32 * sub + lane);
     pdl_wait();     // partial sums of the streaming pass
     pdl_trigger();
     const long long t_step = *d.step + 1;
     if (k < d.n_cams) {
-        float hi[STEP_VALS], lo[STEP_VALS];
+        float hi[NQ], lo[NQ];
 #pragma unroll
-        for (int q = 0; q < STEP_VALS; ++q) hi[q] = lo[q] = 0.f;
+        for (int q = 0; q < NQ; ++q) hi[q] = lo[q] = 0.f;
         for (int base = e_begin; base < e_end; base += 32) {
             if (base != e_begin) {
-                __syncwarp();
+                camera_sync();
                 total = load_chunk(base);
             }
-            for (int t = lane; t < total; t += 32) {
-                int lo_i = 0, hi_i = 31;
-                while (lo_i < hi_i) {
-                    const int mid = (lo_i + hi_i + 1) >> 1;
-                    if (s_item[warp][mid].x <= t) lo_i = mid;
-                    else hi_i = mid - 1;
-                }
-                const int4 it = s_item[warp][lo_i];
-                const float4 *sl = reinterpret_cast<const float4 *>(d.slots + (size_t)(it.y + it.w + (t - it.x)) * SLOT);
-                const float4 sa = sl[0], sb = sl[1], sc = sl[2];
-                const float sum[10] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w, sc.x, sc.y};
+            for (int t0 = 0; t0 < total; t0 += 32 * W) {
+                const int t = t0 + 32 * sub + lane;
                 float contrib[STEP_VALS];
-                pair_chain_rule<FOCAL>(s_geo[warp][lo_i], it.z, sum, gscale, lscale, contrib);
+                if (t < total) {
+                    const int li = t0 == 0 && base == e_begin ? first : find(t);
+                    const int4 it = s_item[cc][li];
+                    const float4 *sl = reinterpret_cast<const float4 *>(d.slots + (size_t)(it.y + it.w + (t - it.x)) * SLOT);
+                    const float4 sa = sl[0], sb = sl[1], sc = sl[2];
+                    const float sum[10] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w, sc.x, sc.y};
+                    pair_chain_rule<FOCAL>(s_geo + (cc * 32 + li) * ROW, it.z, sum, gscale, lscale, contrib);
+                }
+                if (W == 1) {
+                    if (t < total) {
 #pragma unroll
-                for (int q = 0; q < NV; ++q) two_sum_acc(hi[q], lo[q], contrib[q], 0.f);
+                        for (int q = 0; q < NV; ++q) two_sum_acc(hi[q], lo[q], contrib[q], 0.f);
+                    }
+                    continue;
+                }
+                if (t < total) {
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) s_con[cc][sub][q][lane] = contrib[q];
+                }
+                camera_sync();
+#pragma unroll
+                for (int w = 0; w < W; ++w)   // a lane's items in their order
+                    if (t0 + 32 * w + lane < total) {
+#pragma unroll
+                        for (int j = 0; j < NQ; ++j)
+                            if (sub + W * j < NV) two_sum_acc(hi[j], lo[j], s_con[cc][w][sub + W * j][lane], 0.f);
+                    }
+                if (t0 + 32 * W < total) camera_sync();
             }
         }
-        warp_two_sum_spread<NV>(hi, lo, lane);
+        warp_two_sum_spread<NQ>(hi, lo, lane);
 #pragma unroll
-        for (int q = 0; q < NV; ++q)
-            if (lane == spread_lane(NV, q)) {
-                st.hi[q][warp] = hi[0];
-                st.lo[q][warp] = lo[0];
+        for (int j = 0; j < NQ; ++j) {
+            const int q = W == 1 ? j : sub + W * j;
+            if (lane == spread_lane(NQ, j) && q < NV) {
+                st.hi[q][cc] = hi[0];
+                st.lo[q][cc] = lo[0];
             }
+        }
     }
     __syncthreads();
-    if (warp <= rot_roles(STEP_CAMS)) {
+    // blocks of one SM start their roles in different sub-partitions
+    constexpr int ROLES = rot_roles(C) + 1, APART = ROLES == 2 ? 2 : 1;
+    static_assert(ROLES * APART <= C * W, "a warp for each role");
+    const int role = ((warp - (int)(blockIdx.x / 152)) & (C * W - 1)) / APART;
+    if (role < ROLES && ((warp - (int)(blockIdx.x / 152)) & (APART - 1)) == 0) {
         const long long ahead = t_step - 1 - s_step;
         float bc1 = s_bc[ahead & 1][0], bc2 = s_bc[ahead & 1][1];
         if (ahead < 0 || ahead > 1) {   // the count moved by more than that step
             bc1 = bias_correction(st.hyper[2], t_step);
             bc2 = bias_correction(st.hyper[3], t_step);
         }
-        step_update<FOCAL, false>(d, st, blockIdx.x * STEP_CAMS, warp, lane, bc1, bc2, t_step, apply, true, d.cam);
+        step_update<FOCAL, false>(d, st, cam0, role, lane, bc1, bc2, t_step, apply, true, d.cam);
     }
     if (!(apply && next_geo)) return;
     __syncthreads();   // the block's new records are written (the releases below order them for the other blocks)
     if (k < d.n_cams) {
-        for (int e = e_begin + lane; e < e_end; e += 32) {
-            const int n = d.cam_ent[e] >> 1;
-            if (atomic_add_acq_rel(d.pair_cnt + n, 1u) & 1u) pair_geometry(d, n, d.cam_i[n], d.cam_j[n]);
+        for (int e = e_begin + 32 * sub + lane; e < e_end; e += 32 * W) {
+            if (e >= e_begin + 32) {
+                pair0 = d.cam_ent[e] >> 1;
+                ci = d.cam_i[pair0];
+                cj = d.cam_j[pair0];
+            }
+            if (atomic_add_acq_rel(d.pair_cnt + pair0, 1u) & 1u) pair_geometry(d, pair0, ci, cj);
         }
     }
 }
@@ -620,12 +678,27 @@ void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pd
     float gscale, lscale;
     loss_scales(d, gscale, lscale);
     const int ng = next_geo && d.pair_cnt ? 1 : 0;
-    if (d.refine_focal)
-        launch_k(k_camera_step<true>, dim3(blocks_for(d.n_cams, STEP_CAMS)), dim3(STEP_CAMS * 32), s, pdl, d,
-                 gscale, lscale, apply ? 1 : 0, ng);
+    auto go = [&](auto cams, auto warps) {
+        constexpr int C = decltype(cams)::value, W = decltype(warps)::value;
+        const dim3 grid(blocks_for(d.n_cams, C)), block(32 * C * W);
+        if (d.refine_focal) launch_k(k_camera_step<true, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, ng);
+        else launch_k(k_camera_step<false, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, ng);
+    };
+    using std::integral_constant;
+    // Items (range partials of a camera's pairs) a camera: at most 2 (ranges + pairs) / cameras. A block of
+    // one camera and 4 warps while every camera has an SM (152 cameras, 3 M point pairs: 13.2 us an iteration,
+    // 14.0 with 2 x 2), or while the blocks are resident at once and a camera has more than the 64 items that
+    // two warps take in one pass (16 cameras, 5 M: 17.1 against 21.8; 1,000 cameras, 49 M FP32: 143.6
+    // against 146.1; with fewer items 1,000 cameras, 3 M: 31.7 against 25.7). Two cameras of 2 warps while
+    // those are resident (2,000 cameras, 12 M: 34.8, 37.0 with 4 x 1; 3,000 cameras, 6 M: 34.1 against 33.2).
+    // Four cameras of one warp beyond (eight: 4,000 cameras 221.7 against 220.8).
+    const int64_t items = 2 * ((int64_t)d.n_ranges + d.n_pairs);
+    if (d.n_cams <= 152 || (d.n_cams <= 8 * 152 && items > 64 * (int64_t)d.n_cams))
+        go(integral_constant<int, 1>(), integral_constant<int, 4>());
+    else if (d.n_cams <= 16 * 152)
+        go(integral_constant<int, 2>(), integral_constant<int, 2>());
     else
-        launch_k(k_camera_step<false>, dim3(blocks_for(d.n_cams, STEP_CAMS)), dim3(STEP_CAMS * 32), s, pdl, d,
-                 gscale, lscale, apply ? 1 : 0, ng);
+        go(integral_constant<int, 4>(), integral_constant<int, 1>());
 }
 
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {
