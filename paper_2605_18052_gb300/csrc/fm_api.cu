@@ -211,19 +211,21 @@ void time_end(fm_problem *p, int pass, cudaStream_t s) {
     p->tev_used[pass] += 2;
 }
 
-// one optimiser iteration, chained with programmatic dependent launch: the pass over the point
-// pairs, then the camera step, which also writes the geometry records of the new poses; the
-// first iteration of a chain computes the geometry with a pair-setup launch, later ones find
-// it written and their pass finishes the previous step's loss total and step count.
-// `reweight`: the round's reweighting fused into this iteration's pass (always a first one).
-void enqueue_iteration(fm_problem *p, cudaStream_t s, bool timed, bool first, bool reweight = false) {
-    if (first) launch_pair_setup(p->d, s, true, false);
+// optimiser iteration `it` of a chain, with programmatic dependent launch: the pass over the point pairs,
+// then the camera step; both form the pairs' geometry from the camera records, which alternate
+// between two buffers. From the second iteration on, the pass finishes the previous step's loss total and
+// step count. The first pass of a chain reads weights that any launch before it may have written, so
+// it starts after that launch's end, unless it is the round's reweighting (`reweight`), which reads none.
+void enqueue_iteration(fm_problem *p, cudaStream_t s, bool timed, int it, bool reweight) {
+    DevProblem d = p->d;
+    float *dst = d.cam_alt;
+    if (it & 1) std::swap(d.cam, dst);
     const int pass = reweight ? FM_PASS_STREAM_REWEIGHT : FM_PASS_STREAM_LOSS;
     const bool t = timed && time_begin(p, pass, s);
-    if (reweight) launch_stream_reweight(p->d, s, !t);
-    else launch_stream_loss(p->d, s, !t, !first);
+    if (reweight) launch_stream_reweight(d, s, !t);
+    else launch_stream_loss(d, s, !t && it > 0, it > 0);
     if (t) time_end(p, pass, s);
-    launch_camera_step(p->d, true, s, !t, true);
+    launch_camera_step(d, true, dst, s, !t);
 }
 
 // loss and gradient at the current poses, chained like an iteration; the caller's device memory
@@ -231,10 +233,9 @@ void enqueue_iteration(fm_problem *p, cudaStream_t s, bool timed, bool first, bo
 void enqueue_loss_grad(fm_problem *p, double *d_loss, double *d_grad) {
     DevProblem d = p->d;
     if (d_grad) d.grad = d_grad;
-    launch_pair_setup(d, p->s, true, false);
-    launch_stream_loss(d, p->s, true);
-    launch_camera_step(d, false, p->s, true);
-    launch_finalize(d, false, p->s, true, d_loss);
+    launch_stream_loss(d, p->s);
+    launch_camera_step(d, false, nullptr, p->s, true);
+    launch_finalize(d, 0, nullptr, false, p->s, true, d_loss);
 }
 
 // `iters` chained iterations and the closing finalize launch (reweight: the first pass fused
@@ -249,11 +250,11 @@ void enqueue_iterations(fm_problem *p, cudaStream_t s, bool timed, int iters, bo
             launch_quad_step(p->d, it, even ? p->d.cam : p->d.cam_alt, even ? p->d.cam_alt : p->d.cam, true, s,
                              true);
         }
-        launch_finalize_n(p->d, iters, (iters & 1) ? p->d.cam_alt : nullptr, s, true);
+        launch_finalize(p->d, iters, (iters & 1) ? p->d.cam_alt : nullptr, false, s, true);
         return;
     }
-    for (int it = 0; it < iters; ++it) enqueue_iteration(p, s, timed, it == 0, reweight && it == 0);
-    launch_finalize(p->d, true, s, !timed);
+    for (int it = 0; it < iters; ++it) enqueue_iteration(p, s, timed, it, reweight && it == 0);
+    launch_finalize(p->d, 1, (iters & 1) ? p->d.cam_alt : nullptr, true, s, !timed);
 }
 
 // a graph of `iters` chained iterations (reweight: the first pass fused with the reweighting)
@@ -272,8 +273,8 @@ fm_status build_graph(fm_problem *p, int iters, cudaGraphExec_t *out, bool quad 
     return FM_OK;
 }
 
-// n chained iterations as CUDA graphs of whole chains (one pair-setup and one finalize launch
-// per chain), built on first use and kept by length; a chain runs at most CHAIN_MAX
+// n chained iterations as CUDA graphs of whole chains (one finalize launch per chain), built on first
+// use and kept by length; a chain runs at most CHAIN_MAX
 // iterations, and once CHAIN_CACHE lengths are kept, new lengths run as chains of 8 and 1.
 // reweight: the first pass is fused with the round's reweighting.
 fm_status launch_chains(fm_problem *p, int n, bool reweight) {
@@ -353,7 +354,7 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     Arena arena;
     arena.add(&d.R, 9 * nc);         // R, c and the error word are read together (read_params)
     arena.add(&d.c, 3 * nc);
-    arena.add(&d.err, 1);            // from here to pair_cnt: zero at the start
+    arena.add(&d.err, 1);            // from here to the geometry records: zero at the start
     arena.add(&d.m, 6 * nc);
     arena.add(&d.v, 6 * nc);
     arena.add(&d.rho, nc);
@@ -363,10 +364,10 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     arena.add(&d.step, 1);
     arena.add(&d.cen, nc);
     arena.add(&d.geo, GEO * np);
-    arena.add(&d.pair_cnt, np);
     arena.add(&d.cam_loss, nc);
     arena.add(&d.hyper, 8);
     arena.add(&d.cam, CAMREC * nc);
+    arena.add(&d.cam_alt, CAMREC * nc);
     arena.add(&d.cam_i, np);
     arena.add(&d.cam_j, np);
     arena.add(&d.pair_off, np + 1);
@@ -394,7 +395,7 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     d.perm = nullptr;
     d.fbuf = nullptr;
 
-    FM_CUDA(cudaMemsetAsync(d.err, 0, (char *)d.cam_loss - (char *)d.err, p->s));
+    FM_CUDA(cudaMemsetAsync(d.err, 0, (char *)d.geo - (char *)d.err, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_i, cam_i, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_j, cam_j, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_off, cam_off.data(), sizeof(int) * (n_cams + 1), cudaMemcpyHostToDevice, p->s));
@@ -774,8 +775,8 @@ FM_API fm_status fm_step_learned(fm_problem *p, const fm_mlp *net, double tau, d
     launch_learned_loss(p->d, master, wbf, (float)tau, std::isinf(tau_cap) ? INFINITY : (float)tau_cap, round,
                         p->hist_valid, p->s, false);
     if (tl) time_end(p, FM_PASS_LEARNED_LOSS, p->s);
-    launch_camera_step(p->d, true, p->s, !tl);
-    launch_finalize(p->d, true, p->s, !tl);
+    launch_camera_step(p->d, true, p->d.cam_alt, p->s, !tl);
+    launch_finalize(p->d, 1, p->d.cam_alt, false, p->s, !tl);
     FM_CUDA(cudaGetLastError());
     p->quad_valid = false;
     p->hist_valid = 1;
@@ -1034,7 +1035,6 @@ fm_status quad_prepare(fm_problem *p) {
     Arena arena;
     arena.add(&p->d.qslots, (size_t)QSLOT * ((size_t)p->d.n_pairs + p->d.n_ranges));
     arena.add(&p->d.quad, (size_t)QREC * p->d.n_pairs);
-    arena.add(&p->d.cam_alt, (size_t)CAMREC * p->d.n_cams);
     arena.add(&p->d.grid_state, GRID_STATE_WORDS);
     FM_CUDA(arena.commit(p));
     FM_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
@@ -1096,7 +1096,7 @@ FM_API fm_status fm_loss_grad_quadratic(fm_problem *p, double *loss, double *gra
     if (fm_status st = quad_check(p)) return st;
     FM_CUDA(join_in(p));
     launch_quad_step(p->d, 0, p->d.cam, p->d.cam_alt, false, p->s, false);
-    launch_finalize(p->d, false, p->s);
+    launch_finalize(p->d, 0, nullptr, false, p->s);
     FM_CUDA(cudaGetLastError());
     FM_CUDA(cudaMemcpyAsync(loss, p->d.loss_out, sizeof(double), cudaMemcpyDeviceToHost, p->s));
     if (grad)

@@ -88,8 +88,7 @@ struct DevProblem {
     // point: per (pair, range) partials and per pair records
     float *qslots;          // (n_pairs + n_ranges) x QSLOT
     float *quad;            // n_pairs x QREC: c0, g0(9), M(36), e0(9), pad
-    float *cam_alt;         // n_cams x CAMREC: second camera-record buffer of the fused step
-    unsigned *pair_cnt;     // per pair: cameras updated by camera steps with the geometry phase
+    float *cam_alt;         // n_cams x CAMREC: second camera-record buffer of the optimiser steps
     unsigned *grid_state;   // grid barriers of the persistent steps on the form
 };
 
@@ -144,15 +143,12 @@ void launch_set_params(const DevProblem &d, const double *R, const double *c, cu
 cudaError_t launch_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR,
                                  double *gc, cudaStream_t s);
 // pdl: launch with programmatic stream serialisation (overlaps the predecessor's tail)
-// after_step: the previous kernel was an optimiser camera step whose loss total and step
-// count this launch finishes
-void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl = false, bool after_step = false);
-// loss total of the last camera step (and the step count after an optimiser step)
-// (loss_copy: also written to the caller's device memory)
-void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl = false, double *loss_copy = nullptr);
-// the same with `count` steps added, and camera records copied back from copy_src if not null
-void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl,
-                       double *loss_copy = nullptr);
+void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl = false);
+// loss total of the last camera step and `count` added to the step count (loss_copy: also written to the
+// caller's device memory); camera records copied back from copy_src if not null; check: image pairs that
+// the new poses make degenerate are reported
+void launch_finalize(const DevProblem &d, int count, const float *copy_src, bool check, cudaStream_t s, bool pdl = false,
+                     double *loss_copy = nullptr);
 int camera_step_blocks(const DevProblem &d);
 // factors applied to the raw sums of the loss (Sum w eps^2 or Sum |eps|, weights stored as
 // w * s): gradient 2/(Z s) and loss 1/(Z s) for IRLS, 1/Z for L1
@@ -169,9 +165,9 @@ void launch_gather(const DevProblem &d, bool count_step, cudaStream_t s);
 // exponential map, camera record; the last block sums the loss and advances the step count
 // Adam step of every camera with the gradient in d.grad (FP64, n_cams x 6); advances the step
 void launch_apply_gradient(const DevProblem &d, cudaStream_t s);
-// apply = false computes the gradient and loss only (no Adam step, no step count); next_geo
-// (with apply, when d.pair_cnt is allocated): also the geometry records of the new poses
-void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pdl = false, bool next_geo = false);
+// apply = false computes the gradient and loss only; apply: the new camera records go to cam_dst, another
+// buffer than d.cam
+void launch_camera_step(const DevProblem &d, bool apply, float *cam_dst, cudaStream_t s, bool pdl = false);
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s);
 void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s);
 

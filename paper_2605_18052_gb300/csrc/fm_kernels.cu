@@ -11,33 +11,38 @@
 //   irls_weights / residuals: the same streaming walk writing one value per point pair
 #include <math.h>
 
+#include <algorithm>
+
 #include "fm_step.cuh"
 
 namespace fm {
 
-// W warps per block, a range each, staged in shared memory S chunks deep (walk_range_staged). The last
-// block has no range: when the pass follows an optimiser camera step (prev_loss > 0; that step also
-// wrote this pass's geometry records), it finishes the step's loss total (over prev_loss per-camera
-// shares) and step count.
+template <int S>
+constexpr int PASS_BYTES = S * STAGE_BYTES + CameraE::BYTES;   // shared memory of a warp
+
+// A warp per block, a range each, staged in shared memory S chunks deep (walk_range_staged). The last block
+// has no range: when the pass follows an optimiser camera step (prev_loss > 0), it finishes the
+// step's loss total (over prev_loss per-camera shares) and step count.
 // Bound by HBM on large scenes, by the latency of a range's loads and by the launches around the pass
 // on small ones. Loading 4 groups per warp into registers after the wait for the launch before
 // (8 warps a block) left the memory system idle while a pass filled up and drained. An iteration of
-// fm_step, before -> now: 119 k point pairs FP32 18.7 -> 13.7 us, 3.1 M FP32 28.0 -> 18.4, 12 M FP16
-// 39.6 -> 30.8, 49 M FP32 161 -> 153, 49 M FP16 92.3 -> 84, 141 M FP16 227.9 -> 216.
-template <int STORE, int MODE, int S, int W>
-__global__ void __launch_bounds__(32 * W) k_stream_loss(DevProblem d, int prev_loss) {
+// fm_step (this pass, then the camera step), before -> now: 119 k point pairs FP32 18.7 -> 8.5 us,
+// 3.1 M FP32 28.0 -> 11.2, 12 M FP16 39.6 -> 28.6, 49 M FP32 161 -> 142, 49 M FP16 92.3 -> 79.0, 141 M FP16
+// 227.9 -> 218.9.
+template <int STORE, int MODE, int S>
+__global__ void __launch_bounds__(32, 32) k_stream_loss(DevProblem d, int prev_loss) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
+    const int r = blockIdx.x;
     if (r >= d.n_ranges) {
         pdl_wait();
         pdl_trigger();
         if (prev_loss > 0 && blockIdx.x == gridDim.x - 1)
-            finish_step<32 * W>(d, prev_loss, 1, reinterpret_cast<double *>(stage));
+            finish_step<32>(d, prev_loss, 1, reinterpret_cast<double *>(stage));
         return;
     }
     LossBody<MODE> body(d);
-    walk_range_staged<STORE, MODE == MODE_LOSS_IRLS, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {
-        pdl_wait();     // pair geometry of this pass
+    walk_range_staged<STORE, MODE == MODE_LOSS_IRLS, S, STAGE_GROUPS, CameraE>(d, r, threadIdx.x, body, stage, [] {
+        pdl_wait();     // camera records of this pass
         pdl_trigger();  // the per-camera step may be scheduled once the last wave has started
     });
 }
@@ -85,14 +90,13 @@ struct ReweightLossBody {
     }
 };
 
-template <int STORE, int S, int W>
-__global__ void __launch_bounds__(32 * W) k_stream_reweight(DevProblem d) {
+template <int STORE, int S>
+__global__ void __launch_bounds__(32, 32) k_stream_reweight(DevProblem d) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
-    if (r >= d.n_ranges) return;
+    const int r = blockIdx.x;
     ReweightLossBody<STORE> body(d, 0.f);
-    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [&] {
-        pdl_wait();     // pair geometry of this pass, the threshold
+    walk_range_staged<STORE, false, S, STAGE_GROUPS, CameraE>(d, r, threadIdx.x, body, stage, [&] {
+        pdl_wait();     // camera records of this pass, the threshold
         pdl_trigger();
         body.tau = (float)d.hyper[6];
     });
@@ -135,13 +139,12 @@ struct WeightBody {
     }
 };
 
-template <int STORE, int S, int W>
-__global__ void __launch_bounds__(32 * W) k_irls_weights(DevProblem d, float tau) {
+template <int STORE, int S>
+__global__ void __launch_bounds__(32) k_irls_weights(DevProblem d, float tau) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.x * W + warp;
-    if (r >= d.n_ranges) return;
+    const int lane = threadIdx.x, r = blockIdx.x;
     WeightBody<STORE> body(d, tau);
-    walk_range_staged<STORE, false, S>(d, r, lane, body, stage + warp * S * STAGE_BYTES, [] {});
+    walk_range_staged<STORE, false, S>(d, r, lane, body, stage, [] {});
     unsigned k = body.kept;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
@@ -167,13 +170,12 @@ struct ResidualBody {
     }
 };
 
-template <int STORE, int S, int W>
-__global__ void __launch_bounds__(32 * W) k_residuals(DevProblem d, float *out) {
+template <int STORE, int S>
+__global__ void __launch_bounds__(32) k_residuals(DevProblem d, float *out) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
-    if (r >= d.n_ranges) return;
+    const int r = blockIdx.x;
     ResidualBody<STORE> body(d, out);
-    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
+    walk_range_staged<STORE, false, S>(d, r, threadIdx.x, body, stage, [] {});
 }
 
 __global__ void k_cam_prep(DevProblem d) {
@@ -217,17 +219,12 @@ __global__ void k_pose_gradient(int n_cams, const double *grad, const double *R,
     gc[3 * (size_t)k + a] = g[3 + a] * s;
 }
 
-// prev_loss > 0: this pass follows an optimiser step with that many per-camera loss shares;
-// block 0 (with 256 threads) finishes that step's loss total and step count.
-__global__ void __launch_bounds__(256) k_pair_setup(DevProblem d, int prev_loss) {
+__global__ void __launch_bounds__(256) k_pair_setup(DevProblem d) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = n < d.n_pairs ? d.cam_i[n] : 0, j = n < d.n_pairs ? d.cam_j[n] : 0;
     pdl_wait();     // camera records of the previous step
     pdl_trigger();
-    __shared__ double red[FIN_THREADS];
-    if (prev_loss > 0 && blockIdx.x == 0) finish_step(d, prev_loss, 1, red);
-    if (n >= d.n_pairs) return;
-    pair_geometry(d, n, i, j);
+    if (n < d.n_pairs) pair_geometry(d, n, i, j);
 }
 
 // ---- per pair: combine partials and chain rule ----------------------------------------------------
@@ -362,8 +359,8 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // Fused per-camera step, C cameras a block and W warps a camera (all blocks resident at once for up to
 // 4,864 cameras). Before waiting for the streaming pass (griddepcontrol.wait) the block fetches everything
 // that is at least two kernels old: its cameras' Adam moments, poses and the step count, and for
-// each camera the (pair, role) entries, their range-partial counts and the pairs' geometry
-// records (into shared memory). After the wait only the partial sums remain to be read.
+// each camera the (pair, role) entries, their range-partial counts and the pairs' geometry (formed again
+// from the camera records). After the wait only the partial sums remain to be read.
 // Phase 1: the chain rule is linear in a pair's sums, so it is applied to every (pair, warp-range partial)
 // item separately; the items are spread evenly over the lanes of the camera's warps, 32 a pass, W passes
 // at once (a pair that spans many ranges does not hold up one lane). Each sum is carried as an unevaluated
@@ -374,20 +371,13 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // (FP16), on 16 cameras and 119 k 11.6 -> 10.55, on 128 and 3.1 M (FP32) 16.9 -> 12.2.
 // Phase 2: the update of the block's cameras, spread over warps (step_update). The two powers of its
 // bias corrections are formed before the wait.
-// Geometry comes from the pair records, never from another camera's record, which another
-// block may be updating. The loss of a pair is counted by its first camera only; each camera's
-// FP64 loss share goes to cam_loss[camera], and the next kernel (the next pass, pair setup or
-// the finalize kernel) adds them up in a fixed order and advances the step count.
-// Phase 3 (next_geo, with apply): the geometry records of the new poses, so the next pass
-// needs no pair-setup launch. Each camera's warps count its image pairs in d.pair_cnt (one
-// acquire-release atomic per (pair, camera); every such step adds 2 to each pair's count); the
-// camera that finds an odd count is the pair's second, both records are then written, and it
-// computes the pair's record. A record is overwritten only after both of its readers in this
-// launch (the pair's two cameras) have passed phase 1, and the pass that read E'_n has
-// completed before this kernel's wait.
+// The new records go to cam_dst, a second buffer (with apply): other blocks may still read this step's
+// records. The loss of a pair is counted by its first camera only; each camera's FP64 loss share goes to
+// cam_loss[camera], and the next kernel (the next pass or the finalize kernel) adds them up in a fixed
+// order and advances the step count.
 template <bool FOCAL, int C, int W>
 __global__ void __launch_bounds__(32 * C * W, 1024 / (32 * C * W))
-k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo) {
+k_camera_step(DevProblem d, float gscale, float lscale, int apply, float *cam_dst) {
     constexpr int NV = FOCAL ? STEP_VALS : STEP_VALS - 1;      // sums carried per camera
     constexpr int NQ = W == 1 ? NV : (STEP_VALS + W - 1) / W;  // of which a warp adds up
     __shared__ StepState<C> st;
@@ -420,8 +410,7 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
     const int e_begin = k < d.n_cams ? d.cam_off[k] : 0;
     const int e_end = k < d.n_cams ? d.cam_off[k + 1] : 0;
     // this camera's entries, 32 at a time: pair, role, first range and number of ranges; the
-    // pair's geometry record goes to shared memory
-    int pair0 = 0, ci = 0, cj = 0;   // of the lane's first entry, for the geometry at the end
+    // pair's geometry at the records of the pass goes to shared memory
     auto load_chunk = [&](int base) -> int {
         const int e = base + lane;
         int n = 0, role = 0, r0 = 0, cnt = 0;
@@ -431,14 +420,12 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
             role = ent & 1;
             r0 = d.pair_off[n] / WR;
             cnt = (d.pair_off[n + 1] - 1) / WR - r0 + 1;
-            const float4 *gv = reinterpret_cast<const float4 *>(d.geo + (size_t)n * GEO);
-            float4 *dst = reinterpret_cast<float4 *>(s_geo + (cc * 32 + lane) * ROW);
+            if (sub == 0) {
+                float g[GEO];
+                pair_geometry_regs(d.cam, d.cen, d.cam_i[n], d.cam_j[n], g);   // (the pass has reported degenerate pairs)
+                float4 *dst = reinterpret_cast<float4 *>(s_geo + (cc * 32 + lane) * ROW);
 #pragma unroll
-            for (int q = 2 + sub; q < GEO / 4; q += W) dst[q] = gv[q];
-            if (base == e_begin && sub == 0) {
-                pair0 = n;
-                ci = d.cam_i[n];
-                cj = d.cam_j[n];
+                for (int q = 2; q < GEO / 4; ++q) dst[q] = make_float4(g[4 * q], g[4 * q + 1], g[4 * q + 2], g[4 * q + 3]);
             }
         }
         int incl = cnt;
@@ -529,19 +516,7 @@ k_camera_step(DevProblem d, float gscale, float lscale, int apply, int next_geo)
             bc1 = bias_correction(st.hyper[2], t_step);
             bc2 = bias_correction(st.hyper[3], t_step);
         }
-        step_update<FOCAL, false>(d, st, cam0, role, lane, bc1, bc2, t_step, apply, true, d.cam);
-    }
-    if (!(apply && next_geo)) return;
-    __syncthreads();   // the block's new records are written (the releases below order them for the other blocks)
-    if (k < d.n_cams) {
-        for (int e = e_begin + 32 * sub + lane; e < e_end; e += 32 * W) {
-            if (e >= e_begin + 32) {
-                pair0 = d.cam_ent[e] >> 1;
-                ci = d.cam_i[pair0];
-                cj = d.cam_j[pair0];
-            }
-            if (atomic_add_acq_rel(d.pair_cnt + pair0, 1u) & 1u) pair_geometry(d, pair0, ci, cj);
-        }
+        step_update<FOCAL, false>(d, st, cam0, role, lane, bc1, bc2, t_step, apply, true, cam_dst);
     }
 }
 
@@ -566,22 +541,28 @@ __global__ void __launch_bounds__(128) k_apply_gradient(DevProblem d) {
 
 __global__ void k_bump_step(DevProblem d) { *d.step += 1; }
 
-// closes a chain of steps: loss of the last step and `count` steps added to the step count
-// (loss_copy: the caller's loss, or null)
-__global__ void __launch_bounds__(FIN_THREADS) k_finalize(DevProblem d, int n_loss, int count, double *loss_copy) {
+// closes a chain of steps: loss of the last step and `count` steps added to the step count (loss_copy: the
+// caller's loss, or null), by block 0; the others copy the camera records back from the alternate buffer
+// (copy_src, or null: a float4 per thread) and (check) report image pairs that the last step left degenerate
+__global__ void __launch_bounds__(FIN_THREADS) k_finalize(DevProblem d, int n_loss, int count, double *loss_copy,
+                                                          const float *copy_src, int check) {
+    const int i = ((int)blockIdx.x - 1) * FIN_THREADS + threadIdx.x;
+    const bool pair = check && i >= 0 && i < d.n_pairs;
+    const int ci = pair ? d.cam_i[i] : 0, cj = pair ? d.cam_j[i] : 0;
     pdl_wait();
     pdl_trigger();
     __shared__ double red[FIN_THREADS];
-    finish_step(d, n_loss, count, red);
-    if (loss_copy && threadIdx.x == 0) *loss_copy = red[0];
-}
-
-// camera records copied back from the alternate buffer (one float4 per thread)
-__global__ void __launch_bounds__(256) k_copy_records(DevProblem d, const float4 *src) {
-    pdl_wait();
-    pdl_trigger();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < d.n_cams * (CAMREC / 4)) reinterpret_cast<float4 *>(d.cam)[i] = src[i];
+    if (blockIdx.x == 0) {
+        finish_step(d, n_loss, count, red);
+        if (loss_copy && threadIdx.x == 0) *loss_copy = red[0];
+        return;
+    }
+    if (copy_src && i < d.n_cams * (CAMREC / 4))
+        reinterpret_cast<float4 *>(d.cam)[i] = reinterpret_cast<const float4 *>(copy_src)[i];
+    if (pair) {
+        float g[GEO];
+        if (!pair_geometry_regs(copy_src ? copy_src : d.cam, d.cen, ci, cj, g)) atomicOr(d.err, ERR_DEGENERATE);
+    }
 }
 
 // ---- launchers -------------------------------------------------------------------------------------
@@ -593,8 +574,8 @@ void launch_cam_prep(const DevProblem &d, cudaStream_t s) {
     k_cam_prep<<<blocks_for(d.n_cams, 128), 128, 0, s>>>(d);
 }
 
-void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
-    launch_k(k_pair_setup, dim3(blocks_for(d.n_pairs, 256)), dim3(256), s, pdl, d, after_step ? d.n_cams : 0);
+void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl) {
+    launch_k(k_pair_setup, dim3(blocks_for(d.n_pairs, 256)), dim3(256), s, pdl, d);
 }
 
 void launch_set_hyper(const DevProblem &d, const double *h, cudaStream_t s) {
@@ -609,34 +590,30 @@ void launch_set_params(const DevProblem &d, const double *R, const double *c, cu
     k_set_params<<<blocks_for(d.n_cams, 64), 64, 0, s>>>(d, R, c);
 }
 
-void launch_finalize(const DevProblem &d, bool count_step, cudaStream_t s, bool pdl, double *loss_copy) {
-    launch_finalize_n(d, count_step ? 1 : 0, nullptr, s, pdl, loss_copy);
-}
-
-void launch_finalize_n(const DevProblem &d, int count, const float *copy_src, cudaStream_t s, bool pdl, double *loss_copy) {
-    if (copy_src)
-        launch_k(k_copy_records, dim3(blocks_for((int64_t)d.n_cams * (CAMREC / 4), 256)), dim3(256), s, pdl, d,
-                 reinterpret_cast<const float4 *>(copy_src));
-    launch_k(k_finalize, dim3(1), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count, loss_copy);
+void launch_finalize(const DevProblem &d, int count, const float *copy_src, bool check, cudaStream_t s, bool pdl,
+                     double *loss_copy) {
+    const int work = std::max(copy_src ? d.n_cams * (CAMREC / 4) : 0, check ? d.n_pairs : 0);
+    launch_k(k_finalize, dim3(1 + blocks_for(work, FIN_THREADS)), dim3(FIN_THREADS), s, pdl, d, d.n_cams, count, loss_copy,
+             copy_src, check ? 1 : 0);
 }
 
 void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl, bool after_step) {
     const int prev = after_step ? d.n_cams : 0;
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        static_assert(S * W * STAGE_BYTES >= FIN_THREADS * sizeof(double), "the last block finishes a step in its stage");
-        const dim3 grid(blocks_for(d.n_ranges, W) + 1), block(32 * W);
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        static_assert(S * STAGE_BYTES >= FIN_THREADS * sizeof(double), "the last block finishes a step in its stage");
+        const dim3 grid(d.n_ranges + 1), block(32);
         if (d.loss == FM_LOSS_IRLS)
-            launch_smem(k_stream_loss<STORE, MODE_LOSS_IRLS, S, W>, grid, block, S * W * STAGE_BYTES, s, pdl, d, prev);
+            launch_smem(k_stream_loss<STORE, MODE_LOSS_IRLS, S>, grid, block, PASS_BYTES<S>, s, pdl, d, prev);
         else
-            launch_smem(k_stream_loss<STORE, MODE_LOSS_L1, S, W>, grid, block, S * W * STAGE_BYTES, s, pdl, d, prev);
+            launch_smem(k_stream_loss<STORE, MODE_LOSS_L1, S>, grid, block, PASS_BYTES<S>, s, pdl, d, prev);
     });
 }
 
 void launch_stream_reweight(const DevProblem &d, cudaStream_t s, bool pdl) {
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        launch_smem(k_stream_reweight<STORE, S, W>, dim3(blocks_for(d.n_ranges, W)), dim3(32 * W), S * W * STAGE_BYTES, s,
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        launch_smem(k_stream_reweight<STORE, S>, dim3(d.n_ranges), dim3(32), PASS_BYTES<S>, s,
                     pdl, d);
     });
 }
@@ -674,15 +651,14 @@ void launch_apply_gradient(const DevProblem &d, cudaStream_t s) {
     k_bump_step<<<1, 1, 0, s>>>(d);
 }
 
-void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pdl, bool next_geo) {
+void launch_camera_step(const DevProblem &d, bool apply, float *cam_dst, cudaStream_t s, bool pdl) {
     float gscale, lscale;
     loss_scales(d, gscale, lscale);
-    const int ng = next_geo && d.pair_cnt ? 1 : 0;
     auto go = [&](auto cams, auto warps) {
         constexpr int C = decltype(cams)::value, W = decltype(warps)::value;
         const dim3 grid(blocks_for(d.n_cams, C)), block(32 * C * W);
-        if (d.refine_focal) launch_k(k_camera_step<true, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, ng);
-        else launch_k(k_camera_step<false, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, ng);
+        if (d.refine_focal) launch_k(k_camera_step<true, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, cam_dst);
+        else launch_k(k_camera_step<false, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, cam_dst);
     };
     using std::integral_constant;
     // Items (range partials of a camera's pairs) a camera: at most 2 (ranges + pairs) / cameras. A block of
@@ -702,16 +678,16 @@ void launch_camera_step(const DevProblem &d, bool apply, cudaStream_t s, bool pd
 }
 
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        k_irls_weights<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau);
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        k_irls_weights<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, tau);
     });
 }
 
 void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        k_residuals<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, out_input_order);
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        k_residuals<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, out_input_order);
     });
 }
 

@@ -48,13 +48,12 @@ struct StatsBody {
     __device__ __forceinline__ void group_done(int, int, int) {}
 };
 
-template <int STORE, int S, int W>
-__global__ void __launch_bounds__(32 * W) k_pair_stats(DevProblem d, float tau) {
+template <int STORE, int S>
+__global__ void __launch_bounds__(32) k_pair_stats(DevProblem d, float tau) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
-    if (r >= d.n_ranges) return;
+    const int r = blockIdx.x;
     StatsBody body(d, tau);
-    walk_range_staged<STORE, false, S>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
+    walk_range_staged<STORE, false, S>(d, r, threadIdx.x, body, stage, [] {});
 }
 
 __global__ void k_pair_stats_combine(DevProblem d) {
@@ -239,18 +238,17 @@ struct CollectBody {
     }
 };
 
-template <int STORE, int S, int W>
-__global__ void __launch_bounds__(32 * W)
+template <int STORE, int S>
+__global__ void __launch_bounds__(32)
 k_collect_features(DevProblem d, float tau, int round, int hist_valid, __nv_bfloat16 *feat_out) {
     extern __shared__ __align__(16) unsigned char stage[];
-    const int warp = threadIdx.x >> 5, r = blockIdx.x * W + warp;
-    if (r >= d.n_ranges) return;
+    const int r = blockIdx.x;
     CollectBody<STORE> body(d);
     body.log_tau = __logf(tau);
     body.round_f = round * 0.1f;
     body.hist_valid = hist_valid;
     body.feat_out = feat_out;
-    walk_range_staged<STORE, false, S, 1>(d, r, threadIdx.x & 31, body, stage + warp * S * STAGE_BYTES, [] {});
+    walk_range_staged<STORE, false, S, 1>(d, r, threadIdx.x, body, stage, [] {});
 }
 
 // ---- the learned reweighting -------------------------------------------------------------------------
@@ -484,9 +482,9 @@ void launch_learned_loss(const DevProblem &d, const float *master, const __nv_bf
 }
 
 void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        k_pair_stats<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau);
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        k_pair_stats<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, tau);
     });
     k_pair_stats_combine<<<blocks_for(d.n_pairs, 128), 128, 0, s>>>(d);
 }
@@ -502,10 +500,9 @@ void launch_learned_weights(const DevProblem &d, const float *master, const __nv
 
 void launch_collect_features(const DevProblem &d, float tau, int round, int hist_valid,
                              __nv_bfloat16 *feat, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth, auto warps) {
-        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value, W = decltype(warps)::value;
-        k_collect_features<STORE, S, W><<<blocks_for(d.n_ranges, W), 32 * W, S * W * STAGE_BYTES, s>>>(d, tau, round, hist_valid,
-                                                                                                   feat);
+    with_stages(d, [&](auto store, auto depth) {
+        constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
+        k_collect_features<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, tau, round, hist_valid, feat);
     });
 }
 

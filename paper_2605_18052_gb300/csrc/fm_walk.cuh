@@ -140,259 +140,6 @@ __device__ __forceinline__ float epi(const float *E, float x1, float y1, float x
 // set by the residual's FP32 error.
 __device__ __forceinline__ float irls_weight(float a, float delta) { return __fdividef(1.0f, fmaxf(a, delta)); }
 
-// *p += v at GPU scope with acquire-release semantics; returns the old value
-__device__ __forceinline__ unsigned atomic_add_acq_rel(unsigned *p, unsigned v) {
-    unsigned old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-
-// ---- the streaming walk ------------------------------------------------------------------------
-// Warp `r` streams point pairs [r*WR, min((r+1)*WR, n_pp)). Lane l of group g handles PPL
-// consecutive point pairs at g*32*PPL + l*PPL, so every load instruction of the warp reads one
-// contiguous 512 B block. The image pair changes only at sorted boundaries: a group that lies
-// inside the current pair takes the fast path; a group that crosses a boundary is processed in
-// passes, one pass per image pair it meets, and `body.segment_end` closes each finished pair.
-// Positions are 32-bit (n_pp < 2^31 - 2^16, so also past the end of the padded arrays).
-struct WalkState {
-    int p_begin, p_end, seg, seg_end;
-    float E[9];
-    __device__ __forceinline__ WalkState(const DevProblem &d, int r)
-        : p_begin(r * WR), p_end((int)min((int64_t)p_begin + WR, d.n_pp)), seg(d.range_pair[r]),
-          seg_end(d.pair_off[seg + 1]) {}
-};
-
-template <int STORE, class Body>
-__device__ __forceinline__ void walk_group(const DevProblem &d, WalkState &st, const typename Fmt<STORE>::Raw &raw, int gb,
-                                           int r, int lane, Body &body) {
-    using F = Fmt<STORE>;
-    constexpr int PPL = F::PPL;
-    constexpr int GROUP = 32 * PPL;
-    if (gb + GROUP <= st.seg_end) {
-#pragma unroll
-        for (int k = 0; k < PPL; ++k) {
-            float x1, y1, x2, y2, w;
-            F::get(raw, k, x1, y1, x2, y2, w);
-            body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
-        }
-    } else {
-        int lo = gb;
-        const int g_end = min(gb + GROUP, st.p_end);
-        while (true) {
-            const int hi = min(st.seg_end, st.p_end);
-#pragma unroll
-            for (int k = 0; k < PPL; ++k) {
-                const int q = gb + lane * PPL + k;
-                if (q >= lo && q < hi) {
-                    float x1, y1, x2, y2, w;
-                    F::get(raw, k, x1, y1, x2, y2, w);
-                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
-                }
-            }
-            if (st.seg_end >= g_end) break;
-            body.segment_end(st.seg, r, lane, false);
-            lo = st.seg_end;
-            ++st.seg;
-            st.seg_end = d.pair_off[st.seg + 1];
-            load_E(d.geo, st.seg, st.E);
-            body.segment_begin(st.seg);
-        }
-    }
-    body.group_done(gb, st.p_end, lane);
-}
-
-// The walk of a range, staged in shared memory by asynchronous copies, a chunk of 4 groups (2 KB of
-// keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the launch before this one; the first S chunks are requested ahead of it, so they arrive while that
-// launch finishes. (Keypoints are static. Weights are written at least two launches earlier: a pass
-// that writes them is followed by the camera step, which lets this launch start only after its own
-// wait for that pass.)
-constexpr int STAGE_GROUPS = 4;
-constexpr int STAGE_BYTES = STAGE_GROUPS * 32 * (16 + 4);
-
-__device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
-// UNROLL: groups of a chunk in straight code (1 for bodies of many instructions). A chunk inside one image
-// pair takes one branch and reads its four groups before their sums: a warp that checks every group
-// issues the loads of one at a time, and where few warps share an SM the pass is that chain of latencies
-// (an iteration on 119 k point pairs 15.1 -> 13.7 us, 3.1 M FP32 19.2 -> 18.4; 141 M FP16 219.5 -> 216).
-// Where UNROLL is below a chunk (the quadratic-form pass) the second copy of the body costs
-// more than it gives: 403 -> 421 us for a round on 49 M.
-template <int STORE, bool NEED_W, int S, int UNROLL = STAGE_GROUPS, class Body, class Before>
-__device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, int lane, Body &body, unsigned char *stage,
-                                                  Before before) {
-    using F = Fmt<STORE>;
-    constexpr int GROUP = 32 * F::PPL;
-    constexpr int CHUNK = STAGE_GROUPS * GROUP;
-    static_assert(WR % CHUNK == 0, "range must be whole chunks");
-    WalkState st(d, r);
-    const int n_chunks = (st.p_end - st.p_begin + CHUNK - 1) / CHUNK;
-    const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + (size_t)st.p_begin * (16 / F::PPL);
-    const unsigned char *wp = static_cast<const unsigned char *>(d.w) + (size_t)st.p_begin * (4 / F::PPL);
-    auto request = [&](int c) {
-        if (c < n_chunks) {
-            unsigned char *dst = stage + (c % S) * STAGE_BYTES;
-#pragma unroll
-            for (int u = 0; u < STAGE_GROUPS; ++u)
-                cp_async16(dst + (u * 32 + lane) * 16, kp + (size_t)c * (STAGE_GROUPS * 512) + (u * 32 + lane) * 16);
-            if (NEED_W) cp_async16(dst + STAGE_GROUPS * 512 + lane * 16, wp + (size_t)c * (STAGE_GROUPS * 128) + lane * 16);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    for (int c = 0; c < S; ++c) request(c);
-    before();
-    load_E(d.geo, st.seg, st.E);
-    body.segment_begin(st.seg);
-    for (int c = 0; c < n_chunks; ++c) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
-        __syncwarp();   // a lane's weights were copied by another lane
-        const unsigned char *src = stage + (c % S) * STAGE_BYTES;
-        const int cb = st.p_begin + c * CHUNK;
-        if (UNROLL == STAGE_GROUPS && cb + CHUNK <= st.seg_end) {
-            typename F::Raw raw[STAGE_GROUPS];
-#pragma unroll
-            for (int u = 0; u < STAGE_GROUPS; ++u) {
-                raw[u].kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
-                raw[u].w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < STAGE_GROUPS; ++u) {
-#pragma unroll
-                for (int k = 0; k < F::PPL; ++k) {
-                    float x1, y1, x2, y2, w;
-                    F::get(raw[u], k, x1, y1, x2, y2, w);
-                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
-                }
-                body.group_done(cb + u * GROUP, st.p_end, lane);
-            }
-        } else
-#pragma unroll UNROLL
-        for (int u = 0; u < STAGE_GROUPS; ++u) {
-            const int gb = cb + u * GROUP;
-            if (gb >= st.p_end) break;
-            typename F::Raw raw;
-            raw.kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
-            raw.w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
-            walk_group<STORE>(d, st, raw, gb, r, lane, body);
-        }
-        if (S < WR / CHUNK) __syncwarp();   // every lane has read the chunk before it is overwritten
-        request(c + S);
-    }
-    body.segment_end(st.seg, r, lane, true);
-}
-
-// Depth and block size of the staged passes. FP32: 4 chunks (512 point pairs) a warp; the whole range,
-// 16 chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 13.8 ->
-// 13.65 us an iteration, 245 ranges 16.3 -> 16.0; 733 ranges 16.6 -> 18.5). FP16: 2 chunks (512 point
-// pairs; 4 chunks: 5,860 ranges 30.8 -> 32.2, 48,829 ranges 163.5 -> 166.8). One warp per block, so that a
-// finished range makes room for the next at once, but four from 300 ranges per SM on, where the block
-// launches count (FP16: 48,829 ranges 163.5 -> 162.3 us, 68,633 ranges 223.6 -> 219.5, 23,860 ranges
-// 85.5 -> 85.9).
-constexpr int FEW_RANGES = 2 * 152, MANY_RANGES = 300 * 152;
-
-template <class Launch>
-static void with_stages(const DevProblem &d, Launch launch) {
-    using std::integral_constant;
-    if (d.storage == FM_STORE_FP32) {
-        integral_constant<int, FM_STORE_FP32> st;
-        if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>(), integral_constant<int, 1>());
-        else if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 4>(), integral_constant<int, 1>());
-        else launch(st, integral_constant<int, 4>(), integral_constant<int, 4>());
-    } else {
-        integral_constant<int, FM_STORE_FP16> st;
-        if (d.n_ranges < MANY_RANGES) launch(st, integral_constant<int, 2>(), integral_constant<int, 1>());
-        else launch(st, integral_constant<int, 2>(), integral_constant<int, 4>());
-    }
-}
-
-// ---- packed FP32 pairs -----------------------------------------------------------------------------
-// Two lanes of FP32 arithmetic in one instruction (fma/mul/add.rn.f32x2): each lane rounds once,
-// exactly as the scalar operation, so results keep their bits while the streaming passes, which
-// are close to bound by instruction issue, issue one instruction where they issued two.
-__device__ __forceinline__ void fma2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
-    asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
-        "mov.b64 ra, {%2, %3};\n\t"
-        "mov.b64 rb, {%4, %5};\n\t"
-        "mov.b64 rc, {%0, %1};\n\t"
-        "fma.rn.f32x2 rc, ra, rb, rc;\n\t"
-        "mov.b64 {%0, %1}, rc;\n\t}"
-        : "+f"(d0), "+f"(d1)
-        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void mul2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
-    asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
-        "mov.b64 ra, {%2, %3};\n\t"
-        "mov.b64 rb, {%4, %5};\n\t"
-        "mul.rn.f32x2 rc, ra, rb;\n\t"
-        "mov.b64 {%0, %1}, rc;\n\t}"
-        : "=f"(d0), "=f"(d1)
-        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
-}
-// d0 += b0, d1 += b1
-__device__ __forceinline__ void add2(float &d0, float &d1, float b0, float b1) {
-    asm("{\n\t.reg .b64 rb, rc;\n\t"
-        "mov.b64 rb, {%2, %3};\n\t"
-        "mov.b64 rc, {%0, %1};\n\t"
-        "add.rn.f32x2 rc, rc, rb;\n\t"
-        "mov.b64 {%0, %1}, rc;\n\t}"
-        : "+f"(d0), "+f"(d1)
-        : "f"(b0), "f"(b1));
-}
-
-// ---- loss + adjoint -----------------------------------------------------------------------------
-// acc[0..8] = sum s * o2 o1^T (row-major), acc[9] = sum of loss terms, with s = w*eps (IRLS,
-// the factor 2/Z is applied later) or sign(eps) (L1). Each finished (image pair, warp range)
-// intersection is reduced by a warp butterfly into its own slot n + r; no atomics, no fences,
-// a fixed summation order.
-template <int MODE>
-struct LossBody {
-    const DevProblem &d;
-    float acc[10];
-    __device__ explicit LossBody(const DevProblem &dd) : d(dd) {
-#pragma unroll
-        for (int i = 0; i < 10; ++i) acc[i] = 0.f;
-    }
-    __device__ __forceinline__ void point(int, float e, float x1, float y1, float x2, float y2,
-                                          float w) {
-        float s;
-        if (MODE == MODE_LOSS_IRLS) {
-            s = w * e;
-            acc[9] = fmaf(s, e, acc[9]);
-        } else {
-            s = e > 0.f ? 1.f : (e < 0.f ? -1.f : 0.f);
-            acc[9] += fabsf(e);
-        }
-        float a, b;   // s x2, s y2
-        mul2(a, b, s, s, x2, y2);
-        fma2(acc[0], acc[1], a, a, x1, y1);
-        add2(acc[2], acc[5], a, b);
-        fma2(acc[3], acc[4], b, b, x1, y1);
-        fma2(acc[6], acc[7], s, s, x1, y1);
-        acc[8] += s;
-    }
-    __device__ __forceinline__ void segment_begin(int) {}
-    __device__ __forceinline__ void segment_end(int seg, int r, int lane, bool) {
-#pragma unroll
-        for (int i = 0; i < 10; ++i) {
-            float v = acc[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            acc[i] = v;
-        }
-        if (lane == 0) {
-            float4 *s = reinterpret_cast<float4 *>(d.slots + (size_t)(seg + r) * SLOT);
-            s[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-            s[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-            s[2] = make_float4(acc[8], acc[9], 0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < 10; ++i) acc[i] = 0.f;
-    }
-    __device__ __forceinline__ void group_done(int, int, int) {}
-};
-
 // ---- per pair: relative pose and folded essential matrix ------------------------------------------
 // camera record: R (9), centre as hi (3) + lo (3) floats, s = scale of the normalised keypoints.
 // Read at L2 (ld.global.cg): a record may have been written by another block of the same
@@ -500,6 +247,302 @@ __device__ __forceinline__ void pair_geometry(const DevProblem &d, int n, int i,
 #pragma unroll
     for (int k = 0; k < GEO / 4; ++k) out[k] = make_float4(g[4 * k], g[4 * k + 1], g[4 * k + 2], g[4 * k + 3]);
 }
+
+// E' of a walk's image pairs, from their geometry records (written by a launch before).
+struct RecordE {
+    static constexpr int BYTES = 0;
+    const DevProblem &d;
+    __device__ RecordE(const DevProblem &dd, int, int, int, unsigned char *) : d(dd) {}
+    __device__ __forceinline__ void start() {}
+    __device__ __forceinline__ void get(int seg, float *E) { load_E(d.geo, seg, E); }
+};
+
+// The same formed from the camera records, for 16 image pairs of the range at once, a lane each, into a
+// table in shared memory: no launch between the camera step and the pass, no record written and read
+// back, and a range of several image pairs finds the next one's E' without a trip to L2. (Records
+// written by the last camera of a pair cost the camera step an acquire-release atomic per pair and 3,400
+// cycles: a round of 25 iterations took 250 us on 119 k point pairs, 224 now, 335 on 3.1 M, 312 now.)
+struct CameraE {
+    static constexpr int PAIRS = 16, BYTES = PAIRS * 9 * (int)sizeof(float);
+    const DevProblem &d;
+    float *table;
+    int lane, p_end, base, i, j;
+    bool mine;
+    __device__ __forceinline__ CameraE(const DevProblem &dd, int seg, int end, int l, unsigned char *mem)
+        : d(dd), table(reinterpret_cast<float *>(mem)), lane(l), p_end(end) {
+        pairs(seg);
+    }
+    __device__ __forceinline__ void pairs(int seg) {   // static data
+        base = seg;
+        const int n = seg + lane;
+        mine = lane < PAIRS && n < d.n_pairs && d.pair_off[n] < p_end;
+        i = mine ? d.cam_i[n] : 0;
+        j = mine ? d.cam_j[n] : 0;
+    }
+    __device__ __forceinline__ void start() {
+        if (mine) {
+            float g[GEO];
+            if (!pair_geometry_regs(d.cam, d.cen, i, j, g)) atomicOr(d.err, ERR_DEGENERATE);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) table[9 * lane + q] = g[q];
+        }
+        __syncwarp();
+    }
+    __device__ __forceinline__ void get(int seg, float *E) {
+        if (seg - base == PAIRS) {
+            __syncwarp();
+            pairs(seg);
+            start();
+        }
+#pragma unroll
+        for (int q = 0; q < 9; ++q) E[q] = table[9 * (seg - base) + q];
+    }
+};
+
+// ---- the streaming walk ------------------------------------------------------------------------
+// Warp `r` streams point pairs [r*WR, min((r+1)*WR, n_pp)). Lane l of group g handles PPL
+// consecutive point pairs at g*32*PPL + l*PPL, so every load instruction of the warp reads one
+// contiguous 512 B block. The image pair changes only at sorted boundaries: a group that lies
+// inside the current pair takes the fast path; a group that crosses a boundary is processed in
+// passes, one pass per image pair it meets, and `body.segment_end` closes each finished pair.
+// Positions are 32-bit (n_pp < 2^31 - 2^16, so also past the end of the padded arrays).
+struct WalkState {
+    int p_begin, p_end, seg, seg_end;
+    float E[9];
+    __device__ __forceinline__ WalkState(const DevProblem &d, int r)
+        : p_begin(r * WR), p_end((int)min((int64_t)p_begin + WR, d.n_pp)), seg(d.range_pair[r]),
+          seg_end(d.pair_off[seg + 1]) {}
+};
+
+template <int STORE, class Source, class Body>
+__device__ __forceinline__ void walk_group(const DevProblem &d, Source &source, WalkState &st, const typename Fmt<STORE>::Raw &raw, int gb,
+                                           int r, int lane, Body &body) {
+    using F = Fmt<STORE>;
+    constexpr int PPL = F::PPL;
+    constexpr int GROUP = 32 * PPL;
+    if (gb + GROUP <= st.seg_end) {
+#pragma unroll
+        for (int k = 0; k < PPL; ++k) {
+            float x1, y1, x2, y2, w;
+            F::get(raw, k, x1, y1, x2, y2, w);
+            body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+        }
+    } else {
+        int lo = gb;
+        const int g_end = min(gb + GROUP, st.p_end);
+        while (true) {
+            const int hi = min(st.seg_end, st.p_end);
+#pragma unroll
+            for (int k = 0; k < PPL; ++k) {
+                const int q = gb + lane * PPL + k;
+                if (q >= lo && q < hi) {
+                    float x1, y1, x2, y2, w;
+                    F::get(raw, k, x1, y1, x2, y2, w);
+                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+                }
+            }
+            if (st.seg_end >= g_end) break;
+            body.segment_end(st.seg, r, lane, false);
+            lo = st.seg_end;
+            ++st.seg;
+            st.seg_end = d.pair_off[st.seg + 1];
+            source.get(st.seg, st.E);
+            body.segment_begin(st.seg);
+        }
+    }
+    body.group_done(gb, st.p_end, lane);
+}
+
+// The walk of a range, staged in shared memory by asynchronous copies, a chunk of 4 groups (2 KB of
+// keypoints, 512 B of weights) at a time, S chunks in flight. `before` is the wait for the launch before this one; the first S chunks are requested ahead of it, so they arrive while that
+// launch finishes. (Keypoints are static. A pass with weights that is launched ahead of its predecessor's end
+// follows a camera step, and so the pass that wrote them by two launches: the camera step lets this
+// launch start only after its own wait for that pass.)
+constexpr int STAGE_GROUPS = 4;
+constexpr int STAGE_BYTES = STAGE_GROUPS * 32 * (16 + 4);
+
+__device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// UNROLL: groups of a chunk in straight code (1 for bodies of many instructions). A chunk inside one image
+// pair takes one branch and reads its four groups before their sums: a warp that checks every group
+// issues the loads of one at a time, and where few warps share an SM the pass is that chain of latencies
+// (an iteration on 119 k point pairs went from 15.1 to 13.7 us, on 3.1 M FP32 from 19.2 to 18.4).
+// Where UNROLL is below a chunk (the quadratic-form pass) the second copy of the body costs
+// more than it gives: 403 -> 421 us for a round on 49 M.
+// Source: where a pair's E' comes from (its table, Source::BYTES, lies behind the stage).
+template <int STORE, bool NEED_W, int S, int UNROLL = STAGE_GROUPS, class Source = RecordE, class Body, class Before>
+__device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, int lane, Body &body, unsigned char *stage,
+                                                  Before before) {
+    using F = Fmt<STORE>;
+    constexpr int GROUP = 32 * F::PPL;
+    constexpr int CHUNK = STAGE_GROUPS * GROUP;
+    static_assert(WR % CHUNK == 0, "range must be whole chunks");
+    WalkState st(d, r);
+    const int n_chunks = (st.p_end - st.p_begin + CHUNK - 1) / CHUNK;
+    const unsigned char *kp = static_cast<const unsigned char *>(d.kp) + (size_t)st.p_begin * (16 / F::PPL);
+    const unsigned char *wp = static_cast<const unsigned char *>(d.w) + (size_t)st.p_begin * (4 / F::PPL);
+    auto request = [&](int c) {
+        if (c < n_chunks) {
+            unsigned char *dst = stage + (c % S) * STAGE_BYTES;
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u)
+                cp_async16(dst + (u * 32 + lane) * 16, kp + (size_t)c * (STAGE_GROUPS * 512) + (u * 32 + lane) * 16);
+            if (NEED_W) cp_async16(dst + STAGE_GROUPS * 512 + lane * 16, wp + (size_t)c * (STAGE_GROUPS * 128) + lane * 16);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < S; ++c) request(c);
+    Source source(d, st.seg, st.p_end, lane, stage + S * STAGE_BYTES);
+    before();
+    source.start();
+    source.get(st.seg, st.E);
+    body.segment_begin(st.seg);
+    for (int c = 0; c < n_chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
+        __syncwarp();   // a lane's weights were copied by another lane
+        const unsigned char *src = stage + (c % S) * STAGE_BYTES;
+        const int cb = st.p_begin + c * CHUNK;
+        if (UNROLL == STAGE_GROUPS && cb + CHUNK <= st.seg_end) {
+            typename F::Raw raw[STAGE_GROUPS];
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u) {
+                raw[u].kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
+                raw[u].w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < STAGE_GROUPS; ++u) {
+#pragma unroll
+                for (int k = 0; k < F::PPL; ++k) {
+                    float x1, y1, x2, y2, w;
+                    F::get(raw[u], k, x1, y1, x2, y2, w);
+                    body.point(k, epi(st.E, x1, y1, x2, y2), x1, y1, x2, y2, w);
+                }
+                body.group_done(cb + u * GROUP, st.p_end, lane);
+            }
+        } else
+#pragma unroll UNROLL
+        for (int u = 0; u < STAGE_GROUPS; ++u) {
+            const int gb = cb + u * GROUP;
+            if (gb >= st.p_end) break;
+            typename F::Raw raw;
+            raw.kp = *reinterpret_cast<const uint4 *>(src + (u * 32 + lane) * 16);
+            raw.w = NEED_W ? *reinterpret_cast<const unsigned *>(src + STAGE_GROUPS * 512 + (u * 32 + lane) * 4) : 0u;
+            walk_group<STORE>(d, source, st, raw, gb, r, lane, body);
+        }
+        if (S < WR / CHUNK) __syncwarp();   // every lane has read the chunk before it is overwritten
+        request(c + S);
+    }
+    body.segment_end(st.seg, r, lane, true);
+}
+
+// Depth of the staged passes, which run a warp (a range) per block, so that a finished range makes room for
+// the next at once (four to a block, an iteration: FP16 5,860 ranges 28.6 -> 31.3 us, 48,829 ranges 154.3
+// -> 159.0; FP32 23,860 ranges 141.6 -> 144.7). FP32: 4 chunks (512 point pairs); the whole range, 16
+// chunks, up to two ranges per SM, where a warp has its SM's load path to itself (59 ranges 13.8 -> 13.65
+// us, 245 ranges 16.3 -> 16.0; 733 ranges 16.6 -> 18.5). FP16: 2 chunks (512 point pairs; 4 chunks: 5,860
+// ranges 28.6 -> 30.4, 68,634 ranges 218.9 -> 224.3).
+constexpr int FEW_RANGES = 2 * 152;
+
+template <class Launch>
+static void with_stages(const DevProblem &d, Launch launch) {
+    using std::integral_constant;
+    if (d.storage == FM_STORE_FP32) {
+        integral_constant<int, FM_STORE_FP32> st;
+        if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>());
+        else launch(st, integral_constant<int, 4>());
+    } else {
+        launch(integral_constant<int, FM_STORE_FP16>(), integral_constant<int, 2>());
+    }
+}
+
+// ---- packed FP32 pairs -----------------------------------------------------------------------------
+// Two lanes of FP32 arithmetic in one instruction (fma/mul/add.rn.f32x2): each lane rounds once,
+// exactly as the scalar operation, so results keep their bits while the streaming passes, which
+// are close to bound by instruction issue, issue one instruction where they issued two.
+__device__ __forceinline__ void fma2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
+    asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
+        "mov.b64 ra, {%2, %3};\n\t"
+        "mov.b64 rb, {%4, %5};\n\t"
+        "mov.b64 rc, {%0, %1};\n\t"
+        "fma.rn.f32x2 rc, ra, rb, rc;\n\t"
+        "mov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(d0), "+f"(d1)
+        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void mul2(float &d0, float &d1, float a0, float a1, float b0, float b1) {
+    asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
+        "mov.b64 ra, {%2, %3};\n\t"
+        "mov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rc, ra, rb;\n\t"
+        "mov.b64 {%0, %1}, rc;\n\t}"
+        : "=f"(d0), "=f"(d1)
+        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+// d0 += b0, d1 += b1
+__device__ __forceinline__ void add2(float &d0, float &d1, float b0, float b1) {
+    asm("{\n\t.reg .b64 rb, rc;\n\t"
+        "mov.b64 rb, {%2, %3};\n\t"
+        "mov.b64 rc, {%0, %1};\n\t"
+        "add.rn.f32x2 rc, rc, rb;\n\t"
+        "mov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(d0), "+f"(d1)
+        : "f"(b0), "f"(b1));
+}
+
+// ---- loss + adjoint -----------------------------------------------------------------------------
+// acc[0..8] = sum s * o2 o1^T (row-major), acc[9] = sum of loss terms, with s = w*eps (IRLS,
+// the factor 2/Z is applied later) or sign(eps) (L1). Each finished (image pair, warp range)
+// intersection is reduced by a warp butterfly into its own slot n + r; no atomics, no fences,
+// a fixed summation order.
+template <int MODE>
+struct LossBody {
+    const DevProblem &d;
+    float acc[10];
+    __device__ explicit LossBody(const DevProblem &dd) : d(dd) {
+#pragma unroll
+        for (int i = 0; i < 10; ++i) acc[i] = 0.f;
+    }
+    __device__ __forceinline__ void point(int, float e, float x1, float y1, float x2, float y2,
+                                          float w) {
+        float s;
+        if (MODE == MODE_LOSS_IRLS) {
+            s = w * e;
+            acc[9] = fmaf(s, e, acc[9]);
+        } else {
+            s = e > 0.f ? 1.f : (e < 0.f ? -1.f : 0.f);
+            acc[9] += fabsf(e);
+        }
+        float a, b;   // s x2, s y2
+        mul2(a, b, s, s, x2, y2);
+        fma2(acc[0], acc[1], a, a, x1, y1);
+        add2(acc[2], acc[5], a, b);
+        fma2(acc[3], acc[4], b, b, x1, y1);
+        fma2(acc[6], acc[7], s, s, x1, y1);
+        acc[8] += s;
+    }
+    __device__ __forceinline__ void segment_begin(int) {}
+    __device__ __forceinline__ void segment_end(int seg, int r, int lane, bool) {
+#pragma unroll
+        for (int i = 0; i < 10; ++i) {
+            float v = acc[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            acc[i] = v;
+        }
+        if (lane == 0) {
+            float4 *s = reinterpret_cast<float4 *>(d.slots + (size_t)(seg + r) * SLOT);
+            s[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            s[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+            s[2] = make_float4(acc[8], acc[9], 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 10; ++i) acc[i] = 0.f;
+    }
+    __device__ __forceinline__ void group_done(int, int, int) {}
+};
 
 // Loss total of an optimiser step (FP64, fixed order over the n_loss per-camera shares in
 // cam_loss) and `count` steps added to the step count. One block of NT threads (NT divides
