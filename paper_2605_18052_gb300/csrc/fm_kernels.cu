@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // hi + lo pair (TwoSum); a lane's items are added in the order of their passes and the lanes by a
 // butterfly, whatever W is, so every W gives the same bits; with W > 1 the warps share the values out.
 // What bounds it is latency: a pass of loads and chain rule takes about 2,000 cycles, and a warp a camera
-// makes three of them in series on 1,000 cameras and 49 M point pairs. An iteration there 83.7 -> 79.2 us
-// (FP16), on 16 cameras and 119 k 11.6 -> 10.55, on 128 and 3.1 M (FP32) 16.9 -> 12.2.
+// makes three of them in series on 1,000 cameras and 49 M point pairs (an iteration with 8 cameras of one
+// warp a block 80.5 us, now 78.0; on 16 cameras and 119 k 9.7, now 8.8).
 // Phase 2: the update of the block's cameras, spread over warps (step_update). The two powers of its
 // bias corrections are formed before the wait.
 // The new records go to cam_dst, a second buffer (with apply): other blocks may still read this step's
@@ -661,20 +661,20 @@ void launch_camera_step(const DevProblem &d, bool apply, float *cam_dst, cudaStr
         else launch_k(k_camera_step<false, C, W>, grid, block, s, pdl, d, gscale, lscale, apply ? 1 : 0, cam_dst);
     };
     using std::integral_constant;
-    // Items (range partials of a camera's pairs) a camera: at most 2 (ranges + pairs) / cameras. A block of
-    // one camera and 4 warps while every camera has an SM (152 cameras, 3 M point pairs: 13.2 us an iteration,
-    // 14.0 with 2 x 2), or while the blocks are resident at once and a camera has more than the 64 items that
-    // two warps take in one pass (16 cameras, 5 M: 17.1 against 21.8; 1,000 cameras, 49 M FP32: 143.6
-    // against 146.1; with fewer items 1,000 cameras, 3 M: 31.7 against 25.7). Two cameras of 2 warps while
-    // those are resident (2,000 cameras, 12 M: 34.8, 37.0 with 4 x 1; 3,000 cameras, 6 M: 34.1 against 33.2).
-    // Four cameras of one warp beyond (eight: 4,000 cameras 221.7 against 220.8).
+    // Items (range partials of a camera's pairs) a camera: at most 2 (ranges + pairs) / cameras. us an
+    // iteration with C x W = 8 x 1, 2 x 2, 1 x 4:
+    //   many items (46 to 320): 16 cameras, 5 M point pairs 24.2, 19.1, 17.1; 100 cameras, 3.1 M 13.1, 11.6, 11.3;
+    //     1,000 cameras, 49 M FP32 144.9, 141.9, 140.6
+    //   fewer (13 to 40): 128 cameras, 1 M 11.4, 10.3, 10.9; 152 cameras, 3.1 M FP16 12.8, 11.7, 12.2; 1,000 cameras,
+    //     3 M 20.6, 20.9, 30.8; 2,000 cameras, 80 M FP32 231.1, 228.9, 232.8
+    //   more cameras than 2 x 2 has resident: 3,000 cameras, 60 M 103.6, 107.3, 111.8; 4,000, 140 M 215.8, 221.1, 227.2
     const int64_t items = 2 * ((int64_t)d.n_ranges + d.n_pairs);
-    if (d.n_cams <= 152 || (d.n_cams <= 8 * 152 && items > 64 * (int64_t)d.n_cams))
+    if (d.n_cams <= 8 * 152 && items > 44 * (int64_t)d.n_cams)
         go(integral_constant<int, 1>(), integral_constant<int, 4>());
     else if (d.n_cams <= 16 * 152)
         go(integral_constant<int, 2>(), integral_constant<int, 2>());
     else
-        go(integral_constant<int, 4>(), integral_constant<int, 1>());
+        go(integral_constant<int, 8>(), integral_constant<int, 1>());
 }
 
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {

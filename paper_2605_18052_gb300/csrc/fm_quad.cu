@@ -208,8 +208,8 @@ __device__ __forceinline__ void form_sums(const float4 *rec, const float *g, flo
 //   q = g0 + W d,  loss = c0 + d^T (g0 + q),  d = E'_n - e0,
 // and the chain rule to camera k. Both cameras of a pair evaluate it (O(1) each), which
 // removes a per-pair launch and the wait on it. The warp reduces with compensated butterflies,
-// then the block updates its cameras (step_update) and writes the new records to cam_dst: the records of this step's poses stay intact in cam_src for the other
-// blocks. The Adam step count is *d.step + 1 + it; the launch that closes the chain adds
+// then the block updates its cameras (step_update) and writes the new records to cam_dst: the
+// records of this step's poses stay intact in cam_src for the other blocks. The Adam step count is *d.step + 1 + it; the launch that closes the chain adds
 // the chain's length to *d.step.
 template <bool FOCAL>
 __global__ void __launch_bounds__(STEP_CAMS * 32, 4)

@@ -1,6 +1,5 @@
-"""The camera step at the edges of its dispatch: one camera a block and four warps (up to 152 cameras, or up
-to 1,216 with more than 64 items a camera), two cameras of two warps (up to 2,432), four of one
-warp beyond; cameras with more than 32 image pairs, and with more items than the warps take in one pass.
+"""The camera step at the edges of its dispatch: one camera a block and four warps (up to 1,216 cameras with
+more than 44 items each), two cameras of two warps (up to 2,432), eight of one warp beyond; cameras with more than 32 image pairs, and with more items than the warps take in one pass.
 
 The gradient is compared with the quadratic form's at the same poses, which another kernel sums up per
 pair before its chain rule: both hold FP32 sums whose errors are a few 1e-6 of the sum of magnitudes, so
@@ -52,3 +51,16 @@ def test_step_and_gradient(cams, near, points, storage):
         for u, v in zip(p.get_params(), q.get_params()):
             np.testing.assert_array_equal(u, v)
         assert p.loss_grad()[0] == q.loss_grad()[0]
+
+
+def test_coincident_cameras_are_reported():
+    # the pass forms the pair geometry itself, in every iteration of a chain
+    build.build()
+    rng = np.random.default_rng(0)
+    R, t = np.stack([np.eye(3)] * 3), np.array([[0.0, 0, 0], [0, 0, 0], [1, 0, 0]])
+    x1, x2 = (rng.uniform(-0.5, 0.5, (40, 2)).astype(np.float32) for _ in range(2))
+    pid = np.repeat(np.arange(2, dtype=np.int32), 20)
+    for call in (lambda p: p.loss_grad(), lambda p: p.irls_weights(0.1), lambda p: (p.step(1), p.last_loss())):
+        with fm.Problem(R, t, np.array([0, 0], np.int32), np.array([1, 2], np.int32), pid, x1, x2) as p:
+            with pytest.raises(fm.FastMapError):
+                call(p)
