@@ -44,7 +44,7 @@ struct DevRot {
     float *m, *v;            // Adam moments, n_cams x 6
     double *pgrad;           // n_pairs x 18: d d_p / d R_i (9), d d_p / d R_j (9)
     double *pdist;           // n_pairs: d_p
-    double *blk;             // per-block partial sums (loss, CG dot products)
+    double *blk;             // per-block partial sums (loss, CG dot products): two rows of camera blocks
     double *loss;
     double *hyper;           // lr, beta1, beta2, eps
     long long *step;
@@ -182,7 +182,9 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
     const bool single = t.n_cams <= stride;
     if (axis == 1 && (*t.err & ERR_DEGENERATE)) return;   // column 1 vanished: leave the state as it is
     GridBarrier gb(t.grid_state, t.err);
-    double *slot = t.blk, *cam_rz = t.cam_rz;
+    // The groups' sums lie in two rows of t.blk: r.z of the setup in one, p.q of the iterations in the other.
+    // The setup has one barrier: a block may reach the first p.q while another still reads the setup's r.z.
+    double *slot = t.blk, *slot_setup = t.blk + groups, *cam_rz = t.cam_rz;
     // warp 0: lane 3 c + a holds component a of the block's camera c
     const int cc = lane / 3, ca = lane % 3, base = 3 * cc;
     // (its state stays in registers when the block owns one group; it goes through memory otherwise)
@@ -211,11 +213,11 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
             if (lane == spread_lane(3, a)) s_sum[warp][a] = mine;
     };
     // warp 0: a value per camera (in its first lane) summed over the group in camera order
-    auto put_group = [&](int kb, double mine) {
+    auto group_sum = [&](double mine) {
         double b = __shfl_sync(0xffffffffu, mine, 0);
 #pragma unroll
         for (int w = 1; w < RT_CAMS; ++w) b += __shfl_sync(0xffffffffu, mine, 3 * w);
-        if (lane == 0) slot[kb / RT_CAMS] = b;
+        return b;
     };
     // setup: x = 0 except the anchor, r = b - A x = the anchor's contribution, z = M^-1 r, p = 0
     for (int kb = k0; kb < t.n_cams; kb += stride) {
@@ -263,7 +265,8 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
                 t.p2[o3] = 0.0;
                 if (kc == 0 && ca == 0) cam_rz[0] = 0.0;
             }
-            put_group(kb, rz);
+            const double b = group_sum(rz);
+            if (lane == 0) slot_setup[kb / RT_CAMS] = b;
         }
         if (!single) __syncthreads();
     }
@@ -271,7 +274,7 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
     if (warp == 0) {
         gb.arrive();
         ok = gb.wait();
-        const double v = sum_values(slot, groups, lane);
+        const double v = sum_values(slot_setup, groups, lane);
         if (lane == 0) s_out = v;
     }
     if (!__syncthreads_and(ok)) return;
@@ -326,7 +329,8 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
                         p_new[o3] = pk;
                         if (!single) t.q[o3] = qk;
                     }
-                    put_group(kb, on ? pq : 0.0);
+                    const double b = group_sum(on ? pq : 0.0);
+                    if (lane == 0) slot[kb / RT_CAMS] = b;
                 }
                 if (!single) __syncthreads();
             }
@@ -934,7 +938,7 @@ fm_status create_rot(fm_rotation *p, int32_t n_cams, int32_t n_pairs, const int3
     RT_CUDA(coop_blocks(k_rot_steps, RT_CAMS * 32, &p->step_grid));
     p->cg_grid = std::min(p->cg_grid, cam_blocks(n_cams));
     p->step_grid = std::min(p->step_grid, std::max(cam_blocks(n_cams), (n_pairs + 63) / 64));
-    RT_CUDA(ralloc(p, &d.blk, (size_t)cam_blocks(n_cams)));
+    RT_CUDA(ralloc(p, &d.blk, 2 * (size_t)cam_blocks(n_cams)));
     RT_CUDA(ralloc(p, &d.grid_state, (size_t)GRID_STATE_WORDS));
     RT_CUDA(ralloc(p, &d.loss, 1));
     RT_CUDA(ralloc(p, &d.hyper, 4));
