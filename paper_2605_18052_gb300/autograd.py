@@ -11,8 +11,9 @@ g_c. For R the backward returns the tangent-space Euclidean gradient 0.5 [g_phi]
 inner product with any rotation perturbation [dphi]_x R equals g_phi . dphi, so autograd
 through any rotation parameterisation (exponential map, 6D, quaternions) is exact. Contiguous
 float64 inputs take one kernel for this (fm_pose_gradient; as torch operations it was 13 launches,
-one of them a 70 us batched FP64 matrix product); other types and layouts, and a backward that is itself
-differentiated (create_graph), take the torch operations.
+one of them a 70 us batched FP64 matrix product); other types and layouts, tensors whose memory does not
+hold their values (a batched backward), and a backward that is itself differentiated (create_graph), take
+the torch operations.
 """
 from __future__ import annotations
 
@@ -38,6 +39,19 @@ def _loss_grad(problem, R, c):
     return loss, grad
 
 
+def _in_memory(t: torch.Tensor) -> bool:
+    """A plain tensor whose memory holds its values, so that a kernel can be given its address. Not so for the
+    gradients of a batched backward (no storage of their own, though their Python type is torch.Tensor), for
+    a lazily negated tensor (autograd's imaginary parts of conjugates: the memory has the other sign) and
+    for autograd's zeros without memory."""
+    if type(t) is not torch.Tensor or t.is_neg():
+        return False
+    try:
+        return t.data_ptr() != 0
+    except RuntimeError:
+        return False
+
+
 class EpipolarLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, problem, R, c, recompute: bool = False):
@@ -59,7 +73,7 @@ class EpipolarLoss(torch.autograd.Function):
             R, grad = ctx.saved_tensors
         if (not torch.is_grad_enabled() and R.dtype == grad.dtype == grad_out.dtype == torch.float64
                 and R.is_cuda and grad_out.device == R.device and R.is_contiguous()
-                and type(R) is type(grad_out) is torch.Tensor):
+                and _in_memory(R) and _in_memory(grad_out)):
             return None, *pose_gradient(grad, R, grad_out), None
         g = grad * grad_out
         gR = 0.5 * _hat(g[:, :3]) @ R.to(torch.float64)
