@@ -71,9 +71,12 @@ class EpipolarLoss(torch.autograd.Function):
             _, grad = _loss_grad(ctx.problem, R, c)
         else:
             R, grad = ctx.saved_tensors
+        # (saved-tensor hooks may give back other devices, layouts and shapes than were saved)
         if (not torch.is_grad_enabled() and R.dtype == grad.dtype == grad_out.dtype == torch.float64
-                and R.is_cuda and grad_out.device == R.device and R.is_contiguous()
-                and _in_memory(R) and _in_memory(grad_out)):
+                and R.is_cuda and grad_out.device == grad.device == R.device
+                and R.shape == (grad.shape[0], 3, 3) and grad.shape[1:] == (6,)
+                and R.is_contiguous() and grad.is_contiguous()
+                and _in_memory(R) and _in_memory(grad) and _in_memory(grad_out)):
             return None, *pose_gradient(grad, R, grad_out), None
         g = grad * grad_out
         gR = 0.5 * _hat(g[:, :3]) @ R.to(torch.float64)

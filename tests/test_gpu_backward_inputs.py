@@ -53,3 +53,16 @@ def test_zero_gradient_without_memory(scene):
     zero = torch._efficientzerotensor((), dtype=torch.float64, device="cuda")
     for g in torch.autograd.grad(fm.epipolar_loss(p, *leaves), leaves, zero):
         assert not g.any()
+
+
+def test_saved_gradient_in_another_layout(scene):
+    p, R, C, ref = scene
+    leaves = R.clone().requires_grad_(), C.clone().requires_grad_()
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t.transpose(0, 1).contiguous(), lambda t: t.transpose(0, 1)):
+        loss = fm.epipolar_loss(p, *leaves)
+    _same(torch.autograd.grad(loss, leaves), ref)
+    # the gradient alone: R comes back as it was
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t.t().contiguous() if t.dim() == 2 else t,
+                                                  lambda t: t.t() if t.dim() == 2 else t):
+        loss = fm.epipolar_loss(p, *leaves)
+    _same(torch.autograd.grad(loss, leaves), ref)
