@@ -40,11 +40,11 @@ def _loss_grad(problem, R, c):
 
 
 def _in_memory(t: torch.Tensor) -> bool:
-    """A plain tensor whose memory holds its values, so that a kernel can be given its address. Not so for the
+    """A plain tensor or parameter whose memory holds its values, so that a kernel can be given its address. Not so for the
     gradients of a batched backward (no storage of their own, though their Python type is torch.Tensor), for
     a lazily negated tensor (autograd's imaginary parts of conjugates: the memory has the other sign) and
     for autograd's zeros without memory."""
-    if type(t) is not torch.Tensor or t.is_neg():
+    if type(t) not in (torch.Tensor, torch.nn.Parameter) or t.is_neg():
         return False
     try:
         return t.data_ptr() != 0

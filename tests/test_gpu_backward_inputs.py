@@ -6,7 +6,7 @@ import torch
 
 import scenegen
 import paper_2605_18052_gb300 as fm
-from paper_2605_18052_gb300 import build
+from paper_2605_18052_gb300 import autograd, build
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +66,14 @@ def test_saved_gradient_in_another_layout(scene):
                                                   lambda t: t.t() if t.dim() == 2 else t):
         loss = fm.epipolar_loss(p, *leaves)
     _same(torch.autograd.grad(loss, leaves), ref)
+
+
+def test_parameters_take_the_kernel(scene, monkeypatch):
+    p, R, C, ref = scene
+    calls = []
+    kernel = autograd.pose_gradient
+    monkeypatch.setattr(autograd, "pose_gradient", lambda *a: calls.append(a) or kernel(*a))
+    leaves = torch.nn.Parameter(R.clone()), torch.nn.Parameter(C.clone())
+    fm.epipolar_loss(p, *leaves).backward()
+    _same([v.grad for v in leaves], ref)
+    assert len(calls) == 1 and type(leaves[0].grad) is torch.Tensor
