@@ -146,7 +146,8 @@ FM_API fm_status fm_set_poses(fm_problem *p, const double *R, const double *t);
 FM_API fm_status fm_get_params(fm_problem *p, double *R, double *c);
 FM_API fm_status fm_set_params(fm_problem *p, const double *R, const double *c);
 /* fm_set_params from device memory (d_R n_cams x 9, d_c n_cams x 3, FP64), asynchronous and
- * ordered on the caller's stream; R must be a rotation (not checked here). */
+ * ordered on the caller's stream; R must be a rotation (not checked here). A kernel on the problem's
+ * device reads the arrays: memory of another device has to be copied first. */
 FM_API fm_status fm_set_params_device(fm_problem *p, const double *d_R, const double *d_c);
 
 /*
@@ -172,7 +173,8 @@ FM_API fm_status fm_irls_weights(fm_problem *p, double tau, int64_t *n_active);
  * Synchronises.
  */
 FM_API fm_status fm_loss_grad(fm_problem *p, double *loss, double *grad);
-/* Same, asynchronous, into device memory the caller owns (either pointer may be NULL). */
+/* Same, asynchronous, into device memory the caller owns (either pointer may be NULL). Kernels on the
+ * problem's device write it: it has to be memory of that device. */
 FM_API fm_status fm_loss_grad_device(fm_problem *p, double *d_loss, double *d_grad);
 
 /*

@@ -198,6 +198,16 @@ def _current_stream():
     return ctypes.c_void_p(0)
 
 
+def _current_device() -> int:
+    try:
+        import torch
+        if torch.cuda.is_available() and torch.cuda.is_initialized():
+            return torch.cuda.current_device()
+    except Exception:
+        pass
+    return 0
+
+
 class Problem:
     """One epipolar-adjustment problem held on the GPU (see include/fastmap.h)."""
 
@@ -228,6 +238,7 @@ class Problem:
         self.n_pp = int(n_pp)
         self.options = options if options is not None else default_options()
         self.stream = stream if stream is not None else _current_stream()
+        self._device = _current_device()
         h = ctypes.c_void_p()
         _check(lib.fm_create_problem(self.n_cams, _ptr(R), _ptr(t), self.n_pairs, _ptr(ci), _ptr(cj),
                                      self.n_pp, *ptrs, 1 if on_dev else 0, ctypes.byref(self.options),
@@ -282,8 +293,14 @@ class Problem:
         c = _host(c, np.float64)
         _check(load_library().fm_set_params(self._h, _ptr(R), _ptr(c)))
 
+    def _here(self, t) -> bool:
+        # the library's kernels read and write the caller's memory: it has to be the problem's device's
+        return t.is_cuda and t.get_device() == self._device
+
     def set_params_device(self, R, c):
-        """Asynchronous parameter update from contiguous float64 CUDA tensors (N,3,3), (N,3)."""
+        """Asynchronous parameter update from contiguous float64 CUDA tensors (N,3,3), (N,3). Tensors that are
+        not on the problem's device are copied there."""
+        R, c = (v if self._here(v) else v.detach().to(f"cuda:{self._device}") for v in (R, c))
         _check(load_library().fm_set_params_device(self._h, ctypes.c_void_p(R.data_ptr()),
                                                    ctypes.c_void_p(c.data_ptr())))
 
@@ -364,7 +381,18 @@ class Problem:
         return loss.value, g
 
     def loss_grad_device(self, loss_out, grad_out):
-        """Asynchronous loss/gradient into device tensors (float64, sizes 1 and n_cams*6)."""
+        """Asynchronous loss/gradient into device tensors (float64, sizes 1 and n_cams*6). Results for tensors
+        that are not on the problem's device are copied there."""
+        away = [t for t in (loss_out, grad_out) if t is not None and not self._here(t)]
+        if away:
+            import torch
+            with torch.no_grad():
+                near = [None if t is None else torch.empty_like(t, device=f"cuda:{self._device}") for t in (loss_out, grad_out)]
+                self.loss_grad_device(*near)
+                for t, n in zip((loss_out, grad_out), near):
+                    if t is not None:
+                        t.copy_(n)
+            return
         _check(load_library().fm_loss_grad_device(
             self._h, ctypes.c_void_p(loss_out.data_ptr()) if loss_out is not None else None,
             ctypes.c_void_p(grad_out.data_ptr()) if grad_out is not None else None))
