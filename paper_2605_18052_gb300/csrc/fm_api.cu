@@ -437,18 +437,23 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     p->input_was_sorted = (err & ERR_UNSORTED) ? 0 : 1;
 
     const int *keys = d_pid;
-    float4 *sorted = nullptr;   // point pairs in pair order, when they did not come so
+    const int *perm = nullptr;   // where the keypoints of a point pair are in d_x1 and d_x2 (null: in pair order)
     if (!p->input_was_sorted) {
         FM_CUDA(dalloc(p, &d.perm, (size_t)n_pp));
+        perm = d.perm;
         const size_t kb = (sizeof(int) * n_pp + 255) / 256 * 256;
-        const size_t gather = d.storage == FM_STORE_FP16 ? sizeof(float4) * n_pp : 0;
-        FM_CUDA(cudaMallocAsync(&t_sort, kb + std::max(sort_scratch_bytes(n_pp), gather), p->s));
+        FM_CUDA(cudaMallocAsync(&t_sort, kb + sort_scratch_bytes(n_pp), p->s));
         int *sorted_keys = reinterpret_cast<int *>(t_sort);
         FM_CUDA(sort_by_pair(d_pid, n_pp, n_pairs, sorted_keys, d.perm, t_sort + kb, p->s));
         keys = sorted_keys;
-        if (gather) {   // the sort's scratch is free again
-            sorted = reinterpret_cast<float4 *>(t_sort + kb);
-            launch_gather_points(d, d_x1, d_x2, sorted, p->s);
+        if (d.storage == FM_STORE_FP16) {
+            // the centroids and the packing want pair order: x1 in the place of the packed keypoints (8 bytes
+            // a point pair as well), x2 in the sort's scratch, which is free again: no further memory
+            float2 *g1 = static_cast<float2 *>(d.kp), *g2 = reinterpret_cast<float2 *>(t_sort + kb);
+            launch_gather_points(d, d_x1, d_x2, g1, g2, p->s);
+            d_x1 = g1;
+            d_x2 = g2;
+            perm = nullptr;
         }
     }
     launch_pair_offsets(keys, n_pp, n_pairs, d.pair_off, d.err, p->s);
@@ -462,8 +467,8 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     }
     launch_range_pairs(d.pair_off, n_pairs, d.n_ranges, d.range_pair, p->s);
     if (d.storage == FM_STORE_FP16)   // d.grad is free until the first evaluation: the sums of 2 words a camera
-        launch_centroids(d, d_x1, d_x2, sorted, reinterpret_cast<unsigned long long *>(d.grad), p->s);
-    launch_pack(d, keys, d_x1, d_x2, sorted, p->s);
+        launch_centroids(d, d_x1, d_x2, reinterpret_cast<unsigned long long *>(d.grad), p->s);
+    launch_pack(d, keys, d_x1, d_x2, perm, p->s);
     FM_CUDA(cudaGetLastError());
     release_temps();
     FM_CUDA(cudaMemsetAsync(d.err, 0, sizeof(unsigned), p->s));

@@ -184,13 +184,13 @@ void launch_pair_offsets(const int *sorted_keys, int64_t n_pp, int n_pairs, int 
 void launch_range_pairs(const int *pair_off, int n_pairs, int n_ranges, int *range_pair,
                         cudaStream_t s);
 // point pairs in pair order from an unsorted input (d.perm), for the two launches below
-void launch_gather_points(const DevProblem &d, const float2 *x1, const float2 *x2, float4 *out, cudaStream_t s);
+void launch_gather_points(const DevProblem &d, const float2 *x1, const float2 *x2, float2 *o1, float2 *o2, cudaStream_t s);
 // FP16 storage: per-image centroids into d.cen (needs d.cam_off/cam_ent/pair_off/range_pair);
-// `sums` is scratch for 2 * n_cams int64.
-void launch_centroids(const DevProblem &d, const float2 *x1, const float2 *x2, const float4 *sorted,
-                      unsigned long long *sums, cudaStream_t s);
-// keypoints in the streaming format, initial weights, scores and history
-void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2, const float4 *sorted,
+// x1 and x2 in pair order; `sums` is scratch for 2 * n_cams int64.
+void launch_centroids(const DevProblem &d, const float2 *x1, const float2 *x2, unsigned long long *sums, cudaStream_t s);
+// keypoints in the streaming format, initial weights, scores and history; perm: null when x1 and x2 are in
+// pair order
+void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2, const int *perm,
                  cudaStream_t s);
 void launch_set_weights(const DevProblem &d, const float *w_input_order, cudaStream_t s);
 void launch_get_weights(const DevProblem &d, float *w_input_order, cudaStream_t s);

@@ -147,6 +147,7 @@ static size_t sort_hist_words(int64_t n_pp) {
     return (size_t)(n + n / 512 + 64);   // scan levels need < n / 512 extra entries
 }
 
+// at least 8 bytes a point pair, from the start of the scratch on
 size_t sort_scratch_bytes(int64_t n_pp) {
     return 2 * ((sizeof(int) * n_pp + 255) / 256 * 256) + sizeof(unsigned) * sort_hist_words(n_pp);
 }
@@ -242,25 +243,23 @@ __device__ __forceinline__ void centroid_flush(const DevProblem &d, int seg, int
     for (int q = 0; q < 4; ++q) f[q] = 0;
 }
 
-// point pairs of an unsorted input in pair order (x1, y1, x2, y2): one random read per array; the
-// centroids and the packing then read in sequence (reading through the permutation twice took 69 +
-// 29 us on 3.1 M point pairs)
-__global__ void k_gather_points(const int *perm, int64_t n, const float2 *x1, const float2 *x2, float4 *out) {
+// point pairs of an unsorted input in pair order: one random read per array; the centroids and the
+// packing then read in sequence (reading through the permutation twice took 69 + 29 us on 3.1 M
+// point pairs)
+__global__ void k_gather_points(const int *perm, int64_t n, const float2 *x1, const float2 *x2, float2 *o1, float2 *o2) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int64_t src = perm[p];
-    const float2 a = x1[src], b = x2[src];
-    out[p] = make_float4(a.x, a.y, b.x, b.y);
+    o1[p] = x1[src];
+    o2[p] = x2[src];
 }
 
-void launch_gather_points(const DevProblem &d, const float2 *x1, const float2 *x2, float4 *out, cudaStream_t s) {
-    k_gather_points<<<blocks_for(d.n_pp, 256), 256, 0, s>>>(d.perm, d.n_pp, x1, x2, out);
+void launch_gather_points(const DevProblem &d, const float2 *x1, const float2 *x2, float2 *o1, float2 *o2, cudaStream_t s) {
+    k_gather_points<<<blocks_for(d.n_pp, 256), 256, 0, s>>>(d.perm, d.n_pp, x1, x2, o1, o2);
 }
 
-// sorted: the point pairs in pair order, or null when x1 and x2 are in pair order. Four groups are loaded
-// ahead of their sums.
-__global__ void k_centroid_sums(DevProblem d, const float2 *x1, const float2 *x2, const float4 *sorted,
-                                unsigned long long *sums) {
+// x1 and x2 in pair order. Four groups are loaded ahead of their sums.
+__global__ void k_centroid_sums(DevProblem d, const float2 *x1, const float2 *x2, unsigned long long *sums) {
     constexpr int U = 4;
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * 2 + (threadIdx.x >> 5);
@@ -276,8 +275,8 @@ __global__ void k_centroid_sums(DevProblem d, const float2 *x1, const float2 *x2
             const int q = g0 + 32 * u + lane;
             x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (q >= p_end) continue;
-            if (sorted) x[u] = sorted[q];
-            else x[u] = make_float4(x1[q].x, x1[q].y, x2[q].x, x2[q].y);
+            const float2 a = x1[q], b = x2[q];
+            x[u] = make_float4(a.x, a.y, b.x, b.y);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -323,30 +322,27 @@ __global__ void k_centroid_final(const unsigned long long *sums, const int *cam_
     cen[k] = c;
 }
 
-void launch_centroids(const DevProblem &d, const float2 *x1, const float2 *x2, const float4 *sorted,
-                      unsigned long long *sums, cudaStream_t s) {
+void launch_centroids(const DevProblem &d, const float2 *x1, const float2 *x2, unsigned long long *sums, cudaStream_t s) {
     cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * 2 * d.n_cams, s);
-    k_centroid_sums<<<blocks_for(d.n_ranges, 2), 64, 0, s>>>(d, x1, x2, sorted, sums);
+    k_centroid_sums<<<blocks_for(d.n_ranges, 2), 64, 0, s>>>(d, x1, x2, sums);
     k_centroid_final<<<blocks_for(d.n_cams, 128), 128, 0, s>>>(sums, d.cam_off, d.cam_ent,
                                                               d.pair_off, d.n_cams, d.cen);
 }
 
 // ---- packing into the streaming format ------------------------------------------------------------
-// and the initial weights (1), scores (0.5) and residual history (0); padding is zero (score 0.5)
+// and the initial weights (1), scores (0.5) and residual history (0); padding is zero (score 0.5). perm: the
+// input position of each point pair, or null when x1 and x2 are in pair order. (x1 may lie where the FP16
+// offsets go: a thread reads its own 8 bytes before it writes them.)
 template <int STORE>
-__global__ void k_pack(DevProblem d, const int *keys, const float2 *x1, const float2 *x2, const float4 *sorted) {
+__global__ void k_pack(DevProblem d, const int *keys, const float2 *x1, const float2 *x2, const int *perm) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= d.n_pad) return;
     const bool in = p < d.n_pp;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (in) {
-        if (sorted) {
-            v = sorted[p];
-        } else {
-            const int64_t src = d.perm ? d.perm[p] : p;
-            const float2 a = x1[src], b = x2[src];
-            v = make_float4(a.x, a.y, b.x, b.y);
-        }
+        const int64_t src = perm ? perm[p] : p;
+        const float2 a = x1[src], b = x2[src];
+        v = make_float4(a.x, a.y, b.x, b.y);
     }
     if (STORE == FM_STORE_FP32) {
         static_cast<float4 *>(d.kp)[p] = v;
@@ -371,11 +367,11 @@ __global__ void k_pack(DevProblem d, const int *keys, const float2 *x1, const fl
     d.le_hist[p] = __float2half_rn(0.f);
 }
 
-void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2, const float4 *sorted,
+void launch_pack(const DevProblem &d, const int *sorted_keys, const float2 *x1, const float2 *x2, const int *perm,
                  cudaStream_t s) {
     const int grid = blocks_for(d.n_pad, 256);
-    if (d.storage == FM_STORE_FP32) k_pack<FM_STORE_FP32><<<grid, 256, 0, s>>>(d, sorted_keys, x1, x2, sorted);
-    else k_pack<FM_STORE_FP16><<<grid, 256, 0, s>>>(d, sorted_keys, x1, x2, sorted);
+    if (d.storage == FM_STORE_FP32) k_pack<FM_STORE_FP32><<<grid, 256, 0, s>>>(d, sorted_keys, x1, x2, perm);
+    else k_pack<FM_STORE_FP16><<<grid, 256, 0, s>>>(d, sorted_keys, x1, x2, perm);
 }
 
 // ---- weights ------------------------------------------------------------------------------------------
