@@ -174,6 +174,24 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
     if ((int64_t)n_cand > 65535LL * VOTE_CANDS) return fv_fail(FM_EINVAL, "n_cand must be <= 1048560");
     if (!F || !cand || !votes) return fv_fail(FM_EINVAL, "F, cand and votes must not be NULL");
     if (!(tau > 0.0) || !std::isfinite(tau)) return fv_fail(FM_EINVAL, "tau must be finite and > 0");
+    // F is looked at by the device, which reads it anyway; on the host only where a call fails otherwise, so
+    // that a refused F is reported before the arguments behind it and before an error of the device
+    auto check_F = [&]() -> fm_status {
+        for (int n = 0; n < n_pairs; ++n) {
+            double nrm = 0.0;
+            for (int q = 0; q < 9; ++q) {
+                const double v = F[(size_t)n * 9 + q];
+                if (!std::isfinite(v)) return fv_fail(FM_EINVAL, "F must be finite");
+                nrm += v * v;
+            }
+            if (!(nrm > 0.0)) return fv_fail(FM_EINVAL, "F of pair " + std::to_string(n) + " is zero");
+        }
+        return FM_OK;
+    };
+    auto refuse = [&](fm_status st, const char *msg) {
+        if (fm_status bad_F = check_F()) return bad_F;
+        return fv_fail(st, msg);
+    };
     // one host buffer for the small inputs: candidates, then the known focal lengths that are given
     std::vector<float> small(n_cand + (size_t)n_pairs * ((f1_known ? 1 : 0) + (f2_known ? 1 : 0)));
     float *k1 = small.data() + n_cand, *k2 = k1 + (f1_known ? n_pairs : 0);
@@ -186,9 +204,9 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
         return true;
     };
     if (!known(f1_known, k1) || !known(f2_known, k2))
-        return fv_fail(FM_EINVAL, "known focal lengths must be finite and >= 0 (0 = the candidate)");
+        return refuse(FM_EINVAL, "known focal lengths must be finite and >= 0 (0 = the candidate)");
     for (int c = 0; c < n_cand; ++c) {
-        if (!(cand[c] > 0.0) || !std::isfinite(cand[c])) return fv_fail(FM_EINVAL, "candidates must be finite and > 0");
+        if (!(cand[c] > 0.0) || !std::isfinite(cand[c])) return refuse(FM_EINVAL, "candidates must be finite and > 0");
         small[c] = (float)cand[c];
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -239,7 +257,7 @@ extern "C" FM_API fm_status fm_focal_vote(int32_t n_pairs, const double *F, cons
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess)
-        return fv_fail(e == cudaErrorMemoryAllocation ? FM_ENOMEM : FM_ECUDA, cudaGetErrorString(e));
+        return refuse(e == cudaErrorMemoryAllocation ? FM_ENOMEM : FM_ECUDA, cudaGetErrorString(e));
     unsigned long long bad;
     std::memcpy(&bad, &out[n_cand], sizeof bad);
     if (bad != ~0ull)
