@@ -1043,10 +1043,13 @@ fm_status quad_prepare(fm_problem *p) {
     arena.add(&p->d.grid_state, GRID_STATE_WORDS);
     FM_CUDA(arena.commit(p));
     FM_CUDA(cudaMemsetAsync(p->d.grid_state, 0, sizeof(unsigned) * GRID_STATE_WORDS, p->s));
-    int blocks = 0;
-    FM_CUDA(quad_steps_capacity(p->d.refine_focal != 0, &blocks));
-    p->quad_persistent = camera_step_blocks(p->d) <= blocks;
     p->quad_alloc = true;
+    // where the persistent kernel cannot be had (its 60 KB of shared memory, a cooperative launch), the steps
+    // are launched one by one
+    int blocks = 0;
+    const bool capacity = quad_steps_capacity(p->d.refine_focal != 0, &blocks) == cudaSuccess;
+    if (!capacity) cudaGetLastError();
+    p->quad_persistent = capacity && camera_step_blocks(p->d) <= blocks;
     return FM_OK;
 }
 
