@@ -50,6 +50,7 @@ struct fm_problem {
     // fused with the reweighting (key -n)
     std::map<int, cudaGraphExec_t> chains;
     bool timing = false;
+    std::vector<char> host_params;        // R, c and the error word as they come from the device (read_params)
     int hist_valid = 0;                   // d.le_hist holds a previous reweighting's residuals
     double lr_focal = 1e-3;               // Adam step size of rho = log(f0/f)
     bool quad_alloc = false;              // d.qslots, d.quad, d.pair_rec allocated
@@ -82,18 +83,19 @@ cudaError_t dalloc(fm_problem *p, T **ptr, size_t count) {
 // 33 arrays): add() notes where each array's pointer goes, commit() allocates and fills them in.
 // Arrays lie in the order of add(), each on a 256-byte boundary.
 struct Arena {
-    std::vector<std::pair<void **, size_t>> items;
+    std::pair<void **, size_t> items[40];
+    int n = 0;
     size_t bytes = 0;
     template <class T>
     void add(T **ptr, size_t count) {
-        items.emplace_back(reinterpret_cast<void **>(ptr), bytes);
+        items[n++] = {reinterpret_cast<void **>(ptr), bytes};
         bytes += (sizeof(T) * (count ? count : 1) + 255) / 256 * 256;
     }
     cudaError_t commit(fm_problem *p) {
         char *base = nullptr;
         cudaError_t e = dalloc(p, &base, bytes);
         if (e == cudaSuccess)
-            for (auto &it : items) *it.first = base + it.second;
+            for (int i = 0; i < n; ++i) *items[i].first = base + items[i].second;
         return e;
     }
 };
@@ -388,7 +390,9 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     arena.add(&w, w_bytes * d.n_pad);
     arena.add(&d.score, (size_t)d.n_pad);
     arena.add(&d.le_hist, (size_t)d.n_pad);
+    p->allocs.reserve(4);   // the arena, the permutation, the quadratic form
     FM_CUDA(arena.commit(p));
+    p->host_params.resize((char *)d.err - (char *)d.R + sizeof(unsigned));
     d.kp = kp;
     d.w = w;
     d.pstat = reinterpret_cast<float *>(ps);
@@ -483,12 +487,12 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
 // R, c and the device's error word in one copy (they are neighbours in the arena); reports errors as
 // check_device_errors does
 fm_status read_params(fm_problem *p, double *R, double *c) {
-    const size_t n = (size_t)p->d.n_cams, span = (char *)p->d.err - (char *)p->d.R;
-    std::vector<char> buf(span + sizeof(unsigned));
+    const size_t n = (size_t)p->d.n_cams;
+    std::vector<char> &buf = p->host_params;   // allocated with the problem: nothing here can throw
     FM_CUDA(cudaMemcpyAsync(buf.data(), p->d.R, buf.size(), cudaMemcpyDeviceToHost, p->s));
     FM_CUDA(cudaStreamSynchronize(p->s));
     unsigned err;
-    std::memcpy(&err, buf.data() + span, sizeof err);
+    std::memcpy(&err, buf.data() + buf.size() - sizeof err, sizeof err);
     std::memcpy(R, buf.data(), sizeof(double) * 9 * n);
     std::memcpy(c, buf.data() + ((char *)p->d.c - (char *)p->d.R), sizeof(double) * 3 * n);
     return err ? check_device_errors(p) : FM_OK;
