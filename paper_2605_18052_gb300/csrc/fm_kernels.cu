@@ -678,14 +678,14 @@ void launch_camera_step(const DevProblem &d, bool apply, float *cam_dst, cudaStr
 }
 
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth) {
+    with_stages<RECORD_STAGES>(d, [&](auto store, auto depth) {
         constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
         k_irls_weights<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, tau);
     });
 }
 
 void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth) {
+    with_stages<RECORD_STAGES>(d, [&](auto store, auto depth) {
         constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
         k_residuals<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, out_input_order);
     });

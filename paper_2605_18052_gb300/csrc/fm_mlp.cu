@@ -488,7 +488,7 @@ void launch_learned_loss(const DevProblem &d, const float *master, const __nv_bf
 }
 
 void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
-    with_stages(d, [&](auto store, auto depth) {
+    with_stages<RECORD_STAGES>(d, [&](auto store, auto depth) {
         constexpr int STORE = decltype(store)::value, S = decltype(depth)::value;
         k_pair_stats<STORE, S><<<d.n_ranges, 32, S * STAGE_BYTES, s>>>(d, tau);
     });

@@ -445,14 +445,18 @@ __device__ __forceinline__ void walk_range_staged(const DevProblem &d, int r, in
 // us, 245 ranges 16.3 -> 16.0; 733 ranges 16.6 -> 18.5). FP16: 2 chunks (512 point pairs; 4 chunks: 5,860
 // ranges 28.6 -> 30.4, 68,634 ranges 218.9 -> 224.3).
 constexpr int FEW_RANGES = 2 * 152;
+// Passes over geometry records (weights, statistics, residuals), FP32: 3 chunks. An image pair's matrix is read
+// from its record where it begins, which more warps hide better (30 an SM, 22 with 4 chunks): weights of
+// 20.0 M point pairs in 200,000 image pairs 150 -> 134 us (2 chunks 137), in 12,000 the same.
+constexpr int RECORD_STAGES = 3;
 
-template <class Launch>
+template <int DEPTH32 = 4, class Launch>
 static void with_stages(const DevProblem &d, Launch launch) {
     using std::integral_constant;
     if (d.storage == FM_STORE_FP32) {
         integral_constant<int, FM_STORE_FP32> st;
         if (d.n_ranges <= FEW_RANGES) launch(st, integral_constant<int, 16>());
-        else launch(st, integral_constant<int, 4>());
+        else launch(st, integral_constant<int, DEPTH32>());
     } else {
         launch(integral_constant<int, FM_STORE_FP16>(), integral_constant<int, 2>());
     }
