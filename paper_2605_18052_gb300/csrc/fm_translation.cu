@@ -157,8 +157,11 @@ __global__ void __launch_bounds__(TR_CAMS * 32) k_tr_cam(DevTrans t) {
 // instructions remain, the differences of centres and their rounding to FP32: they bound an
 // iteration, 7.7 us there with the barrier, 23.5 us as two launches.
 constexpr int TR_RC = 8;       // most runs of an item
-constexpr int TR_BATCH = 4;    // runs whose loads are in flight together
+// BATCH: runs whose loads are in flight together: 4, and 1 for items of one run, which would read the one
+// centre four times over (100 iterations of one run: 1,000 cameras with 16 image pairs each 433 -> 327 us, 2,000 with 48
+// 806 -> 577, 5,000 with 80 2,444 -> 1,762; as two launches 778, 1,040, 2,058).
 
+template <int BATCH>
 __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int iters, int rc) {
     __shared__ float s_g[TR_CAMS][TR_RC][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -192,11 +195,11 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
                     e_end = t.cam_off[k + 1];
                     if (e_begin + lane < e_end) load_entry(e_begin + lane);
                 }
-                for (int rb = 0; rb < nr; rb += TR_BATCH) {
-                    float g[TR_BATCH][3];
-                    double own[TR_BATCH][3];
+                for (int rb = 0; rb < nr; rb += BATCH) {
+                    float g[BATCH][3];
+                    double own[BATCH][3];
 #pragma unroll
-                    for (int b = 0; b < TR_BATCH; ++b) {
+                    for (int b = 0; b < BATCH; ++b) {
                         const size_t row = (size_t)(r0 + min(rb + b, nr - 1)) * t.n_cams;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
@@ -206,15 +209,15 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
                     }
                     for (int e = e_begin + lane; e < e_end; e += 32) {
                         if (e_end - e_begin > 32) load_entry(e);
-                        double oo[TR_BATCH][3];
+                        double oo[BATCH][3];
 #pragma unroll
-                        for (int b = 0; b < TR_BATCH; ++b) {
+                        for (int b = 0; b < BATCH; ++b) {
                             const size_t row = (size_t)(r0 + min(rb + b, nr - 1)) * t.n_cams;
 #pragma unroll
                             for (int a = 0; a < 3; ++a) oo[b][a] = __ldcg(src + (row + other) * 3 + a);
                         }
 #pragma unroll
-                        for (int b = 0; b < TR_BATCH; ++b) {
+                        for (int b = 0; b < BATCH; ++b) {
                             if (rb + b >= nr) break;
                             float u[3];
 #pragma unroll
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
                         }
                     }
 #pragma unroll
-                    for (int b = 0; b < TR_BATCH; ++b) {
+                    for (int b = 0; b < BATCH; ++b) {
                         if (rb + b >= nr) break;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
@@ -421,9 +424,10 @@ void enqueue_eval(fm_translation *p) {
 // items of rc runs each: as many as fit the resident blocks, so that few runs per block are in series
 cudaError_t enqueue_steps(fm_translation *p, int iters) {
     const int64_t groups = cam_blocks(p->d);
-    const int rc = (int)std::min<int64_t>(TR_RC, (groups * p->d.n_runs + p->step_grid - 1) / p->step_grid);
+    const int fit = (int)std::min<int64_t>(TR_RC, (groups * p->d.n_runs + p->step_grid - 1) / p->step_grid);
+    const int rc = std::min(fit, p->d.n_runs);
     const int64_t items = groups * ((p->d.n_runs + rc - 1) / rc);
-    return launch_coop(k_tr_steps, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, 0, p->s, p->d, iters, rc);
+    return launch_coop(rc == 1 ? k_tr_steps<1> : k_tr_steps<4>, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, 0, p->s, p->d, iters, rc);
 }
 
 constexpr int TR_CHAIN = 4096;
@@ -495,7 +499,10 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     TR_CUDA(talloc(p, &d.o, nc3));
     TR_CUDA(talloc(p, &d.o2, nc3));
     TR_CUDA(talloc(p, &d.grid_state, (size_t)GRID_STATE_WORDS));
-    TR_CUDA(coop_blocks(k_tr_steps, TR_CAMS * 32, &p->step_grid));
+    int blocks1 = 0;
+    TR_CUDA(coop_blocks(k_tr_steps<4>, TR_CAMS * 32, &p->step_grid));
+    TR_CUDA(coop_blocks(k_tr_steps<1>, TR_CAMS * 32, &blocks1));
+    p->step_grid = std::min(p->step_grid, blocks1);
     TR_CUDA(talloc(p, &d.m, nc3));
     TR_CUDA(talloc(p, &d.v, nc3));
     TR_CUDA(talloc(p, &d.pterm, (size_t)n_runs * n_pairs));
