@@ -13,6 +13,7 @@
 // Adam iterations of all runs are one persistent kernel (k_tr_steps). Centres and their update are
 // FP64; the per-pair arithmetic is FP32 on the FP64 difference o_j - o_i.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -161,7 +162,20 @@ constexpr int TR_RC = 8;       // most runs of an item
 // centre four times over (100 iterations of one run: 1,000 cameras with 16 image pairs each 433 -> 327 us, 2,000 with 48
 // 806 -> 577, 5,000 with 80 2,444 -> 1,762; as two launches 778, 1,040, 2,058).
 
-template <int BATCH>
+// PAIRS: a first phase, with a grid barrier behind it, evaluates every pair once, a thread per pair and batch of
+// runs, and the cameras' lanes read the terms. Without it a warp evaluates its camera's pairs 32 at a time, one
+// run after the other, so a camera of many pairs holds up the grid. The phase is taken where more than
+// TR_SERIES such evaluations are in series (rounds of items x runs of an item x 32s of pairs of the largest camera),
+// unless they are the runs of one item, whose loads overlap. us an iteration without / with it, (as two
+// launches):
+//   1: 1,000 cameras, 16 pairs each 3.4 / 5.1 (8.0)     4: 1,000 cameras, 120 pairs each 7.4 / 7.4 (9.7)
+//   2: 3,000 cameras, 24 pairs each 6.9 / 7.3 (11.5)    4: 1,000 cameras, 48 pairs each, 4 runs 9.7 / 8.0 (16.3)
+//   5: 150 cameras, all pairs 8.7 / 7.1 (8.3)           6: 5,000 cameras, 48 pairs each 14.1 / 11.8 (20.4)
+//   10: 300 cameras, all pairs 15.2 / 7.2 (10.1)        157: 5,000 cameras, one in all pairs 175 / 16.8 (34.9)
+//   56: 5,000 cameras, 200 pairs each, 8 runs 159 / 94 (132)
+constexpr int TR_SERIES = 4;
+
+template <int BATCH, bool PAIRS>
 __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int iters, int rc) {
     __shared__ float s_g[TR_CAMS][TR_RC][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -186,6 +200,32 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
     for (int it = 0; it < iters; ++it) {
         const double *src = (it & 1) ? t.o2 : t.o;
         double *dst = (it & 1) ? t.o : t.o2;
+        if (PAIRS) {   // a thread takes BATCH runs of a pair (plain loads: behind the grid barrier's acquire, and
+                       // many pairs share a camera: 1,000 cameras, all pairs, 2 runs 30.2 us from L2, 27.5 so)
+            const size_t run = (size_t)t.n_cams * 3;
+            const size_t work = (size_t)t.n_pairs * ((t.n_runs + BATCH - 1) / BATCH);
+            for (size_t i = blockIdx.x * (TR_CAMS * 32) + threadIdx.x; i < work; i += gridDim.x * (TR_CAMS * 32)) {
+                const int n = (int)(i % t.n_pairs), rb = (int)(i / t.n_pairs) * BATCH;
+                const double *oi = src + (size_t)t.cam_i[n] * 3, *oj = src + (size_t)t.cam_j[n] * 3;
+                const float4 to = t.oij[n];
+                float u[BATCH][3];
+#pragma unroll
+                for (int b = 0; b < BATCH; ++b) {
+                    if (rb + b >= t.n_runs) break;
+                    const size_t row = (rb + b) * run;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) u[b][a] = (float)(oj[row + a] - oi[row + a]);
+                }
+#pragma unroll
+                for (int b = 0; b < BATCH; ++b) {
+                    if (rb + b >= t.n_runs) break;
+                    float4 p;
+                    if (!pair_term(u[b], to, p)) atomicOr(t.err, ERR_DEGENERATE);
+                    t.pterm[(size_t)(rb + b) * t.n_pairs + n] = p;
+                }
+            }
+            if (!gb.sync()) return;
+        }
         for (int item = blockIdx.x; item < items; item += gridDim.x) {
             const int group = item / chunks, r0 = (item % chunks) * rc, nr = min(rc, t.n_runs - r0);
             const int k = group * TR_CAMS + warp;
@@ -193,7 +233,7 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
                 if (!single || it == 0) {
                     e_begin = t.cam_off[k];
                     e_end = t.cam_off[k + 1];
-                    if (e_begin + lane < e_end) load_entry(e_begin + lane);
+                    if (!PAIRS && e_begin + lane < e_end) load_entry(e_begin + lane);
                 }
                 for (int rb = 0; rb < nr; rb += BATCH) {
                     float g[BATCH][3];
@@ -203,10 +243,27 @@ __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int it
                         const size_t row = (size_t)(r0 + min(rb + b, nr - 1)) * t.n_cams;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
-                            own[b][a] = __ldcg(src + (row + k) * 3 + a);
+                            if (!PAIRS) own[b][a] = __ldcg(src + (row + k) * 3 + a);
                             g[b][a] = 0.f;
                         }
                     }
+                    if (PAIRS) {
+#pragma unroll 8 / BATCH
+                        for (int e = e_begin + lane; e < e_end; e += 32) {
+                            const int ent = t.cam_ent[e];
+                            const float se = (ent & 1) ? 1.f : -1.f;
+                            float4 p[BATCH];
+#pragma unroll
+                            for (int b = 0; b < BATCH; ++b)
+                                p[b] = __ldcg(t.pterm + (size_t)(r0 + min(rb + b, nr - 1)) * t.n_pairs + (ent >> 1));
+#pragma unroll
+                            for (int b = 0; b < BATCH; ++b) {
+                                g[b][0] = fmaf(se, p[b].x, g[b][0]);
+                                g[b][1] = fmaf(se, p[b].y, g[b][1]);
+                                g[b][2] = fmaf(se, p[b].z, g[b][2]);
+                            }
+                        }
+                    } else
                     for (int e = e_begin + lane; e < e_end; e += 32) {
                         if (e_end - e_begin > 32) load_entry(e);
                         double oo[BATCH][3];
@@ -358,6 +415,7 @@ struct fm_translation {
     cudaStream_t s = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int step_grid = 0;       // most blocks of the step kernel
+    int chunks = 0;          // image pairs of the camera with the most, in warps' worth
     std::vector<void *> allocs;
 };
 
@@ -421,13 +479,29 @@ void enqueue_eval(fm_translation *p) {
     launch_k(k_tr_cam, gc, dim3(TR_CAMS * 32), p->s, true, p->d);
 }
 
-// items of rc runs each: as many as fit the resident blocks, so that few runs per block are in series
+// items of rc runs each: as many as fit the resident blocks, so that few runs per block are in series (the next
+// rc where the uneven last items would make a nearly empty second round: 849 cameras, 7 runs, 321 items of 3
+// on 304 blocks 11.7 us an iteration, 214 of 4 7.5; 1,617 cameras, 4 runs, 12.2 -> 7.8)
 cudaError_t enqueue_steps(fm_translation *p, int iters) {
-    const int64_t groups = cam_blocks(p->d);
-    const int fit = (int)std::min<int64_t>(TR_RC, (groups * p->d.n_runs + p->step_grid - 1) / p->step_grid);
-    const int rc = std::min(fit, p->d.n_runs);
-    const int64_t items = groups * ((p->d.n_runs + rc - 1) / rc);
-    return launch_coop(rc == 1 ? k_tr_steps<1> : k_tr_steps<4>, (int)std::min<int64_t>(items, p->step_grid), TR_CAMS * 32, 0, p->s, p->d, iters, rc);
+    const DevTrans &d = p->d;
+    const int64_t groups = cam_blocks(d);
+    const int most_runs = std::min(TR_RC, d.n_runs);
+    auto items_of = [&](int rc) { return groups * ((d.n_runs + rc - 1) / rc); };
+    int rc = (int)std::min<int64_t>(most_runs, (groups * d.n_runs + p->step_grid - 1) / p->step_grid);
+    if (items_of(most_runs) <= p->step_grid)
+        while (items_of(rc) > p->step_grid) ++rc;
+    const int64_t items = items_of(rc), rounds = (items + p->step_grid - 1) / p->step_grid;
+    int64_t blocks = items;
+    const int64_t passes = rounds * p->chunks;   // over a warp's pairs, rc runs each
+    const bool pairs = passes > 1 && passes * rc > TR_SERIES;
+    const int batch = rc == 1 ? 1 : (pairs && rc == 2 ? 2 : 4);
+    if (pairs) {
+        const int64_t work = (int64_t)d.n_pairs * ((d.n_runs + batch - 1) / batch);
+        blocks = std::max<int64_t>(blocks, (work + TR_CAMS * 32 - 1) / (TR_CAMS * 32));
+    }
+    auto kernel = pairs ? (batch == 1 ? k_tr_steps<1, true> : (batch == 2 ? k_tr_steps<2, true> : k_tr_steps<4, true>))
+                        : (batch == 1 ? k_tr_steps<1, false> : k_tr_steps<4, false>);
+    return launch_coop(kernel, (int)std::min<int64_t>(blocks, p->step_grid), TR_CAMS * 32, 0, p->s, d, iters, rc);
 }
 
 constexpr int TR_CHAIN = 4096;
@@ -499,10 +573,13 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     TR_CUDA(talloc(p, &d.o, nc3));
     TR_CUDA(talloc(p, &d.o2, nc3));
     TR_CUDA(talloc(p, &d.grid_state, (size_t)GRID_STATE_WORDS));
-    int blocks1 = 0;
-    TR_CUDA(coop_blocks(k_tr_steps<4>, TR_CAMS * 32, &p->step_grid));
-    TR_CUDA(coop_blocks(k_tr_steps<1>, TR_CAMS * 32, &blocks1));
-    p->step_grid = std::min(p->step_grid, blocks1);
+    p->step_grid = INT_MAX;
+    for (auto kernel : {k_tr_steps<1, false>, k_tr_steps<4, false>, k_tr_steps<1, true>, k_tr_steps<2, true>, k_tr_steps<4, true>}) {
+        int most = 0;
+        TR_CUDA(coop_blocks(kernel, TR_CAMS * 32, &most));
+        p->step_grid = std::min(p->step_grid, most);
+    }
+    for (int k = 0; k < n_cams; ++k) p->chunks = std::max(p->chunks, (cam_off[k + 1] - cam_off[k] + 31) / 32);
     TR_CUDA(talloc(p, &d.m, nc3));
     TR_CUDA(talloc(p, &d.v, nc3));
     TR_CUDA(talloc(p, &d.pterm, (size_t)n_runs * n_pairs));
