@@ -117,7 +117,13 @@ struct Vec3 {
     }
     __device__ __forceinline__ double operator[](int a) const { return v[a]; }
 };
-__device__ __forceinline__ double dot(const Vec3 &u, const Vec3 &v) { return u[0] * v[0] + u[1] * v[1] + u[2] * v[2]; }
+// a0 b0 + a1 b1 + a2 b2. The roundings of this and of the other sums of products of the solves are spelled out: which
+// product of a sum the compiler contracts depends on the code around it, and the refinement behind the
+// initialisation amplifies a last bit.
+__device__ __forceinline__ double sum3(double a0, double b0, double a1, double b1, double a2, double b2) {
+    return __fma_rn(a2, b2, __fma_rn(a0, b0, __dmul_rn(a1, b1)));
+}
+__device__ __forceinline__ double dot(const Vec3 &u, const Vec3 &v) { return sum3(u[0], v[0], u[1], v[1], u[2], v[2]); }
 // component a of u x v
 __device__ __forceinline__ double cross(const Vec3 &u, const Vec3 &v, int a) {
     const double p = a == 0 ? u[1] : (a == 1 ? u[2] : u[0]), q = a == 0 ? v[2] : (a == 1 ? v[0] : v[1]);
@@ -165,7 +171,7 @@ __device__ __forceinline__ double sum_values(const double *val, int n, int lane)
 //   p = z + beta p (own camera, and recomputed for the neighbours, so no third phase), q = A p; p.q
 //   x += alpha p, r -= alpha q, z = M^-1 r with M the 3x3 diagonal blocks;               r.z
 // The first phase runs a warp per camera, with the relative rotations in registers from iteration
-// to iteration; what is left per camera runs in warp 0, a lane per component of each of the block's
+// to iteration; what is left per camera runs in one warp, a lane per component of each of the group's
 // cameras. It stops at a multiple of CG_CHUNK iterations, as soon as the preconditioned residual norm has fallen by tol.
 // Then the column is normalised; column 2 (axis 1) is orthogonalised to column 1 first and the
 // rotations [c1 c2 c1 x c2], their parameters and a fresh Adam state are written, unless a column
@@ -173,13 +179,20 @@ __device__ __forceinline__ double sum_values(const double *val, int n, int lane)
 // of which the two barriers take 2.5 us and the serial FP64 instructions of the phases most of the rest.)
 constexpr int CG_CHUNK = 32;
 
+// SINGLE: a group of 8 cameras a block, whose state stays in registers; otherwise (more than 2,432 cameras) the
+// state goes through memory and a block's warps take the per-camera work of its groups in turn. AHEAD: a
+// warp's next pairs are on their way while 32 are used: always without SINGLE, and with it where a camera has
+// more than 256 pairs (below, its registers cost what it gives). us a solve of both columns, one warp for all
+// groups and no reading ahead -> now: 3,000 cameras, 24 pairs each 24.9 -> 23.8 ms, 20,000 with 60 183 -> 169, with 120
+// 202 -> 176, 1,000 cameras, all pairs, 4.1 -> 3.4; 1,000 cameras with 24 4.4 -> 4.3 (z and p by plain loads,
+// behind the barrier's acquire, instead of from L2).
+template <bool SINGLE, bool AHEAD>
 __global__ void __launch_bounds__(RT_CAMS * 32, 2)
 k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, double tol) {
-    __shared__ double s_sum[RT_CAMS][3], s_rz[256], s_out;
+    __shared__ double s_sum[2][RT_CAMS][3], s_rz[256], s_out, s_alpha;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int stride = gridDim.x * RT_CAMS, k0 = blockIdx.x * RT_CAMS;
     const int groups = cam_blocks(t.n_cams), trees = (t.n_cams + 255) / 256;
-    const bool single = t.n_cams <= stride;
     if (axis == 1 && (*t.err & ERR_DEGENERATE)) return;   // column 1 vanished: leave the state as it is
     GridBarrier gb(t.grid_state, t.err);
     // The groups' sums lie in two rows of t.blk: r.z of the setup in one, p.q of the iterations in the other.
@@ -203,14 +216,14 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
     };
     auto mat_v = [&](const double *v, double *o) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) o[a] = M[3 * a] * v[0] + M[3 * a + 1] * v[1] + M[3 * a + 2] * v[2];
+        for (int a = 0; a < 3; ++a) o[a] = sum3(M[3 * a], v[0], M[3 * a + 1], v[1], M[3 * a + 2], v[2]);
     };
-    // a warp's sums over the pairs of its camera to s_sum[warp]
-    auto put_sums = [&](double (&s)[3]) {
+    // a warp's sums over the pairs of its camera to s_sum[half][warp]
+    auto put_sums = [&](double (&s)[3], int half) {
         const double mine = warp_sum_spread<3>(s, lane);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            if (lane == spread_lane(3, a)) s_sum[warp][a] = mine;
+            if (lane == spread_lane(3, a)) s_sum[half][warp][a] = mine;
     };
     // warp 0: a value per camera (in its first lane) summed over the group in camera order
     auto group_sum = [&](double mine) {
@@ -234,8 +247,8 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
 #pragma unroll
                 for (int a = 0; a < 3; ++a) s[a] += o[a];
             }
-            have = single && e_end - e_begin <= 32;
-            put_sums(s);
+            have = SINGLE && e_end - e_begin <= 32;
+            put_sums(s, 0);
         }
         __syncthreads();
         if (warp == 0) {
@@ -243,14 +256,14 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
             const bool on = cc < RT_CAMS && kc < t.n_cams;
             deg = on ? (double)(t.cam_off[kc + 1] - t.cam_off[kc]) : 1.0;
             ck = on ? t.col1[(size_t)kc * 3 + ca] : 0.0;
-            rk = on ? w_pair * s_sum[cc][ca] : 0.0;
+            rk = on ? w_pair * s_sum[0][cc][ca] : 0.0;
             // M = w_pair deg I + w_pen c c^T: M^-1 = (I - beta/(alpha + beta |c|^2) c c^T) / alpha
             const Vec3 cv(ck, base), rv(rk, base);
             al = w_pair * deg;
-            f = w_pen / (al + w_pen * dot(cv, cv));
+            f = w_pen / __fma_rn(w_pen, dot(cv, cv), al);
             y = 1.0 / al;
             const double cr = dot(cv, rv);
-            zk = quotient(rk - f * ck * cr, al, y);
+            zk = quotient(__fma_rn(-__dmul_rn(f, ck), cr, rk), al, y);
             const Vec3 zv(zk, base);
             const double rz = on && kc != 0 ? dot(rv, zv) : 0.0;
             xk = kc == 0 && ca == axis ? 1.0 : 0.0;
@@ -268,7 +281,7 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
             const double b = group_sum(rz);
             if (lane == 0) slot_setup[kb / RT_CAMS] = b;
         }
-        if (!single) __syncthreads();
+        if (!SINGLE) __syncthreads();
     }
     bool ok = true;
     if (warp == 0) {
@@ -285,92 +298,126 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
         for (int c = 0; c < CG_CHUNK; ++c) {
             const double *p_old = (c & 1) ? t.p2 : t.p;
             double *p_new = (c & 1) ? t.p : t.p2;
-            for (int kb = k0; kb < t.n_cams; kb += stride) {
-                const int k = kb + warp;
+            int turn = 0;   // the block's groups one after the other
+            for (int kb = k0; kb < t.n_cams; kb += stride, ++turn) {
+                const int k = kb + warp, half = SINGLE ? 0 : turn & 1;
                 if (k > 0 && k < t.n_cams) {
                     const int e_begin = t.cam_off[k], e_end = t.cam_off[k + 1];
                     double s[3] = {0.0, 0.0, 0.0}, o[3];
-                    for (int e = e_begin + lane; e < e_end; e += 32) {
-                        if (!have) load_entry(e);
-                        if (other == 0) continue;
-                        double vo[3];
+                    if (!AHEAD || have) {
+                        for (int e = e_begin + lane; e < e_end; e += 32) {
+                            if (!have) load_entry(e);
+                            if (other == 0) continue;
+                            double vo[3];
 #pragma unroll
-                        for (int a = 0; a < 3; ++a)
-                            vo[a] = __ldcg(t.z + (size_t)other * 3 + a) + beta * __ldcg(p_old + (size_t)other * 3 + a);
-                        mat_v(vo, o);
-                        if (have) {   // the warp's only chunk
+                            for (int a = 0; a < 3; ++a)
+                                vo[a] = __fma_rn(beta, p_old[(size_t)other * 3 + a], t.z[(size_t)other * 3 + a]);
+                            mat_v(vo, o);
+                            if (have) {   // the warp's only chunk
 #pragma unroll
-                            for (int a = 0; a < 3; ++a) s[a] = o[a];
-                        } else {
+                                for (int a = 0; a < 3; ++a) s[a] = o[a];
+                            } else {
+#pragma unroll
+                                for (int a = 0; a < 3; ++a) s[a] += o[a];
+                            }
+                        }
+                    } else {
+                        if (e_begin + lane < e_end) load_entry(e_begin + lane);
+                        for (int e = e_begin + lane; e < e_end; e += 32) {
+                            double A[9], vo[3];
+                            const int cam = other;
+#pragma unroll
+                            for (int q = 0; q < 9; ++q) A[q] = M[q];
+                            if (e + 32 < e_end) load_entry(e + 32);
+                            if (cam == 0) continue;
+#pragma unroll
+                            for (int a = 0; a < 3; ++a)
+                                vo[a] = __fma_rn(beta, p_old[(size_t)cam * 3 + a], t.z[(size_t)cam * 3 + a]);
+#pragma unroll
+                            for (int a = 0; a < 3; ++a) o[a] = sum3(A[3 * a], vo[0], A[3 * a + 1], vo[1], A[3 * a + 2], vo[2]);
 #pragma unroll
                             for (int a = 0; a < 3; ++a) s[a] += o[a];
                         }
                     }
-                    put_sums(s);
+                    put_sums(s, half);
                 }
                 __syncthreads();
-                if (warp == 0) {
+                // the block's groups in turn by its warps, each while the others go on to the next group
+                // (whose sums take the other half: this half is written again two barriers on)
+                if (warp == (SINGLE ? 0 : turn % RT_CAMS)) {
                     const int kc = kb + cc;
                     const bool on = cc < RT_CAMS && kc > 0 && kc < t.n_cams;
                     const size_t o3 = (size_t)(on ? kc : 0) * 3 + ca;
-                    if (!single) {
+                    if (!SINGLE) {
                         deg = on ? (double)(t.cam_off[kc + 1] - t.cam_off[kc]) : 0.0;
                         ck = on ? t.col1[o3] : 0.0;
-                        zk = on ? t.z[o3] : 0.0;
-                        pk = on ? p_old[o3] : 0.0;
+                        zk = on ? __ldcg(t.z + o3) : 0.0;
+                        pk = on ? __ldcg(p_old + o3) : 0.0;
                     }
-                    pk = zk + beta * pk;
-                    const double sk = on ? s_sum[cc][ca] : 0.0;
+                    pk = __fma_rn(beta, pk, zk);
+                    const double sk = on ? s_sum[half][cc][ca] : 0.0;
                     const Vec3 pv(pk, base);
                     const double cp = dot(Vec3(ck, base), pv);
-                    qk = w_pair * (deg * pk - sk) + w_pen * ck * cp;
+                    // w_pair (deg p - s) + w_pen c (c.p)
+                    qk = __fma_rn(w_pair, __fma_rn(deg, pk, -sk), __dmul_rn(__dmul_rn(w_pen, ck), cp));
                     const double pq = dot(Vec3(qk, base), pv);
                     if (on) {
                         p_new[o3] = pk;
-                        if (!single) t.q[o3] = qk;
+                        if (!SINGLE) t.q[o3] = qk;
                     }
                     const double b = group_sum(on ? pq : 0.0);
                     if (lane == 0) slot[kb / RT_CAMS] = b;
                 }
-                if (!single) __syncthreads();
             }
+            if (!SINGLE) __syncthreads();   // every warp's groups are written
             double y_rz = 0.0;   // for the quotient behind the second sum, while warp 0 is at the first
             if (warp != 0) y_rz = 1.0 / rz;
+            double alpha = 0.0;
             if (warp == 0) {
                 gb.arrive();
                 ok = gb.wait();
                 const double pq = sum_values(slot, groups, lane);
                 // (the shuffle keeps the division out of the divergent code below)
-                const double alpha = __shfl_sync(0xffffffffu, pq > 0.0 ? rz / pq : 0.0, 0);
-                for (int kb = k0; kb < t.n_cams; kb += stride) {
-                    const int kc = kb + cc;
-                    const bool on = cc < RT_CAMS && kc > 0 && kc < t.n_cams;
-                    const size_t o3 = (size_t)(on ? kc : 0) * 3;
-                    if (!single) {
-                        al = on ? t.pre[o3] : 1.0;
-                        y = on ? t.pre[o3 + 1] : 1.0;
-                        f = on ? t.pre[o3 + 2] : 0.0;
-                        ck = on ? t.col1[o3 + ca] : 0.0;
-                        xk = on ? t.x[o3 + ca] : 0.0;
-                        rk = on ? t.r[o3 + ca] : 0.0;
-                        pk = on ? p_new[o3 + ca] : 0.0;
-                        qk = on ? t.q[o3 + ca] : 0.0;
-                    }
-                    xk += alpha * pk;
-                    rk = rk - alpha * qk;
-                    const Vec3 rv(rk, base);
-                    const double cr = dot(Vec3(ck, base), rv);
-                    zk = quotient(rk - f * ck * cr, al, y);
-                    const double rzk = dot(rv, Vec3(zk, base));
-                    if (on) {
-                        t.z[o3 + ca] = zk;
-                        if (ca == 0) cam_rz[kc] = rzk;
-                        if (!single) {
-                            t.x[o3 + ca] = xk;
-                            t.r[o3 + ca] = rk;
-                        }
+                alpha = __shfl_sync(0xffffffffu, pq > 0.0 ? rz / pq : 0.0, 0);
+                if (!SINGLE && lane == 0) s_alpha = alpha;
+            }
+            if (!SINGLE) {
+                __syncthreads();
+                alpha = s_alpha;
+            }
+            turn = 0;
+            for (int kb = k0; kb < t.n_cams; kb += stride, ++turn) {
+                if (warp != (SINGLE ? 0 : turn % RT_CAMS)) continue;
+                const int kc = kb + cc;
+                const bool on = cc < RT_CAMS && kc > 0 && kc < t.n_cams;
+                const size_t o3 = (size_t)(on ? kc : 0) * 3;
+                if (!SINGLE) {
+                    al = on ? t.pre[o3] : 1.0;
+                    y = on ? t.pre[o3 + 1] : 1.0;
+                    f = on ? t.pre[o3 + 2] : 0.0;
+                    ck = on ? t.col1[o3 + ca] : 0.0;
+                    xk = on ? t.x[o3 + ca] : 0.0;
+                    rk = on ? t.r[o3 + ca] : 0.0;
+                    pk = on ? p_new[o3 + ca] : 0.0;
+                    qk = on ? t.q[o3 + ca] : 0.0;
+                }
+                xk = __fma_rn(alpha, pk, xk);
+                rk = __fma_rn(-alpha, qk, rk);
+                const Vec3 rv(rk, base);
+                const double cr = dot(Vec3(ck, base), rv);
+                zk = quotient(__fma_rn(-__dmul_rn(f, ck), cr, rk), al, y);
+                const double rzk = dot(rv, Vec3(zk, base));
+                if (on) {
+                    t.z[o3 + ca] = zk;
+                    if (ca == 0) cam_rz[kc] = rzk;
+                    if (!SINGLE) {
+                        t.x[o3 + ca] = xk;
+                        t.r[o3 + ca] = rk;
                     }
                 }
+            }
+            if (!SINGLE) __syncthreads();
+            if (warp == 0) {
                 gb.arrive();
                 ok = gb.wait() && ok;
             }
@@ -404,7 +451,7 @@ k_cg_solve(DevRot t, int axis, double w_pair, double w_pen, int max_iters, doubl
         t.scal[4 * axis + 2] = (double)it;
     }
     if (warp != 0) return;
-    if (single && cc < RT_CAMS && k0 + cc > 0 && k0 + cc < t.n_cams) t.x[(size_t)(k0 + cc) * 3 + ca] = xk;
+    if (SINGLE && cc < RT_CAMS && k0 + cc > 0 && k0 + cc < t.n_cams) t.x[(size_t)(k0 + cc) * 3 + ca] = xk;
     __syncwarp();
     if (lane >= RT_CAMS) return;
     for (int k = k0 + lane; k < t.n_cams; k += stride) {
@@ -805,6 +852,7 @@ struct fm_rotation {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     double *grad6 = nullptr;
     int step_grid = 0, cg_grid = 0;       // blocks of the persistent kernels
+    void (*cg_solve)(DevRot, int, double, double, int, double) = nullptr;   // the instantiation for the graph
     std::vector<void *> allocs;
     int cg_iters_last = 0;
     double cg_resid_last = 0.0;
@@ -934,7 +982,15 @@ fm_status create_rot(fm_rotation *p, int32_t n_cams, int32_t n_pairs, const int3
     RT_CUDA(ralloc(p, &d.v, 6 * nc));
     RT_CUDA(ralloc(p, &d.pgrad, 18 * (size_t)n_pairs));
     RT_CUDA(ralloc(p, &d.pdist, (size_t)n_pairs));
-    RT_CUDA(coop_blocks(k_cg_solve, RT_CAMS * 32, &p->cg_grid));
+    int most_pairs = 0, most_blocks = 0;
+    for (int k = 0; k < n_cams; ++k) most_pairs = std::max(most_pairs, cam_off[k + 1] - cam_off[k]);
+    p->cg_solve = most_pairs > 256 ? k_cg_solve<true, true> : k_cg_solve<true, false>;
+    RT_CUDA(coop_blocks(p->cg_solve, RT_CAMS * 32, &most_blocks));
+    if (cam_blocks(n_cams) > most_blocks) {
+        p->cg_solve = k_cg_solve<false, true>;
+        RT_CUDA(coop_blocks(p->cg_solve, RT_CAMS * 32, &most_blocks));
+    }
+    p->cg_grid = most_blocks;
     RT_CUDA(coop_blocks(k_rot_steps, RT_CAMS * 32, &p->step_grid));
     p->cg_grid = std::min(p->cg_grid, cam_blocks(n_cams));
     p->step_grid = std::min(p->step_grid, std::max(cam_blocks(n_cams), (n_pairs + 63) / 64));
@@ -1064,9 +1120,9 @@ FM_API fm_status fm_rotation_initialize(fm_rotation *p, int32_t *cg_iters, doubl
     // column 1: sum ||x_j - R_p x_i||^2, anchored x_0 = e1; column 2: (1/|P|) sum ||y_j - R_p y_i||^2 +
     // (1/N) sum (x_k^T y_k)^2, anchored y_0 = e2
     RT_CUDA(cudaMemsetAsync(p->d.scal, 0, sizeof(double) * 8, p->s));
-    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 0, 1.0, 0.0, (int)p->opt.cg_max_iters,
+    RT_CUDA(launch_coop(p->cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 0, 1.0, 0.0, (int)p->opt.cg_max_iters,
                         p->opt.cg_tol));
-    RT_CUDA(launch_coop(k_cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 1, 1.0 / n_pairs, 1.0 / n_cams,
+    RT_CUDA(launch_coop(p->cg_solve, p->cg_grid, RT_CAMS * 32, 0, p->s, p->d, 1, 1.0 / n_pairs, 1.0 / n_cams,
                         (int)p->opt.cg_max_iters, p->opt.cg_tol));
     double sc[8] = {};
     RT_CUDA(cudaMemcpyAsync(sc, p->d.scal, sizeof sc, cudaMemcpyDeviceToHost, p->s));
