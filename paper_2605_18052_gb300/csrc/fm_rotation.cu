@@ -999,14 +999,12 @@ fm_status create_rot(fm_rotation *p, int32_t n_cams, int32_t n_pairs, const int3
     RT_CUDA(ralloc(p, &d.loss, 1));
     RT_CUDA(ralloc(p, &d.hyper, 4));
     RT_CUDA(ralloc(p, &d.step, 1));
-    RT_CUDA(ralloc(p, &d.x, 3 * nc));
-    RT_CUDA(ralloc(p, &d.r, 3 * nc));
-    RT_CUDA(ralloc(p, &d.z, 3 * nc));
-    RT_CUDA(ralloc(p, &d.p, 3 * nc));
-    RT_CUDA(ralloc(p, &d.p2, 3 * nc));
-    RT_CUDA(ralloc(p, &d.q, 3 * nc));
-    RT_CUDA(ralloc(p, &d.pre, 3 * nc));
-    RT_CUDA(ralloc(p, &d.cam_rz, nc));
+    RT_CUDA(ralloc(p, &d.x, 22 * nc));   // the vectors of the solves in one allocation
+    {
+        double **part[] = {&d.r, &d.z, &d.p, &d.p2, &d.q, &d.pre, &d.cam_rz};
+        double *at = d.x;
+        for (double **v : part) *v = at += 3 * nc;
+    }
     RT_CUDA(ralloc(p, &d.col1, 3 * nc));
     RT_CUDA(ralloc(p, &d.col2, 3 * nc));
     RT_CUDA(ralloc(p, &p->grad6, 6 * nc));

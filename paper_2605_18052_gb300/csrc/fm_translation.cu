@@ -570,9 +570,10 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     d.cam_off = co;
     d.cam_ent = ce;
     TR_CUDA(talloc(p, &d.oij, (size_t)n_pairs));
-    TR_CUDA(talloc(p, &d.o, nc3));
-    TR_CUDA(talloc(p, &d.o2, nc3));
-    TR_CUDA(talloc(p, &d.grid_state, (size_t)GRID_STATE_WORDS));
+    TR_CUDA(talloc(p, &d.o, 2 * nc3));
+    d.o2 = d.o + nc3;
+    TR_CUDA(talloc(p, &d.err, 1 + (size_t)GRID_STATE_WORDS));
+    d.grid_state = d.err + 1;
     p->step_grid = INT_MAX;
     for (auto kernel : {k_tr_steps<1, false>, k_tr_steps<4, false>, k_tr_steps<1, true>, k_tr_steps<2, true>, k_tr_steps<4, true>}) {
         int most = 0;
@@ -590,7 +591,6 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
     TR_CUDA(talloc(p, &d.stats, 4 * (size_t)n_runs));
     TR_CUDA(talloc(p, &d.hyper, 4));
     TR_CUDA(talloc(p, &d.step, 1));
-    TR_CUDA(talloc(p, &d.err, 1));
     TR_CUDA(cudaMallocAsync(&Rd, sizeof(double) * 9 * n_cams, p->s));
     TR_CUDA(cudaMallocAsync(&td, sizeof(double) * 3 * n_pairs, p->s));
     TR_CUDA(cudaMemcpyAsync(ci, cam_i, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
