@@ -399,7 +399,7 @@ typedef struct {
     double beta1;       /* 0.9 */
     double beta2;       /* 0.999 */
     double adam_eps;    /* 1e-12 */
-    int32_t use_graph;  /* 1: replay CUDA graphs of chained iterations */
+    int32_t use_graph;  /* 0 or 1, without effect: a call's iterations are one launch */
     int32_t reserved;
 } fm_translation_options;
 
@@ -456,7 +456,7 @@ typedef struct {
     double adam_eps;      /* 1e-12 */
     double cg_tol;        /* stop when the preconditioned residual norm falls by this factor (1e-9) */
     int32_t cg_max_iters; /* per column system (20000) */
-    int32_t use_graph;    /* 1: replay CUDA graphs of chained iterations */
+    int32_t use_graph;    /* 0 or 1, without effect: a call's iterations are one launch */
 } fm_rotation_options;
 
 FM_API void fm_rotation_default_options(fm_rotation_options *opt);

@@ -53,7 +53,7 @@ struct fm_problem {
     std::vector<char> host_params;        // R, c and the error word as they come from the device (read_params)
     int hist_valid = 0;                   // d.le_hist holds a previous reweighting's residuals
     double lr_focal = 1e-3;               // Adam step size of rho = log(f0/f)
-    bool quad_alloc = false;              // d.qslots, d.quad, d.pair_rec allocated
+    bool quad_alloc = false;              // d.qslots, d.quad, d.grid_state allocated
     bool quad_valid = false;              // d.quad holds the form of the current weights
     bool quad_persistent = false;         // the cameras fit the persistent steps on the form
     cudaGraphExec_t qgraph = nullptr, qgraph8 = nullptr;  // quadratic-path iterations
@@ -399,7 +399,6 @@ fm_status create_impl(fm_problem *p, int32_t n_cams, const double *R, const doub
     d.w = w;
     d.pstat = reinterpret_cast<float *>(ps);
     d.perm = nullptr;
-    d.fbuf = nullptr;
 
     FM_CUDA(cudaMemsetAsync(d.err, 0, (char *)d.geo - (char *)d.err, p->s));
     FM_CUDA(cudaMemcpyAsync(d.cam_i, cam_i, sizeof(int) * n_pairs, cudaMemcpyHostToDevice, p->s));
@@ -791,7 +790,7 @@ FM_API fm_status fm_step_learned(fm_problem *p, const fm_mlp *net, double tau, d
     if (ts) time_end(p, FM_PASS_PAIR_STATS, p->s);
     const bool tl = time_begin(p, FM_PASS_LEARNED_LOSS, p->s);
     launch_learned_loss(p->d, master, wbf, (float)tau, std::isinf(tau_cap) ? INFINITY : (float)tau_cap, round,
-                        p->hist_valid, p->s, false);
+                        p->hist_valid, p->s);
     if (tl) time_end(p, FM_PASS_LEARNED_LOSS, p->s);
     launch_camera_step(p->d, true, p->d.cam_alt, p->s, !tl);
     launch_finalize(p->d, 1, p->d.cam_alt, false, p->s, !tl);

@@ -26,15 +26,16 @@ constexpr int PG = 16;             // floats per pair gradient record
 constexpr float COORD_LIMIT = 8.0f;  // |normalized coordinate| bound (fixed-point centroids)
 constexpr int FIXED_SHIFT = 32;    // centroid sums use trunc(x * 2^32) in int64
 
-// geometry record of pair n (written by pair_setup, read by the streaming and combine kernels)
+// geometry of pair n: a record in memory (written by pair_setup, read by the once-per-round passes, the
+// form's anchor and the combine kernel), the same 40 floats in registers or shared memory where a kernel forms
+// them itself from the camera records (the streaming pass, the camera step, the steps on the form)
 //   [0..8]  E'_n = T_j^T E_n T_i (centroid-folded essential matrix, row-major)
 //   [9..17] R_n = R_j R_i^T
 //   [18..20] t_n = R_j (c_i - c_j)
 //   [21] 1/|t_n|, [22..23] centroid of image i, [33..34] centroid of image j
-//   [24..32] R_j (the second camera's rotation, so the per-camera step never reads another
-//            camera's record while that record is being updated)
-// camera record k (written by the per-camera step kernel)
-//   [0..8] R_k (FP32), [9..11] c_k high part, [12..14] c_k low part (c = hi + lo), [15] 0
+//   [24..32] R_j (the second camera's rotation), [35..36] keypoint scales of the two images, [37..39] 0
+// camera record k (written by the step kernels)
+//   [0..8] R_k (FP32), [9..11] c_k high part, [12..14] c_k low part (c = hi + lo), [15] keypoint scale
 // pair gradient record n: [0..2] g_phi_i, [3..5] g_c_i, [6..8] g_phi_j, [9..11] g_c_j, [12] loss
 
 enum StreamMode { MODE_LOSS_IRLS = 0, MODE_LOSS_L1 = 1 };
@@ -79,7 +80,6 @@ struct DevProblem {
     double *grad, *loss_out;
     unsigned *err;
     unsigned long long *counter;
-    float *fbuf;            // n_pad floats of scratch (residual export)
     // learned inlier weights
     __half *score;          // per point pair: matcher confidence (0.5 until set)
     __half *le_hist;        // per point pair: log(|eps| + 1e-6) at the previous reweighting
@@ -133,7 +133,7 @@ void launch_collect_features(const DevProblem &d, float tau, int round, int hist
                              __nv_bfloat16 *feat_input_order, cudaStream_t s);
 // the learned reweighting fused with the loss + adjoint pass (slots, weights, history, kept count)
 void launch_learned_loss(const DevProblem &d, const float *mlp_master, const __nv_bfloat16 *mlp_bf16, float tau,
-                         float tau_cap, int round, int hist_valid, cudaStream_t s, bool pdl);
+                         float tau_cap, int round, int hist_valid, cudaStream_t s);
 
 // ---- kernels launched by the API layer (fm_kernels.cu) ----------------------------------------
 void launch_cam_prep(const DevProblem &d, cudaStream_t s);
@@ -142,8 +142,9 @@ void launch_begin_round(const DevProblem &d, double tau, cudaStream_t s);      /
 void launch_set_params(const DevProblem &d, const double *R, const double *c, cudaStream_t s);
 cudaError_t launch_pose_gradient(int n_cams, const double *grad, const double *R, const double *scale, double *gR,
                                  double *gc, cudaStream_t s);
-// pdl: launch with programmatic stream serialisation (overlaps the predecessor's tail)
-void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl = false);
+// geometry records of all image pairs
+void launch_pair_setup(const DevProblem &d, cudaStream_t s);
+// pdl (here and below): launch with programmatic stream serialisation (overlaps the predecessor's tail)
 // loss total of the last camera step and `count` added to the step count (loss_copy: also written to the
 // caller's device memory); camera records copied back from copy_src if not null; check: image pairs that
 // the new poses make degenerate are reported
@@ -161,12 +162,11 @@ void launch_stream_loss(const DevProblem &d, cudaStream_t s, bool pdl = false, b
 void launch_stream_reweight(const DevProblem &d, cudaStream_t s, bool pdl = false);
 void launch_combine(const DevProblem &d, cudaStream_t s);
 void launch_gather(const DevProblem &d, bool count_step, cudaStream_t s);
-// fused per-camera step: combine this camera's pair partials, chain rule, FP64 sum, Adam,
-// exponential map, camera record; the last block sums the loss and advances the step count
 // Adam step of every camera with the gradient in d.grad (FP64, n_cams x 6); advances the step
 void launch_apply_gradient(const DevProblem &d, cudaStream_t s);
-// apply = false computes the gradient and loss only; apply: the new camera records go to cam_dst, another
-// buffer than d.cam
+// per-camera step: this camera's partial sums, chain rule, compensated sum, Adam, exponential map, camera
+// record. apply = false: the gradient and loss only; apply: the new camera records go to cam_dst, another
+// buffer than d.cam. The next kernel finishes the loss total and the step count
 void launch_camera_step(const DevProblem &d, bool apply, float *cam_dst, cudaStream_t s, bool pdl = false);
 void launch_irls_weights(const DevProblem &d, float tau, cudaStream_t s);
 void launch_residuals(const DevProblem &d, float *out_input_order, cudaStream_t s);

@@ -1,14 +1,14 @@
 // Per-iteration kernels of the epipolar adjustment (Sec. "Epipolar Adjustment").
 //
-//   cam_prep    per camera : FP64 pose -> FP32 camera record (R_k, c_k as hi + lo)
-//   pair_setup  per pair   : R_n, t_n, 1/|t_n| and the centroid-folded essential matrix E'_n
-//   stream_loss per range  : epsilon = o2^T E'_n o1 for every point pair, the loss term and
-//                            the adjoint G'_n += s * o2 o1^T, segmented per image pair
-//   combine     per pair   : sum the range partials (Kahan), unfold centroids, chain rule to
-//                            the two cameras of the pair
-//   gather      per camera : FP64 sum of the pair contributions (fixed order) + FP64 loss sum
-//   adam        per camera : FP64 Adam step, R_k <- Exp(phi_k) R_k, Gram-Schmidt on rows
-//   irls_weights / residuals: the same streaming walk writing one value per point pair
+//   stream_loss per range  : E'_n of the range's pairs from the camera records, epsilon = o2^T E'_n o1 for
+//                            every point pair, the loss term and the adjoint G'_n += s * o2 o1^T, segmented
+//                            per image pair (stream_reweight: with the round's IRLS weights)
+//   camera_step per camera : chain rule of its pairs' partial sums, compensated sum, Adam, R_k <- Exp(phi_k) R_k,
+//                            the new camera record
+//   finalize    per chain  : loss total, step count, camera records back in their first buffer
+// Once per round or call: cam_prep (camera records from the poses), pair_setup (geometry records of the
+// pairs), irls_weights / residuals (the streaming walk writing one value per point pair). combine and gather: the
+// chain rule per pair and its sums per camera, for the evaluation without allocation.
 #include <math.h>
 
 #include <algorithm>
@@ -221,10 +221,7 @@ __global__ void k_pose_gradient(int n_cams, const double *grad, const double *R,
 
 __global__ void __launch_bounds__(256) k_pair_setup(DevProblem d) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = n < d.n_pairs ? d.cam_i[n] : 0, j = n < d.n_pairs ? d.cam_j[n] : 0;
-    pdl_wait();     // camera records of the previous step
-    pdl_trigger();
-    if (n < d.n_pairs) pair_geometry(d, n, i, j);
+    if (n < d.n_pairs) pair_geometry(d, n, d.cam_i[n], d.cam_j[n]);
 }
 
 // ---- per pair: combine partials and chain rule ----------------------------------------------------
@@ -574,8 +571,8 @@ void launch_cam_prep(const DevProblem &d, cudaStream_t s) {
     k_cam_prep<<<blocks_for(d.n_cams, 128), 128, 0, s>>>(d);
 }
 
-void launch_pair_setup(const DevProblem &d, cudaStream_t s, bool pdl) {
-    launch_k(k_pair_setup, dim3(blocks_for(d.n_pairs, 256)), dim3(256), s, pdl, d);
+void launch_pair_setup(const DevProblem &d, cudaStream_t s) {
+    k_pair_setup<<<blocks_for(d.n_pairs, 256), 256, 0, s>>>(d);
 }
 
 void launch_set_hyper(const DevProblem &d, const double *h, cudaStream_t s) {

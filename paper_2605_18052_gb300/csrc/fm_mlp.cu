@@ -275,7 +275,8 @@ k_collect_features(DevProblem d, float tau, int round, int hist_valid, __nv_bflo
 // instructions per point pair; the tensor pipe is 62% busy (8.3 cycles per mma.sync and
 // sub-partition: 415 us on 48.9 M if it never waited), the rest is the latency of a block's phases with
 // four warps per sub-partition. Two tiles interleaved by hand, with 4 or 3 blocks per SM, changed
-// nothing (619, 637 us); 5 blocks spill (818 us).
+// nothing (619, 637 us); 5 blocks an SM spill far more (818 us; at 4, 128 registers, the fused
+// variants spill 28 bytes).
 constexpr int LP_WARPS = 4;
 constexpr int LP_BLOCK = 64;                // point pairs per warp and step
 constexpr int LP_STAGES = 4;                // steps whose loads are in flight
@@ -293,8 +294,7 @@ k_learned_pass(DevProblem d, const float *master, const __nv_bfloat16 *wbf, floa
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 3;
     NetFrag net;
     net.load(master, wbf, lane);
-    pdl_wait();     // pair geometry and statistics of this pass
-    pdl_trigger();
+    pdl_trigger();   // the camera step behind the fused pass may be scheduled
     const int r = blockIdx.x * LP_WARPS + warp;
     if (r >= d.n_ranges) return;
     const float log_tau = __logf(tau), delta = (float)d.delta, wscale = d.w_scale, round_f = round * 0.1f;
@@ -479,12 +479,12 @@ k_learned_pass(DevProblem d, const float *master, const __nv_bfloat16 *wbf, floa
 static inline int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 void launch_learned_loss(const DevProblem &d, const float *master, const __nv_bfloat16 *wbf, float tau,
-                         float tau_cap, int round, int hist_valid, cudaStream_t s, bool pdl) {
+                         float tau_cap, int round, int hist_valid, cudaStream_t s) {
     const dim3 grid(blocks_for(d.n_ranges, LP_WARPS)), block(LP_WARPS * 32);
     if (d.storage == FM_STORE_FP32)
-        launch_k(k_learned_pass<FM_STORE_FP32, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
+        k_learned_pass<FM_STORE_FP32, true><<<grid, block, 0, s>>>(d, master, wbf, tau, tau_cap, round, hist_valid);
     else
-        launch_k(k_learned_pass<FM_STORE_FP16, true>, grid, block, s, pdl, d, master, wbf, tau, tau_cap, round, hist_valid);
+        k_learned_pass<FM_STORE_FP16, true><<<grid, block, 0, s>>>(d, master, wbf, tau, tau_cap, round, hist_valid);
 }
 
 void launch_pair_stats(const DevProblem &d, float tau, cudaStream_t s) {
@@ -499,9 +499,9 @@ void launch_learned_weights(const DevProblem &d, const float *master, const __nv
                             float tau_cap, int round, int hist_valid, cudaStream_t s) {
     const dim3 grid(blocks_for(d.n_ranges, LP_WARPS)), block(LP_WARPS * 32);
     if (d.storage == FM_STORE_FP32)
-        launch_k(k_learned_pass<FM_STORE_FP32, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
+        k_learned_pass<FM_STORE_FP32, false><<<grid, block, 0, s>>>(d, master, wbf, tau, tau_cap, round, hist_valid);
     else
-        launch_k(k_learned_pass<FM_STORE_FP16, false>, grid, block, s, false, d, master, wbf, tau, tau_cap, round, hist_valid);
+        k_learned_pass<FM_STORE_FP16, false><<<grid, block, 0, s>>>(d, master, wbf, tau, tau_cap, round, hist_valid);
 }
 
 void launch_collect_features(const DevProblem &d, float tau, int round, int hist_valid,

@@ -175,7 +175,7 @@ __device__ __forceinline__ double sum_values(const double *val, int n, int lane)
 // cameras. It stops at a multiple of CG_CHUNK iterations, as soon as the preconditioned residual norm has fallen by tol.
 // Then the column is normalised; column 2 (axis 1) is orthogonalised to column 1 first and the
 // rotations [c1 c2 c1 x c2], their parameters and a fresh Adam state are written, unless a column
-// vanished. (As five launches an iteration this took 22 us an iteration on 1,000 cameras; 9.7 us now,
+// vanished. (As five launches an iteration this took 22 us an iteration on 1,000 cameras; 9 us now,
 // of which the two barriers take 2.5 us and the serial FP64 instructions of the phases most of the rest.)
 constexpr int CG_CHUNK = 32;
 

@@ -10,7 +10,7 @@
 namespace fm {
 
 // ---- programmatic dependent launch --------------------------------------------------------------
-// The three kernels of an optimiser iteration are launched with programmatic stream
+// The two kernels of an optimiser iteration (the pass and the camera step) are launched with programmatic stream
 // serialisation, so a kernel's CTAs can be scheduled while its predecessor drains. Every kernel
 // waits (griddepcontrol.wait) before it reads anything its predecessor writes, and lets its own
 // dependents launch (griddepcontrol.launch_dependents) only after that wait: when a kernel
@@ -142,8 +142,8 @@ __device__ __forceinline__ float irls_weight(float a, float delta) { return __fd
 
 // ---- per pair: relative pose and folded essential matrix ------------------------------------------
 // camera record: R (9), centre as hi (3) + lo (3) floats, s = scale of the normalised keypoints.
-// Read at L2 (ld.global.cg): a record may have been written by another block of the same
-// launch (the camera step's geometry phase), and L1 is not coherent across SMs.
+// Read at L2 (ld.global.cg): in the persistent steps on the quadratic form a record was written by
+// another block of the same launch, and L1 is not coherent across SMs.
 __device__ __forceinline__ void load_camrec(const float *rec, float *R, float *hi, float *lo, float &s) {
     const float4 *v = reinterpret_cast<const float4 *>(rec);
     const float4 a = __ldcg(v), b = __ldcg(v + 1), c = __ldcg(v + 2), e = __ldcg(v + 3);
@@ -235,14 +235,9 @@ __device__ __forceinline__ bool pair_geometry_regs(const float *cam, const float
 }
 
 // the geometry record of pair n = (i, j) at the current camera records, written to d.geo
-// (E_out, optional, receives E'_n as well)
-__device__ __forceinline__ void pair_geometry(const DevProblem &d, int n, int i, int j, float *E_out = nullptr) {
+__device__ __forceinline__ void pair_geometry(const DevProblem &d, int n, int i, int j) {
     float g[GEO];
     if (!pair_geometry_regs(d.cam, d.cen, i, j, g)) atomicOr(d.err, ERR_DEGENERATE);
-    if (E_out) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) E_out[k] = g[k];
-    }
     float4 *out = reinterpret_cast<float4 *>(d.geo + (size_t)n * GEO);
 #pragma unroll
     for (int k = 0; k < GEO / 4; ++k) out[k] = make_float4(g[4 * k], g[4 * k + 1], g[4 * k + 2], g[4 * k + 3]);
