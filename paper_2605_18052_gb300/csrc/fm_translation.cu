@@ -163,17 +163,17 @@ constexpr int TR_RC = 8;       // most runs of an item
 // 806 -> 577, 5,000 with 80 2,444 -> 1,762; as two launches 778, 1,040, 2,058).
 
 // PAIRS: a first phase, with a grid barrier behind it, evaluates every pair once, a thread per pair and batch of
-// runs, and the cameras' lanes read the terms. Without it a warp evaluates its camera's pairs 32 at a time, one
-// run after the other, so a camera of many pairs holds up the grid. The phase is taken where more than
-// TR_SERIES such evaluations are in series (rounds of items x runs of an item x 32s of pairs of the largest camera),
-// unless they are the runs of one item, whose loads overlap. us an iteration without / with it, (as two
-// launches):
-//   1: 1,000 cameras, 16 pairs each 3.4 / 5.1 (8.0)     4: 1,000 cameras, 120 pairs each 7.4 / 7.4 (9.7)
-//   2: 3,000 cameras, 24 pairs each 6.9 / 7.3 (11.5)    4: 1,000 cameras, 48 pairs each, 4 runs 9.7 / 8.0 (16.3)
-//   5: 150 cameras, all pairs 8.7 / 7.1 (8.3)           6: 5,000 cameras, 48 pairs each 14.1 / 11.8 (20.4)
-//   10: 300 cameras, all pairs 15.2 / 7.2 (10.1)        157: 5,000 cameras, one in all pairs 175 / 16.8 (34.9)
-//   56: 5,000 cameras, 200 pairs each, 8 runs 159 / 94 (132)
-constexpr int TR_SERIES = 4;
+// runs, and the cameras' lanes read the terms. Without it a warp evaluates its camera's pairs 32 at a time, the
+// runs of its item each time, so a camera of many pairs holds up the grid. The phase is taken (pairs_first)
+// where a warp makes more than 4 such passes with one run or more than 1.5 with several (which take the
+// registers and loads of four), on the average camera, or the largest camera alone more than 4 or 3. us an
+// iteration without / with it (as two launches):
+//   one run, passes: 1: 1,000 cameras, 16 pairs each 3.4 / 5.1 (8.0); 2: 3,000 cameras, 24 each 6.9 / 7.3 (11.5); 4: 1,000
+//     cameras, 120 each 7.4 / 7.4 (9.7); 5: 150 cameras, all pairs 8.7 / 7.1 (8.3); 6: 5,000 cameras, 48 each 14.1 / 11.8
+//     (20.4); 10: 300 cameras, all pairs 15.2 / 7.2 (10.1); the largest 157: 5,000 cameras, one in all pairs 175 / 16.8 (34.9)
+//   several runs: 1: 1,000 cameras, 16 each, 8 runs 7.6 / 10.4 (21.4); 1.1, the largest 2: 1,000 cameras, 23 each, 8 runs
+//     7.7 / 8.1 (21.5); 2: 1,000 cameras, 48 each, 3 runs 8.9 / 7.9 (12.4), 8 runs 12.1 / 11.5 (24.6); 21: 5,000 cameras, 200
+//     each, 8 runs 159 / 94 (132)
 
 template <int BATCH, bool PAIRS>
 __global__ void __launch_bounds__(TR_CAMS * 32, 2) k_tr_steps(DevTrans t, int iters, int rc) {
@@ -415,7 +415,8 @@ struct fm_translation {
     cudaStream_t s = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int step_grid = 0;       // most blocks of the step kernel
-    int chunks = 0;          // image pairs of the camera with the most, in warps' worth
+    int max_chunks = 0;      // image pairs of the largest camera and of the average one, in warps' worth
+    double mean_chunks = 0.0;
     std::vector<void *> allocs;
 };
 
@@ -479,6 +480,12 @@ void enqueue_eval(fm_translation *p) {
     launch_k(k_tr_cam, gc, dim3(TR_CAMS * 32), p->s, true, p->d);
 }
 
+// whether the step kernel evaluates the pairs in a phase of their own (why: at the kernel)
+bool pairs_first(const fm_translation *p, int rc, int rounds) {
+    const double mean = rounds * p->mean_chunks, largest = mean - p->mean_chunks + p->max_chunks;
+    return rc == 1 ? mean > 4.0 || largest > 4.0 : mean > 1.5 || largest > 3.0;
+}
+
 // items of rc runs each: as many as fit the resident blocks, so that few runs per block are in series (the next
 // rc where the uneven last items would make a nearly empty second round: 849 cameras, 7 runs, 321 items of 3
 // on 304 blocks 11.7 us an iteration, 214 of 4 7.5; 1,617 cameras, 4 runs, 12.2 -> 7.8)
@@ -492,8 +499,7 @@ cudaError_t enqueue_steps(fm_translation *p, int iters) {
         while (items_of(rc) > p->step_grid) ++rc;
     const int64_t items = items_of(rc), rounds = (items + p->step_grid - 1) / p->step_grid;
     int64_t blocks = items;
-    const int64_t passes = rounds * p->chunks;   // over a warp's pairs, rc runs each
-    const bool pairs = passes > 1 && passes * rc > TR_SERIES;
+    const bool pairs = pairs_first(p, rc, (int)rounds);
     const int batch = rc == 1 ? 1 : (pairs && rc == 2 ? 2 : 4);
     if (pairs) {
         const int64_t work = (int64_t)d.n_pairs * ((d.n_runs + batch - 1) / batch);
@@ -580,7 +586,11 @@ fm_status create_trans(fm_translation *p, int32_t n_cams, const double *R, int32
         TR_CUDA(coop_blocks(kernel, TR_CAMS * 32, &most));
         p->step_grid = std::min(p->step_grid, most);
     }
-    for (int k = 0; k < n_cams; ++k) p->chunks = std::max(p->chunks, (cam_off[k + 1] - cam_off[k] + 31) / 32);
+    for (int k = 0; k < n_cams; ++k) {
+        const int chunks = (cam_off[k + 1] - cam_off[k] + 31) / 32;
+        p->max_chunks = std::max(p->max_chunks, chunks);
+        p->mean_chunks += chunks / (double)n_cams;
+    }
     TR_CUDA(talloc(p, &d.m, nc3));
     TR_CUDA(talloc(p, &d.v, nc3));
     TR_CUDA(talloc(p, &d.pterm, (size_t)n_runs * n_pairs));
