@@ -73,7 +73,7 @@ class EpipolarLoss(torch.autograd.Function):
             R, grad = ctx.saved_tensors
         # (saved-tensor hooks may give back other devices, layouts and shapes than were saved)
         if (not torch.is_grad_enabled() and R.dtype == grad.dtype == grad_out.dtype == torch.float64
-                and R.is_cuda and grad_out.device == grad.device == R.device
+                and R.is_cuda and grad_out.get_device() == grad.get_device() == R.get_device()
                 and R.shape == (grad.shape[0], 3, 3) and grad.shape[1:] == (6,)
                 and R.is_contiguous() and grad.is_contiguous()
                 and _in_memory(R) and _in_memory(grad) and _in_memory(grad_out)):

@@ -293,14 +293,12 @@ class Problem:
         c = _host(c, np.float64)
         _check(load_library().fm_set_params(self._h, _ptr(R), _ptr(c)))
 
-    def _here(self, t) -> bool:
-        # the library's kernels read and write the caller's memory: it has to be the problem's device's
-        return t.is_cuda and t.get_device() == self._device
-
     def set_params_device(self, R, c):
         """Asynchronous parameter update from contiguous float64 CUDA tensors (N,3,3), (N,3). Tensors that are
         not on the problem's device are copied there."""
-        R, c = (v if self._here(v) else v.detach().to(f"cuda:{self._device}") for v in (R, c))
+        here = self._device     # kernels read the memory themselves (a tensor in host memory has device -1)
+        if R.get_device() != here or c.get_device() != here:
+            R, c = (v.detach().to(f"cuda:{here}") for v in (R, c))
         _check(load_library().fm_set_params_device(self._h, ctypes.c_void_p(R.data_ptr()),
                                                    ctypes.c_void_p(c.data_ptr())))
 
@@ -383,11 +381,12 @@ class Problem:
     def loss_grad_device(self, loss_out, grad_out):
         """Asynchronous loss/gradient into device tensors (float64, sizes 1 and n_cams*6). Results for tensors
         that are not on the problem's device are copied there."""
-        away = [t for t in (loss_out, grad_out) if t is not None and not self._here(t)]
-        if away:
+        here = self._device
+        if ((loss_out is not None and loss_out.get_device() != here)
+                or (grad_out is not None and grad_out.get_device() != here)):
             import torch
             with torch.no_grad():
-                near = [None if t is None else torch.empty_like(t, device=f"cuda:{self._device}") for t in (loss_out, grad_out)]
+                near = [None if t is None else torch.empty_like(t, device=f"cuda:{here}") for t in (loss_out, grad_out)]
                 self.loss_grad_device(*near)
                 for t, n in zip((loss_out, grad_out), near):
                     if t is not None:
