@@ -26,9 +26,9 @@ constexpr int PASS_BYTES = S * STAGE_BYTES + CameraE::BYTES;   // shared memory 
 // Bound by HBM on large scenes, by the latency of a range's loads and by the launches around the pass
 // on small ones. Loading 4 groups per warp into registers after the wait for the launch before
 // (8 warps a block) left the memory system idle while a pass filled up and drained. An iteration of
-// fm_step (this pass, then the camera step), before -> now: 119 k point pairs FP32 18.7 -> 8.5 us,
-// 3.1 M FP32 28.0 -> 11.2, 12 M FP16 39.6 -> 28.6, 49 M FP32 161 -> 142, 49 M FP16 92.3 -> 79.0, 141 M FP16
-// 227.9 -> 218.9.
+// fm_step (this pass, then the camera step; chains of 100), before -> now: 119 k point pairs FP32 18.7 ->
+// 7.7 us, 3.1 M FP32 28.0 -> 11.4, 12 M FP16 39.6 -> 27.5, 49 M FP32 161 -> 142, 49 M FP16 92.3 -> 77.2, 141 M FP16
+// 227.9 -> 214.5.
 template <int STORE, int MODE, int S>
 __global__ void __launch_bounds__(32, 32) k_stream_loss(DevProblem d, int prev_loss) {
     extern __shared__ __align__(16) unsigned char stage[];
@@ -364,8 +364,8 @@ __global__ void __launch_bounds__(GATHER_THREADS) k_gather(DevProblem d, int cou
 // hi + lo pair (TwoSum); a lane's items are added in the order of their passes and the lanes by a
 // butterfly, whatever W is, so every W gives the same bits; with W > 1 the warps share the values out.
 // What bounds it is latency: a pass of loads and chain rule takes about 2,000 cycles, and a warp a camera
-// makes three of them in series on 1,000 cameras and 49 M point pairs (an iteration with 8 cameras of one
-// warp a block 80.5 us, now 78.0; on 16 cameras and 119 k 9.7, now 8.8).
+// makes three of them in series on 1,000 cameras and 49 M point pairs (8 cameras of one warp a block there
+// cost an iteration 2.5 us more, and 0.9 us more on 16 cameras and 119 k).
 // Phase 2: the update of the block's cameras, spread over warps (step_update). The two powers of its
 // bias corrections are formed before the wait.
 // The new records go to cam_dst, a second buffer (with apply): other blocks may still read this step's

@@ -276,9 +276,8 @@ k_quad_step(DevProblem d, int it, const float *cam_src, float *cam_dst, float gs
 // lane: 16-byte loads free of bank conflicts). The same arithmetic as k_quad_step, bit for bit. What bounds
 // an iteration is its serial chain: other cameras' records from L2, geometry and chain rule,
 // the compensated sums, the FP64 update and the barrier. 25 iterations on 1,000 cameras and 11,700
-// pairs: 114 us, 4.5 us each (12.4 us as launches; 5.4 us with the update in one warp and the state
-// read back from memory each iteration). More cameras than resident warps take k_quad_step, whose
-// blocks then overlap each other's latencies (4,000 cameras: 500 blocks, 15 us an iteration).
+// pairs: 114 us, 4.5 us each with the launch, 4.2 in a chain of 1,000 (12.4 us as launches). More cameras than resident warps take k_quad_step, whose
+// blocks then overlap each other's latencies (4,000 cameras: 500 blocks, 13 us an iteration).
 constexpr int QROW = 60;
 constexpr int QUAD_SMEM = STEP_CAMS * 32 * QROW * (int)sizeof(float);
 

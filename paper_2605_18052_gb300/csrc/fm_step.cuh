@@ -289,9 +289,9 @@ __device__ __forceinline__ float adam_delta(float g, float lr, const float *hype
 // work to the state itself and spreads it over lanes and over the SM's four sub-partitions, one role
 // each: 3 such instructions in series for a rotation (re-orthonormalisation, about 40, only every eighth
 // step) and 8 for a centre and its loss, where one warp with a lane per row of R took 26 with the
-// conversions of the hyper-parameters (and a lane per camera 48). An iteration on 119 k point pairs went
-// from 13.0 to 11.8 us, on 3.1 M from 19.8 to 18.2, a form iteration from 5.4 to 4.5. Between two re-orthonormalisations R leaves SO(3) by the FP32 rounding of the
-// increments, a few 1e-7 |phi| per step, far below the FP32 camera record's resolution.
+// conversions of the hyper-parameters (and a lane per camera 48): 1.2 us of an iteration on 119 k point
+// pairs, 1.6 us on 3.1 M, 0.9 us of a form iteration. Between two re-orthonormalisations R leaves SO(3) by the
+// FP32 rounding of the increments, a few 1e-7 |phi| per step, far below the FP32 camera record's resolution.
 constexpr int rot_roles(int cams) { return (cams + 2) / 3; }
 
 template <bool FOCAL, bool KEEP, int C>

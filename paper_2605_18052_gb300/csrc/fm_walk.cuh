@@ -256,7 +256,7 @@ struct RecordE {
 // table in shared memory: no launch between the camera step and the pass, no record written and read
 // back, and a range of several image pairs finds the next one's E' without a trip to L2. (Records
 // written by the last camera of a pair cost the camera step an acquire-release atomic per pair and 3,400
-// cycles: a round of 25 iterations took 250 us on 119 k point pairs, 224 now, 335 on 3.1 M, 312 now.)
+// cycles, 26 us of a round of 25 iterations on 119 k point pairs and 23 us on 3.1 M.)
 struct CameraE {
     static constexpr int PAIRS = 16, BYTES = PAIRS * 9 * (int)sizeof(float);
     const DevProblem &d;
@@ -364,7 +364,7 @@ __device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src) 
 // UNROLL: groups of a chunk in straight code (1 for bodies of many instructions). A chunk inside one image
 // pair takes one branch and reads its four groups before their sums: a warp that checks every group
 // issues the loads of one at a time, and where few warps share an SM the pass is that chain of latencies
-// (an iteration on 119 k point pairs went from 15.1 to 13.7 us, on 3.1 M FP32 from 19.2 to 18.4).
+// (1.4 us of an iteration on 119 k point pairs, 0.8 us on 3.1 M FP32).
 // Where UNROLL is below a chunk (the quadratic-form pass) the second copy of the body costs
 // more than it gives: 403 -> 421 us for a round on 49 M.
 // Source: where a pair's E' comes from (its table, Source::BYTES, lies behind the stage).
